@@ -183,8 +183,8 @@ int saf_fit_marginals(saf_ctx* ctx, int32_t Hf, int32_t T, const float* mean_att
  * and installation": alpha = 0, rho(d) = log max(eta_rel(d)/(T-d), 1e-9), then `steps` Adam steps (beta1 0.9,
  * beta2 0.999, eps 1e-8, bias-corrected) at learning rate `lr` on
  * L = (1/T)[sum_i log Z(i) - sum_j eta_abs(j) alpha(j) - sum_d eta_rel(d) rho(d)]; the paper uses 400 steps at 0.05).
- * All heads are fitted together; nothing of size T x T is allocated (state: 68 bytes per head and position, held by
- * the context and reused).  Exponentials are fp32, the sums that feed Adam and Adam itself fp64.
+ * All heads are fitted together; nothing of size T x T is allocated (state: 56 bytes per head and position, held by
+ * the context and reused).  Exponentials and the terms of the sums are fp32, Adam and its state fp64.
  *   eta_abs, eta_rel : device float64 [Hf, T] (from saf_fit_marginals, or accumulated by the caller)
  *   plogp            : device float64 [Hf] or NULL if kl_out is NULL
  *   alpha_out, rho_out, logZ_out : device float32, row h at offset h*out_stride (out_stride >= T elements): the
@@ -193,7 +193,7 @@ int saf_fit_marginals(saf_ctx* ctx, int32_t Hf, int32_t T, const float* mean_att
  *   kl_out           : device float64 [Hf] or NULL: kappa = mean row KL(P || P^) = L + plogp/T; the paper accepts a
  *                      head when kappa <= 0.2 nats (the caller compares)
  * steps = 0 returns the starting point.  T <= 16384 (SAF_ERR_UNSUPPORTED beyond).  Asynchronous on `stream`
- * (2*steps + 3 kernel launches). */
+ * (one kernel launch). */
 int saf_fit_compact(saf_ctx* ctx, int32_t Hf, int32_t T, const double* eta_abs, const double* eta_rel,
                     const double* plogp, int32_t steps, double lr, float* alpha_out, float* rho_out, float* logZ_out,
                     int64_t out_stride, double* loss_out, double* kl_out, void* stream);

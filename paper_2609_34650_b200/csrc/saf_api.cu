@@ -1222,9 +1222,9 @@ int saf_fit_compact(saf_ctx* ctx, int32_t Hf, int32_t T, const double* eta_abs, 
   if (!g.ok) return SAF_ERR_CUDA;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   ctx->last_stream = st;
-  // state: 6 fp64 and 5 fp32 arrays of [Hf, T]
+  // state: 6 fp64 and 2 fp32 arrays of [Hf, T]
   const size_t n = static_cast<size_t>(Hf) * T;
-  int rc = ensure(ctx->fit_buf, n * (6 * sizeof(double) + 5 * sizeof(float)));
+  int rc = ensure(ctx->fit_buf, n * (6 * sizeof(double) + 2 * sizeof(float)));
   if (rc) return rc;
   FitState s;
   s.T = T;
@@ -1234,7 +1234,7 @@ int saf_fit_compact(saf_ctx* ctx, int32_t Hf, int32_t T, const double* eta_abs, 
   double* d = static_cast<double*>(ctx->fit_buf.ptr);
   s.alpha = d; s.rho = d + n; s.m_a = d + 2 * n; s.v_a = d + 3 * n; s.m_r = d + 4 * n; s.v_r = d + 5 * n;
   float* f = reinterpret_cast<float*>(d + 6 * n);
-  s.a2[0] = f; s.a2[1] = f + n; s.r2[0] = f + 2 * n; s.r2[1] = f + 3 * n; s.nz2 = f + 4 * n;
+  s.a2 = f; s.r2 = f + n;
   ScopedTimer timer(ctx, SAF_KERNEL_FIT, st);
   if (launch_fit(s, Hf, steps, plogp, alpha_out, rho_out, logZ_out, out_stride, loss_out, kl_out, st) != cudaSuccess)
     return SAF_ERR_CUDA;

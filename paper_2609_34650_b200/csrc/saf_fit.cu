@@ -8,16 +8,17 @@
 //              (fitted marginal - target marginal)/T
 //   accept     kappa = mean row KL(P || P^) = L + (1/T) sum P log P   (rows of P sum to one)
 //
-// Nothing of size T x T is formed after the target has been read once.  Every Adam step is two launches:
-//   pass A   rows:      S(i) = sum_{d<=i} exp2(r'(d) + a'(i-d) - z'(i)),  z'(i) += log2 S(i)
-//   pass B   marginals: c(j) = sum_d exp2(r'(d) - z'(j+d) + a'(j))  and  g(d) = sum_j exp2(a'(j) - z'(j+d) + r'(d)),
+// Nothing of size T x T is formed after the target has been read once.  The whole fit is ONE launch: a thread-block
+// cluster per head runs all Adam steps, exchanging vectors of length T through distributed shared memory (normalisers)
+// and L2 (parameters), with two cluster barriers per step:
+//   pass A   rows:      Z(i) = sum_{d<=i} R(d) A(i-d),  W(i) = 1 / Z(i)
+//   pass B   marginals: c(j) = A(j) sum_d R(d) W(j+d)  and  g(d) = R(d) sum_j A(j) W(j+d),
 //            followed in the same thread by the Adam update of alpha(j) / rho(d) (fp64 state)
-// (primes: scaled by log2 e; z' is log2 Z).  All three sums have the same shape
-//   out(x) = sum_y exp2(u[y] + win[x -/+ y] + c[x]),
-// one lane per x, the operand u uniform over the warp, the window operand contiguous over the lanes, so one kernel
-// serves them.  The reference point of the exponentials is the previous step's z' (one Adam step moves every
-// parameter by a fraction of a unit), so no running maximum is needed; the first pass starts from the upper bound
-// max r' (alpha = 0).  The special-function unit (one exp2 per causal pair and pass) bounds the kernel.
+// with A = exp(alpha), R = exp(rho) taken once per parameter and step: the pattern's factorisation turns the three sums
+// into causal convolutions / correlations, one fp32 multiply-add per causal pair and sum instead of an exponential.
+// All terms are positive, so the sums keep the relative accuracy of their terms.  The plain products cannot leave
+// fp32's range while every parameter and normaliser is inside the bounds below; a head that leaves them goes on in the
+// log form (one exp2 per pair, referred to the previous step's normaliser), in the same kernel.
 #include <cuda_runtime.h>
 #include <cstdint>
 #include <cmath>
@@ -30,10 +31,6 @@ namespace {
 
 constexpr double LOG2E_D = 1.4426950408889634074;
 constexpr double LN2_D = 0.6931471805599453094;
-constexpr int XB = 32;             // x values per CTA of the pass kernel (one per lane)
-constexpr int PASS_WARPS = 8;      // warps of a pass CTA; they split the y range in chunks of 32
-constexpr int YC = 4096;           // y values staged in shared memory at a time
-
 __device__ __forceinline__ float ex2f(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -163,159 +160,415 @@ saf_fit_marginals_kernel(const float* __restrict__ Abar, float floor_v, double* 
 }
 #undef SAF_MARG_DISPATCH
 
-// ------------------------------------------------------------------------------------------------ Fit: start
-// One CTA per head: alpha = 0, rho(d) = log max(eta_rel(d)/(T-d), 1e-9), Adam moments zero, and the first
-// reference point of the exponentials: every row starts from the upper bound max_d r'(d) (alpha = 0).
-__global__ void __launch_bounds__(256)
-saf_fit_init_kernel(FitState s) {
-  __shared__ float redm[8];
-  const int h = blockIdx.x, tid = threadIdx.x, T = s.T;
+// ------------------------------------------------------------------------------------------------ Fit
+constexpr int FX = 256;            // x values of a block: 8 consecutive ones per lane
+constexpr int FPAD = 288;          // floats kept neutral in front of A and behind A, R and W
+// Bounds (log2) inside which the product form is used: every factor and product of two stays within 2^+-120, sums of
+// 16384 of them below 2^127, so nothing overflows and nothing is flushed.
+constexpr float A_LO = -50.0f, A_HI = 50.0f, R_LO = -70.0f, R_HI = 50.0f;
+constexpr float Z_LO = 8.6736174e-19f, Z_HI = 1.1258999e15f;      // 2^-60, 2^50
+
+__device__ __forceinline__ uint32_t smem_addr(const void* p) {
+  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
+}
+__device__ __forceinline__ uint32_t cluster_addr(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void st_cluster_f32(uint32_t addr, float v) {
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
+}
+__device__ __forceinline__ void st_cluster_f64(uint32_t addr, double v) {
+  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(addr), "d"(v) : "memory");
+}
+__device__ __forceinline__ void cluster_sync_all() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// 2^x of an fp64 exponent: the integer part goes into the exponent field, so the fp32 exponential sees |f| <= 1/2.
+__device__ __forceinline__ float exp2_split(double x) {
+  const double k = rint(x);
+  return ldexpf(ex2f(static_cast<float>(x - k)), static_cast<int>(k));
+}
+
+// Layout of a vector in shared memory.  A lane reads 8 consecutive values plus a sliding window in 16-byte pieces, so
+// lanes are 32 bytes apart: PADDED inserts 16 bytes after every 32, which makes those reads conflict-free (lanes 48
+// bytes apart) and keeps the pieces at constant offsets.  Indices of a piece: a multiple of 4.
+template <bool PADDED>
+__device__ __forceinline__ int fit_phys(int i) { return PADDED ? i + ((i >> 3) << 2) : i; }
+template <bool PADDED>
+__device__ __forceinline__ constexpr int fit_off(int d) { return PADDED ? d + (d >= 0 ? (d >> 3) : -((7 - d) >> 3)) * 4 : d; }
+
+__device__ __forceinline__ void ld4(const float* p, float* v) {
+  const float4 t = *reinterpret_cast<const float4*>(p);
+  v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+}
+
+// acc[k] += sum over y in [y0, y1) of u(y) * w(x + k -/+ y) for this lane's x .. x+7 (MODE 0: minus, with one u; MODE 1:
+// plus, with two u and two accumulators).  y0, y1: multiples of 16; xl = the lane's x (a multiple of 8).  Per 16 values
+// of y: 4 window pieces and 4 (8) uniform pieces for 128 (256) multiply-adds.  LOG: the vectors hold logarithms and a
+// term is 2^(u + w + c).
+template <int MODE, bool PADDED, bool LOG>
+__device__ __forceinline__ void fit_accumulate(const float* __restrict__ u0, const float* __restrict__ u1,
+                                               const float* __restrict__ w, int xl, int y0, int y1, const float* c0,
+                                               const float* c1, float* acc0, float* acc1) {
+  float win[24];
+  const float* wp = w + fit_phys<PADDED>(MODE == 0 ? xl - y0 : xl + y0);
+  if (y0 < y1) {
+    // the two pieces that consecutive steps share
+    ld4(wp + fit_off<PADDED>(0), MODE == 0 ? win + 16 : win);
+    ld4(wp + fit_off<PADDED>(4), MODE == 0 ? win + 20 : win + 4);
+  }
+  for (int ye = y0; ye < y1;) {
+    // (pieces of 512 values of y are summed on their own, so that no chain of fp32 additions gets long)
+    const int yb = ye;
+    ye = min(y1, yb + 512);
+    float s0[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f}, s1[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll 2
+    for (int y = yb; y < ye; y += 16) {
+      if (MODE == 0) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) ld4(wp + fit_off<PADDED>(-16 + 4 * q), win + 4 * q);
+      } else {
+#pragma unroll
+        for (int q = 2; q < 6; ++q) ld4(wp + fit_off<PADDED>(4 * q), win + 4 * q);
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        float a[4], b[4];
+        ld4(u0 + y + 4 * q, a);
+        if (MODE == 1) ld4(u1 + fit_phys<PADDED>(y) + fit_off<PADDED>(4 * q), b);
+#pragma unroll
+        for (int t = 0; t < 4; ++t)
+#pragma unroll
+          for (int k = 0; k < 8; ++k) {
+            const float wv = win[MODE == 0 ? 16 + k - (4 * q + t) : k + 4 * q + t];
+            if (LOG) {
+              s0[k] += ex2f((a[t] + c0[k]) + wv);
+              if (MODE == 1) s1[k] += ex2f((b[t] + c1[k]) + wv);
+            } else {
+              s0[k] = fmaf(a[t], wv, s0[k]);
+              if (MODE == 1) s1[k] = fmaf(b[t], wv, s1[k]);
+            }
+          }
+      }
+      if (MODE == 0) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) win[16 + k] = win[k];
+      } else {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) win[k] = win[16 + k];
+      }
+      wp += (MODE == 0 ? -1 : 1) * (PADDED ? 24 : 16);
+    }
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      acc0[k] += s0[k];
+      if (MODE == 1) acc1[k] += s1[k];
+    }
+  }
+}
+
+// The x blocks of 256 that a CTA owns in one pass and the segments its NW warps work on.  The 16-wide y chunks of the
+// CTA's blocks are numbered through (in rounds of RB blocks) and split evenly over the warps; warp w's part of block b
+// goes to slot w + b of the partial sums (both only ever move up, so no two segments meet in a slot).
+struct FitPlan {
+  int count;                                     // blocks
+  int total[64];                                 // chunks of round r
+  short xb[64], first[64], n[64];                // block number, first chunk within its round, chunks
+  signed char lo[64], hi[64];                    // warps whose segments touch the block
+};
+
+// One cluster = one head.  A head's x blocks go to the cluster's CTAs in snake order by descending work.  Bound: fp32
+// multiply-adds (128 per clock and SM), 1.5 T^2 per head and step.  Measured (36 heads, T = 4096, 400 steps): 22.3 ms =
+// 55 us per step on 108 SMs, against 100.2 ms for one exponential per pair and sum in two launches per step; the inner
+// loops run at 76 % of the multiply-add peak (148 heads: 64 % over everything).  One head of 256 positions: 5.4 us per
+// step (two cluster barriers, L2 round trips of the parameters, fp64 Adam).
+template <int NW, bool PADDED, int RB>
+__global__ void __launch_bounds__(NW * 32, 1)
+saf_fit_kernel(FitState s, int steps, const double* __restrict__ plogp, float* __restrict__ alpha_out,
+               float* __restrict__ rho_out, float* __restrict__ logZ_out, long long out_stride,
+               double* __restrict__ loss_out, double* __restrict__ kl_out) {
+  extern __shared__ float4 sm_f4[];
+  constexpr int NT = NW * 32;
+  // a parameter (set in pass B, read after its barrier) or a normaliser (pass A) of this head has left the bounds
+  __shared__ int out_par, out_z;
+  __shared__ double redd[NW], part_loss[16];
+  __shared__ float redf[NW];
+  __shared__ FitPlan plan[2];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, T = s.T;
+  uint32_t cs, rank;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(cs));
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+  const int h = blockIdx.x / cs;
   const size_t o = static_cast<size_t>(h) * T;
+  const int Tr = (T + 15) & ~15;
+  const int nA = fit_phys<PADDED>(FPAD + Tr + FPAD), nW = fit_phys<PADDED>(Tr + FPAD);
+  float* Abase = reinterpret_cast<float*>(sm_f4);
+  float* A = Abase + fit_phys<PADDED>(FPAD);     // A[-FPAD .. Tr+FPAD)
+  float* W = Abase + nA;                         // W[0 .. Tr+FPAD)
+  float* R = W + nW;                             // R[0 .. Tr+FPAD), unpadded
+  float* part = R + Tr + FPAD;                   // [NW + RB][2][FX] partial sums
+  const int nxb = (T + FX - 1) / FX;
+  bool slow = false;
+
+  if (tid < 2) {                                 // plan[0]: pass A, plan[1]: pass B
+    FitPlan& p = plan[tid];
+    int cnt = 0;
+    for (int k = 0; k < nxb; ++k) {              // k: blocks in descending order of work
+      const int r = k / static_cast<int>(cs), i = k % static_cast<int>(cs);
+      if (((r & 1) ? static_cast<int>(cs) - 1 - i : i) != static_cast<int>(rank)) continue;
+      const int xb = tid == 0 ? nxb - 1 - k : k;
+      p.xb[cnt] = static_cast<short>(xb);
+      p.n[cnt] = static_cast<short>(((tid == 0 ? min(T, (xb + 1) * FX) : T - xb * FX) + 15) >> 4);
+      ++cnt;
+    }
+    p.count = cnt;
+    for (int i0 = 0, r = 0; i0 < cnt; i0 += RB, ++r) {
+      const int i1 = min(cnt, i0 + RB);
+      int tot = 0;
+      for (int i = i0; i < i1; ++i) {
+        p.first[i] = static_cast<short>(tot);
+        tot += p.n[i];
+      }
+      p.total[r] = tot;
+      for (int i = i0; i < i1; ++i) {
+        int lo = 0, hi = NW - 1;
+        while ((lo + 1) * tot / NW <= p.first[i]) ++lo;
+        while (hi * tot / NW >= p.first[i] + p.n[i]) --hi;
+        p.lo[i] = static_cast<signed char>(lo);
+        p.hi[i] = static_cast<signed char>(hi);
+      }
+    }
+  }
+  // neutral elements around the vectors
+  auto fill_pads = [&](float v) {
+    for (int i = tid; i < FPAD; i += NT) A[fit_phys<PADDED>(i - FPAD)] = v;
+    for (int i = T + tid; i < Tr + FPAD; i += NT) {
+      A[fit_phys<PADDED>(i)] = v;
+      W[fit_phys<PADDED>(i)] = v;
+      R[i] = v;
+    }
+  };
+  // to the log form: parameters from their fp64 values, normalisers as they stand (any nearby reference will do)
+  auto go_slow = [&]() {
+    slow = true;
+    fill_pads(-INFINITY);
+    for (int i = tid; i < T; i += NT) {
+      A[fit_phys<PADDED>(i)] = static_cast<float>(__ldcg(s.alpha + o + i) * LOG2E_D);
+      R[i] = static_cast<float>(__ldcg(s.rho + o + i) * LOG2E_D);
+      W[fit_phys<PADDED>(i)] = __log2f(W[fit_phys<PADDED>(i)]);
+    }
+    cluster_sync_all();                          // nobody's next normalisers may arrive before this is done
+  };
+  auto raise_flag = [&](int* flag) {
+    const uint32_t a = smem_addr(flag);
+    for (uint32_t r = 0; r < cs; ++r)
+      asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(cluster_addr(a, r)), "r"(1) : "memory");
+  };
+
+  // ---- start: alpha = 0, rho(d) = log max(eta_rel(d)/(T-d), 1e-9), Adam moments zero, and a first reference for the
+  // normalisers: the upper bound max rho (alpha = 0)
+  if (tid == 0) out_par = out_z = 0;
   float mx = -INFINITY;
-  for (int d = tid; d < T; d += 256) {
+  bool bad = false;
+  for (int d = tid; d < T; d += NT) {
     const double r = log(fmax(s.eta_rel[o + d] / static_cast<double>(T - d), 1e-9));
-    s.rho[o + d] = r;
-    s.alpha[o + d] = 0.0;
-    s.m_a[o + d] = 0.0; s.v_a[o + d] = 0.0; s.m_r[o + d] = 0.0; s.v_r[o + d] = 0.0;
     const float r2 = static_cast<float>(r * LOG2E_D);
-    s.r2[0][o + d] = r2;
-    s.a2[0][o + d] = 0.0f;
     mx = fmaxf(mx, r2);
+    if (!(r2 >= R_LO && r2 <= R_HI)) bad = true;
+    R[d] = exp2_split(r * LOG2E_D);
+    A[fit_phys<PADDED>(d)] = 1.0f;
+    // (each block's state is written and later read by its owner in pass B only, except for the fp64 parameters)
+    const int k = d / FX, kr = k / static_cast<int>(cs), ki = k % static_cast<int>(cs);
+    if (((kr & 1) ? static_cast<int>(cs) - 1 - ki : ki) == static_cast<int>(rank)) {
+      s.rho[o + d] = r;
+      s.alpha[o + d] = 0.0;
+      s.m_a[o + d] = 0.0; s.v_a[o + d] = 0.0; s.m_r[o + d] = 0.0; s.v_r[o + d] = 0.0;
+    }
   }
 #pragma unroll
   for (int k = 16; k > 0; k >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, k));
-  if ((tid & 31) == 0) redm[tid >> 5] = mx;
-  __syncthreads();
-  mx = redm[0];
+  if (lane == 0) redf[warp] = mx;
+  bad = __syncthreads_or(bad);
+  mx = redf[0];
 #pragma unroll
-  for (int w = 1; w < 8; ++w) mx = fmaxf(mx, redm[w]);
-  for (int i = tid; i < T; i += 256) s.nz2[o + i] = -mx;
-}
+  for (int w = 1; w < NW; ++w) mx = fmaxf(mx, redf[w]);
+  fill_pads(0.0f);
+  for (int i = tid; i < T; i += NT) W[fit_phys<PADDED>(i)] = bad ? -mx : ex2f(-mx);
+  cluster_sync_all();
+  if (bad) {                                     // (the same decision in every CTA of the cluster)
+    go_slow();
+    for (int i = tid; i < T; i += NT) W[fit_phys<PADDED>(i)] = -mx;
+    cluster_sync_all();
+  }
 
-// ------------------------------------------------------------------------------------------------ Fit: the passes
-// MODE 0 (pass A): x = query i, y = distance d <= i:   u = r', window = a'[i-d],  c = -z'(i)   -> z'(i) += log2 S
-// MODE 1 (pass B): blockIdx.z = 0: x = key j, y = d <= T-1-j:  u = r', window = -z'[j+d], c = a'(j) -> Adam on alpha(j)
-//                  blockIdx.z = 1: x = d,     y = j <= T-1-d:  u = a', window = -z'[d+j], c = r'(d) -> Adam on rho(d)
-// CTA = 32 consecutive x (one per lane) x 8 warps that take the 32-wide chunks of y in turn.  Both operands are
-// staged in shared memory, 4096 values of y at a time; window entries outside the causal range are -inf, which is the
-// mask.
-template <int MODE>
-__global__ void __launch_bounds__(PASS_WARPS * 32)
-saf_fit_pass_kernel(FitState s, int cur, double bc1, double bc2) {
-  extern __shared__ float sm_f[];
-  const int T = s.T;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int h = blockIdx.y;
-  const size_t o = static_cast<size_t>(h) * T;
-  const int nxb = (T + XB - 1) / XB;
-  // the longest blocks first: pass A's work grows with x, pass B's shrinks
-  const int xb = (MODE == 0) ? nxb - 1 - static_cast<int>(blockIdx.x) : static_cast<int>(blockIdx.x);
-  const int x0 = xb * XB;
-  const int which = (MODE == 0) ? 0 : static_cast<int>(blockIdx.z);
-  const int ny = (MODE == 0) ? min(T, x0 + XB) : T - x0;          // y = 0 .. ny-1 covers every lane's range
-  const int nyp = (ny + 31) & ~31;
-  const int ycap = min(YC, (T + 31) & ~31);
-  float* us = sm_f;                       // [ycap]
-  float* ws = sm_f + ycap;                // [ycap + 32]
-  const float* a2c = cur ? s.a2[1] : s.a2[0];
-  const float* r2c = cur ? s.r2[1] : s.r2[0];
-  const float* u_g = (MODE == 1 && which == 1) ? a2c + o : r2c + o;
-  const float* w_g = (MODE == 0) ? a2c + o : s.nz2 + o;
-  const int x = x0 + lane;
-  float c = -INFINITY;
-  if (x < T) c = (MODE == 0) ? s.nz2[o + x] : (which == 0 ? a2c[o + x] : r2c[o + x]);
-  float acc0 = 0.0f, acc1 = 0.0f;
-  // the y range in chunks of YC: shared memory per CTA stays at 33 KB whatever T is (six CTAs per SM)
-  for (int yb = 0; yb < nyp; yb += YC) {
-    const int nyc = min(YC, nyp - yb);                 // a multiple of 32
-    if (yb > 0) __syncthreads();                       // the previous chunk has been read
-    for (int y = tid; y < nyc; y += PASS_WARPS * 32) us[y] = (yb + y < ny) ? u_g[yb + y] : -INFINITY;
-    if (MODE == 0) {
-      // lane x at distance y reads a'[x - y]: the chunk's window starts at g0 = x0 - (yb + nyc - 1), and
-      // ws[k] = a'[g0 + k] (-inf below index 0); the lane's entry for y is ws[lane + (yb + nyc - 1 - y)]
-      const int g0 = x0 - (yb + nyc - 1);
-      for (int k = tid; k < nyc + 32; k += PASS_WARPS * 32) {
-        const int g = g0 + k;
-        ws[k] = (g >= 0 && g < ny) ? w_g[g] : -INFINITY;
-      }
-    } else {
-      // lane x at offset y reads -z'[x + y]: ws[k] = -z'[x0 + yb + k] (-inf beyond T); the lane's entry is
-      // ws[lane + (y - yb)]
-      for (int k = tid; k < nyc + 32; k += PASS_WARPS * 32) ws[k] = (x0 + yb + k < T) ? w_g[x0 + yb + k] : -INFINITY;
-    }
-    __syncthreads();
-    for (int y0 = warp * 32; y0 < nyc; y0 += PASS_WARPS * 32) {
-      const float4* u4 = reinterpret_cast<const float4*>(us + y0);
-      const float* wp = (MODE == 0) ? ws + (lane + nyc - 1 - y0) : ws + (lane + y0);
+  double acc = 0.0;                              // this thread's part of T * loss
+  // pass A over this CTA's blocks; `last`: the normalisers of the final parameters (results are written)
+  auto pass_a = [&](bool last) {
+    const FitPlan& p = plan[0];
+    for (int i0 = 0, rd = 0; i0 < p.count; i0 += RB, ++rd) {
+      const int nb = min(RB, p.count - i0), tot = p.total[rd];
+      const int k0 = warp * tot / NW, k1 = (warp + 1) * tot / NW;
+      if (i0 > 0) __syncthreads();
+      for (int b = 0; b < nb; ++b) {
+        const int first = p.first[i0 + b];
+        const int y0 = (max(k0, first) - first) << 4, y1 = (min(k1, first + p.n[i0 + b]) - first) << 4;
+        if (warp < p.lo[i0 + b] || warp > p.hi[i0 + b]) continue;   // (a warp without chunks in between adds zeros)
+        const int xl = p.xb[i0 + b] * FX + 8 * lane;
+        float a8[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+        if (!slow) {
+          fit_accumulate<0, PADDED, false>(R, nullptr, A, xl, y0, y1, nullptr, nullptr, a8, nullptr);
+        } else {
+          float c8[8];
 #pragma unroll
-      for (int t4 = 0; t4 < 8; ++t4) {
-        const float4 u = u4[t4];
-        const int t = 4 * t4;
-        const float w0 = (MODE == 0) ? wp[-t] : wp[t];
-        const float w1 = (MODE == 0) ? wp[-t - 1] : wp[t + 1];
-        const float w2 = (MODE == 0) ? wp[-t - 2] : wp[t + 2];
-        const float w3 = (MODE == 0) ? wp[-t - 3] : wp[t + 3];
-        acc0 += ex2f((u.x + c) + w0);
-        acc1 += ex2f((u.y + c) + w1);
-        acc0 += ex2f((u.z + c) + w2);
-        acc1 += ex2f((u.w + c) + w3);
+          for (int q = 0; q < 8; ++q) c8[q] = xl + q < T ? W[fit_phys<PADDED>(xl + q)] : -INFINITY;
+          fit_accumulate<0, PADDED, true>(R, nullptr, A, xl, y0, y1, c8, nullptr, a8, nullptr);
+        }
+        float4* dst = reinterpret_cast<float4*>(part + (warp + b) * 2 * FX + 8 * lane);
+        dst[0] = make_float4(a8[0], a8[1], a8[2], a8[3]);
+        dst[1] = make_float4(a8[4], a8[5], a8[6], a8[7]);
+      }
+      __syncthreads();
+      for (int q = tid; q < nb * FX; q += NT) {
+        const int b = q / FX, i = i0 + b, x = p.xb[i] * FX + (q & (FX - 1));
+        if (x >= T) continue;
+        float S = 0.0f;
+#pragma unroll 4
+        for (int w = p.lo[i]; w <= p.hi[i]; ++w) S += part[(w + b) * 2 * FX + (q & (FX - 1))];
+        float* slot = W + fit_phys<PADDED>(x);
+        float out;
+        double lz;
+        bool in = true;
+        if (slow) {
+          out = *slot - __log2f(S);
+          lz = -static_cast<double>(out) * LN2_D;
+        } else {
+          in = S >= Z_LO && S <= Z_HI;
+          out = 1.0f / S;
+          lz = last ? log(static_cast<double>(S)) : 0.0;
+        }
+        if (in) {
+          const uint32_t a = smem_addr(slot);
+          for (uint32_t r = 0; r < cs; ++r) st_cluster_f32(cluster_addr(a, r), out);
+        } else {
+          raise_flag(&out_z);
+        }
+        if (last) {
+          logZ_out[static_cast<size_t>(h) * out_stride + x] = static_cast<float>(lz);
+          if (slow || in) acc += lz;
+        }
       }
     }
-  }
-  __shared__ float red[PASS_WARPS][32];
-  red[warp][lane] = acc0 + acc1;
-  __syncthreads();
-  if (warp != 0 || x >= T) return;
-  float S = 0.0f;
-#pragma unroll
-  for (int w = 0; w < PASS_WARPS; ++w) S += red[w][lane];
-  if (MODE == 0) {
-    s.nz2[o + x] = c - __log2f(S);
-  } else {
-    // gradient of Eq. "fit-objective": (fitted marginal - target marginal) / T, then one Adam step in fp64
-    const double eta = (which == 0) ? s.eta_abs[o + x] : s.eta_rel[o + x];
-    double* par = (which == 0) ? s.alpha : s.rho;
-    double* mm = (which == 0) ? s.m_a : s.m_r;
-    double* vv = (which == 0) ? s.v_a : s.v_r;
-    const double g = (static_cast<double>(S) - eta) / static_cast<double>(T);
-    const double m = 0.9 * mm[o + x] + 0.1 * g;
-    const double v = 0.999 * vv[o + x] + 0.001 * g * g;
-    mm[o + x] = m;
-    vv[o + x] = v;
-    const double pnew = par[o + x] - s.lr * (m / bc1) / (sqrt(v / bc2) + 1e-8);
-    par[o + x] = pnew;
-    float* dst = (which == 0) ? (cur ? s.a2[0] : s.a2[1]) : (cur ? s.r2[0] : s.r2[1]);
-    dst[o + x] = static_cast<float>(pnew * LOG2E_D);
-  }
-}
+    cluster_sync_all();
+  };
 
-// ------------------------------------------------------------------------------------------------ Fit: results
-// One CTA per head, fp64: L = (1/T)[sum_i log Z(i) - eta_abs.alpha - eta_rel.rho], kappa = L + (1/T) sum P log P,
-// and the fp32 copies of alpha, rho, log Z that the attention kernels take.
-__global__ void __launch_bounds__(256)
-saf_fit_final_kernel(FitState s, const double* __restrict__ plogp, float* __restrict__ alpha_out,
-                     float* __restrict__ rho_out, float* __restrict__ logZ_out, long long out_stride,
-                     double* __restrict__ loss_out, double* __restrict__ kl_out) {
-  __shared__ double redd[8];
-  const int h = blockIdx.x, tid = threadIdx.x, T = s.T;
-  const size_t o = static_cast<size_t>(h) * T;
+  double p1 = 1.0, p2 = 1.0;
+  for (int t = 1; t <= steps + 1; ++t) {
+    const bool last = t == steps + 1;
+    if (t > 1) {
+      // the parameters of this step, from the owners of their blocks
+      if (!slow && out_par) {
+        go_slow();
+      } else {
+        for (int i = tid; i < T; i += NT) {
+          A[fit_phys<PADDED>(i)] = __ldcg(s.a2 + o + i);
+          R[i] = __ldcg(s.r2 + o + i);
+        }
+        __syncthreads();
+      }
+    }
+    pass_a(last);
+    if (!slow && out_z) {
+      acc = 0.0;
+      go_slow();
+      pass_a(last);
+    }
+    if (last) break;
+    p1 *= 0.9;
+    p2 *= 0.999;
+    const double ib1 = 1.0 / (1.0 - p1), ib2 = 1.0 / (1.0 - p2), iT = 1.0 / static_cast<double>(T);
+    const FitPlan& p = plan[1];
+    for (int i0 = 0, rd = 0; i0 < p.count; i0 += RB, ++rd) {
+      const int nb = min(RB, p.count - i0), tot = p.total[rd];
+      const int k0 = warp * tot / NW, k1 = (warp + 1) * tot / NW;
+      if (i0 > 0) __syncthreads();
+      for (int b = 0; b < nb; ++b) {
+        const int first = p.first[i0 + b];
+        const int y0 = (max(k0, first) - first) << 4, y1 = (min(k1, first + p.n[i0 + b]) - first) << 4;
+        if (warp < p.lo[i0 + b] || warp > p.hi[i0 + b]) continue;   // (a warp without chunks in between adds zeros)
+        const int xl = p.xb[i0 + b] * FX + 8 * lane;
+        float c8[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f}, g8[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+        if (!slow) {
+          fit_accumulate<1, PADDED, false>(R, A, W, xl, y0, y1, nullptr, nullptr, c8, g8);
+        } else {
+          float ca[8], cr[8];
+#pragma unroll
+          for (int q = 0; q < 8; ++q) {
+            ca[q] = A[fit_phys<PADDED>(xl + q)];
+            cr[q] = R[xl + q];
+          }
+          fit_accumulate<1, PADDED, true>(R, A, W, xl, y0, y1, ca, cr, c8, g8);
+        }
+        float4* dst = reinterpret_cast<float4*>(part + (warp + b) * 2 * FX + 8 * lane);
+        dst[0] = make_float4(c8[0], c8[1], c8[2], c8[3]);
+        dst[1] = make_float4(c8[4], c8[5], c8[6], c8[7]);
+        dst[FX / 4] = make_float4(g8[0], g8[1], g8[2], g8[3]);
+        dst[FX / 4 + 1] = make_float4(g8[4], g8[5], g8[6], g8[7]);
+      }
+      __syncthreads();
+      // one Adam step in fp64 on Eq. "fit-objective": gradient = (fitted marginal - target marginal) / T
+#pragma unroll 2
+      for (int q = tid; q < nb * 2 * FX; q += NT) {
+        const int b = q / (2 * FX), i = i0 + b, x = p.xb[i] * FX + (q & (FX - 1));
+        const bool is_rho = (q & FX) != 0;
+        if (x >= T) continue;
+        double* par = (is_rho ? s.rho : s.alpha) + o + x;
+        double* mm = (is_rho ? s.m_r : s.m_a) + o + x;
+        double* vv = (is_rho ? s.v_r : s.v_a) + o + x;
+        const double eta = (is_rho ? s.eta_rel : s.eta_abs)[o + x];
+        const double m0 = *mm, v0 = *vv, x_old = *par;
+        float S = 0.0f;
+#pragma unroll 4
+        for (int w = p.lo[i]; w <= p.hi[i]; ++w) S += part[(w + b) * 2 * FX + (q & (2 * FX - 1))];
+        if (!slow) S *= is_rho ? R[x] : A[fit_phys<PADDED>(x)];
+        const double g = (static_cast<double>(S) - eta) * iT;
+        const double m = 0.9 * m0 + 0.1 * g;
+        const double v = 0.999 * v0 + 0.001 * g * g;
+        *mm = m;
+        *vv = v;
+        const double pnew = x_old - s.lr * (m * ib1) / (sqrt(v * ib2) + 1e-8);
+        *par = pnew;
+        const double e = pnew * LOG2E_D;
+        (is_rho ? s.r2 : s.a2)[o + x] = slow ? static_cast<float>(e) : exp2_split(e);
+        if (!slow && !(e >= (is_rho ? R_LO : A_LO) && e <= (is_rho ? R_HI : A_HI))) raise_flag(&out_par);
+      }
+    }
+    cluster_sync_all();
+  }
+
+  // ---- results: L = (1/T)[sum_i log Z(i) - eta_abs.alpha - eta_rel.rho], kappa = L + (1/T) sum P log P
   const size_t oo = static_cast<size_t>(h) * static_cast<size_t>(out_stride);
-  double acc = 0.0;
-  for (int k = tid; k < T; k += 256) {
-    const double a = s.alpha[o + k], r = s.rho[o + k];
-    const double lz = -static_cast<double>(s.nz2[o + k]) * LN2_D;
-    acc += lz - s.eta_abs[o + k] * a - s.eta_rel[o + k] * r;
+  for (int k = static_cast<int>(rank) * NT + tid; k < T; k += static_cast<int>(cs) * NT) {
+    const double a = __ldcg(s.alpha + o + k), r = __ldcg(s.rho + o + k);
+    acc -= s.eta_abs[o + k] * a + s.eta_rel[o + k] * r;
     alpha_out[oo + k] = static_cast<float>(a);
     rho_out[oo + k] = static_cast<float>(r);
-    logZ_out[oo + k] = static_cast<float>(lz);
   }
 #pragma unroll
   for (int k = 16; k > 0; k >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, k);
-  if ((tid & 31) == 0) redd[tid >> 5] = acc;
+  if (lane == 0) redd[warp] = acc;
   __syncthreads();
   if (tid == 0) {
     double t = 0.0;
-    for (int w = 0; w < 8; ++w) t += redd[w];
+    for (int w = 0; w < NW; ++w) t += redd[w];
+    st_cluster_f64(cluster_addr(smem_addr(part_loss + rank), 0), t);
+  }
+  cluster_sync_all();
+  if (rank == 0 && tid == 0) {
+    double t = 0.0;
+    for (uint32_t r = 0; r < cs; ++r) t += part_loss[r];
     const double loss = t / static_cast<double>(T);
     if (loss_out) loss_out[h] = loss;
     if (kl_out) kl_out[h] = loss + plogp[h] / static_cast<double>(T);
@@ -356,31 +609,67 @@ cudaError_t launch_fit_marginals(const float* Abar, float floor_v, double* eta_a
   return cudaGetLastError();
 }
 
+namespace {
+
+template <int NW, bool PADDED, int RB>
+size_t fit_smem(int T) {
+  const size_t Tr = (T + 15) & ~15;
+  auto ph = [](size_t i) { return PADDED ? i + ((i >> 3) << 2) : i; };
+  return (ph(2 * FPAD + Tr) + ph(Tr + FPAD) + Tr + FPAD + 2 * (NW + RB) * FX) * sizeof(float);
+}
+
+template <int NW, bool PADDED, int RB, typename... Args>
+cudaError_t launch_fit_clusters(const FitState& s, int Hf, cudaStream_t st, Args... args) {
+  auto kern = saf_fit_kernel<NW, PADDED, RB>;
+  const size_t smem = fit_smem<NW, PADDED, RB>(s.T);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.blockDim = dim3(NW * 32);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  // Cluster size: the shortest of (waves of clusters) x (a head's multiply-adds over its CTAs + a fixed cost per step).
+  // Clusters stay inside a GPC, so fewer than 148 / size fit at once (measured with one CTA per SM: 74 of two, 45 of
+  // three, 33 of four, 26 of five, 22 of six, 15 of eight): 36 heads run faster on three CTAs each, in one wave, than
+  // on four.
+  const int nxb = (s.T + FX - 1) / FX;
+  double best = 0.0;
+  int best_cs = 0;
+  for (int cs = 1; cs <= std::min(8, nxb); ++cs) {
+    attr[0].val.clusterDim.x = cs;
+    cfg.gridDim = dim3(static_cast<unsigned>(Hf) * cs);
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess || n < 1) {
+      cudaGetLastError();
+      continue;
+    }
+    const double waves = (Hf + n - 1) / n;
+    const double cost = waves * (1.5 * s.T * static_cast<double>(s.T) / 128.0 / cs + 5000.0);
+    if (best_cs == 0 || cost < best) {
+      best = cost;
+      best_cs = cs;
+    }
+  }
+  if (best_cs == 0) return cudaErrorInvalidConfiguration;
+  attr[0].val.clusterDim.x = best_cs;
+  cfg.gridDim = dim3(static_cast<unsigned>(Hf) * best_cs);
+  return cudaLaunchKernelEx(&cfg, kern, s, args...);
+}
+
+}  // namespace
+
 cudaError_t launch_fit(const FitState& s, int Hf, int steps, const double* plogp, float* alpha_out, float* rho_out,
                        float* logZ_out, long long out_stride, double* loss_out, double* kl_out, cudaStream_t st) {
-  const int T = s.T;
-  const int nxb = (T + XB - 1) / XB;
-  const size_t smem = (2 * static_cast<size_t>(std::min((T + 31) & ~31, YC)) + 32) * sizeof(float);
-  cudaError_t e;
-  if ((e = cudaFuncSetAttribute(saf_fit_pass_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                static_cast<int>(smem))) != cudaSuccess)
-    return e;
-  if ((e = cudaFuncSetAttribute(saf_fit_pass_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                static_cast<int>(smem))) != cudaSuccess)
-    return e;
-  saf_fit_init_kernel<<<Hf, 256, 0, st>>>(s);
-  int cur = 0;
-  double p1 = 1.0, p2 = 1.0;
-  for (int t = 1; t <= steps; ++t) {
-    p1 *= 0.9;
-    p2 *= 0.999;
-    saf_fit_pass_kernel<0><<<dim3(nxb, Hf, 1), PASS_WARPS * 32, smem, st>>>(s, cur, 1.0, 1.0);
-    saf_fit_pass_kernel<1><<<dim3(nxb, Hf, 2), PASS_WARPS * 32, smem, st>>>(s, cur, 1.0 - p1, 1.0 - p2);
-    cur ^= 1;
-  }
-  saf_fit_pass_kernel<0><<<dim3(nxb, Hf, 1), PASS_WARPS * 32, smem, st>>>(s, cur, 1.0, 1.0);
-  saf_fit_final_kernel<<<Hf, 256, 0, st>>>(s, plogp, alpha_out, rho_out, logZ_out, out_stride, loss_out, kl_out);
-  return cudaGetLastError();
+  // up to 8192 positions the padded vectors fit beside the partial sums of 16 warps; the longest sequences keep them
+  // unpadded (two-way bank conflicts on the window reads) and run 8 warps
+  if (s.T <= 8192)
+    return launch_fit_clusters<16, true, 16>(s, Hf, st, steps, plogp, alpha_out, rho_out, logZ_out, out_stride, loss_out, kl_out);
+  return launch_fit_clusters<8, false, 4>(s, Hf, st, steps, plogp, alpha_out, rho_out, logZ_out, out_stride, loss_out, kl_out);
 }
 
 }  // namespace saf

@@ -223,8 +223,7 @@ struct FitState {
   const double* eta_rel;
   double* alpha; double* rho;          // fp64 parameters
   double* m_a; double* v_a; double* m_r; double* v_r;   // Adam moments
-  float* a2[2]; float* r2[2];          // log2e-scaled fp32 copies, double-buffered over the steps
-  float* nz2;                          // -log2 Z(i) of the current parameters
+  float* a2; float* r2;                // exp (in the log form: log2e-scaled copy) of the current parameters
 };
 int fit_max_T();
 cudaError_t launch_fit_marginals(const float* Abar, float floor_v, double* eta_abs, double* eta_rel, double* plogp,

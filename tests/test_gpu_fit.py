@@ -241,3 +241,33 @@ def test_fit_no_heads_and_bad_arguments():
         ctx.saf_fit_compact(1, 16385, z, z, z, 1, 0.05, f, f, f, 16385, None, None)
     assert e.value.code == saf.SAF_ERR_UNSUPPORTED
     _status(ctx)
+
+
+# One launch per call: a cluster of CTAs per head.  Edges: blocks of 256 positions (one, two, a partial one), more heads
+# than clusters fit at once, the longest sequences (vectors kept unpadded), two to eight CTAs per cluster.
+@pytest.mark.parametrize("Hf,T,steps", [(1, 255, 3), (2, 257, 3), (1, 2304, 2), (150, 272, 2), (40, 300, 2), (1, 10300, 1)])
+def test_fit_cluster_edges(Hf, T, steps):
+    base = si.mean_attention_maps(1, T, 40 + T)
+    P, ea, er, pl = _oracle_stats(base)
+    rep = lambda v: _dev(np.repeat(v, Hf, axis=0))
+    a, r, z, loss, kl = _gpu_fit(_ctx(), rep(ea), rep(er), rep(pl), steps)
+    for x in (a, r, z, loss, kl):
+        assert np.array_equal(x, np.broadcast_to(x[:1], x.shape))             # every head ran the same program
+    wa, wr, wz = fo.fit_compact(ea[0], er[0], steps=steps)
+    assert np.max(np.abs(a[0] - wa)) < 2e-4 and np.max(np.abs(r[0] - wr)) < 2e-4 and np.max(np.abs(z[0] - wz)) < 1e-4
+    assert abs(kl[0] - fo.fit_kl_dense(P[0], wa, wr)) < 1e-4
+
+
+# Parameters beyond 2^+-50 (2^-70): the head goes on with logarithms.  Steps of 10 nats cross the bounds within four
+# steps; magnitudes reach a few hundred nats, where an fp32 exponent argument carries 2^-24 * 2^9 = 3e-5 nats per
+# rounding, so 5e-4 is asserted on log Z (about ten roundings) against the fp64 normalisers at the returned parameters.
+@pytest.mark.parametrize("T,steps", [(100, 12), (700, 8)])
+def test_fit_leaves_the_product_range(T, steps):
+    A = si.mean_attention_maps(2, T, 50 + T)
+    P, ea, er, pl = _oracle_stats(A)
+    a, r, z, loss, kl = _gpu_fit(_ctx(), _dev(ea), _dev(er), _dev(pl), steps, lr=10.0)
+    assert max(np.abs(a).max(), np.abs(r).max()) > 50 * np.log(2)
+    for h in range(2):
+        want_z, _ = fo._logZ_and_P(a[h], r[h])
+        assert np.max(np.abs(z[h] - want_z)) < 5e-4
+        assert abs(loss[h] - fo.fit_objective(a[h], r[h], ea[h], er[h])) < 5e-4 * max(1.0, abs(loss[h]))
