@@ -22,7 +22,7 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
 struct WorklistEntry {
-  int B, H, T, backward, grid, wide;
+  int B, H, T, D, backward, grid;
   std::vector<uint8_t> mask;
   std::vector<WorkItem> items_host;       // kept alive: the upload is asynchronous on the caller's stream
   std::vector<int> offsets_host;
@@ -284,6 +284,37 @@ void build_worklist_host(int B, int H, int T, const uint8_t* mask, int backward,
   offsets[n_ctas] = static_cast<int>(items.size());
 }
 
+// Work queue of the 128-wide forward, whose items are two consecutive query blocks of one (batch, head) unit (the first
+// block of an odd count goes alone).  CTAs claim items in this order at run time, so longest-first within groups of
+// units keeps both the tail short and a group's K and V in L2 while its items run: a group is as many units as have
+// 32 MB of K and V together.  While the items would not fill the SMs, blocks go one by one: a pair takes longer than a
+// single block and there are SMs to spare.
+void build_pair_order(int B, int H, int T, int D, const uint8_t* mask, int num_sms, std::vector<WorkItem>& order) {
+  const int nblk = (T + BLK - 1) / BLK;
+  const bool pair = static_cast<long long>(B) * H * nblk > num_sms;
+  const long long unit_bytes = static_cast<long long>(T) * D * 4;
+  const int group = static_cast<int>(std::max<long long>(1, (32ll << 20) / unit_bytes));
+  order.clear();
+  std::vector<std::pair<long long, WorkItem>> items;
+  auto flush = [&] {
+    std::stable_sort(items.begin(), items.end(),
+                     [](const std::pair<long long, WorkItem>& a, const std::pair<long long, WorkItem>& b) { return a.first > b.first; });
+    for (const auto& it : items) order.push_back(it.second);
+    items.clear();
+  };
+  for (int u = 0; u < B * H; ++u) {
+    const int b = u / H, h = u % H;
+    const int kind = mask[h] ? KIND_FROZEN : KIND_ORDINARY;
+    for (int q = nblk - 1; q >= 0; q -= pair ? 2 : 1) {
+      const bool two = pair && q > 0;
+      const long long tiles = two ? 2 * q + 1 : q + 1;
+      items.push_back({(mask[h] ? 50 : 100) * tiles + 100, WorkItem{b, h, q, kind | (two ? KIND_PAIR : 0)}});
+    }
+    if ((u + 1) % group == 0) flush();
+  }
+  flush();
+}
+
 // Measured cost-model defaults: `wide` = the 128-wide kernels (head dimension 96 or 128), else the 64-wide ones.
 void sched_defaults(int wide, int backward, int* frozen_pct, int* overhead_pct, int* overhead_frozen_pct) {
   if (backward) {
@@ -296,10 +327,10 @@ void sched_defaults(int wide, int backward, int* frozen_pct, int* overhead_pct, 
   }
 }
 
-int get_worklist(saf_ctx* ctx, int B, int H, int T, const uint8_t* mask, int backward, int grid, int wide,
-                 cudaStream_t st, const WorklistEntry** out) {
+int get_worklist(saf_ctx* ctx, int B, int H, int T, int D, const uint8_t* mask, int backward, int grid, cudaStream_t st,
+                 const WorklistEntry** out) {
   for (const WorklistEntry& e : ctx->worklists)
-    if (e.B == B && e.H == H && e.T == T && e.backward == backward && e.grid == grid && e.wide == wide &&
+    if (e.B == B && e.H == H && e.T == T && e.D == D && e.backward == backward && e.grid == grid &&
         std::memcmp(e.mask.data(), mask, H) == 0) {
       *out = &e;
       return SAF_OK;
@@ -313,6 +344,7 @@ int get_worklist(saf_ctx* ctx, int B, int H, int T, const uint8_t* mask, int bac
   }
   std::vector<WorkItem> items;
   std::vector<int> offsets;
+  const int wide = D != 64;
   int frozen_pct, overhead_pct, overhead_frozen_pct;
   sched_defaults(wide, backward, &frozen_pct, &overhead_pct, &overhead_frozen_pct);
   const int fw = backward ? ctx->frozen_weight_bwd_pct : ctx->frozen_weight_pct;
@@ -323,9 +355,10 @@ int get_worklist(saf_ctx* ctx, int B, int H, int T, const uint8_t* mask, int bac
   WorklistEntry e;
   build_worklist_host(B, H, T, mask, backward, grid, frozen_pct, overhead_pct, overhead_frozen_pct, second_wave, items,
                       offsets, &e.order_host);
-  e.B = B; e.H = H; e.T = T; e.backward = backward; e.grid = grid; e.wide = wide;
+  if (wide && !backward) build_pair_order(B, H, T, D, mask, ctx->num_sms, e.order_host);
+  e.B = B; e.H = H; e.T = T; e.D = D; e.backward = backward; e.grid = grid;
   e.mask.assign(mask, mask + H);
-  e.n_items = static_cast<int>(items.size());
+  e.n_items = static_cast<int>(e.order_host.size());
   if (cudaMalloc(&e.items_dev, items.size() * sizeof(WorkItem)) != cudaSuccess) return SAF_ERR_NOMEM;
   if (cudaMalloc(&e.offsets_dev, offsets.size() * sizeof(int)) != cudaSuccess) {
     cudaFree(e.items_dev);
@@ -620,9 +653,10 @@ int saf_hybrid_attn_fwd(saf_ctx* ctx, const saf_problem* p, const void* Q, const
   }
   const int nblk = (p->T + BLK - 1) / BLK;
   const long long n_items = static_cast<long long>(p->B) * p->H * nblk;
-  const int grid = static_cast<int>(std::min<long long>(2LL * ctx->num_sms, n_items));
+  // (head dimension 64: two CTAs per SM; the 128-wide kernel: one)
+  const int grid = static_cast<int>(std::min<long long>((p->D == 64 ? 2LL : 1LL) * ctx->num_sms, n_items));
   const WorklistEntry* wl = nullptr;
-  rc = get_worklist(ctx, p->B, p->H, p->T, frozen_mask_host, 0, grid, p->D != 64, st, &wl);
+  rc = get_worklist(ctx, p->B, p->H, p->T, p->D, frozen_mask_host, 0, grid, st, &wl);
   if (rc) return rc;
 
   CUtensorMap mq, mk, mv;
@@ -792,7 +826,7 @@ int saf_hybrid_attn_bwd(saf_ctx* ctx, const saf_problem* p, const void* Q, const
   const long long n_items = static_cast<long long>(p->B) * p->H * nblk;
   const int grid = static_cast<int>(std::min<long long>(ctx->num_sms, n_items));
   const WorklistEntry* wl = nullptr;
-  rc = get_worklist(ctx, p->B, p->H, p->T, frozen_mask_host, 1, grid, p->D != 64, st, &wl);
+  rc = get_worklist(ctx, p->B, p->H, p->T, p->D, frozen_mask_host, 1, grid, st, &wl);
   if (rc) return rc;
 
   CUtensorMap mq, mk, mv, mdo;

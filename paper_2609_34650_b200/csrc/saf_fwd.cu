@@ -1,36 +1,54 @@
-// Forward of the hybrid causal attention layer on sm_100a: one persistent kernel for ordinary
-// (flash-style online softmax) and frozen (pattern rebuilt from alpha/rho/logZ) heads.
+// Forward of the hybrid causal attention layer on sm_100a, two query blocks per work item: one persistent kernel for
+// ordinary (flash-style online softmax) and frozen (pattern rebuilt from alpha/rho/logZ) heads.
 //
-// Per CTA (320 threads): warps 0-7 = compute, warp 8 = TMA producer, warp 9 = tcgen05 issuer and TMEM
-// owner.  Two compute threads share a query row (= TMEM lane): warps 0-3 own key columns 0-63 of a
-// tile, warps 4-7 columns 64-127; row maxima and row sums are exchanged through shared memory.  Two
-// CTAs share an SM, so one CTA's softmax and bookkeeping overlap the other's MMAs.
-// TMEM columns: [0,128) S (fp32) / P (bf16 pairs in [0,32) and [64,96): each warp writes into the
-// columns it has consumed itself), [128,128+D) O accumulator.
+// One CTA per SM, 512 threads: warps 0-3 softmax of query block 0 of the item, warps 4-7 of query block 1 (one thread
+// per query row = TMEM lane, all 128 scores of a tile in registers), warps 8-11 epilogue, warp 12 TMA producer,
+// warp 13 tcgen05 issuer and TMEM owner.  Registers are moved to the softmax warps (192 a thread) from the others (64):
+// 256 x 192 + 256 x 64 = the 512 x 128 of the launch.
 //
-// Ordinary item (b,h,I): for J = 0..I: S = Q_I K_J^T (tcgen05, operands in 128B-swizzled smem via TMA),
-//   row max / lazy rescale / exp2 / row sum in registers, P -> TMEM as bf16, O += P V_J (A from TMEM,
-//   V as MN-major B); epilogue O / l and LSE.
-// Frozen item (b,h,I): for J = 0..I: P^(i,j) = exp(alpha(j) + rho(i-j) - logZ(i)) for j <= i
-//   (Eq. "compact-prior" with the stored normaliser) generated into TMEM, O += P^ V_J.  No Q/K loads,
-//   no score MMA, no max/sum.  The exponential is factorised per tile as
-//   w(i) * a(j) * r(i-j) with a = exp(alpha - max_tile alpha), r = exp(rho - max_band rho),
-//   w = exp(max alpha + max rho - logZ(i)); a tile whose exponent range would leave fp32 falls back to
-//   one exp per element.
+// Why this shape: a 128x128 tile of an ordinary head costs 1024 clk of special-function unit (16 ex2/clk/SM) and, at
+// D = 128, 1024 clk of tensor pipe.  With one score buffer per CTA the two alternate; with the two query blocks
+// of an item sharing each K/V tile, the tensor pipe works on one block while the other is in its softmax, and
+// each K/V tile is loaded once for 256 queries.  TMEM: S/P of the two blocks [0,128) [128,256), O [256,256+D) and
+// [256+D,256+2D).
+//
+// Ordinary item (b,h,q1): query blocks q1 and (pair) q1-1; for J = 0..: S_t = Q_t K_J^T, row max / lazy rescale / exp2 /
+//   row sum in registers, P_t -> TMEM as bf16 over S_t, O_t += P_t V_J; the next score MMA of a block is queued
+//   directly behind the MMA that consumes its P (MMAs of one thread execute in order).  The first scores of the next
+//   item go out as soon as block 0 of this one has its last P V MMA, so no softmax warp idles between items.
 // Frozen item, tensor-core form (pattern tables prepared and the head's flag set): with global maxima,
-//   O = diag(w) R (diag(a) V), R(i,j) = r(i-j).  A tile of R with reversed rows is a Hankel matrix that the
-//   tensor core reads straight from a 4 KB band table (no-swizzle descriptor, both strides 128 bytes), so
-//   a tile is one bulk copy of the band, one TMA load of the a-scaled V tile and 8 MMAs; the compute warps
-//   only scale the finished rows by w(i) (TMEM lane m holds query 127-m of the block).
+//   O = diag(w) R (diag(a) V), R(i,j) = r(i-j).  A tile of R with reversed rows is a Hankel matrix that the tensor
+//   core reads straight from a 4 KB band table (no-swizzle descriptor, both strides 128 bytes), so a tile is two bulk
+//   copies of bands, one TMA load of the a-scaled V tile and 16 MMAs; the epilogue scales the finished rows by w(i)
+//   (TMEM lane m holds query 127-m of the block).
+// Frozen item, general form: P^(i,j) = exp(alpha(j) + rho(i-j) - logZ(i)) for j <= i (Eq. "compact-prior" with the
+//   stored normaliser) generated into TMEM by the softmax warps, O_t += P^ V_J.  The exponential is factorised per
+//   tile as w(i) a(j) r(i-j) with a = exp(alpha - max_tile alpha), r = exp(rho - max_band rho),
+//   w = exp(max alpha + max rho - logZ(i)); a tile whose exponent range would leave fp32 falls back to one exp per
+//   element.
 #include <cuda_bf16.h>
 #include "ptx.cuh"
 #include "saf_internal.h"
 
+#ifdef SAF_TRACE
+__device__ unsigned long long g_saf_trace_fwd128[3][16384];
+#define TRF(role, id)                                                                                  \
+  do {                                                                                                 \
+    if (blockIdx.x == 0 && (threadIdx.x & 31) == 0 && tr_n < 16380)                                    \
+      g_saf_trace_fwd128[role][tr_n++] = (static_cast<unsigned long long>(id) << 48) | (clock64() & 0xffffffffffffULL); \
+  } while (0)
+extern "C" int saf_debug_read_trace_fwd128(unsigned long long* out) {
+  return static_cast<int>(cudaMemcpyFromSymbol(out, g_saf_trace_fwd128, sizeof(g_saf_trace_fwd128)));
+}
+#else
 #define TRF(role, id)
+#endif
 
 SAF_SPAN_DEFINE(fwd128)
 
 namespace saf {
+
+namespace {
 
 constexpr float LOG2E_F = 1.4426950408889634f;
 constexpr float LN2_F = 0.6931471805599453f;
@@ -40,72 +58,106 @@ struct FwdCfg {
   static constexpr int NPANEL = D / 64;                 // 64-column bf16 panels: 128-byte rows, one swizzle atom
   static constexpr int PANEL_BYTES = 128 * 64 * 2;      // 16 KB
   static constexpr int TILE_BYTES = NPANEL * PANEL_BYTES;
-  static constexpr int NS = (D == 64) ? 2 : 1;          // K and V ring depth
-  static constexpr int OFF_Q = 0;
-  static constexpr int OFF_K = TILE_BYTES;
-  static constexpr int OFF_V = OFF_K + NS * TILE_BYTES;
-  static constexpr int OFF_TAB = OFF_V + NS * TILE_BYTES;
-  // floats: aJ[128] rband[256] a2raw[128] r2raw[256] red[32] xch[2][2][128] lx[2][128]
-  static constexpr int TAB_FLOATS = 128 + 256 + 128 + 256 + 32 + 512 + 256;
-  static constexpr int OFF_BAR = OFF_TAB + TAB_FLOATS * 4;
-  static constexpr int NBAR = 2 + 4 * NS + 4;
-  static constexpr int SMEM = OFF_BAR + NBAR * 8 + 16 + 1024;   // + slack for 1024-byte alignment
-  static constexpr int TMEM_COLS = 256;
-  static constexpr int COL_S = 0, COL_P = 0, COL_O = 128;
-  static constexpr int NTHREADS = 320;
-  // A thread keeps its 64 scores in registers between the max and the exp pass (reading them from TMEM
-  // twice instead measured almost twice as slow at D = 128).
-  static constexpr bool SCORES_IN_REGS = true;
+  static constexpr int NS = 4;                          // ring of K and V tiles (K_0 V_0 K_1 V_1 ...)
+  static constexpr int OFF_Q = 0;                       // Q of the two query blocks (general frozen form: tables)
+  static constexpr int OFF_KV = 2 * TILE_BYTES;
+  static constexpr int OFF_BAND = OFF_KV + NS * TILE_BYTES;   // 2 x 4 KB of Hankel bands per ring stage
+  static constexpr int OFF_LINV = OFF_BAND + NS * 8192;       // [2][128] 1 / row sum
+  static constexpr int OFF_BAR = OFF_LINV + 2 * 128 * 4;
+  static constexpr int NRING = 4;                       // work-item records in flight
+  static constexpr int NBAR = 2 * NS + 14 + 2 * NRING;
+  static constexpr int OFF_RING = (OFF_BAR + NBAR * 8 + 16 + 15) / 16 * 16;
+  static constexpr int SMEM = OFF_RING + NRING * 16 + 1024;   // + slack for 1024-byte alignment
+  static constexpr int TMEM_COLS = 512;
+  static constexpr int COL_S = 0, COL_O = 256;          // + 128 t, + D t
+  static constexpr int NTHREADS = 512;
 };
 
-enum FwdSite { SITE_Q_EMPTY = 1, SITE_K_EMPTY, SITE_V_EMPTY, SITE_Q_FULL, SITE_K_FULL, SITE_P_FULL, SITE_V_FULL,
-               SITE_O_FREE, SITE_S_FULL, SITE_PV_DONE };
+enum FwdSite { SITE_Q_EMPTY = 1, SITE_KV_EMPTY, SITE_Q_FULL, SITE_KV_FULL, SITE_P_FULL, SITE_O_FREE, SITE_S_FULL,
+               SITE_O_FULL, SITE_L_FULL, SITE_RING_EMPTY, SITE_RING_FULL };
+
+constexpr int RING_FAST = 1 << 8;
+constexpr int RING_END = -1;
+
+// A work item as the roles see it.  n1 = key tiles of query block `blk` (tile 1), n0 = key tiles of query block blk - 1
+// (tile 0; 0: the item has one query block).
+struct ItemView {
+  int b, h, blk, kind, n0, n1;
+  bool fast;
+};
+
+template <int NRING>
+__device__ __forceinline__ bool ring_take(const int4* ring, uint64_t* ring_full, uint64_t* ring_empty, uint32_t n,
+                                          const WaitCtx& wc, ItemView& v) {
+  const uint32_t slot = n % NRING;
+  if (!mbar_wait_warp(ring_full + slot, (n / NRING) & 1, wc, SITE_RING_FULL)) return false;
+  const int4 raw = ring[slot];
+  warp_arrive(ring_empty + slot);
+  v.b = raw.x;
+  v.h = raw.y;
+  v.blk = raw.z;
+  v.kind = raw.w < 0 ? RING_END : (raw.w & 0x7f);
+  v.fast = raw.w >= 0 && (raw.w & RING_FAST) != 0;
+  v.n1 = raw.z + 1;
+  v.n0 = (raw.w & KIND_PAIR) ? raw.z : 0;
+  return true;
+}
+
+}  // namespace
 
 template <int D>
-__global__ void __launch_bounds__(320, 2)
+__global__ void __launch_bounds__(512, 1)
 saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ CUtensorMap mk,
                const __grid_constant__ CUtensorMap mv, const __grid_constant__ CUtensorMap mvt, const FwdParams p) {
   using C = FwdCfg<D>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::OFF_BAR);
-  uint64_t* q_full = bars;
-  uint64_t* q_empty = bars + 1;
-  uint64_t* k_full = bars + 2;
-  uint64_t* k_empty = k_full + C::NS;
-  uint64_t* v_full = k_empty + C::NS;
-  uint64_t* v_empty = v_full + C::NS;
-  uint64_t* s_full = v_empty + C::NS;
-  uint64_t* p_full = s_full + 1;
-  uint64_t* pv_done = p_full + 1;
-  uint64_t* o_free = pv_done + 1;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(o_free + 1);
+  uint64_t* kv_full = bars;                      // [NS]
+  uint64_t* kv_empty = kv_full + C::NS;          // [NS]
+  uint64_t* q_full = kv_empty + C::NS;           // [2] Q of block t has landed
+  uint64_t* q_empty = q_full + 2;                // [2] the item's last use of Q t's memory has completed
+  uint64_t* s_full = q_empty + 2;                // [2] scores of block t (general form: buffer t may be written)
+  uint64_t* p_full = s_full + 2;                 // [2] P of block t written (4 warp arrivals)
+  uint64_t* o_full = p_full + 2;                 // [2] last MMA into O_t has completed
+  uint64_t* o_free = o_full + 2;                 // [2] epilogue has read O_t (4 warp arrivals)
+  uint64_t* l_full = o_free + 2;                 // [2] 1 / row sum of block t written (4 warp arrivals)
+  uint64_t* ring_full = l_full + 2;              // [NRING] record n has been published by the producer
+  uint64_t* ring_empty = ring_full + C::NRING;   // [NRING] issuer + 8 softmax warps + 4 epilogue warps have copied it
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(ring_empty + C::NRING);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  float* tab = reinterpret_cast<float*>(smem + C::OFF_TAB);
+  int4* ring = reinterpret_cast<int4*>(smem + C::OFF_RING);
+  float* linv = reinterpret_cast<float*>(smem + C::OFF_LINV);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const WaitCtx wc{abort_flag, p.status, p.wait_limit_ns};
   SAF_SPAN(fwd128, 0);
+#ifdef SAF_TRACE
   int tr_n = 0;
-  (void)tr_n;
+#endif
 
   if (tid == 0) {
     *abort_flag = 0;
-    mbar_init(q_full, 1);
-    mbar_init(q_empty, 1);
     for (int s = 0; s < C::NS; ++s) {
-      mbar_init(k_full + s, 1);
-      mbar_init(k_empty + s, 1);
-      mbar_init(v_full + s, 1);
-      mbar_init(v_empty + s, 1);
+      mbar_init(kv_full + s, 1);
+      mbar_init(kv_empty + s, 1);
     }
-    mbar_init(s_full, 1);
-    mbar_init(p_full, 8);                        // one arrival per compute warp
-    mbar_init(pv_done, 1);
-    mbar_init(o_free, 8);
+    for (int t = 0; t < 2; ++t) {
+      mbar_init(q_full + t, 1);
+      mbar_init(q_empty + t, 1);
+      mbar_init(s_full + t, 1);
+      mbar_init(p_full + t, 4);
+      mbar_init(o_full + t, 1);
+      mbar_init(o_free + t, 4);
+      mbar_init(l_full + t, 4);
+    }
+    for (int k = 0; k < C::NRING; ++k) {
+      mbar_init(ring_full + k, 1);
+      mbar_init(ring_empty + k, 13);
+    }
     mbar_fence_init();
   }
-  if (warp == 9) {
+  if (warp == 13) {
     tmem_alloc(tmem_slot, C::TMEM_COLS);
     tmem_relinquish();
   }
@@ -117,414 +169,521 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
   pdl_launch_dependents();
   pdl_wait();
 
-  const int it_begin = p.cta_offsets[blockIdx.x], it_end = p.cta_offsets[blockIdx.x + 1];
-
-  if (warp == 8) {
-    // ------------------------------------------------------------------ TMA producer
-    if (lane == 0) {
-      tma_prefetch_desc(&mq);
-      tma_prefetch_desc(&mk);
-      tma_prefetch_desc(&mv);
-      tma_prefetch_desc(&mvt);
-      uint32_t nq = 0, nk = 0, nv = 0;
-      bool ok = true;
-      for (int it = it_begin; it < it_end && ok; ++it) {
-        const WorkItem w = p.items[it];
-        const int ntiles = w.blk + 1;
-        if (w.kind == KIND_FROZEN && p.band_f != nullptr && p.fast_ok[w.h] != 0 && p.ovf[w.h] != p.call_id) {
-          // tensor-core form: per tile the Hankel band of distance block (I - J) and the scaled V tile
-          const int ord = p.hord[w.h];
-          const uint8_t* bands = static_cast<const uint8_t*>(p.band_f) + static_cast<size_t>(w.h) * p.nblkp * 4096;
-          for (int j = 0; j < ntiles; ++j) {
-            const int sk = nk % C::NS;
-            ok = mbar_wait(k_empty + sk, ((nk / C::NS) & 1) ^ 1, wc, SITE_K_EMPTY);
-            if (!ok) break;
-            mbar_expect_tx(k_full + sk, 4096);
-            bulk_load(smem + C::OFF_K + sk * C::TILE_BYTES, bands + static_cast<size_t>(w.blk - j) * 4096, 4096,
-                      k_full + sk);
-            ++nk;
-            const int sv = nv % C::NS;
-            ok = mbar_wait(v_empty + sv, ((nv / C::NS) & 1) ^ 1, wc, SITE_V_EMPTY);
-            if (!ok) break;
-            mbar_expect_tx(v_full + sv, C::TILE_BYTES);
+  // (each warpgroup sets its register share at the top of its own branch)
+  if (warp >= 12) {
+    reg_dec<64>();
+    if (warp == 12) {
+      // ---------------------------------------------------------------- TMA producer
+      if (lane == 0) {
+        tma_prefetch_desc(&mq);
+        tma_prefetch_desc(&mk);
+        tma_prefetch_desc(&mv);
+        tma_prefetch_desc(&mvt);
+        uint32_t n = 0;                            // ring position
+        uint32_t nq0 = 0, nq1 = 0;                 // uses of the two Q areas
+        bool ok = true;
+        for (uint32_t nclaim = 0; ok; ++nclaim) {
+          // claim the next item of the queue and publish it to the other roles
+          const uint32_t slot = nclaim % C::NRING;
+          ok = mbar_wait(ring_empty + slot, ((nclaim / C::NRING) & 1) ^ 1, wc, SITE_RING_EMPTY);
+          if (!ok) break;
+          const int idx = atomicAdd(p.queue, 1);
+          int4 rec = make_int4(0, 0, 0, RING_END);
+          bool fast = false;
+          if (idx < p.n_items) {
+            rec = __ldg(reinterpret_cast<const int4*>(p.order + idx));
+            fast = (rec.w & 0x7f) != KIND_ORDINARY && p.band_f != nullptr && __ldg(p.fast_ok + rec.y) != 0 &&
+                   __ldg(p.ovf + rec.y) != p.call_id;
+            if (fast) rec.w |= RING_FAST;
+          }
+          ring[slot] = rec;
+          mbar_arrive(ring_full + slot);                 // (release: the record is visible to whoever sees the phase)
+          if (idx >= p.n_items) break;
+          const int b = rec.x, h = rec.y, n1 = rec.z + 1;
+          const bool pair = (rec.w & KIND_PAIR) != 0;
+          auto load_kv = [&](const CUtensorMap* m, int j, int head) {
+            const uint32_t s = n % C::NS;
+            ok = mbar_wait(kv_empty + s, ((n / C::NS) & 1) ^ 1, wc, SITE_KV_EMPTY);
+            if (!ok) return;
+            mbar_expect_tx(kv_full + s, C::TILE_BYTES);
             for (int pn = 0; pn < C::NPANEL; ++pn)
-              tma_load_4d(smem + C::OFF_V + sv * C::TILE_BYTES + pn * C::PANEL_BYTES, &mvt, v_full + sv, pn * 64,
-                          j * BLK, ord, w.b);
-            ++nv;
-          }
-          continue;
-        }
-        if (w.kind == KIND_ORDINARY) {
-          ok = mbar_wait(q_empty, (nq & 1) ^ 1, wc, SITE_Q_EMPTY);
-          if (!ok) break;
-          mbar_expect_tx(q_full, C::TILE_BYTES);
-          for (int pn = 0; pn < C::NPANEL; ++pn)
-            tma_load_4d(smem + C::OFF_Q + pn * C::PANEL_BYTES, &mq, q_full, pn * 64, w.blk * BLK,
-                        p.qslot ? p.qslot[w.h] : w.h, w.b);
-          ++nq;
-        }
-        for (int j = 0; j < ntiles && ok; ++j) {
-          if (w.kind == KIND_ORDINARY) {
-            const int s = nk % C::NS;
-            ok = mbar_wait(k_empty + s, ((nk / C::NS) & 1) ^ 1, wc, SITE_K_EMPTY);
-            if (!ok) break;
-            mbar_expect_tx(k_full + s, C::TILE_BYTES);
-            for (int pn = 0; pn < C::NPANEL; ++pn)
-              tma_load_4d(smem + C::OFF_K + s * C::TILE_BYTES + pn * C::PANEL_BYTES, &mk, k_full + s, pn * 64,
-                          j * BLK, p.qslot ? p.qslot[w.h] : w.h / p.kv_group, w.b);
-            ++nk;
-          }
-          const int s = nv % C::NS;
-          ok = mbar_wait(v_empty + s, ((nv / C::NS) & 1) ^ 1, wc, SITE_V_EMPTY);
-          if (!ok) break;
-          mbar_expect_tx(v_full + s, C::TILE_BYTES);
-          for (int pn = 0; pn < C::NPANEL; ++pn)
-            tma_load_4d(smem + C::OFF_V + s * C::TILE_BYTES + pn * C::PANEL_BYTES, &mv, v_full + s, pn * 64,
-                        j * BLK, w.h / p.kv_group, w.b);
-          ++nv;
-        }
-      }
-    }
-  } else if (warp == 9) {
-    // ------------------------------------------------------------------ tcgen05 issuer
-    // The whole warp walks the loops (warp-uniform operands); one elected lane issues.
-    const bool leader = elect_one() != 0;
-    const uint32_t sb = smem_u32(smem);
-    constexpr uint32_t idesc_s = umma_idesc_bf16(128, 128, 0, 0);
-    // (head dimension 96 runs here with features 96..127 zero-filled by TMA: its MMAs skip the two empty k-steps of
-    // the scores and produce only 96 output columns)
-    const uint32_t idesc_o = umma_idesc_bf16(128, p.d_real, 0, 1);
-    const int nk16 = p.d_real / 16;
-    const uint32_t idesc_hk = umma_idesc_f16(128, p.d_real, 0, 1);  // tensor-core frozen form: fp16 band x fp16 scaled V
-    uint32_t nq = 0, nk = 0, nv = 0, np = 0, nitem = 0;
-    bool ok = true;
-    // descriptor halves for smem offset 0: K-major tiles (k-step +32 B within a 64-column panel) and
-    // the MN-major V tile (k-step +2048 B, LBO = panel stride)
-    const uint64_t d_kmaj = umma_smem_desc(sb, 16, 1024, UMMA_LAYOUT_SW128);
-    const uint64_t d_mn = umma_smem_desc(sb, C::PANEL_BYTES, 1024, UMMA_LAYOUT_SW128);
-    const uint32_t lo_k = desc_lo(d_kmaj), hi_k = desc_hi(d_kmaj), lo_m = desc_lo(d_mn), hi_m = desc_hi(d_mn);
-    const uint32_t q_lo = lo_k + (C::OFF_Q >> 4);
-    // Hankel band: no-swizzle K-major, core matrices 128 bytes apart in both directions
-    const uint64_t d_band = umma_smem_desc(sb, 128, 128, UMMA_LAYOUT_NONE);
-    const uint32_t lo_b = desc_lo(d_band), hi_b = desc_hi(d_band);
-    for (int it = it_begin; it < it_end && ok; ++it, ++nitem) {
-      const WorkItem w = p.items[it];
-      const int ntiles = w.blk + 1;
-      const bool ord = w.kind == KIND_ORDINARY;
-      if (w.kind == KIND_FROZEN && p.band_f != nullptr && p.fast_ok[w.h] != 0 && p.ovf[w.h] != p.call_id) {
-        for (int j = 0; j < ntiles && ok; ++j) {
-          const uint32_t sk = nk % C::NS, sv = nv % C::NS;
-          ok = mbar_wait_warp(k_full + sk, (nk / C::NS) & 1, wc, SITE_K_FULL);
-          if (!ok) break;
-          ++nk;
-          ok = mbar_wait_warp(v_full + sv, (nv / C::NS) & 1, wc, SITE_V_FULL);
-          if (!ok) break;
-          ++nv;
-          if (j == 0) {
-            ok = mbar_wait_warp(o_free, (nitem & 1) ^ 1, wc, SITE_O_FREE);
-            if (!ok) break;
-          }
-          tc_fence_after();
-          const uint32_t band_lo = lo_b + ((C::OFF_K + sk * C::TILE_BYTES) >> 4);
-          const uint32_t v_lo = lo_m + ((C::OFF_V + sv * C::TILE_BYTES) >> 4);
-          const uint32_t acc0 = j > 0 ? 1u : 0u;
-          if (leader) {
-#pragma unroll
-            for (int kc = 0; kc < 8; ++kc)
-              umma_ss2(tmem + C::COL_O, band_lo + 16 * kc, hi_b, v_lo + 128 * kc, hi_m, idesc_hk, kc > 0 ? 1u : acc0);
-            umma_commit(k_empty + sk);
-            umma_commit(v_empty + sv);
-            if (j == ntiles - 1) umma_commit(pv_done);
-          }
-          __syncwarp();
-        }
-        continue;
-      }
-      if (ord) {
-        ok = mbar_wait_warp(q_full, nq & 1, wc, SITE_Q_FULL);
-        if (!ok) break;
-        ++nq;
-      }
-      for (int j = 0; j < ntiles && ok; ++j) {
-        if (ord) {
-          const uint32_t s = nk % C::NS;
-          TRF(0, 1);
-          ok = mbar_wait_warp(k_full + s, (nk / C::NS) & 1, wc, SITE_K_FULL);
-          if (!ok) break;
-          ++nk;
-          tc_fence_after();
-          TRF(0, 2);
-          const uint32_t k_lo = lo_k + ((C::OFF_K + s * C::TILE_BYTES) >> 4);
-          if (leader) {
-#pragma unroll
-            for (int kc = 0; kc < D / 16; ++kc) {
-              if (kc >= nk16) break;
-              const uint32_t off = ((kc >> 2) * C::PANEL_BYTES + (kc & 3) * 32) >> 4;
-              umma_ss2(tmem + C::COL_S, q_lo + off, hi_k, k_lo + off, hi_k, idesc_s, kc > 0);
+              tma_load_4d(smem + C::OFF_KV + s * C::TILE_BYTES + pn * C::PANEL_BYTES, m, kv_full + s, pn * 64, j * BLK, head, b);
+            ++n;
+          };
+          if (fast) {
+            // tensor-core form: per tile the scaled V tile and the Hankel bands of distance blocks q1 - J, q1 - 1 - J
+            const int ord = p.hord[h];
+            const uint8_t* bands = static_cast<const uint8_t*>(p.band_f) + static_cast<size_t>(h) * p.nblkp * 4096;
+            for (int j = 0; j < n1; ++j) {
+              const uint32_t s = n % C::NS;
+              ok = mbar_wait(kv_empty + s, ((n / C::NS) & 1) ^ 1, wc, SITE_KV_EMPTY);
+              if (!ok) break;
+              const int d = n1 - 1 - j;
+              const bool two = pair && d > 0;
+              mbar_expect_tx(kv_full + s, C::TILE_BYTES + (two ? 8192 : 4096));
+              for (int pn = 0; pn < C::NPANEL; ++pn)
+                tma_load_4d(smem + C::OFF_KV + s * C::TILE_BYTES + pn * C::PANEL_BYTES, &mvt, kv_full + s, pn * 64, j * BLK,
+                            ord, b);
+              bulk_load(smem + C::OFF_BAND + s * 8192 + 4096, bands + static_cast<size_t>(d) * 4096, 4096, kv_full + s);
+              if (two) bulk_load(smem + C::OFF_BAND + s * 8192, bands + static_cast<size_t>(d - 1) * 4096, 4096, kv_full + s);
+              ++n;
             }
-            umma_commit(s_full);
-            umma_commit(k_empty + s);
-            if (j == ntiles - 1) umma_commit(q_empty);
+            continue;
           }
-          __syncwarp();
-          TRF(0, 3);
+          const int hv = h / p.kv_group;
+          if ((rec.w & 0x7f) == KIND_ORDINARY) {
+            const int hq = p.qslot ? p.qslot[h] : h, hk = p.qslot ? hq : hv;
+            // Q_0 and K_0 first: block 0's first scores are issued before this item's predecessor has finished with Q_1
+            if (pair) {
+              ok = mbar_wait(q_empty, (nq0 & 1) ^ 1, wc, SITE_Q_EMPTY);
+              if (!ok) break;
+              mbar_expect_tx(q_full, C::TILE_BYTES);
+              for (int pn = 0; pn < C::NPANEL; ++pn)
+                tma_load_4d(smem + C::OFF_Q + pn * C::PANEL_BYTES, &mq, q_full, pn * 64, (rec.z - 1) * BLK, hq, b);
+              ++nq0;
+            }
+            load_kv(&mk, 0, hk);
+            if (!ok) break;
+            ok = mbar_wait(q_empty + 1, (nq1 & 1) ^ 1, wc, SITE_Q_EMPTY);
+            if (!ok) break;
+            mbar_expect_tx(q_full + 1, C::TILE_BYTES);
+            for (int pn = 0; pn < C::NPANEL; ++pn)
+              tma_load_4d(smem + C::OFF_Q + C::TILE_BYTES + pn * C::PANEL_BYTES, &mq, q_full + 1, pn * 64, rec.z * BLK, hq, b);
+            ++nq1;
+            load_kv(&mv, 0, hv);
+            for (int j = 1; j < n1 && ok; ++j) {
+              load_kv(&mk, j, hk);
+              if (ok) load_kv(&mv, j, hv);
+            }
+          } else {
+            // general frozen form: the Q areas hold the tables of the softmax warps; an area counts as used by this item
+            if (pair) {
+              ok = mbar_wait(q_empty, (nq0 & 1) ^ 1, wc, SITE_Q_EMPTY);
+              ++nq0;
+            }
+            if (ok) ok = mbar_wait(q_empty + 1, (nq1 & 1) ^ 1, wc, SITE_Q_EMPTY);
+            ++nq1;
+            for (int j = 0; j < n1 && ok; ++j) load_kv(&mv, j, hv);
+          }
         }
-        ok = mbar_wait_warp(p_full, np & 1, wc, SITE_P_FULL);
-        if (!ok) break;
-        ++np;
-        TRF(0, 4);
-        const uint32_t s = nv % C::NS;
-        ok = mbar_wait_warp(v_full + s, (nv / C::NS) & 1, wc, SITE_V_FULL);
-        if (!ok) break;
-        ++nv;
-        if (j == 0) {
-          ok = mbar_wait_warp(o_free, (nitem & 1) ^ 1, wc, SITE_O_FREE);
-          if (!ok) break;
-        }
-        tc_fence_after();
-        TRF(0, 5);
-        const uint32_t v_lo = lo_m + ((C::OFF_V + s * C::TILE_BYTES) >> 4);
-        const uint32_t acc0 = j > 0 ? 1u : 0u;
+      }
+    } else if (warp == 13) {
+      // ---------------------------------------------------------------- tcgen05 issuer
+      // The whole warp walks the loops (warp-uniform operands); one elected lane issues.
+      const bool leader = elect_one() != 0;
+      const uint32_t sb = smem_u32(smem);
+      constexpr uint32_t idesc_s = umma_idesc_bf16(128, 128, 0, 0);
+      // (head dimension 96 runs here with features 96..127 zero-filled by TMA: its MMAs skip the two empty k-steps of
+      // the scores and produce only 96 output columns)
+      const uint32_t idesc_o = umma_idesc_bf16(128, p.d_real, 0, 1);
+      const int nk16 = p.d_real / 16;
+      const uint32_t idesc_hk = umma_idesc_f16(128, p.d_real, 0, 1);  // tensor-core frozen form: fp16 band x fp16 scaled V
+      // descriptor halves for smem offset 0: K-major tiles (k-step +32 B within a 64-column panel) and
+      // the MN-major V tile (k-step +2048 B, LBO = panel stride)
+      const uint64_t d_kmaj = umma_smem_desc(sb, 16, 1024, UMMA_LAYOUT_SW128);
+      const uint64_t d_mn = umma_smem_desc(sb, C::PANEL_BYTES, 1024, UMMA_LAYOUT_SW128);
+      const uint32_t lo_k = desc_lo(d_kmaj), hi_k = desc_hi(d_kmaj), lo_m = desc_lo(d_mn), hi_m = desc_hi(d_mn);
+      // Hankel band: no-swizzle K-major, core matrices 128 bytes apart in both directions
+      const uint64_t d_band = umma_smem_desc(sb, 128, 128, UMMA_LAYOUT_NONE);
+      const uint32_t lo_b = desc_lo(d_band), hi_b = desc_hi(d_band);
+      auto kv_wait = [&](uint32_t pos) {
+        return mbar_wait_warp(kv_full + pos % C::NS, (pos / C::NS) & 1, wc, SITE_KV_FULL);
+      };
+      // (all callers sit between two warp-uniform points; `leader` alone issues)
+      auto issue_qk = [&](uint32_t t, uint32_t pos) {
+        const uint32_t q_lo = lo_k + ((C::OFF_Q + t * C::TILE_BYTES) >> 4);
+        const uint32_t k_lo = lo_k + ((C::OFF_KV + (pos % C::NS) * C::TILE_BYTES) >> 4);
         if (leader) {
-          // bf16 P pairs: keys 0-63 in columns [0,32), keys 64-127 in columns [64,96)
+#pragma unroll
+          for (int kc = 0; kc < D / 16; ++kc) {
+            if (kc >= nk16) break;
+            const uint32_t off = ((kc >> 2) * C::PANEL_BYTES + (kc & 3) * 32) >> 4;
+            umma_ss2(tmem + C::COL_S + 128 * t, q_lo + off, hi_k, k_lo + off, hi_k, idesc_s, kc > 0);
+          }
+          umma_commit(s_full + t);
+        }
+      };
+      auto issue_pv = [&](uint32_t t, uint32_t pos, uint32_t acc0) {
+        const uint32_t v_lo = lo_m + ((C::OFF_KV + (pos % C::NS) * C::TILE_BYTES) >> 4);
+        if (leader) {
 #pragma unroll
           for (int kc = 0; kc < 8; ++kc)
-            umma_ts2(tmem + C::COL_O, tmem + C::COL_P + 8 * kc + (kc >= 4 ? 32u : 0u), v_lo + 128 * kc, hi_m, idesc_o,
+            umma_ts2(tmem + C::COL_O + D * t, tmem + C::COL_S + 128 * t + 8 * kc, v_lo + 128 * kc, hi_m, idesc_o,
                      kc > 0 ? 1u : acc0);
-          umma_commit(v_empty + s);
-          umma_commit(pv_done);
         }
-        __syncwarp();
-        TRF(0, 6);
+      };
+      uint32_t n = 0, nrec = 0;
+      uint32_t nqf0 = 0, nqf1 = 0, np0 = 0, np1 = 0, no0 = 0, no1 = 0;   // phases of q_full, p_full, o_free by block
+      bool early = false;                          // block 0's first scores of `cur` are already issued
+      ItemView cur;
+      bool ok = ring_take<C::NRING>(ring, ring_full, ring_empty, nrec++, wc, cur);
+      while (ok && cur.kind != RING_END) {
+        ItemView nxt;
+        bool have_next = false;
+        const int n0 = cur.n0, n1 = cur.n1;
+        if (cur.fast) {
+          for (int j = 0; j < n1 && ok; ++j) {
+            ok = kv_wait(n);
+            if (!ok) break;
+            const uint32_t s = n % C::NS;
+            const uint32_t band_lo = lo_b + ((C::OFF_BAND + s * 8192) >> 4);
+            const uint32_t v_lo = lo_m + ((C::OFF_KV + s * C::TILE_BYTES) >> 4);
+            const uint32_t acc0 = j > 0 ? 1u : 0u;
+            if (j < n0) {
+              if (j == 0) {
+                ok = mbar_wait_warp(o_free, (no0++ & 1) ^ 1, wc, SITE_O_FREE);
+                if (!ok) break;
+              }
+              tc_fence_after();
+              if (leader) {
+#pragma unroll
+                for (int kc = 0; kc < 8; ++kc)
+                  umma_ss2(tmem + C::COL_O, band_lo + 16 * kc, hi_b, v_lo + 128 * kc, hi_m, idesc_hk, kc > 0 ? 1u : acc0);
+                if (j == n0 - 1) umma_commit(o_full);
+              }
+              __syncwarp();
+            }
+            if (j == 0) {
+              ok = mbar_wait_warp(o_free + 1, (no1++ & 1) ^ 1, wc, SITE_O_FREE);
+              if (!ok) break;
+            }
+            tc_fence_after();
+            if (leader) {
+#pragma unroll
+              for (int kc = 0; kc < 8; ++kc)
+                umma_ss2(tmem + C::COL_O + D, band_lo + 256 + 16 * kc, hi_b, v_lo + 128 * kc, hi_m, idesc_hk,
+                         kc > 0 ? 1u : acc0);
+              umma_commit(kv_empty + s);
+              if (j == n1 - 1) umma_commit(o_full + 1);
+            }
+            __syncwarp();
+            ++n;
+          }
+        } else if (cur.kind == KIND_ORDINARY) {
+          if (n0 > 0 && !early) {
+            ok = mbar_wait_warp(q_full, nqf0++ & 1, wc, SITE_Q_FULL) && kv_wait(n);
+            if (!ok) break;
+            tc_fence_after();
+            issue_qk(0, n);
+            if (leader && n0 == 1) umma_commit(q_empty);
+            __syncwarp();
+          }
+          early = false;
+          ok = mbar_wait_warp(q_full + 1, nqf1++ & 1, wc, SITE_Q_FULL) && kv_wait(n);
+          if (!ok) break;
+          tc_fence_after();
+          issue_qk(1, n);
+          if (leader) {
+            umma_commit(kv_empty + n % C::NS);
+            if (n1 == 1) umma_commit(q_empty + 1);
+          }
+          __syncwarp();
+          for (int j = 0; j < n1 && ok; ++j) {
+            const uint32_t pv = n + 2 * j + 1, pk = pv + 1;        // ring positions of V_j and K_{j+1}
+            const bool more1 = j + 1 < n1;
+            const uint32_t acc0 = j > 0 ? 1u : 0u;
+            // the tiles' loads land long before P is ready: test their barriers first, so that only one test
+            // stands between "P is ready" and the MMAs that wait for it
+            ok = kv_wait(pv) && (!more1 || kv_wait(pk));
+            if (!ok) break;
+            if (j < n0) {
+              if (j == 0) ok = mbar_wait_warp(o_free, (no0++ & 1) ^ 1, wc, SITE_O_FREE);
+              if (ok) ok = mbar_wait_warp(p_full, np0++ & 1, wc, SITE_P_FULL);
+              if (!ok) break;
+              tc_fence_after();
+              TRF(0, 2);
+              issue_pv(0, pv, acc0);
+              if (j + 1 < n0) {
+                issue_qk(0, pk);                         // executes after P V: same thread, in order
+                if (leader && j + 2 == n0) umma_commit(q_empty);
+                __syncwarp();
+                TRF(0, 3);
+              } else {
+                if (leader) umma_commit(o_full);
+                __syncwarp();
+                // block 0 is through: its first scores of the next item go out now
+                ok = ring_take<C::NRING>(ring, ring_full, ring_empty, nrec++, wc, nxt);
+                if (!ok) break;
+                have_next = true;
+                if (nxt.kind == KIND_ORDINARY && nxt.n0 > 0) {
+                  const uint32_t pn = n + 2 * n1;
+                  ok = mbar_wait_warp(q_full, nqf0++ & 1, wc, SITE_Q_FULL) && kv_wait(pn);
+                  if (!ok) break;
+                  tc_fence_after();
+                  issue_qk(0, pn);
+                  if (leader && nxt.n0 == 1) umma_commit(q_empty);
+                  __syncwarp();
+                  early = true;
+                }
+              }
+            }
+            if (j == 0) {
+              ok = mbar_wait_warp(o_free + 1, (no1++ & 1) ^ 1, wc, SITE_O_FREE);
+              if (!ok) break;
+            }
+            ok = mbar_wait_warp(p_full + 1, np1++ & 1, wc, SITE_P_FULL);
+            if (!ok) break;
+            tc_fence_after();
+            TRF(0, 4);
+            issue_pv(1, pv, acc0);
+            if (leader) umma_commit(kv_empty + pv % C::NS);
+            __syncwarp();
+            if (more1) {
+              issue_qk(1, pk);
+              if (leader) {
+                umma_commit(kv_empty + pk % C::NS);
+                if (j + 2 == n1) umma_commit(q_empty + 1);
+              }
+              TRF(0, 5);
+            } else if (leader) {
+              umma_commit(o_full + 1);
+            }
+            __syncwarp();
+          }
+          n += 2 * n1;
+        } else {
+          // general frozen form: P^ written by the softmax warps, one P V per block and tile; s_full says that a
+          // block's P^ buffer may be written (everything issued before has completed)
+          if (leader) {
+            if (n0 > 0) umma_commit(s_full);
+            umma_commit(s_full + 1);
+          }
+          __syncwarp();
+          for (int j = 0; j < n1 && ok; ++j) {
+            ok = kv_wait(n);
+            if (!ok) break;
+            const uint32_t acc0 = j > 0 ? 1u : 0u;
+            if (j < n0) {
+              if (j == 0) ok = mbar_wait_warp(o_free, (no0++ & 1) ^ 1, wc, SITE_O_FREE);
+              if (ok) ok = mbar_wait_warp(p_full, np0++ & 1, wc, SITE_P_FULL);
+              if (!ok) break;
+              tc_fence_after();
+              issue_pv(0, n, acc0);
+              if (leader) {
+                if (j + 1 < n0) {
+                  umma_commit(s_full);
+                } else {
+                  umma_commit(o_full);
+                  umma_commit(q_empty);
+                }
+              }
+              __syncwarp();
+            }
+            if (j == 0) ok = mbar_wait_warp(o_free + 1, (no1++ & 1) ^ 1, wc, SITE_O_FREE);
+            if (ok) ok = mbar_wait_warp(p_full + 1, np1++ & 1, wc, SITE_P_FULL);
+            if (!ok) break;
+            tc_fence_after();
+            issue_pv(1, n, acc0);
+            if (leader) {
+              umma_commit(kv_empty + n % C::NS);
+              if (j + 1 < n1) {
+                umma_commit(s_full + 1);
+              } else {
+                umma_commit(o_full + 1);
+                umma_commit(q_empty + 1);
+              }
+            }
+            __syncwarp();
+            ++n;
+          }
+        }
+        if (!ok) break;
+        if (have_next) cur = nxt;
+        else ok = ring_take<C::NRING>(ring, ring_full, ring_empty, nrec++, wc, cur);
       }
     }
-  } else {
-    // ------------------------------------------------------------------ compute warps (256 threads)
-    const int q4 = warp & 3, hh = warp >> 2;
-    const int rowl = q4 * 32 + lane;                   // query row within the tile = TMEM lane
-    const int pair_bar = 1 + q4;                       // named barrier of the two warps sharing this lane quarter
+  } else if (warp < 8) {
+    // ------------------------------------------------------------------ softmax warps (2 x 128 threads)
+    reg_inc<192>();
+    const int q4 = warp & 3, t = warp >> 2;
+    const int rowl = q4 * 32 + lane;                   // query row within the block = TMEM lane
     const uint32_t lane_base = static_cast<uint32_t>(q4 * 32) << 16;
-    const uint32_t t_s = tmem + lane_base + C::COL_S + 64 * hh;       // this thread's 64 score columns
-    const uint32_t t_p = tmem + lane_base + C::COL_P + 64 * hh;       // ... and where its bf16 pairs go
-    const uint32_t t_o = tmem + lane_base + C::COL_O + (D / 2) * hh;  // this thread's half of the O row
-    float* aJ = tab;
-    float* rband = tab + 128;
-    float* a2raw = tab + 384;
-    float* r2raw = tab + 512;
-    float* red = tab + 768;
-    float* xch = tab + 800;                            // [tile parity][hh][row]
-    float* lx = tab + 1312;                            // [hh][row]
-    uint32_t ns = 0, npv = 0;
+    const uint32_t t_s = tmem + lane_base + C::COL_S + 128 * t;       // scores, then bf16 pairs of P in the first 64
+    const uint32_t t_o = tmem + lane_base + C::COL_O + D * t;
+    const int wg_bar = 1 + t, wg_bar2 = 3 + t;
+    uint32_t ns = 0, nof = 0;                          // phases of s_full[t]; items of this block so far
     bool ok = true;
-    const int trr = 1 + hh;
-    (void)trr;
-    // A compute warp whose wait was abandoned keeps walking (without storing) until the next
-    // agreement barrier, where all eight leave together; none is ever left alone at a barrier.
-    for (int it = it_begin; it < it_end; ++it) {
-      const WorkItem w = p.items[it];
-      const int ntiles = w.blk + 1;
-      int row = w.blk * BLK + rowl;
-      float inv_l = 1.0f, lse = 0.0f;
-      if (named_bar_or(5, 256, !ok)) break;
-      if (w.kind == KIND_FROZEN && p.band_f != nullptr && p.fast_ok[w.h] != 0 && p.ovf[w.h] != p.call_id) {
-        // tensor-core form: nothing to do per tile; lane m holds query 127-m, scaled by w(i) below
-        row = w.blk * BLK + 127 - rowl;
-        inv_l = (row < p.T) ? p.wvec[static_cast<size_t>(w.h) * p.Tp + row] * (1.0f / (HK_BAND_SCALE * HK_A_SCALE)) : 0.0f;
-      } else if (w.kind == KIND_ORDINARY) {
-        float m_ref = -INFINITY, l = 0.0f;
+    // A softmax warp whose wait was abandoned keeps walking (without storing) until the next
+    // agreement barrier, where its four leave together; none is ever left alone at a barrier.
+    for (uint32_t nrec = 0;; ++nrec) {
+      ItemView w;
+      if (!ring_take<C::NRING>(ring, ring_full, ring_empty, nrec, wc, w)) {
+        ok = false;
+        w.kind = KIND_ORDINARY; w.n0 = w.n1 = 0; w.fast = false; w.b = w.h = w.blk = 0;
+      }
+      if (named_bar_or(wg_bar, 128, !ok) || w.kind == RING_END) break;
+      const int nt = t == 0 ? w.n0 : w.n1;
+      if (nt == 0) continue;
+      const int blk = nt - 1;
+      const int row = blk * BLK + rowl;
+      if (w.fast) {
+        ++nof;
+        continue;
+      }
+      if (w.kind == KIND_ORDINARY) {
+        float m_ref = -INFINITY;
+        uint64_t l2a = 0, l2b = 0;                     // packed pairs of partial row sums
         const float c = p.scale_log2;
-        for (int j = 0; j < ntiles; ++j) {
-          TRF(trr, 11);
-          if (!mbar_wait_warp(s_full, ns & 1, wc, SITE_S_FULL)) ok = false;
+        const uint64_t c2 = pk2(c, c);
+        for (int j = 0; j < nt; ++j) {
+          if (q4 == 0) TRF(1 + t, 11);
+          // (the completion of this score MMA also covers the block's previous P V MMA, issued before it)
+          if (!mbar_wait_warp(s_full + t, ns & 1, wc, SITE_S_FULL)) ok = false;
           ++ns;
-          if (j > 0) {
-            if (!mbar_wait_warp(pv_done, npv & 1, wc, SITE_PV_DONE)) ok = false;
-            ++npv;
-          }
           tc_fence_after();
-          TRF(trr, 12);
-          const bool diag = (j == w.blk);
-          uint32_t r0[C::SCORES_IN_REGS ? 32 : 1], r1[C::SCORES_IN_REGS ? 32 : 1];
-          float mx;
-          if constexpr (C::SCORES_IN_REGS) {
-            tmem_ld32(t_s, r0);
-            tmem_ld32(t_s + 32, r1);
-            tmem_wait_ld();
-            if (diag) {
+          if (q4 == 0) TRF(1 + t, 12);
+          uint32_t r[4][32];
+          float mx0, mx1;
+          tmem_ld32(t_s, r[0]);
+          tmem_ld32(t_s + 32, r[1]);
+          tmem_wait_ld();
+          tmem_ld32(t_s + 64, r[2]);
+          tmem_ld32(t_s + 96, r[3]);
+          if (j == blk) {
 #pragma unroll
-              for (int e = 0; e < 32; ++e) {
-                if (64 * hh + e > rowl) r0[e] = 0xff800000u;        // -inf above the diagonal
-                if (64 * hh + 32 + e > rowl) r1[e] = 0xff800000u;
-              }
-            }
-            float mx0 = -INFINITY, mx1 = -INFINITY;
-#pragma unroll
-            for (int e = 0; e < 32; ++e) {
-              mx0 = fmaxf(mx0, __uint_as_float(r0[e]));
-              mx1 = fmaxf(mx1, __uint_as_float(r1[e]));
-            }
-            mx = fmaxf(mx0, mx1);
-          } else {
-            mx = -INFINITY;
-#pragma unroll
-            for (int cc = 0; cc < 2; ++cc) {
-              uint32_t r[32];
-              tmem_ld32(t_s + 32 * cc, r);
-              tmem_wait_ld();
-              float m0 = -INFINITY, m1 = -INFINITY;
-#pragma unroll
-              for (int e = 0; e < 16; ++e) {
-                float s0 = __uint_as_float(r[2 * e]), s1 = __uint_as_float(r[2 * e + 1]);
-                if (diag) {
-                  if (64 * hh + 32 * cc + 2 * e > rowl) s0 = -INFINITY;
-                  if (64 * hh + 32 * cc + 2 * e + 1 > rowl) s1 = -INFINITY;
-                }
-                m0 = fmaxf(m0, s0);
-                m1 = fmaxf(m1, s1);
-              }
-              mx = fmaxf(mx, fmaxf(m0, m1));
-            }
+            for (int e = 0; e < 64; ++e)
+              if (e > rowl) r[e >> 5][e & 31] = 0xff800000u;          // -inf above the diagonal
           }
-          TRF(trr, 13);
-          // row maximum over both column halves
-          float* xs = xch + (j & 1) * 256;
-          xs[hh * 128 + rowl] = mx;
-          named_bar_sync(pair_bar, 64);
-          mx = fmaxf(mx, xs[(hh ^ 1) * 128 + rowl]);
-          TRF(trr, 14);
-          const float m_new = fmaxf(m_ref, mx * c);
+          mx0 = __uint_as_float(r[0][0]);
+          mx1 = __uint_as_float(r[1][0]);
+#pragma unroll
+          for (int e = 1; e < 32; ++e) {
+            mx0 = fmaxf(mx0, __uint_as_float(r[0][e]));
+            mx1 = fmaxf(mx1, __uint_as_float(r[1][e]));
+          }
+          tmem_wait_ld();
+          if (j == blk) {
+#pragma unroll
+            for (int e = 64; e < 128; ++e)
+              if (e > rowl) r[e >> 5][e & 31] = 0xff800000u;
+          }
+#pragma unroll
+          for (int e = 0; e < 32; ++e) {
+            mx0 = fmaxf(mx0, __uint_as_float(r[2][e]));
+            mx1 = fmaxf(mx1, __uint_as_float(r[3][e]));
+          }
+          if (q4 == 0) TRF(1 + t, 13);
+          const float m_new = fmaxf(m_ref, fmaxf(mx0, mx1) * c);   // finite: key 0 is visible to every row
           if (j == 0) {
             m_ref = m_new;
           } else {
             const bool need = (m_new - m_ref) > 8.0f;
             if (__any_sync(0xffffffffu, need)) {
               const float f = need ? ex2_approx(m_ref - m_new) : 1.0f;
-              l *= f;
+              l2a = mul2(l2a, pk2(f, f));
+              l2b = mul2(l2b, pk2(f, f));
               if (need) m_ref = m_new;
 #pragma unroll
-              for (int cc = 0; cc < D / 32; ++cc) {
-                uint32_t r[16];
-                tmem_ld16(t_o + 16 * cc, r);
+              for (int cc = 0; cc < D / 16; ++cc) {
+                uint32_t o[16];
+                tmem_ld16(t_o + 16 * cc, o);
                 tmem_wait_ld();
 #pragma unroll
-                for (int e = 0; e < 16; ++e) r[e] = __float_as_uint(__uint_as_float(r[e]) * f);
-                tmem_st16(t_o + 16 * cc, r);
+                for (int e = 0; e < 16; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * f);
+                tmem_st16(t_o + 16 * cc, o);
               }
             }
           }
-          const float neg_m = -m_ref;
-          float l0 = 0.0f, l1 = 0.0f;
-          if constexpr (C::SCORES_IN_REGS) {
-            uint32_t pk0[16], pk1[16];
+          const uint64_t nm2 = pk2(-m_ref, -m_ref);
+#pragma unroll
+          for (int cc = 0; cc < 4; ++cc) {
+            uint32_t pk[16];
 #pragma unroll
             for (int e = 0; e < 16; ++e) {
-              const float a0 = ex2_approx(fmaf(__uint_as_float(r0[2 * e]), c, neg_m));
-              const float a1 = ex2_approx(fmaf(__uint_as_float(r0[2 * e + 1]), c, neg_m));
-              const float b0 = ex2_approx(fmaf(__uint_as_float(r1[2 * e]), c, neg_m));
-              const float b1 = ex2_approx(fmaf(__uint_as_float(r1[2 * e + 1]), c, neg_m));
-              l0 += a0 + a1;
-              l1 += b0 + b1;
-              pk0[e] = pack_bf16x2(a0, a1);
-              pk1[e] = pack_bf16x2(b0, b1);
+              const uint64_t x2 = fma2(pk2(__uint_as_float(r[cc][2 * e]), __uint_as_float(r[cc][2 * e + 1])), c2, nm2);
+              float a0, a1;
+              upk2(x2, a0, a1);
+              a0 = ex2_approx(a0);
+              a1 = ex2_approx(a1);
+              const uint64_t a2 = pk2(a0, a1);
+              if (e & 1) l2b = add2(l2b, a2);
+              else l2a = add2(l2a, a2);
+              pk[e] = pack_bf16x2(a0, a1);
             }
-            tmem_st16(t_p, pk0);
-            tmem_st16(t_p + 16, pk1);
-          } else {
-#pragma unroll
-            for (int cc = 0; cc < 2; ++cc) {
-              uint32_t r[32];
-              tmem_ld32(t_s + 32 * cc, r);
-              tmem_wait_ld();
-              uint32_t pk[16];
-#pragma unroll
-              for (int e = 0; e < 16; ++e) {
-                float a0 = ex2_approx(fmaf(__uint_as_float(r[2 * e]), c, neg_m));
-                float a1 = ex2_approx(fmaf(__uint_as_float(r[2 * e + 1]), c, neg_m));
-                if (diag) {
-                  if (64 * hh + 32 * cc + 2 * e > rowl) a0 = 0.0f;
-                  if (64 * hh + 32 * cc + 2 * e + 1 > rowl) a1 = 0.0f;
-                }
-                l0 += a0;
-                l1 += a1;
-                pk[e] = pack_bf16x2(a0, a1);
-              }
-              tmem_st16(t_p + 16 * cc, pk);
-            }
+            tmem_st16(t_s + 16 * cc, pk);
           }
-          l += l0 + l1;
-          TRF(trr, 15);
+          if (q4 == 0) TRF(1 + t, 14);
           tmem_wait_st();
           tc_fence_before();
-          warp_arrive(p_full);
-          TRF(trr, 16);
+          warp_arrive(p_full + t);
+          if (q4 == 0) TRF(1 + t, 15);
         }
-        // row sum over both column halves
-        lx[hh * 128 + rowl] = l;
-        named_bar_sync(pair_bar, 64);
-        l += lx[(hh ^ 1) * 128 + rowl];
-        inv_l = 1.0f / l;
-        lse = (m_ref + log2f(l)) * LN2_F;
+        float la, lb, lc, ld;
+        upk2(l2a, la, lb);
+        upk2(l2b, lc, ld);
+        const float l = (la + lb) + (lc + ld);
+        // the epilogue has read the previous item's row sums once it has released O_t
+        if (nof > 0 && !mbar_wait_warp(o_free + t, (nof - 1) & 1, wc, SITE_O_FREE)) ok = false;
+        linv[t * 128 + rowl] = 1.0f / l;
+        warp_arrive(l_full + t);
+        if (p.LSE != nullptr && row < p.T && ok)
+          p.LSE[(static_cast<size_t>(w.b) * p.H + w.h) * p.T + row] = (m_ref + log2f(l)) * LN2_F;
       } else {
-        // ---------------- frozen head: generate P^ tiles
+        // ---------------- frozen head, general form: generate P^ tiles
+        float* tab = reinterpret_cast<float*>(smem + C::OFF_Q + t * C::TILE_BYTES);
+        float* aJ = tab;                               // [128] a of the tile's keys
+        float* rband = tab + 128;                      // [256] r of the tile's distances
+        float* a2raw = tab + 384;                      // [128]
+        float* r2raw = tab + 512;                      // [256]
+        float* red = tab + 768;                        // [8]
+        const int wt = tid & 127;
         const float* alpha_h = p.alpha + static_cast<size_t>(w.h) * p.Tp;
         const float* rho_h = p.rho + static_cast<size_t>(w.h) * p.Tp;
         const float z2 = (row < p.T) ? p.logZ[static_cast<size_t>(w.h) * p.Tp + row] * LOG2E_F : INFINITY;
         bool leave = false;
-        for (int j = 0; j < ntiles; ++j) {
-          // previous tile's table readers are done; the compute warps also agree whether to go on
-          if (named_bar_or(5, 256, !ok)) {
+        for (int j = 0; j < nt; ++j) {
+          // previous P^ tile consumed (first tile: everything issued before this item has completed)
+          if (!mbar_wait_warp(s_full + t, ns & 1, wc, SITE_S_FULL)) ok = false;
+          ++ns;
+          tc_fence_after();
+          // previous tile's table readers are done; the four warps also agree whether to go on
+          if (named_bar_or(wg_bar, 128, !ok)) {
             ok = false;
             leave = true;
             break;
           }
-          const int d0 = (w.blk - j) * BLK - 127;      // band covers distances d0 .. d0+254
-          float a2 = -INFINITY, r2 = -INFINITY;
-          if (tid < 128) {
-            const int key = j * BLK + tid;
-            if (key < p.T) a2 = alpha_h[key] * LOG2E_F;
-            a2raw[tid] = a2;
-          }
+          const int d0 = (blk - j) * BLK - 127;        // band covers distances d0 .. d0+254
+          float ma = -INFINITY, mr = -INFINITY, a2 = -INFINITY, r2[2];
           {
-            const int d = d0 + tid;                    // one band entry per compute thread (255 used)
-            if (tid < 255 && d >= 0 && d < p.T) r2 = rho_h[d] * LOG2E_F;
-            r2raw[tid] = r2;
+            const int key = j * BLK + wt;
+            if (key < p.T) a2 = alpha_h[key] * LOG2E_F;
+            a2raw[wt] = a2;
+            ma = a2;
           }
-          float ma = a2, mr = r2;
+#pragma unroll
+          for (int k = 0; k < 2; ++k) {
+            const int x = wt + 128 * k, d = d0 + x;
+            r2[k] = (x < 255 && d >= 0 && d < p.T) ? rho_h[d] * LOG2E_F : -INFINITY;
+            r2raw[x] = r2[k];
+            mr = fmaxf(mr, r2[k]);
+          }
 #pragma unroll
           for (int o = 16; o > 0; o >>= 1) {
             ma = fmaxf(ma, __shfl_xor_sync(0xffffffffu, ma, o));
             mr = fmaxf(mr, __shfl_xor_sync(0xffffffffu, mr, o));
           }
           if (lane == 0) {
-            red[warp] = ma;                            // warps 4-7 contribute -inf
-            red[8 + warp] = mr;
+            red[q4] = ma;
+            red[4 + q4] = mr;
           }
-          named_bar_sync(6, 256);
+          named_bar_sync(wg_bar2, 128);
           ma = fmaxf(fmaxf(red[0], red[1]), fmaxf(red[2], red[3]));
-          mr = fmaxf(fmaxf(fmaxf(red[8], red[9]), fmaxf(red[10], red[11])),
-                     fmaxf(fmaxf(red[12], red[13]), fmaxf(red[14], red[15])));
+          mr = fmaxf(fmaxf(red[4], red[5]), fmaxf(red[6], red[7]));
           const float ew = ma + mr - z2;               // -inf for rows beyond T
-          const unsigned anybad = __any_sync(0xffffffffu, ew > 100.0f);   // factorised form would overflow / flush
-          if (lane == 0) red[16 + warp] = anybad ? 1.0f : 0.0f;
-          if (tid < 128) aJ[tid] = ex2_approx(a2 - ma);
-          rband[tid] = ex2_approx(r2 - mr);
-          named_bar_sync(7, 256);
-          const bool exact = (red[16] + red[17] + red[18] + red[19] + red[20] + red[21] + red[22] + red[23]) > 0.0f;
-          if (j > 0) {
-            if (!mbar_wait_warp(pv_done, npv & 1, wc, SITE_PV_DONE)) ok = false;   // previous P^ tile consumed
-            ++npv;
-            tc_fence_after();
-          }
+          aJ[wt] = ex2_approx(a2 - ma);
+          rband[wt] = ex2_approx(r2[0] - mr);
+          rband[wt + 128] = ex2_approx(r2[1] - mr);
+          // (agreement on the form: the factorised one would overflow or flush for some row)
+          const bool exact = named_bar_or(wg_bar2, 128, ew > 100.0f);
 #pragma unroll
-          for (int cc = 0; cc < 2; ++cc) {
-            const int k0c = 64 * hh + 32 * cc;         // first key column of this chunk
+          for (int cc = 0; cc < 4; ++cc) {
             uint32_t pk[16];
             if (!exact) {
               const float wv = ex2_approx(ew);
               const float* rb = rband + rowl + 127;    // rb[-k] = r(distance of key k in this tile)
 #pragma unroll
               for (int e4 = 0; e4 < 8; ++e4) {
-                const int k0 = k0c + 4 * e4;
+                const int k0 = 32 * cc + 4 * e4;
                 const float4 a4 = *reinterpret_cast<const float4*>(aJ + k0);
                 const float p0 = wv * a4.x * rb[-k0], p1 = wv * a4.y * rb[-k0 - 1];
                 const float p2 = wv * a4.z * rb[-k0 - 2], p3 = wv * a4.w * rb[-k0 - 3];
@@ -535,56 +694,89 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
               const float* rb = r2raw + rowl + 127;
 #pragma unroll
               for (int e = 0; e < 16; ++e) {
-                const int k0 = k0c + 2 * e;
+                const int k0 = 32 * cc + 2 * e;
                 const float p0 = ex2_approx(a2raw[k0] + rb[-k0] - z2);
                 const float p1 = ex2_approx(a2raw[k0 + 1] + rb[-k0 - 1] - z2);
                 pk[e] = pack_bf16x2(p0, p1);
               }
             }
-            tmem_st16(t_p + 16 * cc, pk);
+            tmem_st16(t_s + 16 * cc, pk);
           }
           tmem_wait_st();
           tc_fence_before();
-          warp_arrive(p_full);
+          fence_proxy_async_smem();                    // the tables' memory is a TMA destination of a later item
+          warp_arrive(p_full + t);
         }
         if (leave) break;
       }
-      // ---------------- epilogue: wait for the last P V, scale, store this thread's half of the row
-      if (!mbar_wait_warp(pv_done, npv & 1, wc, SITE_PV_DONE)) ok = false;
-      ++npv;
-      tc_fence_after();
-      __nv_bfloat16* orow = reinterpret_cast<__nv_bfloat16*>(p.O) + w.b * p.o_strides[0] + w.h * p.o_strides[1] +
-                            static_cast<int64_t>(row) * p.o_strides[2] + (D / 2) * hh;
+      ++nof;
+    }
+  } else {
+    // ------------------------------------------------------------------ epilogue warps
+    reg_dec<64>();
+    const int q4 = warp & 3;
+    const int rowl = q4 * 32 + lane;
+    const uint32_t lane_base = static_cast<uint32_t>(q4 * 32) << 16;
+    uint32_t nof0 = 0, nof1 = 0, nl0 = 0, nl1 = 0;
+    bool ok = true;
+    for (uint32_t nrec = 0; ok; ++nrec) {
+      ItemView w;
+      ok = ring_take<C::NRING>(ring, ring_full, ring_empty, nrec, wc, w);
+      if (!ok || w.kind == RING_END) break;
+#pragma unroll 1
+      for (int t = 0; t < 2 && ok; ++t) {
+        const int nt = t == 0 ? w.n0 : w.n1;
+        if (nt == 0) continue;
+        const int blk = nt - 1;
+        int row = blk * BLK + rowl;
+        float f = 1.0f;
+        if (w.fast) {
+          row = blk * BLK + 127 - rowl;                // tensor-core form: lane m holds query 127-m, scaled by w(i)
+          f = (row < p.T) ? p.wvec[static_cast<size_t>(w.h) * p.Tp + row] * (1.0f / (HK_BAND_SCALE * HK_A_SCALE)) : 0.0f;
+        } else if (w.kind == KIND_ORDINARY) {
+          ok = mbar_wait_warp(l_full + t, (t == 0 ? nl0++ : nl1++) & 1, wc, SITE_L_FULL);
+          if (!ok) break;
+          f = linv[t * 128 + rowl];
+        }
+        ok = mbar_wait_warp(o_full + t, (t == 0 ? nof0++ : nof1++) & 1, wc, SITE_O_FULL);
+        if (!ok) break;
+        tc_fence_after();
+        const uint32_t t_o = tmem + lane_base + C::COL_O + D * t;
+        const int64_t off = w.b * p.o_strides[0] + w.h * p.o_strides[1] + static_cast<int64_t>(row) * p.o_strides[2];
 #pragma unroll
-      for (int cc = 0; cc < D / 64; ++cc) {
-        uint32_t r[32];
-        tmem_ld32(t_o + 32 * cc, r);
-        tmem_wait_ld();
-        if (row < p.T && ok && p.o_f32) {
-          float* orow32 = static_cast<float*>(p.O) + w.b * p.o_strides[0] + w.h * p.o_strides[1] +
-                          static_cast<int64_t>(row) * p.o_strides[2] + (D / 2) * hh + 32 * cc;
+        for (int cc = 0; cc < D / 32; ++cc) {
+          uint32_t r[32];
+          tmem_ld32(t_o + 32 * cc, r);
+          tmem_wait_ld();
+          if (cc == D / 32 - 1) {
+            tc_fence_before();
+            warp_arrive(o_free + t);                   // the accumulator and linv may be overwritten
+          }
+          if (row < p.T && 32 * cc < p.d_real) {
+            if (p.o_f32) {
+              float* orow = static_cast<float*>(p.O) + off + 32 * cc;
 #pragma unroll
-          for (int g = 0; g < 8; ++g)
-            if ((D / 2) * hh + 32 * cc + 4 * g < p.d_real)
-              *reinterpret_cast<float4*>(orow32 + 4 * g) =
-                  make_float4(__uint_as_float(r[4 * g + 0]) * inv_l, __uint_as_float(r[4 * g + 1]) * inv_l,
-                              __uint_as_float(r[4 * g + 2]) * inv_l, __uint_as_float(r[4 * g + 3]) * inv_l);
-        } else if (row < p.T && ok) {
+              for (int g = 0; g < 8; ++g)
+                *reinterpret_cast<float4*>(orow + 4 * g) =
+                    make_float4(__uint_as_float(r[4 * g + 0]) * f, __uint_as_float(r[4 * g + 1]) * f,
+                                __uint_as_float(r[4 * g + 2]) * f, __uint_as_float(r[4 * g + 3]) * f);
+            } else {
+              __nv_bfloat16* orow = static_cast<__nv_bfloat16*>(p.O) + off + 32 * cc;
 #pragma unroll
-          for (int g = 0; g < 4; ++g) {
-            uint4 o;
-            o.x = pack_bf16x2(__uint_as_float(r[8 * g + 0]) * inv_l, __uint_as_float(r[8 * g + 1]) * inv_l);
-            o.y = pack_bf16x2(__uint_as_float(r[8 * g + 2]) * inv_l, __uint_as_float(r[8 * g + 3]) * inv_l);
-            o.z = pack_bf16x2(__uint_as_float(r[8 * g + 4]) * inv_l, __uint_as_float(r[8 * g + 5]) * inv_l);
-            o.w = pack_bf16x2(__uint_as_float(r[8 * g + 6]) * inv_l, __uint_as_float(r[8 * g + 7]) * inv_l);
-            if ((D / 2) * hh + 32 * cc + 8 * g < p.d_real) *reinterpret_cast<uint4*>(orow + 32 * cc + 8 * g) = o;
+              for (int g = 0; g < 4; ++g) {
+                uint4 o;
+                o.x = pack_bf16x2(__uint_as_float(r[8 * g + 0]) * f, __uint_as_float(r[8 * g + 1]) * f);
+                o.y = pack_bf16x2(__uint_as_float(r[8 * g + 2]) * f, __uint_as_float(r[8 * g + 3]) * f);
+                o.z = pack_bf16x2(__uint_as_float(r[8 * g + 4]) * f, __uint_as_float(r[8 * g + 5]) * f);
+                o.w = pack_bf16x2(__uint_as_float(r[8 * g + 6]) * f, __uint_as_float(r[8 * g + 7]) * f);
+                *reinterpret_cast<uint4*>(orow + 8 * g) = o;
+              }
+            }
           }
         }
+        if (w.kind != KIND_ORDINARY && p.LSE != nullptr && row < p.T)
+          p.LSE[(static_cast<size_t>(w.b) * p.H + w.h) * p.T + row] = 0.0f;
       }
-      if (p.LSE != nullptr && hh == 0 && row < p.T && ok)
-        p.LSE[(static_cast<size_t>(w.b) * p.H + w.h) * p.T + row] = lse;
-      tc_fence_before();
-      warp_arrive(o_free);
     }
   }
 
@@ -598,21 +790,27 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
   tc_fence_before();
   __syncthreads();
   SAF_SPAN(fwd128, 1);
-  if (warp == 9) tmem_dealloc(tmem, C::TMEM_COLS);
+  if (warp == 13) tmem_dealloc(tmem, C::TMEM_COLS);
+  if (tid == 0) {
+    // this CTA claims nothing more; the last CTA to get here rewinds the queue for the next launch
+    __threadfence();
+    if (atomicAdd(p.queue + 1, 1) == static_cast<int>(gridDim.x) - 1) {
+      p.queue[0] = 0;
+      p.queue[1] = 0;
+      __threadfence();
+    }
+  }
 }
 
 int fwd_smem_bytes(int D) { return D == 64 ? fwd64_smem_bytes() : FwdCfg<128>::SMEM; }
 
 cudaError_t launch_fwd(int D, const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv,
                        const CUtensorMap& mvt, const CUtensorMap& mo, const FwdParams& p, int grid, cudaStream_t st) {
-  cudaError_t e;
-  if (D == 64) {
-    return launch_fwd64(mq, mk, mv, mvt, mo, p, grid, st);   // head dimension 64 has its own kernel
-  } else {
-    e = cudaFuncSetAttribute(saf_fwd_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdCfg<128>::SMEM);
-    if (e != cudaSuccess) return e;
-    return launch_pdl(PDL_FWD, saf_fwd_kernel<128>, dim3(grid), dim3(320), FwdCfg<128>::SMEM, st, mq, mk, mv, mvt, p);
-  }
+  if (D == 64) return launch_fwd64(mq, mk, mv, mvt, mo, p, grid, st);   // head dimension 64 has its own kernel
+  cudaError_t e = cudaFuncSetAttribute(saf_fwd_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdCfg<128>::SMEM);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(PDL_FWD, saf_fwd_kernel<128>, dim3(grid), dim3(FwdCfg<128>::NTHREADS), FwdCfg<128>::SMEM, st, mq, mk, mv,
+                    mvt, p);
 }
 
 }  // namespace saf

@@ -50,6 +50,7 @@ cudaError_t launch_pdl(int which, void (*kernel)(KArgs...), dim3 grid, dim3 bloc
 constexpr int BLK = 128;            // query rows per item and keys per tile
 constexpr int KIND_ORDINARY = 0;
 constexpr int KIND_FROZEN = 1;
+constexpr int KIND_PAIR = 1 << 7;   // 128-wide forward: the item is query blocks blk - 1 and blk
 
 struct WorkItem { int32_t b, h, blk, kind; };
 
@@ -79,7 +80,7 @@ struct FwdParams {
   int nblkp;
   const WorkItem* items;            // grouped by CTA
   const int* cta_offsets;           // [grid+1]
-  // D = 64 forward: the items in queue order, claimed at run time.  queue[0] = next unclaimed item, queue[1] = CTAs
+  // The items in queue order, claimed at run time.  queue[0] = next unclaimed item, queue[1] = CTAs
   // that have finished; the last CTA to finish sets both back to zero for the next launch.
   const WorkItem* order;
   int n_items;
