@@ -88,6 +88,33 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, c
   return __all_sync(0xffffffffu, mbar_wait(bar, parity, w, site));
 }
 
+// The same waits with the clock and the give-up in one out-of-line function that is called every 64 polls.  Inlined at
+// each of its ~40 waits they made up a quarter of the 128-wide forward's code, which then did not fit the instruction
+// caches (the backward kernels are smaller and measured 2-4 % slower with this form: they keep the inline one).
+__device__ __noinline__ static bool wait_expired(volatile int* abort_flag, int* status_word, uint64_t limit_ns, uint64_t& t0,
+                                                 int site) {
+  if (*abort_flag) return true;
+  const uint64_t now = globaltimer_ns();
+  if (t0 == 0) {
+    t0 = now;
+  } else if (now - t0 > limit_ns) {
+    *abort_flag = 1;
+    atomicCAS(status_word, 0, (DEV_TIMEOUT << 24) | (site << 16) | (int)(blockIdx.x & 0xffff));
+    return true;
+  }
+  return false;
+}
+__device__ __forceinline__ bool mbar_wait_compact(uint64_t* bar, uint32_t parity, const WaitCtx& w, int site) {
+  uint64_t t0 = 0;
+  for (uint32_t spin = 1;; ++spin) {
+    if (mbar_try_wait(bar, parity)) return true;
+    if ((spin & 63u) == 0u && wait_expired(w.abort_flag, w.status_word, w.limit_ns, t0, site)) return false;
+  }
+}
+__device__ __forceinline__ bool mbar_wait_warp_compact(uint64_t* bar, uint32_t parity, const WaitCtx& w, int site) {
+  return __all_sync(0xffffffffu, mbar_wait_compact(bar, parity, w, site));
+}
+
 // ------------------------------------------------------------------ proxies / fences
 __device__ __forceinline__ void fence_proxy_async_smem() {   // generic-proxy smem writes -> async proxy (UMMA/TMA)
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -329,6 +356,33 @@ __device__ __forceinline__ float ex2_approx(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
+}
+// 2^x of two values (each <= 127) on the FMA pipes instead of the special-function unit: x = n + r with n the nearest
+// integer and |r| <= 1/2 (adding 1.5 * 2^23 rounds), 2^r by the degree-5 polynomial of least relative error on
+// [-1/2, 1/2] (Remez exchange in double precision: 7.5e-8; 2.1e-7 with the fp32 arithmetic below, the order of
+// ex2.approx itself), n added to the exponent field.  Arguments below -126 (masked keys) give 2^-126, not a flushed zero.
+__device__ __forceinline__ void ex2_poly2(uint64_t x2, float& y0, float& y1) {
+  float x0, x1;
+  upk2(x2, x0, x1);
+  x2 = pk2(fmaxf(x0, -126.0f), fmaxf(x1, -126.0f));
+  const uint64_t t2 = add2(x2, pk2(12582912.0f, 12582912.0f));
+  const uint64_t r2 = fma2(add2(t2, pk2(-12582912.0f, -12582912.0f)), pk2(-1.0f, -1.0f), x2);
+  uint64_t p2 = pk2(0.0013276472454890609f, 0.0013276472454890609f);
+  p2 = fma2(p2, r2, pk2(0.009675540961325169f, 0.009675540961325169f));
+  p2 = fma2(p2, r2, pk2(0.05550713092088699f, 0.05550713092088699f));
+  p2 = fma2(p2, r2, pk2(0.24022120237350464f, 0.24022120237350464f));
+  p2 = fma2(p2, r2, pk2(0.6931469440460205f, 0.6931469440460205f));
+  p2 = fma2(p2, r2, pk2(1.0000001192092896f, 1.0000001192092896f));
+  float t0, t1, p0, p1;
+  upk2(t2, t0, t1);
+  upk2(p2, p0, p1);
+  y0 = __uint_as_float(__float_as_uint(p0) + (__float_as_uint(t0) << 23));
+  y1 = __uint_as_float(__float_as_uint(p1) + (__float_as_uint(t1) << 23));
+}
+__device__ __forceinline__ float max3(float a, float b, float c) {   // one instruction
+  float d;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
 }
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {   // RNE; lo -> bits [0,16)
   uint32_t r;

@@ -65,6 +65,7 @@ struct FwdCfg {
   static constexpr int OFF_LINV = OFF_BAND + NS * 8192;       // [2][128] 1 / row sum
   static constexpr int OFF_BAR = OFF_LINV + 2 * 128 * 4;
   static constexpr int NRING = 4;                       // work-item records in flight
+  static constexpr int CLAIM_AHEAD = 4;
   static constexpr int NBAR = 2 * NS + 14 + 2 * NRING;
   static constexpr int OFF_RING = (OFF_BAR + NBAR * 8 + 16 + 15) / 16 * 16;
   static constexpr int SMEM = OFF_RING + NRING * 16 + 1024;   // + slack for 1024-byte alignment
@@ -90,7 +91,7 @@ template <int NRING>
 __device__ __forceinline__ bool ring_take(const int4* ring, uint64_t* ring_full, uint64_t* ring_empty, uint32_t n,
                                           const WaitCtx& wc, ItemView& v) {
   const uint32_t slot = n % NRING;
-  if (!mbar_wait_warp(ring_full + slot, (n / NRING) & 1, wc, SITE_RING_FULL)) return false;
+  if (!mbar_wait_warp_compact(ring_full + slot, (n / NRING) & 1, wc, SITE_RING_FULL)) return false;
   const int4 raw = ring[slot];
   warp_arrive(ring_empty + slot);
   v.b = raw.x;
@@ -182,28 +183,39 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
         uint32_t n = 0;                            // ring position
         uint32_t nq0 = 0, nq1 = 0;                 // uses of the two Q areas
         bool ok = true;
-        for (uint32_t nclaim = 0; ok; ++nclaim) {
-          // claim the next item of the queue and publish it to the other roles
+        // Claim the next item of the queue and publish it to the other roles.  Claimed CLAIM_AHEAD tiles before the current
+        // item's last: the claim's two global round trips and the loads of Q_0 and K_0 behind it then fit under the
+        // tiles that are left (claimed behind the item's last load they cost ~13000 clk an item).
+        int4 next;
+        uint32_t nclaim = 0;
+        bool claimed = false;
+        auto claim = [&] {
           const uint32_t slot = nclaim % C::NRING;
-          ok = mbar_wait(ring_empty + slot, ((nclaim / C::NRING) & 1) ^ 1, wc, SITE_RING_EMPTY);
-          if (!ok) break;
+          ok = mbar_wait_compact(ring_empty + slot, ((nclaim / C::NRING) & 1) ^ 1, wc, SITE_RING_EMPTY);
+          if (!ok) return;
+          ++nclaim;
+          claimed = true;
           const int idx = atomicAdd(p.queue, 1);
-          int4 rec = make_int4(0, 0, 0, RING_END);
-          bool fast = false;
+          next = make_int4(0, 0, 0, RING_END);
           if (idx < p.n_items) {
-            rec = __ldg(reinterpret_cast<const int4*>(p.order + idx));
-            fast = (rec.w & 0x7f) != KIND_ORDINARY && p.band_f != nullptr && __ldg(p.fast_ok + rec.y) != 0 &&
-                   __ldg(p.ovf + rec.y) != p.call_id;
-            if (fast) rec.w |= RING_FAST;
+            next = __ldg(reinterpret_cast<const int4*>(p.order + idx));
+            if ((next.w & 0x7f) != KIND_ORDINARY && p.band_f != nullptr && __ldg(p.fast_ok + next.y) != 0 &&
+                __ldg(p.ovf + next.y) != p.call_id)
+              next.w |= RING_FAST;
           }
-          ring[slot] = rec;
+          ring[slot] = next;
           mbar_arrive(ring_full + slot);                 // (release: the record is visible to whoever sees the phase)
-          if (idx >= p.n_items) break;
+        };
+        for (;;) {
+          if (!claimed) claim();
+          if (!ok || next.w < 0) break;
+          const int4 rec = next;
+          claimed = false;
           const int b = rec.x, h = rec.y, n1 = rec.z + 1;
-          const bool pair = (rec.w & KIND_PAIR) != 0;
+          const bool fast = (rec.w & RING_FAST) != 0, pair = (rec.w & KIND_PAIR) != 0;
           auto load_kv = [&](const CUtensorMap* m, int j, int head) {
             const uint32_t s = n % C::NS;
-            ok = mbar_wait(kv_empty + s, ((n / C::NS) & 1) ^ 1, wc, SITE_KV_EMPTY);
+            ok = mbar_wait_compact(kv_empty + s, ((n / C::NS) & 1) ^ 1, wc, SITE_KV_EMPTY);
             if (!ok) return;
             mbar_expect_tx(kv_full + s, C::TILE_BYTES);
             for (int pn = 0; pn < C::NPANEL; ++pn)
@@ -216,7 +228,7 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
             const uint8_t* bands = static_cast<const uint8_t*>(p.band_f) + static_cast<size_t>(h) * p.nblkp * 4096;
             for (int j = 0; j < n1; ++j) {
               const uint32_t s = n % C::NS;
-              ok = mbar_wait(kv_empty + s, ((n / C::NS) & 1) ^ 1, wc, SITE_KV_EMPTY);
+              ok = mbar_wait_compact(kv_empty + s, ((n / C::NS) & 1) ^ 1, wc, SITE_KV_EMPTY);
               if (!ok) break;
               const int d = n1 - 1 - j;
               const bool two = pair && d > 0;
@@ -227,7 +239,10 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
               bulk_load(smem + C::OFF_BAND + s * 8192 + 4096, bands + static_cast<size_t>(d) * 4096, 4096, kv_full + s);
               if (two) bulk_load(smem + C::OFF_BAND + s * 8192, bands + static_cast<size_t>(d - 1) * 4096, 4096, kv_full + s);
               ++n;
+              if (!claimed && j + C::CLAIM_AHEAD >= n1) claim();
+              if (!ok) break;
             }
+            if (!ok) break;
             continue;
           }
           const int hv = h / p.kv_group;
@@ -235,7 +250,7 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
             const int hq = p.qslot ? p.qslot[h] : h, hk = p.qslot ? hq : hv;
             // Q_0 and K_0 first: block 0's first scores are issued before this item's predecessor has finished with Q_1
             if (pair) {
-              ok = mbar_wait(q_empty, (nq0 & 1) ^ 1, wc, SITE_Q_EMPTY);
+              ok = mbar_wait_compact(q_empty, (nq0 & 1) ^ 1, wc, SITE_Q_EMPTY);
               if (!ok) break;
               mbar_expect_tx(q_full, C::TILE_BYTES);
               for (int pn = 0; pn < C::NPANEL; ++pn)
@@ -244,24 +259,26 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
             }
             load_kv(&mk, 0, hk);
             if (!ok) break;
-            ok = mbar_wait(q_empty + 1, (nq1 & 1) ^ 1, wc, SITE_Q_EMPTY);
+            ok = mbar_wait_compact(q_empty + 1, (nq1 & 1) ^ 1, wc, SITE_Q_EMPTY);
             if (!ok) break;
             mbar_expect_tx(q_full + 1, C::TILE_BYTES);
             for (int pn = 0; pn < C::NPANEL; ++pn)
               tma_load_4d(smem + C::OFF_Q + C::TILE_BYTES + pn * C::PANEL_BYTES, &mq, q_full + 1, pn * 64, rec.z * BLK, hq, b);
             ++nq1;
             load_kv(&mv, 0, hv);
-            for (int j = 1; j < n1 && ok; ++j) {
+            for (int j = 1;; ++j) {
+              if (ok && !claimed && j + C::CLAIM_AHEAD > n1) claim();
+              if (j == n1 || !ok) break;
               load_kv(&mk, j, hk);
               if (ok) load_kv(&mv, j, hv);
             }
           } else {
             // general frozen form: the Q areas hold the tables of the softmax warps; an area counts as used by this item
             if (pair) {
-              ok = mbar_wait(q_empty, (nq0 & 1) ^ 1, wc, SITE_Q_EMPTY);
+              ok = mbar_wait_compact(q_empty, (nq0 & 1) ^ 1, wc, SITE_Q_EMPTY);
               ++nq0;
             }
-            if (ok) ok = mbar_wait(q_empty + 1, (nq1 & 1) ^ 1, wc, SITE_Q_EMPTY);
+            if (ok) ok = mbar_wait_compact(q_empty + 1, (nq1 & 1) ^ 1, wc, SITE_Q_EMPTY);
             ++nq1;
             for (int j = 0; j < n1 && ok; ++j) load_kv(&mv, j, hv);
           }
@@ -287,9 +304,9 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
       const uint64_t d_band = umma_smem_desc(sb, 128, 128, UMMA_LAYOUT_NONE);
       const uint32_t lo_b = desc_lo(d_band), hi_b = desc_hi(d_band);
       auto kv_wait = [&](uint32_t pos) {
-        return mbar_wait_warp(kv_full + pos % C::NS, (pos / C::NS) & 1, wc, SITE_KV_FULL);
+        return mbar_wait_warp_compact(kv_full + pos % C::NS, (pos / C::NS) & 1, wc, SITE_KV_FULL);
       };
-      // (all callers sit between two warp-uniform points; `leader` alone issues)
+      // (the warp converges behind every burst: without that the two bursts of block 0 took 1560 clk instead of 1050)
       auto issue_qk = [&](uint32_t t, uint32_t pos) {
         const uint32_t q_lo = lo_k + ((C::OFF_Q + t * C::TILE_BYTES) >> 4);
         const uint32_t k_lo = lo_k + ((C::OFF_KV + (pos % C::NS) * C::TILE_BYTES) >> 4);
@@ -302,6 +319,7 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
           }
           umma_commit(s_full + t);
         }
+        __syncwarp();
       };
       auto issue_pv = [&](uint32_t t, uint32_t pos, uint32_t acc0) {
         const uint32_t v_lo = lo_m + ((C::OFF_KV + (pos % C::NS) * C::TILE_BYTES) >> 4);
@@ -311,9 +329,17 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
             umma_ts2(tmem + C::COL_O + D * t, tmem + C::COL_S + 128 * t + 8 * kc, v_lo + 128 * kc, hi_m, idesc_o,
                      kc > 0 ? 1u : acc0);
         }
+        __syncwarp();
       };
+      // (One copy of each burst and wait, the block t a run-time value: with the bursts inlined per block and case the
+      // kernel's code was 133 KB, and every item boundary fetched instructions for ~10000 clk.)
       uint32_t n = 0, nrec = 0;
-      uint32_t nqf0 = 0, nqf1 = 0, np0 = 0, np1 = 0, no0 = 0, no1 = 0;   // phases of q_full, p_full, o_free by block
+      uint32_t ph_q = 0, ph_p = 0, ph_o = 3;       // bit t: parity of the next phase of q_full[t], p_full[t], o_free[t]
+      auto wait_t = [&](uint64_t* bar, uint32_t& ph, uint32_t t, int site) {
+        const bool r = mbar_wait_warp_compact(bar + t, (ph >> t) & 1, wc, site);
+        ph ^= 1u << t;
+        return r;
+      };
       bool early = false;                          // block 0's first scores of `cur` are already issued
       ItemView cur;
       bool ok = ring_take<C::NRING>(ring, ring_full, ring_empty, nrec++, wc, cur);
@@ -322,170 +348,104 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
         bool have_next = false;
         const int n0 = cur.n0, n1 = cur.n1;
         if (cur.fast) {
-          for (int j = 0; j < n1 && ok; ++j) {
+          for (int j = 0; j < n1 && ok; ++j, ++n) {
             ok = kv_wait(n);
-            if (!ok) break;
             const uint32_t s = n % C::NS;
             const uint32_t band_lo = lo_b + ((C::OFF_BAND + s * 8192) >> 4);
             const uint32_t v_lo = lo_m + ((C::OFF_KV + s * C::TILE_BYTES) >> 4);
             const uint32_t acc0 = j > 0 ? 1u : 0u;
-            if (j < n0) {
-              if (j == 0) {
-                ok = mbar_wait_warp(o_free, (no0++ & 1) ^ 1, wc, SITE_O_FREE);
-                if (!ok) break;
-              }
+#pragma unroll 1
+            for (uint32_t t = j < n0 ? 0 : 1; t < 2 && ok; ++t) {
+              if (j == 0) ok = wait_t(o_free, ph_o, t, SITE_O_FREE);
+              if (!ok) break;
               tc_fence_after();
               if (leader) {
 #pragma unroll
                 for (int kc = 0; kc < 8; ++kc)
-                  umma_ss2(tmem + C::COL_O, band_lo + 16 * kc, hi_b, v_lo + 128 * kc, hi_m, idesc_hk, kc > 0 ? 1u : acc0);
-                if (j == n0 - 1) umma_commit(o_full);
+                  umma_ss2(tmem + C::COL_O + D * t, band_lo + 256 * t + 16 * kc, hi_b, v_lo + 128 * kc, hi_m, idesc_hk,
+                           kc > 0 ? 1u : acc0);
+                if (j == (t ? n1 : n0) - 1) umma_commit(o_full + t);
               }
               __syncwarp();
             }
-            if (j == 0) {
-              ok = mbar_wait_warp(o_free + 1, (no1++ & 1) ^ 1, wc, SITE_O_FREE);
-              if (!ok) break;
-            }
-            tc_fence_after();
-            if (leader) {
-#pragma unroll
-              for (int kc = 0; kc < 8; ++kc)
-                umma_ss2(tmem + C::COL_O + D, band_lo + 256 + 16 * kc, hi_b, v_lo + 128 * kc, hi_m, idesc_hk,
-                         kc > 0 ? 1u : acc0);
-              umma_commit(kv_empty + s);
-              if (j == n1 - 1) umma_commit(o_full + 1);
-            }
-            __syncwarp();
-            ++n;
-          }
-        } else if (cur.kind == KIND_ORDINARY) {
-          if (n0 > 0 && !early) {
-            ok = mbar_wait_warp(q_full, nqf0++ & 1, wc, SITE_Q_FULL) && kv_wait(n);
-            if (!ok) break;
-            tc_fence_after();
-            issue_qk(0, n);
-            if (leader && n0 == 1) umma_commit(q_empty);
+            if (leader) umma_commit(kv_empty + s);
             __syncwarp();
           }
-          early = false;
-          ok = mbar_wait_warp(q_full + 1, nqf1++ & 1, wc, SITE_Q_FULL) && kv_wait(n);
-          if (!ok) break;
-          tc_fence_after();
-          issue_qk(1, n);
-          if (leader) {
-            umma_commit(kv_empty + n % C::NS);
-            if (n1 == 1) umma_commit(q_empty + 1);
-          }
-          __syncwarp();
-          for (int j = 0; j < n1 && ok; ++j) {
-            const uint32_t pv = n + 2 * j + 1, pk = pv + 1;        // ring positions of V_j and K_{j+1}
-            const bool more1 = j + 1 < n1;
-            const uint32_t acc0 = j > 0 ? 1u : 0u;
-            // the tiles' loads land long before P is ready: test their barriers first, so that only one test
-            // stands between "P is ready" and the MMAs that wait for it
-            ok = kv_wait(pv) && (!more1 || kv_wait(pk));
-            if (!ok) break;
-            if (j < n0) {
-              if (j == 0) ok = mbar_wait_warp(o_free, (no0++ & 1) ^ 1, wc, SITE_O_FREE);
-              if (ok) ok = mbar_wait_warp(p_full, np0++ & 1, wc, SITE_P_FULL);
+        } else {
+          const bool ord = cur.kind == KIND_ORDINARY;
+          if (ord) {
+            // first scores
+#pragma unroll 1
+            for (uint32_t t = n0 > 0 && !early ? 0 : 1; t < 2 && ok; ++t) {
+              ok = wait_t(q_full, ph_q, t, SITE_Q_FULL) && kv_wait(n);
               if (!ok) break;
               tc_fence_after();
-              TRF(0, 2);
-              issue_pv(0, pv, acc0);
-              if (j + 1 < n0) {
-                issue_qk(0, pk);                         // executes after P V: same thread, in order
-                if (leader && j + 2 == n0) umma_commit(q_empty);
-                __syncwarp();
-                TRF(0, 3);
-              } else {
-                if (leader) umma_commit(o_full);
-                __syncwarp();
-                // block 0 is through: its first scores of the next item go out now
-                ok = ring_take<C::NRING>(ring, ring_full, ring_empty, nrec++, wc, nxt);
-                if (!ok) break;
-                have_next = true;
-                if (nxt.kind == KIND_ORDINARY && nxt.n0 > 0) {
-                  const uint32_t pn = n + 2 * n1;
-                  ok = mbar_wait_warp(q_full, nqf0++ & 1, wc, SITE_Q_FULL) && kv_wait(pn);
-                  if (!ok) break;
-                  tc_fence_after();
-                  issue_qk(0, pn);
-                  if (leader && nxt.n0 == 1) umma_commit(q_empty);
-                  __syncwarp();
-                  early = true;
-                }
-              }
+              issue_qk(t, n);
+              if (leader && (t ? n1 : n0) == 1) umma_commit(q_empty + t);
             }
-            if (j == 0) {
-              ok = mbar_wait_warp(o_free + 1, (no1++ & 1) ^ 1, wc, SITE_O_FREE);
-              if (!ok) break;
-            }
-            ok = mbar_wait_warp(p_full + 1, np1++ & 1, wc, SITE_P_FULL);
-            if (!ok) break;
-            tc_fence_after();
-            TRF(0, 4);
-            issue_pv(1, pv, acc0);
-            if (leader) umma_commit(kv_empty + pv % C::NS);
-            __syncwarp();
-            if (more1) {
-              issue_qk(1, pk);
-              if (leader) {
-                umma_commit(kv_empty + pk % C::NS);
-                if (j + 2 == n1) umma_commit(q_empty + 1);
-              }
-              TRF(0, 5);
-            } else if (leader) {
-              umma_commit(o_full + 1);
-            }
-            __syncwarp();
-          }
-          n += 2 * n1;
-        } else {
-          // general frozen form: P^ written by the softmax warps, one P V per block and tile; s_full says that a
-          // block's P^ buffer may be written (everything issued before has completed)
-          if (leader) {
+            if (leader) umma_commit(kv_empty + n % C::NS);
+            early = false;
+          } else if (leader) {
+            // general frozen form: P^ written by the softmax warps, one P V per block and tile; s_full says that a
+            // block's P^ buffer may be written (everything issued before has completed)
             if (n0 > 0) umma_commit(s_full);
             umma_commit(s_full + 1);
           }
           __syncwarp();
           for (int j = 0; j < n1 && ok; ++j) {
-            ok = kv_wait(n);
-            if (!ok) break;
+            const uint32_t pv = ord ? n + 2 * j + 1 : n + j;       // ring position of V_j; K_{j+1} follows
             const uint32_t acc0 = j > 0 ? 1u : 0u;
-            if (j < n0) {
-              if (j == 0) ok = mbar_wait_warp(o_free, (no0++ & 1) ^ 1, wc, SITE_O_FREE);
-              if (ok) ok = mbar_wait_warp(p_full, np0++ & 1, wc, SITE_P_FULL);
+            // the tiles' loads land long before P is ready: test their barriers first, so that only one test
+            // stands between "P is ready" and the MMAs that wait for it
+            ok = kv_wait(pv) && (!ord || j + 1 == n1 || kv_wait(pv + 1));
+#pragma unroll 1
+            for (uint32_t t = j < n0 ? 0 : 1; t < 2 && ok; ++t) {
+              const int nt = t ? n1 : n0;
+              if (j == 0) ok = wait_t(o_free, ph_o, t, SITE_O_FREE);
+              if (ok) ok = wait_t(p_full, ph_p, t, SITE_P_FULL);
               if (!ok) break;
               tc_fence_after();
-              issue_pv(0, n, acc0);
-              if (leader) {
-                if (j + 1 < n0) {
-                  umma_commit(s_full);
-                } else {
-                  umma_commit(o_full);
-                  umma_commit(q_empty);
+              TRF(0, 2 + 2 * t);
+              issue_pv(t, pv, acc0);
+              if (leader && t == 1) umma_commit(kv_empty + pv % C::NS);
+              uint32_t pos = pv + 1;
+              bool qk = ord && j + 1 < nt, last_qk = j + 2 == nt;
+              if (j + 1 == nt) {
+                if (leader) {
+                  umma_commit(o_full + t);
+                  if (!ord) umma_commit(q_empty + t);
+                }
+                __syncwarp();
+                if (ord && t == 0) {
+                  // block 0 is through: its first scores of the next item go out now
+                  ok = ring_take<C::NRING>(ring, ring_full, ring_empty, nrec++, wc, nxt);
+                  if (!ok) break;
+                  have_next = true;
+                  if (nxt.kind == KIND_ORDINARY && nxt.n0 > 0) {
+                    pos = n + 2 * n1;
+                    ok = wait_t(q_full, ph_q, 0, SITE_Q_FULL) && kv_wait(pos);
+                    if (!ok) break;
+                    tc_fence_after();
+                    early = qk = true;
+                    last_qk = nxt.n0 == 1;
+                  }
+                }
+              } else if (!ord && leader) {
+                umma_commit(s_full + t);
+              }
+              __syncwarp();
+              if (qk) {
+                issue_qk(t, pos);                        // executes after P V: same thread, in order
+                if (leader) {
+                  if (t == 1) umma_commit(kv_empty + pos % C::NS);
+                  if (last_qk) umma_commit(q_empty + t);
                 }
               }
               __syncwarp();
+              TRF(0, 3 + 2 * t);
             }
-            if (j == 0) ok = mbar_wait_warp(o_free + 1, (no1++ & 1) ^ 1, wc, SITE_O_FREE);
-            if (ok) ok = mbar_wait_warp(p_full + 1, np1++ & 1, wc, SITE_P_FULL);
-            if (!ok) break;
-            tc_fence_after();
-            issue_pv(1, n, acc0);
-            if (leader) {
-              umma_commit(kv_empty + n % C::NS);
-              if (j + 1 < n1) {
-                umma_commit(s_full + 1);
-              } else {
-                umma_commit(o_full + 1);
-                umma_commit(q_empty + 1);
-              }
-            }
-            __syncwarp();
-            ++n;
           }
+          n += ord ? 2 * n1 : n1;
         }
         if (!ok) break;
         if (have_next) cur = nxt;
@@ -528,12 +488,11 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
         for (int j = 0; j < nt; ++j) {
           if (q4 == 0) TRF(1 + t, 11);
           // (the completion of this score MMA also covers the block's previous P V MMA, issued before it)
-          if (!mbar_wait_warp(s_full + t, ns & 1, wc, SITE_S_FULL)) ok = false;
+          if (!mbar_wait_warp_compact(s_full + t, ns & 1, wc, SITE_S_FULL)) ok = false;
           ++ns;
           tc_fence_after();
           if (q4 == 0) TRF(1 + t, 12);
           uint32_t r[4][32];
-          float mx0, mx1;
           tmem_ld32(t_s, r[0]);
           tmem_ld32(t_s + 32, r[1]);
           tmem_wait_ld();
@@ -544,13 +503,18 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
             for (int e = 0; e < 64; ++e)
               if (e > rowl) r[e >> 5][e & 31] = 0xff800000u;          // -inf above the diagonal
           }
-          mx0 = __uint_as_float(r[0][0]);
-          mx1 = __uint_as_float(r[1][0]);
+          // (four chains of three-input maxima: two chains of 64 two-input ones cost ~300 clk of latency a tile)
+          float mx[4];
 #pragma unroll
-          for (int e = 1; e < 32; ++e) {
-            mx0 = fmaxf(mx0, __uint_as_float(r[0][e]));
-            mx1 = fmaxf(mx1, __uint_as_float(r[1][e]));
+          for (int k = 0; k < 2; ++k) {
+            mx[2 * k] = fmaxf(__uint_as_float(r[k][0]), __uint_as_float(r[k][1]));
+            mx[2 * k + 1] = fmaxf(__uint_as_float(r[k][2]), __uint_as_float(r[k][3]));
           }
+#pragma unroll
+          for (int e = 4; e < 32; e += 4)
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+              mx[k] = max3(mx[k], __uint_as_float(r[k >> 1][e + 2 * (k & 1)]), __uint_as_float(r[k >> 1][e + 2 * (k & 1) + 1]));
           tmem_wait_ld();
           if (j == blk) {
 #pragma unroll
@@ -558,12 +522,12 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
               if (e > rowl) r[e >> 5][e & 31] = 0xff800000u;
           }
 #pragma unroll
-          for (int e = 0; e < 32; ++e) {
-            mx0 = fmaxf(mx0, __uint_as_float(r[2][e]));
-            mx1 = fmaxf(mx1, __uint_as_float(r[3][e]));
-          }
+          for (int e = 0; e < 32; e += 4)
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+              mx[k] = max3(mx[k], __uint_as_float(r[2 + (k >> 1)][e + 2 * (k & 1)]), __uint_as_float(r[2 + (k >> 1)][e + 2 * (k & 1) + 1]));
           if (q4 == 0) TRF(1 + t, 13);
-          const float m_new = fmaxf(m_ref, fmaxf(mx0, mx1) * c);   // finite: key 0 is visible to every row
+          const float m_new = fmaxf(m_ref, fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * c);   // finite: key 0 is visible to every row
           if (j == 0) {
             m_ref = m_new;
           } else {
@@ -573,7 +537,7 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
               l2a = mul2(l2a, pk2(f, f));
               l2b = mul2(l2b, pk2(f, f));
               if (need) m_ref = m_new;
-#pragma unroll
+#pragma unroll 1
               for (int cc = 0; cc < D / 16; ++cc) {
                 uint32_t o[16];
                 tmem_ld16(t_o + 16 * cc, o);
@@ -613,7 +577,7 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
         upk2(l2b, lc, ld);
         const float l = (la + lb) + (lc + ld);
         // the epilogue has read the previous item's row sums once it has released O_t
-        if (nof > 0 && !mbar_wait_warp(o_free + t, (nof - 1) & 1, wc, SITE_O_FREE)) ok = false;
+        if (nof > 0 && !mbar_wait_warp_compact(o_free + t, (nof - 1) & 1, wc, SITE_O_FREE)) ok = false;
         linv[t * 128 + rowl] = 1.0f / l;
         warp_arrive(l_full + t);
         if (p.LSE != nullptr && row < p.T && ok)
@@ -633,7 +597,7 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
         bool leave = false;
         for (int j = 0; j < nt; ++j) {
           // previous P^ tile consumed (first tile: everything issued before this item has completed)
-          if (!mbar_wait_warp(s_full + t, ns & 1, wc, SITE_S_FULL)) ok = false;
+          if (!mbar_wait_warp_compact(s_full + t, ns & 1, wc, SITE_S_FULL)) ok = false;
           ++ns;
           tc_fence_after();
           // previous tile's table readers are done; the four warps also agree whether to go on
@@ -675,7 +639,7 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
           rband[wt + 128] = ex2_approx(r2[1] - mr);
           // (agreement on the form: the factorised one would overflow or flush for some row)
           const bool exact = named_bar_or(wg_bar2, 128, ew > 100.0f);
-#pragma unroll
+#pragma unroll 1
           for (int cc = 0; cc < 4; ++cc) {
             uint32_t pk[16];
             if (!exact) {
@@ -734,16 +698,16 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
           row = blk * BLK + 127 - rowl;                // tensor-core form: lane m holds query 127-m, scaled by w(i)
           f = (row < p.T) ? p.wvec[static_cast<size_t>(w.h) * p.Tp + row] * (1.0f / (HK_BAND_SCALE * HK_A_SCALE)) : 0.0f;
         } else if (w.kind == KIND_ORDINARY) {
-          ok = mbar_wait_warp(l_full + t, (t == 0 ? nl0++ : nl1++) & 1, wc, SITE_L_FULL);
+          ok = mbar_wait_warp_compact(l_full + t, (t == 0 ? nl0++ : nl1++) & 1, wc, SITE_L_FULL);
           if (!ok) break;
           f = linv[t * 128 + rowl];
         }
-        ok = mbar_wait_warp(o_full + t, (t == 0 ? nof0++ : nof1++) & 1, wc, SITE_O_FULL);
+        ok = mbar_wait_warp_compact(o_full + t, (t == 0 ? nof0++ : nof1++) & 1, wc, SITE_O_FULL);
         if (!ok) break;
         tc_fence_after();
         const uint32_t t_o = tmem + lane_base + C::COL_O + D * t;
         const int64_t off = w.b * p.o_strides[0] + w.h * p.o_strides[1] + static_cast<int64_t>(row) * p.o_strides[2];
-#pragma unroll
+#pragma unroll 1
         for (int cc = 0; cc < D / 32; ++cc) {
           uint32_t r[32];
           tmem_ld32(t_o + 32 * cc, r);
