@@ -203,6 +203,14 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
                 __ldg(p.ovf + next.y) != p.call_id)
               next.w |= RING_FAST;
           }
+          if (next.w >= 0 && (next.w & 0x7f) == KIND_ORDINARY) {
+            // (its Q tiles are read by no other item, so nobody has brought them into L2)
+            const int hq = p.qslot ? p.qslot[next.y] : next.y;
+            for (int pn = 0; pn < C::NPANEL; ++pn) {
+              if (next.w & KIND_PAIR) tma_prefetch_4d(&mq, pn * 64, (next.z - 1) * BLK, hq, next.x);
+              tma_prefetch_4d(&mq, pn * 64, next.z * BLK, hq, next.x);
+            }
+          }
           ring[slot] = next;
           mbar_arrive(ring_full + slot);                 // (release: the record is visible to whoever sees the phase)
         };
