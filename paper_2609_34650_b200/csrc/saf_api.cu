@@ -841,17 +841,14 @@ int saf_hybrid_attn_bwd(saf_ctx* ctx, const saf_problem* p, const void* Q, const
     mq = mdo; mk = mdo; mv = mdo;
   }
   if (p->D != 64) {
-    // ---- 128-wide kernel: Q / dO travel as 64-row half tiles, dK / dV leave with plain stores
-    CUtensorMap mqh = mdo, mdoh, mdoth, mdq128;
-    if ((rc = make_map(ctx, &mdoh, dO, p, p->o_strides, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 0, 64))) return rc;
-    if (no > 0 && (rc = make_map(ctx, &mqh, Q, p, p->q_strides, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, nqh, 64))) return rc;
-    mdoth = mdoh;
+    // ---- 128-wide kernel: dK / dV leave with plain stores
+    CUtensorMap mdot = mdo, mdq128;
     {
       const cuuint64_t Dd = static_cast<cuuint64_t>(p->D), Tt = static_cast<cuuint64_t>(p->T);
       const cuuint64_t Hq = static_cast<cuuint64_t>(std::max(nqh, 1));
       cuuint64_t dims[4] = {Dd, Tt, Hq, static_cast<cuuint64_t>(p->B)};
       cuuint64_t gs[3] = {Dd * 4, Tt * Dd * 4, Tt * Dd * 4 * Hq};
-      cuuint32_t box[4] = {32, BLK, 1, 1};
+      cuuint32_t box[4] = {32, 32, 1, 1};              // (every drain warp reduces the rows of its own lane quarter)
       cuuint32_t es[4] = {1, 1, 1, 1};
       if (ctx->encode(&mdq128, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, dqacc, dims, gs, box, es,
                       CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
@@ -862,7 +859,7 @@ int saf_hybrid_attn_bwd(saf_ctx* ctx, const saf_problem* p, const void* Q, const
     bp.band_b = nullptr; bp.avec = nullptr; bp.fast_ok = nullptr; bp.hord = nullptr; bp.ovf = nullptr; bp.call_id = 0;
     bp.nblkp = (p->Tp + 127) / 128;
     if (tensor_form) {
-      if ((rc = make_map_contig(ctx, &mdoth, ctx->dot_buf.ptr, p, nf, 64))) return rc;
+      if ((rc = make_map_contig(ctx, &mdot, ctx->dot_buf.ptr, p, nf))) return rc;
       bp.band_b = ctx->pat_bandb.ptr;
       bp.avec = static_cast<const float*>(ctx->pat_avec.ptr);
       bp.fast_ok = fz.pat_ok;
@@ -889,7 +886,7 @@ int saf_hybrid_attn_bwd(saf_ctx* ctx, const saf_problem* p, const void* Q, const
     bp.wait_limit_ns = ctx->wait_limit_ns;
     {
       ScopedTimer timer(ctx, SAF_KERNEL_BWD, st);
-      if (launch_bwd128(mk, mv, mqh, mdoh, mdoth, mdq128, bp, grid, st) != cudaSuccess) return SAF_ERR_CUDA;
+      if (launch_bwd128(mk, mv, mq, mdo, mdot, mdq128, bp, grid, st) != cudaSuccess) return SAF_ERR_CUDA;
     }
     if (!grad_f32) {
       ScopedTimer timer(ctx, SAF_KERNEL_BWD_FINALIZE, st);

@@ -1,29 +1,46 @@
 // Backward of the hybrid causal attention layer on sm_100a, head dimension 128 (96 runs here too: TMA zero-fills
-// features 96..127): one persistent kernel, one work item per (batch, head, 128-key block J), looping over
-// 64-query half tiles u of the query blocks I >= J.
+// features 96..127): one persistent kernel, one work item per (batch, head, 128-key block J), looping over the
+// 128-query tiles I >= J.  TMEM (512 columns): dV 128, dK 128, X = S^T then P^T, Y = dP^T then dQ.
+//   S(t)  = K_J Q_t^T -> X          dP(t) = V_J dO_t^T -> Y                      (operands in smem)
+//   P^T   = exp2(c S^T - lse) over X (bf16 pairs),  dS^T = P^T o (dP^T - delta) -> smem
+//   dV_J += P^T dO_t (A from TMEM),  dQ_t = dS K_J -> Y (A = the smem dS^T tile read M-major),  dK_J += dS^T Q_t (A = the
+//   same smem tile, K-major)
+// Issue order of a tile: dP(t) | dV(t), S(t+1) | dQ(t), dK(t).  S(t+1) is queued behind the MMA that consumes P(t), so
+// the exponentials of tile t+1 run while tile t's dS, dQ and dK are in flight, and dK(t) runs while dQ(t) is drained
+// out of Y; MMAs of one thread execute in order, which is all that protects X, Y and the dS tile.
 //
-// With 128 features the two gradient accumulators of a key block take half of TMEM, so there is room for one
-// S^T / dP^T buffer only (64 query columns) and the half tiles go through it one after the other:
-//   A(u):       S'^T = K_J Q_u^T + 1 (-LSE/scale)^T,  dP'^T = V_J dO_u^T + 1 (-delta)^T      (operands in smem; the
-//               row terms ride on one extra 16-wide reduction step, as at head dimension 64)
-//   compute(u): P^T = exp2(c S'^T), dS^T = P^T o dP'^T (bf16 back into the buffer's own columns; dS^T also to smem)
-//   B(u):       dV_J += P^T dO_u,  dK_J += dS^T Q_u       (A from TMEM, 128-wide MMAs), then A(u+1) right behind it
-//   C(t):       dQ_t = dS K_J once per full tile           (A = the smem dS^T tile read M-major, B = K_J MN-major)
-// Appendix E.2 (key-block programs accumulate dV and dK; dQ here comes out of the same loop and is accumulated
-// across key blocks with TMA reduce-adds).  Frozen items (Sec. 3.3: dV = P^^T dO, no query/key gradients) use the
-// tensor-core form (Hankel band x scaled dO, see the forward) or generate P^^T half tiles with one exponential per
-// element.
+// What bounds it: the five MMAs of a tile are 2900 clk of tensor pipe (512 with A in TMEM, 600 with both operands in
+// smem) and the chain through Y (dP, dS, dQ, drain) is about as long.  The 64-query half tiles that this replaces went
+// through one S / dP buffer in sequence, two full round trips a tile.
 //
-// CTA = 704 threads: warps 0-15 compute (TMEM lane = key row; four warps per lane quarter, 16 query columns each),
-// warps 16-19 dQ drain, warp 20 TMA producer, warp 21 tcgen05 issuer and TMEM owner.
-// TMEM columns: [0,128) dV, [128,256) dK, [256,320) S^T / P^T, [320,384) dP^T / dS^T, [384,512) dQ.
-// Q and dO travel as 64-row half tiles through a ring of two stages, so the next half tile loads while the
-// current one is in the tensor core.  Every wait is bounded.
+// Row terms: LSE and delta reach the compute warps as fp32 vectors with each Q tile (columns of S^T are queries, so a
+// value is a broadcast load).  Appendix E.2 (key-block programs accumulate dV and dK; dQ here comes out of the same loop
+// and is accumulated across key blocks with TMA reduce-adds).  Frozen items (Sec. 3.3: dV = P^^T dO, no query/key
+// gradients) use the tensor-core form (Hankel band x scaled dO, see the forward) or generate P^^T tiles with one
+// exponential per element; their dO tiles go through the Q stages.
+//
+// CTA = 896 threads: warps 0-15 compute (TMEM lane = key row; four warps per lane quarter, 32 query columns each),
+// warps 16-23 dQ drain (two per lane quarter, 64 feature columns each), warp 24 TMA producer, warp 25 tcgen05 issuer and
+// TMEM owner.  Registers: 512 x 80 + 256 x 72 + 128 x 40 = the 896 x 72 of the launch.  Every wait is bounded.
 #include <cuda_bf16.h>
 #include "ptx.cuh"
 #include "saf_internal.h"
 
 SAF_SPAN_DEFINE(bwd128)
+
+#ifdef SAF_TRACE
+__device__ unsigned long long g_saf_trace_bwd128[3][16384];
+#define TRB(role, id)                                                                                  \
+  do {                                                                                                 \
+    if (blockIdx.x == 0 && (threadIdx.x & 31) == 0 && tr_n < 16380)                                    \
+      g_saf_trace_bwd128[role][tr_n++] = (static_cast<unsigned long long>(id) << 48) | (clock64() & 0xffffffffffffULL); \
+  } while (0)
+extern "C" int saf_debug_read_trace_bwd128(unsigned long long* out) {
+  return static_cast<int>(cudaMemcpyFromSymbol(out, g_saf_trace_bwd128, sizeof(g_saf_trace_bwd128)));
+}
+#else
+#define TRB(role, id)
+#endif
 
 namespace saf {
 
@@ -33,28 +50,26 @@ constexpr float LOG2E_W = 1.4426950408889634f;
 
 struct W128 {
   static constexpr int PANEL = 128 * 64 * 2;         // [128 rows][64 cols] bf16, 16 KB
-  static constexpr int HP = 64 * 64 * 2;             // half-tile panel [64 rows][64 cols], 8 KB
-  static constexpr int NS = 2;                       // half-tile stages of Q / dO
-  static constexpr int OFF_K = 0;                    // 2 panels
-  static constexpr int OFF_V = 2 * PANEL;            // 2 panels
-  static constexpr int OFF_QH = 4 * PANEL;           // NS x 2 half panels
-  static constexpr int OFF_DOH = OFF_QH + NS * 2 * HP;
-  static constexpr int OFF_DS = OFF_DOH + NS * 2 * HP;   // 2 panels: [query half][128 key rows][64 queries]
-  static constexpr int OFF_DQ = OFF_DS + 2 * PANEL;      // fp32 staging box [128 rows][32 floats]
-  static constexpr int OFF_AUX = OFF_DQ + PANEL;         // NS x 4 KB: row-term images of Q | dO (2 KB each), or a band
-  static constexpr int OFF_ONES = OFF_AUX + NS * 4096;   // 4 KB constant tile: columns 0..2 one, rest zero
-  static constexpr int OFF_TAB = OFF_ONES + 4096;
-  static constexpr int TAB_FLOATS = 256 + 128;           // r2raw[256] z2s[128]
-  static constexpr int OFF_BAR = OFF_TAB + TAB_FLOATS * 4;
-  static constexpr int NBAR = 2 + 2 * NS + 9;
-  static constexpr int SMEM = OFF_BAR + NBAR * 8 + 16 + 1024;
+  static constexpr int TILE = 2 * PANEL;
+  static constexpr int NS = 2;                       // stages of Q (frozen items: of dO)
+  static constexpr int OFF_K = 0;
+  static constexpr int OFF_V = TILE;
+  static constexpr int OFF_Q = 2 * TILE;
+  static constexpr int OFF_DO = OFF_Q + NS * TILE;   // one dO tile; tensor-core frozen form: bands, 4 KB per stage
+  static constexpr int OFF_DS = OFF_DO + TILE;       // [query half][128 key rows][64 queries]; general frozen form: tables
+  static constexpr int OFF_DQ = OFF_DS + TILE;       // fp32 staging boxes of the drain warps, 8 x [32 rows][32 floats]
+  static constexpr int OFF_AUX = OFF_DQ + 8 * 4096;  // NS x { -LSE log2 e [128], -delta [128] }
+  static constexpr int OFF_BAR = OFF_AUX + NS * 1024;
+  static constexpr int NBAR = 2 + 2 * NS + 2 + 9;
+  static constexpr int SMEM = OFF_BAR + NBAR * 8 + 16;
   static constexpr int TMEM_COLS = 512;
-  static constexpr int COL_DV = 0, COL_DK = 128, COL_S = 256, COL_DP = 320, COL_DQ = 384;
-  static constexpr int NTHREADS = 704;
+  static constexpr int COL_DV = 0, COL_DK = 128, COL_X = 256, COL_Y = 384;
+  static constexpr int NTHREADS = 896;
 };
+static_assert(W128::SMEM <= 227 * 1024, "shared memory");
 
-enum W128Site { W_KV_EMPTY = 81, W_H_EMPTY, W_KV_FULL, W_H_FULL, W_PDS_FULL, W_ACC_FREE, W_DQ_FREE, W_S_FULL,
-                W_SDP_FULL, W_DQ_FULL, W_ACC_FULL, W_PFREE, W_C_DONE };
+enum W128Site { W_KV_EMPTY = 81, W_Q_EMPTY, W_KV_FULL, W_Q_FULL, W_P_FULL, W_ACC_FREE, W_DQ_FREE, W_S_FULL,
+                W_DP_FULL, W_DQ_FULL, W_ACC_FULL, W_PFREE, W_DO_EMPTY, W_DO_FULL, W_DS_FULL, W_ALIGN };
 
 __device__ __forceinline__ void red_add_v4(float* addr, float a, float b, float c, float d) {
   asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(addr), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
@@ -82,68 +97,67 @@ __device__ __forceinline__ ItemW load_item_w(const BwdParams& p, int it, int it_
 
 __global__ void __launch_bounds__(W128::NTHREADS, 1)
 saf_bwd128_kernel(const __grid_constant__ CUtensorMap mk, const __grid_constant__ CUtensorMap mv,
-                  const __grid_constant__ CUtensorMap mqh, const __grid_constant__ CUtensorMap mdoh,
-                  const __grid_constant__ CUtensorMap mdoth, const __grid_constant__ CUtensorMap mdq,
+                  const __grid_constant__ CUtensorMap mq, const __grid_constant__ CUtensorMap mdo,
+                  const __grid_constant__ CUtensorMap mdot, const __grid_constant__ CUtensorMap mdq,
                   const BwdParams p) {
   using C = W128;
-  extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  extern __shared__ __align__(1024) uint8_t smem[];
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::OFF_BAR);
   uint64_t* kv_full = bars;
   uint64_t* kv_empty = bars + 1;
-  uint64_t* h_full = bars + 2;                   // [NS] a half tile of Q / dO (or band + scaled dO) has landed
-  uint64_t* h_empty = h_full + C::NS;            // [NS]
-  uint64_t* s_full = h_empty + C::NS;            // S'^T is complete
-  uint64_t* sdp_full = s_full + 1;               // ... and dP'^T
-  uint64_t* pds_full = sdp_full + 1;             // the compute warps have written P^T / dS^T (16 warp arrivals)
-  uint64_t* dq_full = pds_full + 1;
-  uint64_t* dq_free = dq_full + 1;               // 4 drain warps
+  uint64_t* q_full = bars + 2;                   // [NS] Q tile and its row terms (frozen: dO tile, band)
+  uint64_t* q_empty = q_full + C::NS;            // [NS]
+  uint64_t* do_full = q_empty + C::NS;
+  uint64_t* do_empty = do_full + 1;
+  uint64_t* s_full = do_empty + 1;
+  uint64_t* dp_full = s_full + 1;
+  uint64_t* p_full = dp_full + 1;                // P^T written (16 warp arrivals)
+  uint64_t* ds_full = p_full + 1;                // dS^T written (16 warp arrivals)
+  uint64_t* dq_full = ds_full + 1;
+  uint64_t* dq_free = dq_full + 1;               // dQ is in the drain warps' registers (8 warp arrivals)
   uint64_t* acc_full = dq_free + 1;
   uint64_t* acc_free = acc_full + 1;             // 16 compute warps
-  uint64_t* pfree = acc_free + 1;                // generic frozen form: the P^^T half tile has been consumed
-  uint64_t* c_done = pfree + 1;                  // the dQ MMAs have read the smem dS^T tile
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(c_done + 1);
+  uint64_t* pfree = acc_free + 1;                // general frozen form: the P^^T tile has been consumed
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(pfree + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const WaitCtx wc{abort_flag, p.status, p.wait_limit_ns};
   SAF_SPAN(bwd128, 0);
+#ifdef SAF_TRACE
+  int tr_n = 0;
+#endif
   const int nblk = p.nblk;
+  if ((smem_u32(smem) & 1023u) != 0) {           // (the swizzled tiles need it; there is no room for a slack)
+    if (tid == 0) atomicCAS(p.status, 0, (DEV_TIMEOUT << 24) | (W_ALIGN << 16) | static_cast<int>(blockIdx.x & 0xffff));
+    return;
+  }
 
   if (tid == 0) {
     *abort_flag = 0;
     mbar_init(kv_full, 1);
     mbar_init(kv_empty, 1);
     for (int s = 0; s < C::NS; ++s) {
-      mbar_init(h_full + s, 1);
-      mbar_init(h_empty + s, 1);
+      mbar_init(q_full + s, 1);
+      mbar_init(q_empty + s, 1);
     }
+    mbar_init(do_full, 1);
+    mbar_init(do_empty, 1);
     mbar_init(s_full, 1);
-    mbar_init(sdp_full, 1);
-    mbar_init(pds_full, 16);
+    mbar_init(dp_full, 1);
+    mbar_init(p_full, 16);
+    mbar_init(ds_full, 16);
     mbar_init(dq_full, 1);
-    mbar_init(dq_free, 4);
+    mbar_init(dq_free, 8);
     mbar_init(acc_full, 1);
     mbar_init(acc_free, 16);
     mbar_init(pfree, 1);
-    mbar_init(c_done, 1);
     mbar_fence_init();
   }
-  // constant tile of ones (columns 0..2) in the no-swizzle K-major core-matrix layout
-  for (int i = tid; i < 256; i += C::NTHREADS) {
-    const int k8 = (i >> 3) & 1;                 // 16-byte unit i: row group i>>4, k-half k8, row-in-group i&7
-    uint4 v = make_uint4(0, 0, 0, 0);
-    if (k8 == 0) {
-      v.x = 0x3F803F80u;                         // bf16 1.0, 1.0
-      v.y = 0x00003F80u;                         // bf16 1.0, 0
-    }
-    reinterpret_cast<uint4*>(smem + C::OFF_ONES)[i] = v;
-  }
-  if (warp == 21) {
+  if (warp == 25) {
     tmem_alloc(tmem_slot, C::TMEM_COLS);
     tmem_relinquish();
   }
-  fence_proxy_async_smem();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -153,288 +167,273 @@ saf_bwd128_kernel(const __grid_constant__ CUtensorMap mk, const __grid_constant_
   pdl_wait();
   const int it_begin = p.cta_offsets[blockIdx.x], it_end = p.cta_offsets[blockIdx.x + 1];
 
-  if (warp == 20) {
-    // ------------------------------------------------------------------ TMA producer
-    if (lane == 0) {
-      tma_prefetch_desc(&mk);
-      tma_prefetch_desc(&mv);
-      tma_prefetch_desc(&mqh);
-      tma_prefetch_desc(&mdoh);
-      tma_prefetch_desc(&mdoth);
-      uint32_t nkv = 0, nh = 0;
-      bool ok = true;
-      ItemW nxt = load_item_w(p, it_begin, it_end);
-      for (int it = it_begin; it < it_end && ok; ++it) {
-        const WorkItem w = nxt.w;
-        const bool fast = nxt.fast;
-        nxt = load_item_w(p, it + 1, it_end);
-        const bool ord = w.kind == KIND_ORDINARY;
-        const size_t bh = static_cast<size_t>(w.b) * p.H + w.h;
-        const int qh = (ord && p.qslot) ? p.qslot[w.h] : w.h;          // head index in the Q tensor
-        if (ord) {
-          const int kh = p.qslot ? p.qslot[w.h] : w.h / p.kv_group;    // ... in the K tensor
-          ok = mbar_wait(kv_empty, (nkv & 1) ^ 1, wc, W_KV_EMPTY);
-          if (!ok) break;
-          mbar_expect_tx(kv_full, 4 * C::PANEL);
-          for (int pn = 0; pn < 2; ++pn) {
-            tma_load_4d(smem + C::OFF_K + pn * C::PANEL, &mk, kv_full, pn * 64, w.blk * BLK, kh, w.b);
-            tma_load_4d(smem + C::OFF_V + pn * C::PANEL, &mv, kv_full, pn * 64, w.blk * BLK, w.h / p.kv_group, w.b);
-          }
-          ++nkv;
-        }
-        const int fo = fast ? p.hord[w.h] : 0;
-        const uint8_t* bands = static_cast<const uint8_t*>(p.band_b) + static_cast<size_t>(w.h) * p.nblkp * 4096;
-        const int U = 2 * (nblk - w.blk);
-        for (int u = 0; u < U; ++u, ++nh) {
-          const int I = w.blk + (u >> 1), row0 = I * BLK + 64 * (u & 1);
-          const uint32_t s = nh % C::NS;
-          ok = mbar_wait(h_empty + s, ((nh / C::NS) & 1) ^ 1, wc, W_H_EMPTY);
-          if (!ok) break;
-          uint8_t* qdst = smem + C::OFF_QH + s * 2 * C::HP;
-          uint8_t* ddst = smem + C::OFF_DOH + s * 2 * C::HP;
-          uint8_t* aux = smem + C::OFF_AUX + s * 4096;
-          if (fast) {
-            // tensor-core form: the Hankel band of distance block (I - J) and the scaled dO half tile
-            mbar_expect_tx(h_full + s, 2 * C::HP + 4096);
-            bulk_load(aux, bands + static_cast<size_t>(I - w.blk) * 4096, 4096, h_full + s);
-            for (int pn = 0; pn < 2; ++pn) tma_load_4d(ddst + pn * C::HP, &mdoth, h_full + s, pn * 64, row0, fo, w.b);
-          } else if (ord) {
-            mbar_expect_tx(h_full + s, 4 * C::HP + 4096);
-            const size_t img = (bh * nblk + I) * 4096 + (u & 1) * 2048;
-            bulk_load(aux, static_cast<const uint8_t*>(p.q_ext) + img, 2048, h_full + s);
-            bulk_load(aux + 2048, static_cast<const uint8_t*>(p.do_ext) + img, 2048, h_full + s);
-            for (int pn = 0; pn < 2; ++pn) {
-              tma_load_4d(qdst + pn * C::HP, &mqh, h_full + s, pn * 64, row0, qh, w.b);
-              tma_load_4d(ddst + pn * C::HP, &mdoh, h_full + s, pn * 64, row0, w.h, w.b);
+  if (warp >= 24) {
+    reg_dec<40>();
+    if (warp == 24) {
+      // ---------------------------------------------------------------- TMA producer
+      if (lane == 0) {
+        tma_prefetch_desc(&mk);
+        tma_prefetch_desc(&mv);
+        tma_prefetch_desc(&mq);
+        tma_prefetch_desc(&mdo);
+        tma_prefetch_desc(&mdot);
+        uint32_t nkv = 0, nq = 0, ndo = 0;
+        bool ok = true, bands_open = false;
+        ItemW nxt = load_item_w(p, it_begin, it_end);
+        for (int it = it_begin; it < it_end && ok; ++it) {
+          const WorkItem w = nxt.w;
+          const bool fast = nxt.fast;
+          nxt = load_item_w(p, it + 1, it_end);
+          const bool ord = w.kind == KIND_ORDINARY;
+          const size_t bh = static_cast<size_t>(w.b) * p.H + w.h;
+          const int qh = (ord && p.qslot) ? p.qslot[w.h] : w.h;          // head index in the Q tensor
+          auto load_tile = [&](const CUtensorMap* m, int off, uint64_t* bar, int row0, int head) {
+            for (int pn = 0; pn < 2; ++pn)
+              tma_load_4d(smem + off + pn * C::PANEL, m, bar, pn * 64, row0, head, w.b);
+          };
+          if (ord) {
+            const int kh = p.qslot ? p.qslot[w.h] : w.h / p.kv_group;    // ... in the K tensor
+            ok = mbar_wait(kv_empty, (nkv & 1) ^ 1, wc, W_KV_EMPTY);
+            if (!ok) break;
+            mbar_expect_tx(kv_full, 2 * C::TILE);
+            load_tile(&mk, C::OFF_K, kv_full, w.blk * BLK, kh);
+            load_tile(&mv, C::OFF_V, kv_full, w.blk * BLK, w.h / p.kv_group);
+            ++nkv;
+            if (bands_open) {
+              // the bands (in the dO tile's place) of the last frozen tiles have been consumed
+              for (uint32_t n = nq > C::NS ? nq - C::NS : 0; n < nq && ok; ++n)
+                ok = mbar_wait(q_empty + n % C::NS, (n / C::NS) & 1, wc, W_Q_EMPTY);
+              if (!ok) break;
+              bands_open = false;
             }
-          } else {
-            mbar_expect_tx(h_full + s, 2 * C::HP);
-            for (int pn = 0; pn < 2; ++pn) tma_load_4d(ddst + pn * C::HP, &mdoh, h_full + s, pn * 64, row0, w.h, w.b);
+          } else if (fast && !bands_open) {
+            // the last dO tile has been consumed
+            if (ndo > 0) ok = mbar_wait(do_empty, (ndo - 1) & 1, wc, W_DO_EMPTY);
+            if (!ok) break;
+            bands_open = true;
+          }
+          const int fo = fast ? p.hord[w.h] : 0;
+          const uint8_t* bands = static_cast<const uint8_t*>(p.band_b) + static_cast<size_t>(w.h) * p.nblkp * 4096;
+          for (int I = w.blk; I < nblk; ++I, ++nq) {
+            const uint32_t s = nq % C::NS;
+            ok = mbar_wait(q_empty + s, ((nq / C::NS) & 1) ^ 1, wc, W_Q_EMPTY);
+            if (!ok) break;
+            const int qoff = C::OFF_Q + s * C::TILE;
+            if (ord) {
+              mbar_expect_tx(q_full + s, C::TILE + 1024);
+              load_tile(&mq, qoff, q_full + s, I * BLK, qh);
+              uint8_t* aux = smem + C::OFF_AUX + s * 1024;
+              const size_t vec = (bh * nblk + I) * 512;
+              bulk_load(aux, static_cast<const uint8_t*>(p.q_ext) + vec, 512, q_full + s);
+              bulk_load(aux + 512, static_cast<const uint8_t*>(p.do_ext) + vec, 512, q_full + s);
+              ok = mbar_wait(do_empty, (ndo & 1) ^ 1, wc, W_DO_EMPTY);
+              if (!ok) break;
+              mbar_expect_tx(do_full, C::TILE);
+              load_tile(&mdo, C::OFF_DO, do_full, I * BLK, w.h);
+              ++ndo;
+            } else if (fast) {
+              // tensor-core form: the Hankel band of distance block (I - J) and the scaled dO tile
+              mbar_expect_tx(q_full + s, C::TILE + 4096);
+              bulk_load(smem + C::OFF_DO + s * 4096, bands + static_cast<size_t>(I - w.blk) * 4096, 4096, q_full + s);
+              load_tile(&mdot, qoff, q_full + s, I * BLK, fo);
+            } else {
+              mbar_expect_tx(q_full + s, C::TILE);
+              load_tile(&mdo, qoff, q_full + s, I * BLK, w.h);
+            }
           }
         }
       }
-    }
-  }
-  else if (warp == 21) {
-    // ------------------------------------------------------------------ tcgen05 issuer
-    // The whole warp walks the loops (warp-uniform operands); one elected lane issues.  MMAs issued by one thread
-    // execute in issue order: A(u+1) is queued right behind B(u), which reads the bf16 contents of the same buffer.
-    const bool leader = elect_one() != 0;
-    const uint32_t sb = smem_u32(smem);
-    constexpr uint32_t id_s = umma_idesc_bf16(128, 64, 0, 0);      // S^T, dP^T half tiles: both operands K-major
-    // (head dimension 96 runs here with features 96..127 zero-filled by TMA: the gradient MMAs produce only 96
-    // columns and the score MMAs skip the two empty k-steps)
-    const uint32_t id_acc = umma_idesc_bf16(128, p.d_real, 0, 1);  // dV, dK: A from TMEM, B MN-major
-    const uint32_t id_dq = umma_idesc_bf16(128, p.d_real, 1, 1);   // dQ: A (dS^T tile) M-major, B MN-major
-    const uint32_t id_hk = umma_idesc_f16(128, p.d_real, 0, 1);    // fp16 band x fp16 scaled dO
-    const int nk16 = p.d_real / 16;
-    // descriptor halves for smem offset 0: 128B-swizzled K-major (k-step +32 B inside a 64-feature panel), the
-    // no-swizzle K-major row-term tiles (LBO 128 B, SBO 256 B), 128B-swizzled MN-major tiles whose two 64-wide
-    // halves are a half panel (Q / dO stages) or a panel (K_J, dS^T) apart, and the Hankel band
-    const uint64_t d_k = umma_smem_desc(sb, 16, 1024, UMMA_LAYOUT_SW128);
-    const uint64_t d_x = umma_smem_desc(sb, 128, 256, UMMA_LAYOUT_NONE);
-    const uint64_t d_mh = umma_smem_desc(sb, C::HP, 1024, UMMA_LAYOUT_SW128);
-    const uint64_t d_m = umma_smem_desc(sb, C::PANEL, 1024, UMMA_LAYOUT_SW128);
-    const uint64_t d_band = umma_smem_desc(sb, 128, 128, UMMA_LAYOUT_NONE);
-    const uint32_t lo_k = desc_lo(d_k), hi_k = desc_hi(d_k), lo_x = desc_lo(d_x), hi_x = desc_hi(d_x);
-    const uint32_t lo_mh = desc_lo(d_mh), hi_mh = desc_hi(d_mh), lo_m = desc_lo(d_m), hi_m = desc_hi(d_m);
-    const uint32_t lo_b = desc_lo(d_band), hi_b = desc_hi(d_band);
-    const uint32_t ones_lo = lo_x + (C::OFF_ONES >> 4);
-    const uint32_t k_lo = lo_k + (C::OFF_K >> 4), v_lo = lo_k + (C::OFF_V >> 4);
-    const uint32_t km_lo = lo_m + (C::OFF_K >> 4), ds_lo = lo_m + (C::OFF_DS >> 4);
-    const uint32_t t_s = tmem + C::COL_S, t_dp = tmem + C::COL_DP;
-    uint32_t nkv = 0, nh = 0, nitem = 0, ndq = 0, npds = 0;
-    bool ok = true;
-    ItemW nxt = load_item_w(p, it_begin, it_end);
-    for (int it = it_begin; it < it_end && ok; ++it, ++nitem) {
-      const WorkItem w = nxt.w;
-      const bool fast = nxt.fast;
-      nxt = load_item_w(p, it + 1, it_end);
-      const bool ord = w.kind == KIND_ORDINARY;
-      const int U = 2 * (nblk - w.blk);
-      if (ord) {
-        ok = mbar_wait_warp(kv_full, nkv & 1, wc, W_KV_FULL);
-        if (!ok) break;
-        ++nkv;
-        // score MMAs of the half tile in ring position pos
-        auto issue_A = [&](uint32_t pos) {
-          const uint32_t s = pos % C::NS;
-          const uint32_t q_lo = lo_k + ((C::OFF_QH + s * 2 * C::HP) >> 4);
-          const uint32_t do_lo = lo_k + ((C::OFF_DOH + s * 2 * C::HP) >> 4);
-          const uint32_t qx_lo = lo_x + ((C::OFF_AUX + s * 4096) >> 4);
-          if (leader) {
+    } else if (warp == 25) {
+      // ---------------------------------------------------------------- tcgen05 issuer
+      // The whole warp walks the loops (warp-uniform operands); one elected lane issues.
+      const bool leader = elect_one() != 0;
+      const uint32_t sb = smem_u32(smem);
+      constexpr uint32_t id_s = umma_idesc_bf16(128, 128, 0, 0);     // S^T, dP^T: both operands K-major
+      // (head dimension 96 runs here with features 96..127 zero-filled by TMA: the gradient MMAs produce only 96
+      // columns and the score MMAs skip the two empty k-steps)
+      const uint32_t id_acc = umma_idesc_bf16(128, p.d_real, 0, 1);  // dV, dK: A K-major, B MN-major
+      const uint32_t id_dq = umma_idesc_bf16(128, p.d_real, 1, 1);   // dQ: A (dS^T tile) M-major, B MN-major
+      const uint32_t id_hk = umma_idesc_f16(128, p.d_real, 0, 1);    // fp16 band x fp16 scaled dO
+      const int nk16 = p.d_real / 16;
+      // descriptor halves for smem offset 0: 128B-swizzled K-major tiles (k-step +32 B inside a 64-wide panel), MN-major
+      // tiles whose two 64-wide halves are a panel apart (k-step +2048 B), and the Hankel band
+      const uint64_t d_k = umma_smem_desc(sb, 16, 1024, UMMA_LAYOUT_SW128);
+      const uint64_t d_m = umma_smem_desc(sb, C::PANEL, 1024, UMMA_LAYOUT_SW128);
+      const uint64_t d_band = umma_smem_desc(sb, 128, 128, UMMA_LAYOUT_NONE);
+      const uint32_t lo_k = desc_lo(d_k), hi_k = desc_hi(d_k), lo_m = desc_lo(d_m), hi_m = desc_hi(d_m);
+      const uint32_t lo_b = desc_lo(d_band), hi_b = desc_hi(d_band);
+      const uint32_t t_x = tmem + C::COL_X, t_y = tmem + C::COL_Y;
+      uint32_t nkv = 0, nq = 0, ndo = 0, nitem = 0, np = 0, nds = 0;
+      bool ok = true;
+      auto q_wait = [&](uint32_t pos) {
+        return mbar_wait_warp(q_full + pos % C::NS, (pos / C::NS) & 1, wc, W_Q_FULL);
+      };
+      // (scores) d = a b^T over the features; a, b: smem offsets of K-major tiles
+      auto issue_kk = [&](uint32_t d, uint32_t a_off, uint32_t b_off, uint64_t* bar) {
+        if (leader) {
 #pragma unroll
-            for (int kc = 0; kc < 8; ++kc) {
-              if (kc >= nk16) break;
-              const uint32_t ok_ = ((kc >> 2) * C::PANEL + (kc & 3) * 32) >> 4;
-              const uint32_t oh_ = ((kc >> 2) * C::HP + (kc & 3) * 32) >> 4;
-              umma_ss2(t_s, k_lo + ok_, hi_k, q_lo + oh_, hi_k, id_s, kc > 0);
-            }
-            umma_ss2(t_s, ones_lo, hi_x, qx_lo, hi_x, id_s, 1);
-            umma_commit(s_full);                         // the exponentials start while dP'^T is computed
-#pragma unroll
-            for (int kc = 0; kc < 8; ++kc) {
-              if (kc >= nk16) break;
-              const uint32_t ok_ = ((kc >> 2) * C::PANEL + (kc & 3) * 32) >> 4;
-              const uint32_t oh_ = ((kc >> 2) * C::HP + (kc & 3) * 32) >> 4;
-              umma_ss2(t_dp, v_lo + ok_, hi_k, do_lo + oh_, hi_k, id_s, kc > 0);
-            }
-            umma_ss2(t_dp, ones_lo, hi_x, qx_lo + (2048 >> 4), hi_x, id_s, 1);
-            umma_commit(sdp_full);
+          for (int kc = 0; kc < 8; ++kc) {
+            if (kc >= nk16) break;
+            const uint32_t off = ((kc >> 2) * C::PANEL + (kc & 3) * 32) >> 4;
+            umma_ss2(d, lo_k + (a_off >> 4) + off, hi_k, lo_k + (b_off >> 4) + off, hi_k, id_s, kc > 0);
           }
-          __syncwarp();
-        };
-        ok = mbar_wait_warp(h_full + nh % C::NS, (nh / C::NS) & 1, wc, W_H_FULL);
-        if (!ok) break;
-        tc_fence_after();
-        issue_A(nh);
-        for (int u = 0; u < U && ok; ++u) {
-          const uint32_t pos = nh + u, s = pos % C::NS;
-          ok = mbar_wait_warp(pds_full, npds & 1, wc, W_PDS_FULL);
-          ++npds;
-          if (ok && u == 0) ok = mbar_wait_warp(acc_free, (nitem & 1) ^ 1, wc, W_ACC_FREE);
+          umma_commit(bar);
+        }
+        __syncwarp();
+      };
+      ItemW nxt = load_item_w(p, it_begin, it_end);
+      for (int it = it_begin; it < it_end && ok; ++it, ++nitem) {
+        const WorkItem w = nxt.w;
+        const bool fast = nxt.fast;
+        nxt = load_item_w(p, it + 1, it_end);
+        const int nt = nblk - w.blk;
+        if (w.kind == KIND_ORDINARY) {
+          ok = mbar_wait_warp(kv_full, nkv++ & 1, wc, W_KV_FULL) && q_wait(nq);
           if (!ok) break;
           tc_fence_after();
-          const uint32_t doh_lo = lo_mh + ((C::OFF_DOH + s * 2 * C::HP) >> 4);
-          const uint32_t qh_lo = lo_mh + ((C::OFF_QH + s * 2 * C::HP) >> 4);
-          const uint32_t acc0 = u > 0 ? 1u : 0u;
-          if (leader) {
-#pragma unroll
-            for (int kc = 0; kc < 4; ++kc)
-              umma_ts2(tmem + C::COL_DV, t_s + 16 * kc, doh_lo + 128 * kc, hi_mh, id_acc, kc > 0 ? 1u : acc0);
-#pragma unroll
-            for (int kc = 0; kc < 4; ++kc)
-              umma_ts2(tmem + C::COL_DK, t_dp + 16 * kc, qh_lo + 128 * kc, hi_mh, id_acc, kc > 0 ? 1u : acc0);
-            umma_commit(h_empty + s);
-          }
-          __syncwarp();
-          if (u + 1 < U) {
-            ok = mbar_wait_warp(h_full + (pos + 1) % C::NS, ((pos + 1) / C::NS) & 1, wc, W_H_FULL);
+          issue_kk(t_x, C::OFF_K, C::OFF_Q + (nq % C::NS) * C::TILE, s_full);
+          for (int t = 0; t < nt && ok; ++t, ++nq) {
+            // dP(t): the dQ that was in Y is out
+            ok = mbar_wait_warp(do_full, ndo & 1, wc, W_DO_FULL) && mbar_wait_warp(dq_free, (ndo & 1) ^ 1, wc, W_DQ_FREE);
+            if (!ok) break;
+            ++ndo;
+            tc_fence_after();
+            TRB(0, 1);
+            issue_kk(t_y, C::OFF_V, C::OFF_DO, dp_full);
+            TRB(0, 2);
+            // dV(t), S(t+1)
+            ok = (t > 0 || mbar_wait_warp(acc_free, (nitem & 1) ^ 1, wc, W_ACC_FREE)) &&
+                 (t + 1 == nt || q_wait(nq + 1)) && mbar_wait_warp(p_full, np++ & 1, wc, W_P_FULL);
             if (!ok) break;
             tc_fence_after();
-            issue_A(pos + 1);
-          }
-          if (u & 1) {
-            // full tile done: dQ of the tile
-            ok = mbar_wait_warp(dq_free, (ndq & 1) ^ 1, wc, W_DQ_FREE);
-            if (!ok) break;
-            ++ndq;
-            tc_fence_after();
+            TRB(0, 3);
             if (leader) {
 #pragma unroll
               for (int kc = 0; kc < 8; ++kc)
-                umma_ss2(tmem + C::COL_DQ, ds_lo + 128 * kc, hi_m, km_lo + 128 * kc, hi_m, id_dq, kc > 0);
+                umma_ts2(tmem + C::COL_DV, t_x + 32 * (kc >> 1) + 8 * (kc & 1), lo_m + (C::OFF_DO >> 4) + 128 * kc, hi_m, id_acc,
+                         kc > 0 || t > 0 ? 1u : 0u);
+              umma_commit(do_empty);
+            }
+            __syncwarp();
+            if (t + 1 < nt) issue_kk(t_x, C::OFF_K, C::OFF_Q + ((nq + 1) % C::NS) * C::TILE, s_full);
+            TRB(0, 4);
+            // dQ(t), dK(t)
+            ok = mbar_wait_warp(ds_full, nds++ & 1, wc, W_DS_FULL);
+            if (!ok) break;
+            tc_fence_after();
+            TRB(0, 5);
+            if (leader) {
+#pragma unroll
+              for (int kc = 0; kc < 8; ++kc)
+                umma_ss2(t_y, lo_m + (C::OFF_DS >> 4) + 128 * kc, hi_m, lo_m + (C::OFF_K >> 4) + 128 * kc, hi_m, id_dq, kc > 0);
               umma_commit(dq_full);
-              umma_commit(c_done);
+            }
+            __syncwarp();
+            const uint32_t q_lo = lo_m + ((C::OFF_Q + (nq % C::NS) * C::TILE) >> 4);
+            if (leader) {
+#pragma unroll
+              for (int kc = 0; kc < 8; ++kc)
+                umma_ss2(tmem + C::COL_DK, lo_k + (C::OFF_DS >> 4) + (((kc >> 2) * C::PANEL + (kc & 3) * 32) >> 4), hi_k,
+                         q_lo + 128 * kc, hi_m, id_acc, kc > 0 || t > 0 ? 1u : 0u);
+              umma_commit(q_empty + nq % C::NS);
+              if (t + 1 == nt) umma_commit(kv_empty);
+            }
+            __syncwarp();
+            TRB(0, 6);
+          }
+        } else {
+          // frozen item: dV only.  Tensor-core form: A = Hankel band, B = scaled dO tile; general form: A = the P^^T tile
+          // the compute warps wrote into X.
+          for (int t = 0; t < nt && ok; ++t, ++nq) {
+            const uint32_t s = nq % C::NS;
+            ok = q_wait(nq) && (t > 0 || mbar_wait_warp(acc_free, (nitem & 1) ^ 1, wc, W_ACC_FREE)) &&
+                 (fast || mbar_wait_warp(p_full, np++ & 1, wc, W_P_FULL));
+            if (!ok) break;
+            tc_fence_after();
+            const uint32_t do_lo = lo_m + ((C::OFF_Q + s * C::TILE) >> 4);
+            const uint32_t band_lo = lo_b + ((C::OFF_DO + s * 4096) >> 4);
+            if (leader) {
+              if (fast) {
+#pragma unroll
+                for (int kc = 0; kc < 8; ++kc)
+                  umma_ss2(tmem + C::COL_DV, band_lo + 16 * kc, hi_b, do_lo + 128 * kc, hi_m, id_hk, kc > 0 || t > 0 ? 1u : 0u);
+              } else {
+#pragma unroll
+                for (int kc = 0; kc < 8; ++kc)
+                  umma_ts2(tmem + C::COL_DV, t_x + 32 * (kc >> 1) + 8 * (kc & 1), do_lo + 128 * kc, hi_m, id_acc,
+                           kc > 0 || t > 0 ? 1u : 0u);
+                umma_commit(pfree);
+              }
+              umma_commit(q_empty + s);
             }
             __syncwarp();
           }
         }
         if (!ok) break;
-        nh += U;
-        if (leader) umma_commit(kv_empty);
-      } else {
-        // frozen item: dV only.  Tensor-core form: A = Hankel band rows of this query half, B = scaled dO half tile;
-        // general form: A = the P^^T half tile the compute warps wrote into the S^T buffer.
-        for (int u = 0; u < U && ok; ++u, ++nh) {
-          const uint32_t s = nh % C::NS;
-          ok = mbar_wait_warp(h_full + s, (nh / C::NS) & 1, wc, W_H_FULL);
-          if (ok && !fast) {
-            ok = mbar_wait_warp(pds_full, npds & 1, wc, W_PDS_FULL);
-            ++npds;
-          }
-          if (ok && u == 0) ok = mbar_wait_warp(acc_free, (nitem & 1) ^ 1, wc, W_ACC_FREE);
-          if (!ok) break;
-          tc_fence_after();
-          const uint32_t doh_lo = lo_mh + ((C::OFF_DOH + s * 2 * C::HP) >> 4);
-          const uint32_t band_lo = lo_b + ((C::OFF_AUX + s * 4096) >> 4) + 16 * 4 * (u & 1);
-          const uint32_t acc0 = u > 0 ? 1u : 0u;
-          if (leader) {
-            if (fast) {
-#pragma unroll
-              for (int kc = 0; kc < 4; ++kc)
-                umma_ss2(tmem + C::COL_DV, band_lo + 16 * kc, hi_b, doh_lo + 128 * kc, hi_mh, id_hk, kc > 0 ? 1u : acc0);
-            } else {
-#pragma unroll
-              for (int kc = 0; kc < 4; ++kc)
-                umma_ts2(tmem + C::COL_DV, t_s + 16 * kc, doh_lo + 128 * kc, hi_mh, id_acc, kc > 0 ? 1u : acc0);
-              umma_commit(pfree);
-            }
-            umma_commit(h_empty + s);
-          }
-          __syncwarp();
-        }
-        if (!ok) break;
+        if (leader) umma_commit(acc_full);
+        __syncwarp();
       }
-      if (leader) umma_commit(acc_full);
-      __syncwarp();
     }
-  }
-  else if (warp >= 16 && warp < 20) {
-    // ------------------------------------------------------------------ dQ drain warps (128 threads)
-    // dQ of a tile (128 queries x 128 features, fp32) leaves in four [128][32] boxes through one staging box.
-    const int q4 = warp & 3;
-    const int rowl = q4 * 32 + lane;                    // query row within the tile
+  } else if (warp >= 16) {
+    // ------------------------------------------------------------------ dQ drain warps
+    // A warp takes 32 query rows x 64 features into registers at once, so that Y is free again, and sends them as
+    // two [32][32] boxes through its own staging box.
+    const int q4 = warp & 3, hh = (warp - 16) >> 2;
     const uint32_t lane_base = static_cast<uint32_t>(q4 * 32) << 16;
-    const uint32_t stage_row = smem_u32(smem + C::OFF_DQ) + rowl * 128;
-    const int nbox = p.d_real > 96 ? 4 : 3;             // head dimension 96: the fourth box does not exist
+    uint8_t* box = smem + C::OFF_DQ + (warp - 16) * 4096;
+    const uint32_t stage_row = smem_u32(box) + lane * 128;
     uint32_t ndq = 0;
-    bool ok = true, leave = false;
-    for (int it = it_begin; it < it_end && !leave; ++it) {
+    bool ok = true;
+    for (int it = it_begin; it < it_end && ok; ++it) {
       const WorkItem w = p.items[it];
       if (w.kind != KIND_ORDINARY) continue;
       const int qh = p.qslot ? p.qslot[w.h] : w.h;      // head index in the dQ accumulator
-      for (int I = w.blk; I < nblk && !leave; ++I) {
-        for (int k = 0; k < 4; ++k) {
-          // the previous reduce has finished reading the staging box (thread 512 waits for it before arriving
-          // here); the drain warps also agree here whether a wait has been abandoned
-          if (named_bar_or(2, 128, !ok)) {
-            leave = true;
-            break;
-          }
-          if (k == 0) {
-            if (!mbar_wait_warp(dq_full, ndq & 1, wc, W_DQ_FULL)) ok = false;
-            ++ndq;
-            tc_fence_after();
-          }
-          uint32_t r[32];
-          tmem_ld32(tmem + lane_base + C::COL_DQ + 32 * k, r);
-          tmem_wait_ld();
-          if (k == 3) {
-            tc_fence_before();
-            warp_arrive(dq_free);                       // the tensor core may overwrite dQ
-          }
+      for (int I = w.blk; I < nblk; ++I) {
+        ok = mbar_wait_warp(dq_full, ndq++ & 1, wc, W_DQ_FULL);
+        if (!ok) break;
+        tc_fence_after();
+        uint32_t r[2][32];
+        tmem_ld32(tmem + lane_base + C::COL_Y + 64 * hh, r[0]);
+        tmem_ld32(tmem + lane_base + C::COL_Y + 64 * hh + 32, r[1]);
+        tmem_wait_ld();
+        tc_fence_before();
+        warp_arrive(dq_free);                           // the tensor core may overwrite Y
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          const int col = 64 * hh + 32 * k;
+          if (col >= p.d_real) break;                   // head dimension 96: the fourth box does not exist
+          if (lane == 0) bulk_wait_group_read0();       // the box's previous contents have been read
+          __syncwarp();
 #pragma unroll
           for (int g = 0; g < 8; ++g) {
-            const uint32_t chunk = static_cast<uint32_t>(g ^ (rowl & 7)) * 16;
-            st_shared_v4w(stage_row + chunk, __float_as_uint(__uint_as_float(r[4 * g]) * p.scale),
-                          __float_as_uint(__uint_as_float(r[4 * g + 1]) * p.scale),
-                          __float_as_uint(__uint_as_float(r[4 * g + 2]) * p.scale),
-                          __float_as_uint(__uint_as_float(r[4 * g + 3]) * p.scale));
+            const uint32_t chunk = static_cast<uint32_t>(g ^ (lane & 7)) * 16;
+            st_shared_v4w(stage_row + chunk, __float_as_uint(__uint_as_float(r[k][4 * g]) * p.scale),
+                          __float_as_uint(__uint_as_float(r[k][4 * g + 1]) * p.scale),
+                          __float_as_uint(__uint_as_float(r[k][4 * g + 2]) * p.scale),
+                          __float_as_uint(__uint_as_float(r[k][4 * g + 3]) * p.scale));
           }
           fence_proxy_async_smem();
-          named_bar_sync(3, 128);
-          if (tid == 512 && ok && k < nbox) {
-            tma_reduce_add_4d(&mdq, smem + C::OFF_DQ, 32 * k, I * BLK, qh, w.b);
+          __syncwarp();
+          if (lane == 0) {
+            tma_reduce_add_4d(&mdq, box, col, I * BLK + 32 * q4, qh, w.b);
             bulk_commit_group();
-            bulk_wait_group_read0();
           }
         }
       }
     }
-    if (tid == 512) bulk_wait_group0();                 // all reduce-adds have landed before the kernel ends
-  }
-  else {
+    if (lane == 0) bulk_wait_group0();                  // all reduce-adds have landed before the kernel ends
+  } else {
     // ------------------------------------------------------------------ compute warps (16 x 32 threads)
-    // warp = 4 cq + q4: lane quarter q4 (TMEM lane = key row), 16 query columns cq of the 64-column half tile
+    // warp = 4 cq + q4: lane quarter q4 (TMEM lane = key row), query columns 32 cq .. 32 cq + 31 of the tile
+    reg_inc<80>();
     const int q4 = warp & 3, cq = warp >> 2;
     const int rowl = q4 * 32 + lane;
     const uint32_t lane_base = static_cast<uint32_t>(q4 * 32) << 16;
-    const uint32_t t_s = tmem + lane_base + C::COL_S + 16 * cq;
-    const uint32_t t_dp = tmem + lane_base + C::COL_DP + 16 * cq;
-    float* r2raw = reinterpret_cast<float*>(smem + C::OFF_TAB);   // [256] rho' over the tile's band of distances
+    const uint32_t t_x = tmem + lane_base + C::COL_X + 32 * cq;
+    const uint32_t t_y = tmem + lane_base + C::COL_Y + 32 * cq;
+    float* r2raw = reinterpret_cast<float*>(smem + C::OFF_DS);     // [256] rho' over the tile's band of distances
     float* z2s = r2raw + 256;                                      // [128] logZ' of the tile's queries
-    uint32_t nsdp = 0, nacc = 0, gt = 0, npf = 0;
+    uint32_t ns = 0, nacc = 0, nq = 0, npf = 0;
     bool ok = true;
     // A warp whose wait was abandoned keeps walking (without storing) to the next agreement barrier, where all
     // sixteen leave together; none is ever left alone at a named barrier.
@@ -443,7 +442,7 @@ saf_bwd128_kernel(const __grid_constant__ CUtensorMap mk, const __grid_constant_
       const WorkItem w = nxt.w;
       const bool fast = nxt.fast;                        // (the next item is fetched under the epilogue's wait)
       const bool ord = w.kind == KIND_ORDINARY;
-      const int U = 2 * (nblk - w.blk);
+      const int nt = nblk - w.blk;
       int key = w.blk * BLK + rowl;
       float dv_mul = 1.0f;
       if (named_bar_or(1, 512, !ok)) break;
@@ -451,103 +450,125 @@ saf_bwd128_kernel(const __grid_constant__ CUtensorMap mk, const __grid_constant_
         // tensor-core form: nothing to do per tile; lane m holds key 127-m, scaled by a(j) below
         key = w.blk * BLK + 127 - rowl;
         dv_mul = (key < p.T) ? p.avec[static_cast<size_t>(w.h) * p.Tp + key] * (1.0f / HK_BAND_SCALE) : 0.0f;
+        nq += nt;
       } else if (ord) {
-        const float c = p.scale_log2;
-        for (int u = 0; u < U; ++u) {
-          const int b = u & 1;
-          if (!mbar_wait_warp(s_full, nsdp & 1, wc, W_S_FULL)) ok = false;
+        const uint64_t c2 = pk2(p.scale_log2, p.scale_log2);
+        for (int t = 0; t < nt; ++t, ++nq, ++ns) {
+          const uint32_t aux = smem_u32(smem + C::OFF_AUX) + (nq % C::NS) * 1024 + cq * 128;
+          if (warp == 0) TRB(1, 11);
+          // (the Q tile's barrier also covers its row terms: this thread reads them, so it waits for it itself)
+          if (!mbar_wait_warp(q_full + nq % C::NS, (nq / C::NS) & 1, wc, W_Q_FULL)) ok = false;
+          if (!mbar_wait_warp(s_full, ns & 1, wc, W_S_FULL)) ok = false;
           tc_fence_after();
-          // P^T of this warp's 16 query columns from S'^T alone; dP'^T is still on the tensor core
-          uint32_t rs[16];
-          tmem_ld16(t_s, rs);
+          if (warp == 0) TRB(1, 12);
+          uint32_t rs[32];
+          tmem_ld32(t_x, rs);
           tmem_wait_ld();
           {
-            uint32_t pk[8];
+            uint32_t pk[16];
 #pragma unroll
-            for (int e = 0; e < 8; ++e) {
-              float p0 = ex2_approx(__uint_as_float(rs[2 * e]) * c);
-              float p1 = ex2_approx(__uint_as_float(rs[2 * e + 1]) * c);
-              if (u < 2) {                                 // diagonal tile: query index >= key index
-                const int qa = 64 * b + 16 * cq + 2 * e;
-                if (qa < rowl) p0 = 0.0f;
-                if (qa + 1 < rowl) p1 = 0.0f;
+            for (int e4 = 0; e4 < 8; ++e4) {
+              float z[4];
+              ld_shared_v4f(aux + e4 * 16, z[0], z[1], z[2], z[3]);       // -LSE log2 e of four queries
+#pragma unroll
+              for (int k = 0; k < 2; ++k) {
+                const int e = 2 * e4 + k;
+                float p0, p1;
+                upk2(fma2(pk2(__uint_as_float(rs[2 * e]), __uint_as_float(rs[2 * e + 1])), c2, pk2(z[2 * k], z[2 * k + 1])), p0, p1);
+                p0 = ex2_approx(p0);
+                p1 = ex2_approx(p1);
+                if (t == 0) {                              // diagonal tile: query index >= key index
+                  const int qa = 32 * cq + 2 * e;
+                  if (qa < rowl) p0 = 0.0f;
+                  if (qa + 1 < rowl) p1 = 0.0f;
+                }
+                rs[2 * e] = __float_as_uint(p0);
+                rs[2 * e + 1] = __float_as_uint(p1);
+                pk[e] = pack_bf16x2(p0, p1);
               }
-              rs[2 * e] = __float_as_uint(p0);
-              rs[2 * e + 1] = __float_as_uint(p1);
-              pk[e] = pack_bf16x2(p0, p1);
             }
-            tmem_st8(t_s, pk);                             // bf16 pairs re-use columns this warp has consumed
-          }
-          if (!mbar_wait_warp(sdp_full, nsdp & 1, wc, W_SDP_FULL)) ok = false;
-          ++nsdp;
-          tc_fence_after();
-          if (b == 0) {
-            // the dQ MMAs of the previous tile have read the smem dS^T tile
-            if (!mbar_wait_warp(c_done, (gt & 1) ^ 1, wc, W_C_DONE)) ok = false;
-          }
-          uint32_t rd[16], dk[8];
-          tmem_ld16(t_dp, rd);
-          tmem_wait_ld();
-#pragma unroll
-          for (int e = 0; e < 8; ++e)
-            dk[e] = pack_bf16x2(__uint_as_float(rs[2 * e]) * __uint_as_float(rd[2 * e]),
-                                __uint_as_float(rs[2 * e + 1]) * __uint_as_float(rd[2 * e + 1]));
-          tmem_st8(t_dp, dk);
-          // dS^T row (this key) -> smem panel of this query half, 128-byte swizzle (chunk ^= row & 7)
-          const uint32_t rowaddr = smem_u32(smem + C::OFF_DS + b * C::PANEL) + rowl * 128;
-#pragma unroll
-          for (int g = 0; g < 2; ++g) {
-            const uint32_t chunk = static_cast<uint32_t>((2 * cq + g) ^ (rowl & 7));
-            st_shared_v4w(rowaddr + chunk * 16, dk[4 * g], dk[4 * g + 1], dk[4 * g + 2], dk[4 * g + 3]);
+            tmem_st16(t_x, pk);                            // bf16 pairs re-use columns this warp has consumed
           }
           tmem_wait_st();
+          tc_fence_before();
+          warp_arrive(p_full);
+          if (warp == 0) TRB(1, 13);
+          if (!mbar_wait_warp(dp_full, ns & 1, wc, W_DP_FULL)) ok = false;
+          tc_fence_after();
+          if (warp == 0) TRB(1, 14);
+          // dS^T row (this key) -> smem panel of this query half, 128-byte swizzle (chunk ^= row & 7).  (The MMAs that read
+          // the tile's previous contents were issued before dP(t): they have completed.)
+          const uint32_t rowaddr = smem_u32(smem + C::OFF_DS + (cq >> 1) * C::PANEL) + rowl * 128;
+#pragma unroll
+          for (int hf = 0; hf < 2; ++hf) {
+            uint32_t rd[16], dk[8];
+            tmem_ld16(t_y + 16 * hf, rd);
+            tmem_wait_ld();
+#pragma unroll
+            for (int e4 = 0; e4 < 4; ++e4) {
+              float z[4];
+              ld_shared_v4f(aux + 512 + hf * 64 + e4 * 16, z[0], z[1], z[2], z[3]);     // -delta of four queries
+#pragma unroll
+              for (int k = 0; k < 2; ++k) {
+                const int e = 2 * e4 + k;
+                float d0, d1;
+                upk2(mul2(add2(pk2(__uint_as_float(rd[2 * e]), __uint_as_float(rd[2 * e + 1])), pk2(z[2 * k], z[2 * k + 1])),
+                          pk2(__uint_as_float(rs[16 * hf + 2 * e]), __uint_as_float(rs[16 * hf + 2 * e + 1]))),
+                     d0, d1);
+                dk[e] = pack_bf16x2(d0, d1);
+              }
+            }
+#pragma unroll
+            for (int g = 0; g < 2; ++g) {
+              const uint32_t chunk = static_cast<uint32_t>((4 * (cq & 1) + 2 * hf + g) ^ (rowl & 7));
+              st_shared_v4w(rowaddr + chunk * 16, dk[4 * g], dk[4 * g + 1], dk[4 * g + 2], dk[4 * g + 3]);
+            }
+          }
           fence_proxy_async_smem();
           tc_fence_before();
-          warp_arrive(pds_full);
-          if (b == 1) ++gt;
+          warp_arrive(ds_full);
+          if (warp == 0) TRB(1, 15);
         }
       } else {
-        // ---------------- frozen head, general form: P^^T half tiles, one exponential per element
+        // ---------------- frozen head, general form: P^^T tiles, one exponential per element
+        nq += nt;
         const float* alpha_h = p.alpha + static_cast<size_t>(w.h) * p.Tp;
         const float* rho_h = p.rho + static_cast<size_t>(w.h) * p.Tp;
         const float* logz_h = p.logZ + static_cast<size_t>(w.h) * p.Tp;
         const float a2 = (key < p.T) ? alpha_h[key] * LOG2E_W : -INFINITY;
         bool leave = false;
-        for (int u = 0; u < U; ++u) {
-          const int b = u & 1, t = u >> 1;
-          if (b == 0) {
-            if (named_bar_or(1, 512, !ok)) {               // previous tile's table readers are done; agree to go on
-              ok = false;
-              leave = true;
-              break;
-            }
-            const int d = t * BLK - 127 + tid;             // band entry x = tid: distance of (query - key + 127)
-            if (tid < 256) r2raw[tid] = (tid < 255 && d >= 0 && d < p.T) ? rho_h[d] * LOG2E_W : -INFINITY;
-            if (tid < 128) {
-              const int qi = (w.blk + t) * BLK + tid;
-              z2s[tid] = (qi < p.T) ? logz_h[qi] * LOG2E_W : INFINITY;
-            }
-            named_bar_sync(2, 512);
+        for (int t = 0; t < nt; ++t) {
+          if (named_bar_or(1, 512, !ok)) {                 // previous tile's table readers are done; agree to go on
+            ok = false;
+            leave = true;
+            break;
           }
-          if (u > 0) {                                     // the previous P^^T half tile has been consumed
+          const int d = t * BLK - 127 + tid;               // band entry x = tid: distance of (query - key + 127)
+          if (tid < 256) r2raw[tid] = (tid < 255 && d >= 0 && d < p.T) ? rho_h[d] * LOG2E_W : -INFINITY;
+          if (tid < 128) {
+            const int qi = (w.blk + t) * BLK + tid;
+            z2s[tid] = (qi < p.T) ? logz_h[qi] * LOG2E_W : INFINITY;
+          }
+          named_bar_sync(2, 512);
+          if (t > 0) {                                     // the previous P^^T tile has been consumed
             if (!mbar_wait_warp(pfree, npf & 1, wc, W_PFREE)) ok = false;
             ++npf;
             tc_fence_after();
           }
-          const int q0 = 64 * b + 16 * cq;
+          const int q0 = 32 * cq;
           const float* rb = r2raw + (q0 - rowl + 127);
-          uint32_t pk[8];
+          uint32_t pk[16];
 #pragma unroll
-          for (int e = 0; e < 8; ++e)
+          for (int e = 0; e < 16; ++e)
             pk[e] = pack_bf16x2(ex2_approx(a2 + rb[2 * e] - z2s[q0 + 2 * e]),
                                 ex2_approx(a2 + rb[2 * e + 1] - z2s[q0 + 2 * e + 1]));
-          tmem_st8(t_s, pk);
+          tmem_st16(t_x, pk);
           tmem_wait_st();
           tc_fence_before();
-          warp_arrive(pds_full);
+          warp_arrive(p_full);
         }
         if (leave) break;
-        // keep the barrier in step: absorb the completion of the last half tile
+        // keep the barrier in step: absorb the completion of the last tile
         if (!mbar_wait_warp(pfree, npf & 1, wc, W_PFREE)) ok = false;
         ++npf;
       }
@@ -607,18 +628,18 @@ saf_bwd128_kernel(const __grid_constant__ CUtensorMap mk, const __grid_constant_
   tc_fence_before();
   __syncthreads();
   SAF_SPAN(bwd128, 1);
-  if (warp == 21) tmem_dealloc(tmem, C::TMEM_COLS);
+  if (warp == 25) tmem_dealloc(tmem, C::TMEM_COLS);
 }
 
 int bwd128_smem_bytes() { return W128::SMEM; }
 
-cudaError_t launch_bwd128(const CUtensorMap& mk, const CUtensorMap& mv, const CUtensorMap& mqh, const CUtensorMap& mdoh,
-                          const CUtensorMap& mdoth, const CUtensorMap& mdq, const BwdParams& p, int grid,
+cudaError_t launch_bwd128(const CUtensorMap& mk, const CUtensorMap& mv, const CUtensorMap& mq, const CUtensorMap& mdo,
+                          const CUtensorMap& mdot, const CUtensorMap& mdq, const BwdParams& p, int grid,
                           cudaStream_t st) {
   cudaError_t e =
       cudaFuncSetAttribute(saf_bwd128_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, W128::SMEM);
   if (e != cudaSuccess) return e;
-  return launch_pdl(PDL_BWD, saf_bwd128_kernel, dim3(grid), dim3(W128::NTHREADS), W128::SMEM, st, mk, mv, mqh, mdoh, mdoth, mdq, p);
+  return launch_pdl(PDL_BWD, saf_bwd128_kernel, dim3(grid), dim3(W128::NTHREADS), W128::SMEM, st, mk, mv, mq, mdo, mdot, mdq, p);
 }
 
 }  // namespace saf

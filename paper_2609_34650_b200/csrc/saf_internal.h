@@ -207,10 +207,11 @@ cudaError_t launch_bwd_finalize(const float* dQacc, void* dQ, size_t n, cudaStre
 cudaError_t launch_fwd64(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv, const CUtensorMap& mvt,
                          const CUtensorMap& mo, const FwdParams& p, int grid, cudaStream_t st);
 int fwd64_smem_bytes();
-// head dimension 128 / 96 (saf_bwd128.cu): mqh / mdoh / mdoth are maps with 64-row boxes (half tiles), mdq the fp32 dQ
-// accumulator [B][Hq][T][D]; dK / dV are written with plain stores (reduce-adds for shared heads)
-cudaError_t launch_bwd128(const CUtensorMap& mk, const CUtensorMap& mv, const CUtensorMap& mqh, const CUtensorMap& mdoh,
-                          const CUtensorMap& mdoth, const CUtensorMap& mdq, const BwdParams& p, int grid,
+// head dimension 128 / 96 (saf_bwd128.cu): mdot as in launch_bwd, mdq the fp32 dQ accumulator [B][Hq][T][D] in boxes of 32
+// rows; q_ext / do_ext of the parameters are fp32 vectors [B][H][128 nblk] (-LSE log2 e, -delta); dK / dV are written with
+// plain stores (reduce-adds for shared heads)
+cudaError_t launch_bwd128(const CUtensorMap& mk, const CUtensorMap& mv, const CUtensorMap& mq, const CUtensorMap& mdo,
+                          const CUtensorMap& mdot, const CUtensorMap& mdq, const BwdParams& p, int grid,
                           cudaStream_t st);
 int bwd128_smem_bytes();
 int fwd_smem_bytes(int D);

@@ -246,6 +246,7 @@ __device__ __forceinline__ uint4 split3_bf16(float x) {
 //                  rows beyond T: q_ext = most negative bf16 (their probabilities become 0), do_ext = 0
 //   every head   : dQacc row = 0 (it is accumulated by reduce-adds of the main kernel)
 //   frozen head  : dK row = 0 (no key gradient; Sec. 3.3); with the tensor-core form, the row w(i) dO in fp16
+//   (D != 64: q_ext = -LSE log2 e and do_ext = -delta as fp32 vectors over the rows instead of images)
 // Image layout per 128-row block (4 KB): byte (n/8)*256 + (k/8)*128 + (n%8)*16 + (k%8)*2 for row n, column k < 16.
 // (TPR threads per row: D / 8, or 16 with four idle ones at D = 96 so that a row stays inside a warp)
 // (OF32: O is fp32 instead of bf16, same element strides)
@@ -357,6 +358,12 @@ __global__ void __launch_bounds__(256, 8) saf_bwd_prep_kernel(const void* __rest
   for (int o = TPR / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
   if (inrange && part == 0 && !frozen) {
     const size_t bh = static_cast<size_t>(b) * H + h;
+    if constexpr (D != 64) {
+      // 128-wide backward: plain fp32 vectors over the padded rows (-inf: probabilities of rows beyond T become 0)
+      reinterpret_cast<float*>(q_ext)[bh * Tpad + t] = valid ? -LSE[bh * T + t] * 1.4426950408889634f : -INFINITY;
+      reinterpret_cast<float*>(do_ext)[bh * Tpad + t] = valid ? -acc : 0.0f;
+      return;
+    }
     const size_t img = (bh * (Tpad / 128) + t / 128) * 4096 + ((t % 128) / 8) * 256 + (t % 8) * 16;
     uint4 qv, dv;
     if (valid) {
