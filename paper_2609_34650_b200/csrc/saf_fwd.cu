@@ -184,8 +184,8 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
         uint32_t nq0 = 0, nq1 = 0;                 // uses of the two Q areas
         bool ok = true;
         // Claim the next item of the queue and publish it to the other roles.  Claimed CLAIM_AHEAD tiles before the current
-        // item's last: the claim's two global round trips and the loads of Q_0 and K_0 behind it then fit under the
-        // tiles that are left (claimed behind the item's last load they cost ~13000 clk an item).
+        // item's last, but behind the loads of its first two: the claim's global round trips and the loads of Q_0 and K_0
+        // behind it then fit under the tiles that are left (claimed behind the item's last load they cost ~13000 clk an item).
         int4 next;
         uint32_t nclaim = 0;
         bool claimed = false;
@@ -195,7 +195,9 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
           if (!ok) return;
           ++nclaim;
           claimed = true;
-          const int idx = atomicAdd(p.queue, 1);
+          // (a CTA's first item is its own number; a grid of one item per CTA does not touch the queue)
+          const int grid = static_cast<int>(gridDim.x);
+          const int idx = nclaim == 1 ? static_cast<int>(blockIdx.x) : p.n_items <= grid ? p.n_items : grid + atomicAdd(p.queue, 1);
           next = make_int4(0, 0, 0, RING_END);
           if (idx < p.n_items) {
             next = __ldg(reinterpret_cast<const int4*>(p.order + idx));
@@ -247,7 +249,7 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
               bulk_load(smem + C::OFF_BAND + s * 8192 + 4096, bands + static_cast<size_t>(d) * 4096, 4096, kv_full + s);
               if (two) bulk_load(smem + C::OFF_BAND + s * 8192, bands + static_cast<size_t>(d - 1) * 4096, 4096, kv_full + s);
               ++n;
-              if (!claimed && j + C::CLAIM_AHEAD >= n1) claim();
+              if (!claimed && j + C::CLAIM_AHEAD >= n1 && (j > 0 || n1 == 1)) claim();
               if (!ok) break;
             }
             if (!ok) break;
@@ -275,7 +277,7 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
             ++nq1;
             load_kv(&mv, 0, hv);
             for (int j = 1;; ++j) {
-              if (ok && !claimed && j + C::CLAIM_AHEAD > n1) claim();
+              if (ok && !claimed && j + C::CLAIM_AHEAD > n1 && (j > 1 || j == n1)) claim();
               if (j == n1 || !ok) break;
               load_kv(&mk, j, hk);
               if (ok) load_kv(&mv, j, hv);
@@ -763,7 +765,7 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
   __syncthreads();
   SAF_SPAN(fwd128, 1);
   if (warp == 13) tmem_dealloc(tmem, C::TMEM_COLS);
-  if (tid == 0) {
+  if (tid == 0 && p.n_items > static_cast<int>(gridDim.x)) {
     // this CTA claims nothing more; the last CTA to get here rewinds the queue for the next launch
     __threadfence();
     if (atomicAdd(p.queue + 1, 1) == static_cast<int>(gridDim.x) - 1) {
@@ -781,7 +783,7 @@ cudaError_t launch_fwd(int D, const CUtensorMap& mq, const CUtensorMap& mk, cons
   if (D == 64) return launch_fwd64(mq, mk, mv, mvt, mo, p, grid, st);   // head dimension 64 has its own kernel
   cudaError_t e = cudaFuncSetAttribute(saf_fwd_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdCfg<128>::SMEM);
   if (e != cudaSuccess) return e;
-  return launch_pdl(PDL_FWD, saf_fwd_kernel<128>, dim3(grid), dim3(FwdCfg<128>::NTHREADS), FwdCfg<128>::SMEM, st, mq, mk, mv,
+  return launch_pdl(PDL_FWD128, saf_fwd_kernel<128>, dim3(grid), dim3(FwdCfg<128>::NTHREADS), FwdCfg<128>::SMEM, st, mq, mk, mv,
                     mvt, p);
 }
 
