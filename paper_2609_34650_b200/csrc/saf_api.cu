@@ -83,12 +83,19 @@ struct saf_ctx {
   cudaStream_t mask_stream = nullptr, qslot_stream = nullptr;
   // tensor-core form of frozen heads: tables built by saf_pattern_prepare, scaled V / dO per call
   PatternCache pat;
+  std::vector<int> pat_heads_host;         // what pat_heads holds (and its upload source), and the stream that wrote it
+  cudaStream_t pat_heads_stream = nullptr;
   bool tensor_pattern = true;              // SAF_DISABLE_TENSOR_PATTERN=1 turns the form off
   bool selftest_drop_load = false;         // SAF_SELFTEST_DROP_LOAD=1: see FwdParams::selftest_drop_load
-  DevBuf pat_consts, pat_ok, pat_avec, pat_wvec, pat_bandf, pat_bandb, pat_hord, pat_hlist, pat_snap, vt_buf, dot_buf, ok_fwd, ok_bwd, pg_hlist, pg_delta, pg_items, pg_offsets, fit_buf, calib_tmp;
+  DevBuf pat_consts, pat_ok, pat_avec, pat_wvec, pat_bandf, pat_bandb, pat_heads, pat_snap, pat_marks, vt_buf, dot_buf, pg_hlist, pg_delta, pg_items, pg_offsets, fit_buf, calib_tmp;
   std::vector<int> pg_hlist_host, pg_offsets_host;   // host copies of the pattern-gradient tables (upload sources)
   std::vector<PgItem> pg_items_host;
   std::array<int, 5> pg_key = {0, 0, 0, 0, 0};      // (B, frozen heads, T, D, grid) the work list was built for
+  // pat_heads: hord[H] (head -> ordinal among the frozen heads, -1), then hlist; pat_marks: overflow marks of the forward,
+  // of the backward, counters of the normaliser kernel, a third of the buffer each
+  const int* pat_hord() const { return static_cast<const int*>(pat_heads.ptr); }
+  const int* pat_hlist() const { return pat_hord() + pat.H; }
+  int* pat_mark(int which) const { return static_cast<int*>(pat_marks.ptr) + which * (pat_marks.bytes / 3 / sizeof(int)); }
   bool profiling = false;
   std::vector<TimedLaunch> timed;          // event pairs recorded since the last query
   std::vector<cudaEvent_t> event_pool;
@@ -523,7 +530,7 @@ int saf_destroy(saf_ctx* ctx) {
     cudaFree(e.order_dev);
   }
   DevBuf* pbufs[] = {&ctx->pat_consts, &ctx->pat_ok, &ctx->pat_avec, &ctx->pat_wvec, &ctx->pat_bandf, &ctx->pat_bandb,
-                     &ctx->pat_hord, &ctx->pat_hlist, &ctx->pat_snap, &ctx->vt_buf, &ctx->dot_buf, &ctx->ok_fwd, &ctx->ok_bwd, &ctx->pg_hlist, &ctx->pg_delta, &ctx->pg_items, &ctx->pg_offsets, &ctx->fit_buf, &ctx->calib_tmp};
+                     &ctx->pat_heads, &ctx->pat_snap, &ctx->pat_marks, &ctx->vt_buf, &ctx->dot_buf, &ctx->pg_hlist, &ctx->pg_delta, &ctx->pg_items, &ctx->pg_offsets, &ctx->fit_buf, &ctx->calib_tmp};
   for (DevBuf* b : pbufs) release(*b);
   DevBuf* bufs[] = {&ctx->mask_buf, &ctx->logz_buf, &ctx->delta_buf, &ctx->dqacc_buf, &ctx->dkacc_buf, &ctx->dvacc_buf, &ctx->qslot_buf, &ctx->hq, &ctx->hk, &ctx->hv,
                     &ctx->hdo, &ctx->ho, &ctx->hlse, &ctx->hdq, &ctx->hdk, &ctx->hdv, &ctx->halpha, &ctx->hrho,
@@ -559,58 +566,59 @@ int saf_pattern_prepare(saf_ctx* ctx, int32_t H, int32_t Tp, const uint8_t* froz
   int rc = upload_mask(ctx, frozen_mask_host, H, st);
   if (rc) return rc;
   ctx->last_stream = st;
-  {
-    ScopedTimer timer(ctx, SAF_KERNEL_LOGZ, st);
-    if (launch_logz(alpha_dev, rho_dev, logZ_dev_out, static_cast<const uint8_t*>(ctx->mask_buf.ptr), H, Tp, st) !=
-        cudaSuccess)
-      return SAF_ERR_CUDA;
-  }
   ctx->pat.valid = false;
-  if (!ctx->tensor_pattern) return SAF_OK;
-  // tables of the tensor-core form (Hankel bands of exp(rho), key scale a, row scale w, per-head flag)
+  if (!ctx->tensor_pattern) {
+    ScopedTimer timer(ctx, SAF_KERNEL_LOGZ, st);
+    return launch_logz(alpha_dev, rho_dev, logZ_dev_out, static_cast<const uint8_t*>(ctx->mask_buf.ptr), H, Tp, nullptr,
+                       nullptr, nullptr, st) == cudaSuccess ? SAF_OK : SAF_ERR_CUDA;
+  }
+  // tables of the tensor-core form (Hankel bands of exp(rho), key scale a, row scale w, per-head flag) and the snapshot of
+  // the three vectors: the tables are matched to a later call by these pointers, and the staging kernels compare the
+  // bits, so a head whose vectors were rewritten in place since (by the caller, by the fitter, by the allocation-free
+  // normaliser entry point) falls back to the general form instead of using stale tables
   const int nblkp = (Tp + 127) / 128;
   const size_t vecb = static_cast<size_t>(H) * Tp * sizeof(float);
   const size_t bandb = static_cast<size_t>(H) * nblkp * 4096;
-  if ((rc = ensure(ctx->pat_consts, static_cast<size_t>(H) * 2 * sizeof(float))) ||
-      (rc = ensure(ctx->pat_ok, static_cast<size_t>(H) * sizeof(int))) || (rc = ensure(ctx->pat_avec, vecb)) ||
+  const size_t hb = static_cast<size_t>(std::max(H, 64)) * sizeof(int);
+  const size_t marks_before = ctx->pat_marks.bytes, heads_before = ctx->pat_heads.bytes;
+  if ((rc = ensure(ctx->pat_consts, 2 * hb)) || (rc = ensure(ctx->pat_ok, hb)) || (rc = ensure(ctx->pat_avec, vecb)) ||
       (rc = ensure(ctx->pat_wvec, vecb)) || (rc = ensure(ctx->pat_bandf, bandb)) ||
-      (rc = ensure(ctx->pat_bandb, bandb)) || (rc = ensure(ctx->pat_hord, static_cast<size_t>(H) * sizeof(int))) ||
-      (rc = ensure(ctx->pat_hlist, static_cast<size_t>(H) * sizeof(int))) || (rc = ensure(ctx->pat_snap, 3 * vecb)) ||
-      (rc = ensure(ctx->ok_fwd, static_cast<size_t>(H) * sizeof(int))) ||
-      (rc = ensure(ctx->ok_bwd, static_cast<size_t>(H) * sizeof(int))))
+      (rc = ensure(ctx->pat_bandb, bandb)) || (rc = ensure(ctx->pat_heads, 2 * hb)) || (rc = ensure(ctx->pat_snap, 3 * vecb)) ||
+      (rc = ensure(ctx->pat_marks, 3 * hb)))
     return rc;
-  // per-head overflow marks of the forward / backward staging kernels (a mark is the id of the call that set it)
-  if (cudaMemsetAsync(ctx->ok_fwd.ptr, 0, static_cast<size_t>(H) * sizeof(int), st) != cudaSuccess ||
-      cudaMemsetAsync(ctx->ok_bwd.ptr, 0, static_cast<size_t>(H) * sizeof(int), st) != cudaSuccess)
-    return SAF_ERR_CUDA;
-  std::vector<int> hord(H, -1), hlist(H, 0);
-  int ord = 0;
-  for (int h = 0; h < H; ++h)
+  // A new buffer starts at zero: per-head overflow marks of the forward / backward staging kernels (a mark is the id of the
+  // call that set it, ids only grow) and the counters of the normaliser kernel (which returns them to zero).
+  if (ctx->pat_heads.bytes != heads_before) ctx->pat_heads_host.clear();
+  if (ctx->pat_marks.bytes != marks_before) {
+    if (cudaMemsetAsync(ctx->pat_marks.ptr, 0, ctx->pat_marks.bytes, st) != cudaSuccess) return SAF_ERR_CUDA;
+  }
+  // ordinals of the frozen heads, uploaded when the mask (or the stream) is another one: hord[H], then hlist
+  std::vector<int> heads(2 * static_cast<size_t>(H), 0);
+  for (int h = 0, ord = 0; h < H; ++h) {
+    heads[h] = -1;
     if (frozen_mask_host[h]) {
-      hlist[ord] = h;
-      hord[h] = ord++;
+      heads[H + ord] = h;
+      heads[h] = ord++;
     }
-  if (cudaMemcpyAsync(ctx->pat_hord.ptr, hord.data(), static_cast<size_t>(H) * sizeof(int), cudaMemcpyHostToDevice, st) !=
-          cudaSuccess ||
-      cudaMemcpyAsync(ctx->pat_hlist.ptr, hlist.data(), static_cast<size_t>(H) * sizeof(int), cudaMemcpyHostToDevice,
-                      st) != cudaSuccess)
-    return SAF_ERR_CUDA;
+  }
+  if (heads != ctx->pat_heads_host || ctx->pat_heads_stream != st) {
+    ctx->pat_heads_host = heads;
+    ctx->pat_heads_stream = st;
+    if (cudaMemcpyAsync(ctx->pat_heads.ptr, ctx->pat_heads_host.data(), heads.size() * sizeof(int), cudaMemcpyHostToDevice,
+                        st) != cudaSuccess) {
+      ctx->pat_heads_host.clear();
+      return SAF_ERR_CUDA;
+    }
+  }
   {
     ScopedTimer timer(ctx, SAF_KERNEL_LOGZ, st);
-    if (launch_pattern_tables(alpha_dev, rho_dev, logZ_dev_out, static_cast<const uint8_t*>(ctx->mask_buf.ptr), H, Tp,
-                              static_cast<float*>(ctx->pat_consts.ptr), static_cast<int*>(ctx->pat_ok.ptr),
+    float* consts = static_cast<float*>(ctx->pat_consts.ptr);
+    if (launch_logz(alpha_dev, rho_dev, logZ_dev_out, static_cast<const uint8_t*>(ctx->mask_buf.ptr), H, Tp, consts,
+                    static_cast<int*>(ctx->pat_ok.ptr), reinterpret_cast<unsigned*>(ctx->pat_mark(2)), st) != cudaSuccess ||
+        launch_pattern_tables(alpha_dev, rho_dev, logZ_dev_out, static_cast<const uint8_t*>(ctx->mask_buf.ptr), H, Tp, consts,
                               static_cast<float*>(ctx->pat_avec.ptr), static_cast<float*>(ctx->pat_wvec.ptr),
-                              ctx->pat_bandf.ptr, ctx->pat_bandb.ptr, st) != cudaSuccess)
-      return SAF_ERR_CUDA;
-  }
-  // Snapshot of the three vectors: the tables are matched to a later call by these pointers, and the staging kernels
-  // compare the bits, so a head whose vectors were rewritten in place since (by the caller, by the fitter, by the
-  // allocation-free normaliser entry point) falls back to the general form instead of using stale tables.
-  {
-    uint8_t* snap = static_cast<uint8_t*>(ctx->pat_snap.ptr);
-    if (cudaMemcpyAsync(snap, alpha_dev, vecb, cudaMemcpyDeviceToDevice, st) != cudaSuccess ||
-        cudaMemcpyAsync(snap + vecb, rho_dev, vecb, cudaMemcpyDeviceToDevice, st) != cudaSuccess ||
-        cudaMemcpyAsync(snap + 2 * vecb, logZ_dev_out, vecb, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
+                              ctx->pat_bandf.ptr, ctx->pat_bandb.ptr, static_cast<uint32_t*>(ctx->pat_snap.ptr),
+                              st) != cudaSuccess)
       return SAF_ERR_CUDA;
   }
   ctx->pat.valid = true;
@@ -686,8 +694,8 @@ int saf_hybrid_attn_fwd(saf_ctx* ctx, const saf_problem* p, const void* Q, const
     {
       ScopedTimer timer(ctx, SAF_KERNEL_SCALE, st);
       if (launch_scale_rows(V, p->v_strides, static_cast<const float*>(ctx->pat_avec.ptr), HK_A_SCALE, p->Tp,
-                            static_cast<const int*>(ctx->pat_hlist.ptr), static_cast<const int*>(ctx->pat_ok.ptr),
-                            static_cast<int*>(ctx->ok_fwd.ptr), fp.call_id, ctx->vt_buf.ptr, p->B, nf, p->T, p->D,
+                            ctx->pat_hlist(), static_cast<const int*>(ctx->pat_ok.ptr),
+                            ctx->pat_mark(0), fp.call_id, ctx->vt_buf.ptr, p->B, nf, p->T, p->D,
                             kvg, pattern_check(ctx, alpha, rho, logZ), st) != cudaSuccess)
         return SAF_ERR_CUDA;
     }
@@ -696,8 +704,8 @@ int saf_hybrid_attn_fwd(saf_ctx* ctx, const saf_problem* p, const void* Q, const
     fp.band_f = ctx->pat_bandf.ptr;
     fp.wvec = static_cast<const float*>(ctx->pat_wvec.ptr);
     fp.fast_ok = static_cast<const int*>(ctx->pat_ok.ptr);
-    fp.ovf = static_cast<const int*>(ctx->ok_fwd.ptr);
-    fp.hord = static_cast<const int*>(ctx->pat_hord.ptr);
+    fp.ovf = ctx->pat_mark(0);
+    fp.hord = ctx->pat_hord();
   }
   fp.B = p->B; fp.H = p->H; fp.T = p->T; fp.Tp = p->Tp;
   fp.kv_group = kvg;
@@ -805,9 +813,9 @@ int saf_hybrid_attn_bwd(saf_ctx* ctx, const saf_problem* p, const void* Q, const
     rc = ensure(ctx->dot_buf, static_cast<size_t>(p->B) * nf * p->T * p->D * 2);
     if (rc) return rc;
     fz.wvec = static_cast<const float*>(ctx->pat_wvec.ptr);
-    fz.hord = static_cast<const int*>(ctx->pat_hord.ptr);
+    fz.hord = ctx->pat_hord();
     fz.pat_ok = static_cast<const int*>(ctx->pat_ok.ptr);
-    fz.ovf = static_cast<int*>(ctx->ok_bwd.ptr);
+    fz.ovf = ctx->pat_mark(1);
     fz.call_id = ++ctx->call_counter;
     fz.dot_dst = ctx->dot_buf.ptr;
     fz.Hf = nf;
@@ -1103,10 +1111,13 @@ int saf_pattern_grad(saf_ctx* ctx, const saf_problem* p, const void* V, const vo
   if (!g.ok) return SAF_ERR_CUDA;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   ctx->last_stream = st;
-  const size_t pbytes = static_cast<size_t>(p->H) * p->Tp * sizeof(float);
-  if (cudaMemsetAsync(dalpha_out, 0, pbytes, st) != cudaSuccess || cudaMemsetAsync(drho_out, 0, pbytes, st) != cudaSuccess)
-    return SAF_ERR_CUDA;
-  if (nf == 0) return SAF_OK;
+  const size_t n_vec = static_cast<size_t>(p->H) * p->Tp;
+  if (nf == 0) {
+    if (cudaMemsetAsync(dalpha_out, 0, n_vec * sizeof(float), st) != cudaSuccess ||
+        cudaMemsetAsync(drho_out, 0, n_vec * sizeof(float), st) != cudaSuccess)
+      return SAF_ERR_CUDA;
+    return SAF_OK;
+  }
   if (!V || !O || !dO || !alpha || !rho || !logZ) return SAF_ERR_INVALID_ARG;
   if (!aligned16(V) || !aligned16(O) || !aligned16(dO)) return SAF_ERR_INVALID_ARG;
   if (check_strides(p->v_strides, p->D) || check_strides(p->o_strides, p->D)) return SAF_ERR_INVALID_ARG;
@@ -1131,7 +1142,8 @@ int saf_pattern_grad(saf_ctx* ctx, const saf_problem* p, const void* V, const vo
   {
     ScopedTimer timer(ctx, SAF_KERNEL_BWD_PREP, st);
     if (launch_rowdot(O, p->o_dtype == SAF_F32, dO, p->o_strides, static_cast<const int*>(ctx->pg_hlist.ptr),
-                      static_cast<float*>(ctx->pg_delta.ptr), p->B, p->H, nf, p->T, p->D, st) != cudaSuccess)
+                      static_cast<float*>(ctx->pg_delta.ptr), dalpha_out, drho_out, static_cast<long long>(n_vec), p->B, p->H, nf,
+                      p->T, p->D, st) != cudaSuccess)
       return SAF_ERR_CUDA;
   }
   // Work list: (frozen-head ordinal, key block J, run of query blocks, run of batch entries), dealt longest first to

@@ -203,7 +203,9 @@ saf_fwd64_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
         const uint32_t slot = nclaim % C::NRING;
         ok = mbar_wait(ring_empty + slot, ((nclaim / C::NRING) & 1) ^ 1, wc, F_RING_EMPTY);
         if (!ok) break;
-        const int idx = atomicAdd(p.queue, 1);
+        // (a CTA's first item is its own number; a grid of one item per CTA does not touch the queue)
+        const int grid = static_cast<int>(gridDim.x);
+        const int idx = nclaim == 0 ? static_cast<int>(blockIdx.x) : p.n_items <= grid ? p.n_items : grid + atomicAdd(p.queue, 1);
         int4 rec = make_int4(0, 0, 0, RING_END);
         bool fast = false;
         if (idx < p.n_items) {
@@ -774,7 +776,7 @@ saf_fwd64_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
   __syncthreads();
   SAF_SPAN(fwd64, 1);
   if (warp == 9) tmem_dealloc(tmem, C::TMEM_COLS);
-  if (tid == 0) {
+  if (tid == 0 && p.n_items > static_cast<int>(gridDim.x)) {
     // this CTA claims nothing more; the last CTA to get here rewinds the queue for the next launch
     __threadfence();
     if (atomicAdd(p.queue + 1, 1) == static_cast<int>(gridDim.x) - 1) {

@@ -153,7 +153,8 @@ struct PgradParams {
   unsigned long long wait_limit_ns;
 };
 cudaError_t launch_rowdot(const void* O, int o_f32, const void* dO, const int64_t* o_strides, const int* hlist,
-                          float* delta, int B, int H, int Hf, int T, int D, cudaStream_t st);
+                          float* delta, float* zero0, float* zero1, long long n_zero, int B, int H, int Hf, int T, int D,
+                          cudaStream_t st);   // zero0 / zero1: n_zero floats each, set to zero
 cudaError_t launch_pgrad(int D, const CUtensorMap& mv, const CUtensorMap& mdo, const PgradParams& p, int grid,
                          cudaStream_t st);
 
@@ -167,11 +168,12 @@ struct PatternCheck {
   size_t vec_elems;                 // H * Tp
 };
 // Launchers (defined in the .cu files).  All return the launch error.
-cudaError_t launch_logz(const float* alpha, const float* rho, float* logZ, const uint8_t* mask_dev, int H,
-                        int Tp, cudaStream_t st);
+// (consts, fast_ok, counters: the head's constants of the tensor-core form, formed behind the normalisers; NULL to leave out)
+cudaError_t launch_logz(const float* alpha, const float* rho, float* logZ, const uint8_t* mask_dev, int H, int Tp,
+                        float* consts, int* fast_ok, unsigned* counters, cudaStream_t st);
 cudaError_t launch_pattern_tables(const float* alpha, const float* rho, const float* logZ, const uint8_t* mask_dev,
-                                  int H, int Tp, float* consts, int* fast_ok, float* avec, float* wvec, void* band_f,
-                                  void* band_b, cudaStream_t st);
+                                  int H, int Tp, const float* consts, float* avec, float* wvec, void* band_f,
+                                  void* band_b, uint32_t* snap, cudaStream_t st);
 cudaError_t launch_scale_rows(const void* src, const int64_t* strides, const float* vec, float extra, int Tp,
                               const int* hlist, const int* pat_ok, int* ovf, int call_id, void* dst, int B, int Hf,
                               int T, int D, int src_group, const PatternCheck& chk, cudaStream_t st);   // src head = h / src_group

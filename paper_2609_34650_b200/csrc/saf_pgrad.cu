@@ -324,8 +324,11 @@ template <int D, int TPR, bool OF32>
 __global__ void __launch_bounds__(256) saf_rowdot_kernel(const void* __restrict__ O,
                                                          const __nv_bfloat16* __restrict__ dO, int64_t s0, int64_t s1,
                                                          int64_t s2, const int* __restrict__ hlist,
-                                                         float* __restrict__ delta, int B, int H, int Hf, int T, int VB) {
+                                                         float* __restrict__ delta, float* __restrict__ zero0,
+                                                         float* __restrict__ zero1, long long n_zero, int B, int H, int Hf,
+                                                         int T, int VB) {
   const long long gid = static_cast<long long>(blockIdx.x) * 256 + threadIdx.x;
+  for (long long x = gid; x < n_zero; x += static_cast<long long>(gridDim.x) * 256) zero0[x] = zero1[x] = 0.0f;
   const long long rowid = gid / TPR;               // over [chunks][Hf][T]
   const int part = static_cast<int>(gid % TPR);
   const int nbc = (B + VB - 1) / VB;
@@ -372,6 +375,7 @@ __global__ void __launch_bounds__(256) saf_rowdot_kernel(const void* __restrict_
 }
 
 cudaError_t launch_rowdot(const void* O, int o_f32, const void* dO, const int64_t* os, const int* hlist, float* delta,
+                          float* zero0, float* zero1, long long n_zero,
                           int B, int H, int Hf, int T, int D, cudaStream_t st) {
   const int tpr = D == 96 ? 16 : D / 8;
   const int vb = pgrad_batch_chunk(D);
@@ -379,7 +383,7 @@ cudaError_t launch_rowdot(const void* O, int o_f32, const void* dO, const int64_
   const unsigned grid = static_cast<unsigned>((nthreads + 255) / 256);
 #define SAF_ROWDOT(DD, TT, FF) \
   saf_rowdot_kernel<DD, TT, FF><<<grid, 256, 0, st>>>(O, static_cast<const __nv_bfloat16*>(dO), os[0], os[1], os[2], \
-                                                      hlist, delta, B, H, Hf, T, vb)
+                                                      hlist, delta, zero0, zero1, n_zero, B, H, Hf, T, vb)
   if (D == 64) { if (o_f32) SAF_ROWDOT(64, 8, true); else SAF_ROWDOT(64, 8, false); }
   else if (D == 96) { if (o_f32) SAF_ROWDOT(96, 16, true); else SAF_ROWDOT(96, 16, false); }
   else { if (o_f32) SAF_ROWDOT(128, 16, true); else SAF_ROWDOT(128, 16, false); }

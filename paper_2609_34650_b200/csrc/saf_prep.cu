@@ -12,40 +12,133 @@
 namespace saf {
 
 // logZ[h][i] = log sum_{k<=i} exp(alpha[h][k] + rho[h][i-k])   (Eq. "compact-prior", the normaliser Z(i)).
-// One warp per row; two passes (row maximum, then the sum of exponentials); lane partials in fp32,
-// the 32 partials and the logarithm in fp64.
+// A block takes 32 consecutive rows (lane = row) and its eight warps take slices of the keys in turn; alpha and rho pass
+// through shared memory in chunks (alpha[k] is the same for a warp, rho[i-k] contiguous over its lanes), -inf where the
+// causal range ends.  The exponentials are taken relative to max alpha[0..] + max rho[0..] over the block's range, an upper
+// bound that needs no pass of its own; a row whose sum is then too small for fp32 (every term 2^-100 below the bound) is
+// done again relative to its own maximum.  fp32 sums of 32 terms, fp64 from there.  Bound: one ex2 per causal pair.
+// (One warp per row with two passes over global memory: 19.4 us for 6 heads x 2048, now see the launcher.)
+// The last block of a head to finish also forms the head's constants (consts != NULL): max alpha, max rho, and
+// whether the tensor-core form's range holds (see below); counters return to zero.
+constexpr int LZ_KC = 1024;
+__device__ __forceinline__ float block_max(float v, float* red) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  v = red[0];
+#pragma unroll
+  for (int k = 1; k < 8; ++k) v = fmaxf(v, red[k]);
+  return v;
+}
 __global__ void __launch_bounds__(256) saf_logz_kernel(const float* __restrict__ alpha, const float* __restrict__ rho,
-                                                       float* __restrict__ logZ, const uint8_t* __restrict__ mask,
-                                                       int Tp) {
-  const int h = blockIdx.y;
-  if (!mask[h]) return;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+                                                       float* logZ, const uint8_t* __restrict__ mask, int Tp,
+                                                       float* __restrict__ consts, int* __restrict__ fast_ok,
+                                                       unsigned* __restrict__ counters) {
+  __shared__ float sa[LZ_KC], sr[LZ_KC + 32], red[8];
+  __shared__ double part[8][32];
+  __shared__ int last;
+  const int h = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (!mask[h]) {
+    if (consts != nullptr && blockIdx.x == 0 && tid == 0) fast_ok[h] = 0;
+    return;
+  }
   // heavy (late) rows first so that the tail of the grid is cheap
-  const int i = Tp - 1 - (blockIdx.x * 8 + warp);
-  if (i < 0) return;
+  const int i0 = (static_cast<int>(gridDim.x) - 1 - static_cast<int>(blockIdx.x)) * 32;
+  const int i = i0 + lane, iend = min(Tp, i0 + 32);
   const float* a = alpha + static_cast<size_t>(h) * Tp;
   const float* r = rho + static_cast<size_t>(h) * Tp;
-  float m = -INFINITY;
-  for (int k = lane; k <= i; k += 32) m = fmaxf(m, a[k] + r[i - k]);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  float s0 = 0.0f, s1 = 0.0f;
-  int k = lane;
-  for (; k + 32 <= i; k += 64) {
-    s0 += __expf(a[k] + r[i - k] - m);
-    s1 += __expf(a[k + 32] + r[i - k - 32] - m);
+  float* z = logZ + static_cast<size_t>(h) * Tp;
+  float ma = -INFINITY, mr = -INFINITY;
+  for (int k = tid; k < iend; k += 256) {
+    ma = fmaxf(ma, a[k]);
+    mr = fmaxf(mr, r[k]);
   }
-  if (k <= i) s0 += __expf(a[k] + r[i - k] - m);
-  double s = static_cast<double>(s0) + static_cast<double>(s1);
+  const float bound = block_max(ma, red) + block_max(mr, red);
+  const float L2E = 1.4426950408889634f;
+  const float nb = -bound * L2E;
+  double s = 0.0;
+  for (int k0 = 0; k0 < iend; k0 += LZ_KC) {
+    __syncthreads();
+    for (int x = tid; x < LZ_KC; x += 256) sa[x] = k0 + x < iend ? a[k0 + x] : 0.0f;
+    // sr[x] = rho[i0 + x - (k0 + LZ_KC - 1)]
+    for (int x = tid; x < LZ_KC + 31; x += 256) {
+      const int d = i0 + x - (k0 + LZ_KC - 1);
+      sr[x] = d >= 0 && d < Tp ? r[d] : -INFINITY;
+    }
+    __syncthreads();
+    const int kb = warp * (LZ_KC / 8);                  // this warp's keys k0 + kb ...
+    if (k0 + kb >= iend) continue;
+    const float* rp = sr + lane + LZ_KC - 1 - kb;       // rp[-k] = rho[i - (k0 + kb + k)]
+#pragma unroll 1
+    for (int k = 0; k < LZ_KC / 8; k += 32) {
+      float p[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if (lane == 0) logZ[static_cast<size_t>(h) * Tp + i] = static_cast<float>(static_cast<double>(m) + log(s));
+      for (int e = 0; e < 32; e += 4) {
+        const float4 a4 = *reinterpret_cast<const float4*>(sa + kb + k + e);
+        p[0] += ex2_approx(fmaf(a4.x + rp[-k - e], L2E, nb));
+        p[1] += ex2_approx(fmaf(a4.y + rp[-k - e - 1], L2E, nb));
+        p[2] += ex2_approx(fmaf(a4.z + rp[-k - e - 2], L2E, nb));
+        p[3] += ex2_approx(fmaf(a4.w + rp[-k - e - 3], L2E, nb));
+      }
+      s += static_cast<double>((p[0] + p[1]) + (p[2] + p[3]));
+    }
+  }
+  part[warp][lane] = s;
+  __syncthreads();
+  for (int rr = 0; rr < 4; ++rr) {                      // four rows per warp
+    const int row = i0 + warp * 4 + rr;
+    double t = lane < 8 ? part[lane][warp * 4 + rr] : 0.0;
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    t = __shfl_sync(0xffffffffu, t, 0);
+    if (row >= Tp) continue;
+    float ref = bound;
+    if (!(t > 1e-30)) {
+      // the bound is too far above this row: two passes relative to its own maximum
+      float m = -INFINITY;
+      for (int k = lane; k <= row; k += 32) m = fmaxf(m, a[k] + r[row - k]);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+      float s0 = 0.0f;
+      for (int k = lane; k <= row; k += 32) s0 += __expf(a[k] + r[row - k] - m);
+      t = static_cast<double>(s0);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+      ref = m;
+    }
+    if (lane == 0) z[row] = static_cast<float>(static_cast<double>(ref) + log(t));
+  }
+  if (consts == nullptr) return;
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) last = atomicInc(counters + h, gridDim.x - 1) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  float mz = -INFINITY;
+  ma = mr = -INFINITY;
+  for (int t = tid; t < Tp; t += 256) {
+    ma = fmaxf(ma, a[t]);
+    mr = fmaxf(mr, r[t]);
+    mz = fmaxf(mz, -__ldcg(z + t));
+  }
+  ma = block_max(ma, red);
+  mr = block_max(mr, red);
+  mz = block_max(mz, red);
+  if (tid == 0) {
+    consts[2 * h] = ma;
+    consts[2 * h + 1] = mr;
+    const float wmax = ma + mr + mz;
+    fast_ok[h] = (wmax <= 9.0f && wmax > -1e30f && ma < 1e30f && mr < 1e30f) ? 1 : 0;
+  }
 }
 
 cudaError_t launch_logz(const float* alpha, const float* rho, float* logZ, const uint8_t* mask_dev, int H, int Tp,
-                        cudaStream_t st) {
-  dim3 grid((Tp + 7) / 8, H);
-  saf_logz_kernel<<<grid, 256, 0, st>>>(alpha, rho, logZ, mask_dev, Tp);
+                        float* consts, int* fast_ok, unsigned* counters, cudaStream_t st) {
+  dim3 grid((Tp + 31) / 32, H);
+  saf_logz_kernel<<<grid, 256, 0, st>>>(alpha, rho, logZ, mask_dev, Tp, consts, fast_ok, counters);
   return cudaGetLastError();
 }
 
@@ -67,52 +160,6 @@ cudaError_t launch_logz(const float* alpha, const float* rho, float* logZ, const
 // scaled units, i.e. the pattern entry w a r by at most w 2^-39: the form is used for a head only if
 // max_i (c_a + c_r - logZ(i)) <= 9 (fast_ok), which keeps that below 1e-8 and leaves w dO room in fp16
 // (the scaling kernel checks the staged values against fp16's range on every call).
-__global__ void __launch_bounds__(256) saf_pattern_consts_kernel(const float* __restrict__ alpha,
-                                                                 const float* __restrict__ rho,
-                                                                 const float* __restrict__ logZ,
-                                                                 const uint8_t* __restrict__ mask, int Tp,
-                                                                 float* __restrict__ consts, int* __restrict__ fast_ok) {
-  const int h = blockIdx.x;
-  if (!mask[h]) {
-    if (threadIdx.x == 0) fast_ok[h] = 0;
-    return;
-  }
-  __shared__ float red[3][8];
-  const float* a = alpha + static_cast<size_t>(h) * Tp;
-  const float* r = rho + static_cast<size_t>(h) * Tp;
-  const float* z = logZ + static_cast<size_t>(h) * Tp;
-  float ma = -INFINITY, mr = -INFINITY, mz = INFINITY;
-  for (int t = threadIdx.x; t < Tp; t += 256) {
-    ma = fmaxf(ma, a[t]);
-    mr = fmaxf(mr, r[t]);
-    mz = fminf(mz, z[t]);
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    ma = fmaxf(ma, __shfl_xor_sync(0xffffffffu, ma, o));
-    mr = fmaxf(mr, __shfl_xor_sync(0xffffffffu, mr, o));
-    mz = fminf(mz, __shfl_xor_sync(0xffffffffu, mz, o));
-  }
-  const int warp = threadIdx.x >> 5;
-  if ((threadIdx.x & 31) == 0) {
-    red[0][warp] = ma;
-    red[1][warp] = mr;
-    red[2][warp] = mz;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int k = 1; k < 8; ++k) {
-      ma = fmaxf(ma, red[0][k]);
-      mr = fmaxf(mr, red[1][k]);
-      mz = fminf(mz, red[2][k]);
-    }
-    consts[2 * h] = ma;
-    consts[2 * h + 1] = mr;
-    const float wmax = ma + mr - mz;
-    fast_ok[h] = (wmax <= 9.0f && wmax > -1e30f && ma < 1e30f && mr < 1e30f) ? 1 : 0;
-  }
-}
-
 __global__ void __launch_bounds__(256) saf_pattern_tables_kernel(const float* __restrict__ alpha,
                                                                  const float* __restrict__ rho,
                                                                  const float* __restrict__ logZ,
@@ -120,15 +167,22 @@ __global__ void __launch_bounds__(256) saf_pattern_tables_kernel(const float* __
                                                                  const float* __restrict__ consts,
                                                                  float* __restrict__ avec, float* __restrict__ wvec,
                                                                  __half* __restrict__ band_f,
-                                                                 __half* __restrict__ band_b, int nblkp) {
+                                                                 __half* __restrict__ band_b, uint32_t* __restrict__ snap,
+                                                                 int nblkp) {
   const int h = blockIdx.y, dblk = blockIdx.x;
   if (!mask[h]) return;
   const float ca = consts[2 * h], cr = consts[2 * h + 1];
   const size_t row = static_cast<size_t>(h) * Tp;
   const int t = dblk * 128 + threadIdx.x;
   if (threadIdx.x < 128 && t < Tp) {
-    avec[row + t] = __expf(alpha[row + t] - ca);
-    wvec[row + t] = __expf(ca + cr - logZ[row + t]);
+    const float at = alpha[row + t], rt = rho[row + t], zt = logZ[row + t];
+    avec[row + t] = __expf(at - ca);
+    wvec[row + t] = __expf(ca + cr - zt);
+    // the bits these tables stand for (see pattern_row_changed)
+    const size_t n = static_cast<size_t>(gridDim.y) * Tp;
+    snap[row + t] = __float_as_uint(at);
+    snap[n + row + t] = __float_as_uint(rt);
+    snap[2 * n + row + t] = __float_as_uint(zt);
   }
   const size_t band = (static_cast<size_t>(h) * nblkp + dblk) * 2048;
   for (int idx = threadIdx.x; idx < 2048; idx += 256) {
@@ -144,15 +198,12 @@ __global__ void __launch_bounds__(256) saf_pattern_tables_kernel(const float* __
 }
 
 cudaError_t launch_pattern_tables(const float* alpha, const float* rho, const float* logZ, const uint8_t* mask_dev, int H,
-                                  int Tp, float* consts, int* fast_ok, float* avec, float* wvec, void* band_f,
-                                  void* band_b, cudaStream_t st) {
+                                  int Tp, const float* consts, float* avec, float* wvec, void* band_f, void* band_b,
+                                  uint32_t* snap, cudaStream_t st) {
   const int nblkp = (Tp + 127) / 128;
-  saf_pattern_consts_kernel<<<H, 256, 0, st>>>(alpha, rho, logZ, mask_dev, Tp, consts, fast_ok);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
   saf_pattern_tables_kernel<<<dim3(nblkp, H), 256, 0, st>>>(alpha, rho, logZ, mask_dev, Tp, consts, avec, wvec,
                                                             static_cast<__half*>(band_f),
-                                                            static_cast<__half*>(band_b), nblkp);
+                                                            static_cast<__half*>(band_b), snap, nblkp);
   return cudaGetLastError();
 }
 
@@ -485,7 +536,7 @@ extern "C" int saf_pattern_logz_static(int32_t device, int32_t H, int32_t Tp, co
     if (cudaMemcpyAsync(scratch, g_static_mask_host, static_cast<size_t>(H), cudaMemcpyHostToDevice, st) != cudaSuccess)
       rc = SAF_ERR_CUDA;
   }
-  if (rc == SAF_OK && saf::launch_logz(alpha_dev, rho_dev, logZ_dev_out, scratch, H, Tp, st) != cudaSuccess)
+  if (rc == SAF_OK && saf::launch_logz(alpha_dev, rho_dev, logZ_dev_out, scratch, H, Tp, nullptr, nullptr, nullptr, st) != cudaSuccess)
     rc = SAF_ERR_CUDA;
   if (prev != device) cudaSetDevice(prev);
   return rc;
