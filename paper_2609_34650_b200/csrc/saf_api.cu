@@ -92,10 +92,10 @@ struct saf_ctx {
   std::vector<PgItem> pg_items_host;
   std::array<int, 5> pg_key = {0, 0, 0, 0, 0};      // (B, frozen heads, T, D, grid) the work list was built for
   // pat_heads: hord[H] (head -> ordinal among the frozen heads, -1), then hlist; pat_marks: overflow marks of the forward,
-  // of the backward, counters of the normaliser kernel, a third of the buffer each
+  // of the backward (a quarter of the buffer each), counters of the normaliser kernel (two per head)
   const int* pat_hord() const { return static_cast<const int*>(pat_heads.ptr); }
   const int* pat_hlist() const { return pat_hord() + pat.H; }
-  int* pat_mark(int which) const { return static_cast<int*>(pat_marks.ptr) + which * (pat_marks.bytes / 3 / sizeof(int)); }
+  int* pat_mark(int which) const { return static_cast<int*>(pat_marks.ptr) + which * (pat_marks.bytes / 4 / sizeof(int)); }
   bool profiling = false;
   std::vector<TimedLaunch> timed;          // event pairs recorded since the last query
   std::vector<cudaEvent_t> event_pool;
@@ -584,7 +584,7 @@ int saf_pattern_prepare(saf_ctx* ctx, int32_t H, int32_t Tp, const uint8_t* froz
   if ((rc = ensure(ctx->pat_consts, 2 * hb)) || (rc = ensure(ctx->pat_ok, hb)) || (rc = ensure(ctx->pat_avec, vecb)) ||
       (rc = ensure(ctx->pat_wvec, vecb)) || (rc = ensure(ctx->pat_bandf, bandb)) ||
       (rc = ensure(ctx->pat_bandb, bandb)) || (rc = ensure(ctx->pat_heads, 2 * hb)) || (rc = ensure(ctx->pat_snap, 3 * vecb)) ||
-      (rc = ensure(ctx->pat_marks, 3 * hb)))
+      (rc = ensure(ctx->pat_marks, 4 * hb)))
     return rc;
   // A new buffer starts at zero: per-head overflow marks of the forward / backward staging kernels (a mark is the id of the
   // call that set it, ids only grow) and the counters of the normaliser kernel (which returns them to zero).

@@ -19,26 +19,20 @@ namespace saf {
 // done again relative to its own maximum.  fp32 sums of 32 terms, fp64 from there.  Bound: one ex2 per causal pair.
 // (One warp per row with two passes over global memory: 19.4 us for 6 heads x 2048, now see the launcher.)
 // The last block of a head to finish also forms the head's constants (consts != NULL): max alpha, max rho, and
-// whether the tensor-core form's range holds (see below); counters return to zero.
-constexpr int LZ_KC = 1024;
-__device__ __forceinline__ float block_max(float v, float* red) {
+// whether the tensor-core form's range holds (see below); counters (two per head) return to zero.
+constexpr int LZ_KC = 4096;
+__device__ __forceinline__ float warp_max(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  v = red[0];
-#pragma unroll
-  for (int k = 1; k < 8; ++k) v = fmaxf(v, red[k]);
   return v;
 }
 __global__ void __launch_bounds__(256) saf_logz_kernel(const float* __restrict__ alpha, const float* __restrict__ rho,
-                                                       float* logZ, const uint8_t* __restrict__ mask, int Tp,
-                                                       float* __restrict__ consts, int* __restrict__ fast_ok,
+                                                       float* __restrict__ logZ, const uint8_t* __restrict__ mask, int Tp,
+                                                       float* consts, int* __restrict__ fast_ok,
                                                        unsigned* __restrict__ counters) {
-  __shared__ float sa[LZ_KC], sr[LZ_KC + 32], red[8];
+  __shared__ __align__(16) float sa[LZ_KC];
+  __shared__ float sr[LZ_KC + 32], red[2][8];
   __shared__ double part[8][32];
-  __shared__ int last;
   const int h = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (!mask[h]) {
     if (consts != nullptr && blockIdx.x == 0 && tid == 0) fast_ok[h] = 0;
@@ -46,92 +40,120 @@ __global__ void __launch_bounds__(256) saf_logz_kernel(const float* __restrict__
   }
   // heavy (late) rows first so that the tail of the grid is cheap
   const int i0 = (static_cast<int>(gridDim.x) - 1 - static_cast<int>(blockIdx.x)) * 32;
-  const int i = i0 + lane, iend = min(Tp, i0 + 32);
+  const int iend = min(Tp, i0 + 32);
   const float* a = alpha + static_cast<size_t>(h) * Tp;
   const float* r = rho + static_cast<size_t>(h) * Tp;
   float* z = logZ + static_cast<size_t>(h) * Tp;
-  float ma = -INFINITY, mr = -INFINITY;
-  for (int k = tid; k < iend; k += 256) {
-    ma = fmaxf(ma, a[k]);
-    mr = fmaxf(mr, r[k]);
-  }
-  const float bound = block_max(ma, red) + block_max(mr, red);
   const float L2E = 1.4426950408889634f;
-  const float nb = -bound * L2E;
+  float ma = -INFINITY, mr = -INFINITY;
+  if (iend > LZ_KC) {                                   // (up to LZ_KC the maxima come out of the staging below)
+#pragma unroll 4
+    for (int k = tid; k < iend; k += 256) {
+      ma = fmaxf(ma, a[k]);
+      mr = fmaxf(mr, r[k]);
+    }
+  }
+  float bound = 0.0f, nb = 0.0f;
   double s = 0.0;
   for (int k0 = 0; k0 < iend; k0 += LZ_KC) {
+    const int n = (min(LZ_KC, iend - k0) + 31) / 32 * 32;      // keys of this chunk, in whole groups of 32
     __syncthreads();
-    for (int x = tid; x < LZ_KC; x += 256) sa[x] = k0 + x < iend ? a[k0 + x] : 0.0f;
-    // sr[x] = rho[i0 + x - (k0 + LZ_KC - 1)]
-    for (int x = tid; x < LZ_KC + 31; x += 256) {
-      const int d = i0 + x - (k0 + LZ_KC - 1);
-      sr[x] = d >= 0 && d < Tp ? r[d] : -INFINITY;
+    // sa[x] = alpha[k0 + x], sr[x] = rho[i0 + x - (k0 + n - 1)]
+#pragma unroll 4
+    for (int x = tid; x < n; x += 256) {
+      const bool in = k0 + x < iend;
+      const float v = in ? a[k0 + x] : 0.0f;
+      sa[x] = v;
+      ma = fmaxf(ma, in ? v : -INFINITY);
+    }
+#pragma unroll 4
+    for (int x = tid; x < n + 31; x += 256) {
+      const int d = i0 + x - (k0 + n - 1);
+      const float v = d >= 0 && d < iend ? r[d] : -INFINITY;
+      sr[x] = v;
+      mr = fmaxf(mr, v);
+    }
+    if (k0 == 0) {
+      ma = warp_max(ma);
+      mr = warp_max(mr);
+      if (lane == 0) {
+        red[0][warp] = ma;
+        red[1][warp] = mr;
+      }
     }
     __syncthreads();
-    const int kb = warp * (LZ_KC / 8);                  // this warp's keys k0 + kb ...
-    if (k0 + kb >= iend) continue;
-    const float* rp = sr + lane + LZ_KC - 1 - kb;       // rp[-k] = rho[i - (k0 + kb + k)]
-#pragma unroll 1
-    for (int k = 0; k < LZ_KC / 8; k += 32) {
+    if (k0 == 0) {
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        ma = fmaxf(ma, red[0][k]);
+        mr = fmaxf(mr, red[1][k]);
+      }
+      bound = ma + mr;
+      nb = -bound * L2E;
+    }
+    for (int kb = 32 * warp; kb < n; kb += 256) {       // groups of 32 keys, in turn over the warps
+      const float* rp = sr + lane + n - 1 - kb;         // rp[-e] = rho[i0 + lane - (k0 + kb + e)]
       float p[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
       for (int e = 0; e < 32; e += 4) {
-        const float4 a4 = *reinterpret_cast<const float4*>(sa + kb + k + e);
-        p[0] += ex2_approx(fmaf(a4.x + rp[-k - e], L2E, nb));
-        p[1] += ex2_approx(fmaf(a4.y + rp[-k - e - 1], L2E, nb));
-        p[2] += ex2_approx(fmaf(a4.z + rp[-k - e - 2], L2E, nb));
-        p[3] += ex2_approx(fmaf(a4.w + rp[-k - e - 3], L2E, nb));
+        const float4 a4 = *reinterpret_cast<const float4*>(sa + kb + e);
+        p[0] += ex2_approx(fmaf(a4.x + rp[-e], L2E, nb));
+        p[1] += ex2_approx(fmaf(a4.y + rp[-e - 1], L2E, nb));
+        p[2] += ex2_approx(fmaf(a4.z + rp[-e - 2], L2E, nb));
+        p[3] += ex2_approx(fmaf(a4.w + rp[-e - 3], L2E, nb));
       }
       s += static_cast<double>((p[0] + p[1]) + (p[2] + p[3]));
     }
   }
   part[warp][lane] = s;
   __syncthreads();
-  for (int rr = 0; rr < 4; ++rr) {                      // four rows per warp
-    const int row = i0 + warp * 4 + rr;
-    double t = lane < 8 ? part[lane][warp * 4 + rr] : 0.0;
+  if (warp != 0) return;
+  double t = 0.0;
 #pragma unroll
-    for (int o = 4; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-    t = __shfl_sync(0xffffffffu, t, 0);
-    if (row >= Tp) continue;
-    float ref = bound;
-    if (!(t > 1e-30)) {
-      // the bound is too far above this row: two passes relative to its own maximum
-      float m = -INFINITY;
-      for (int k = lane; k <= row; k += 32) m = fmaxf(m, a[k] + r[row - k]);
+  for (int k = 0; k < 8; ++k) t += part[k][lane];
+  const int row = i0 + lane;
+  const bool valid = row < Tp;
+  float ref = bound;
+  unsigned redo = __ballot_sync(0xffffffffu, valid && !(t > 1e-30));
+  while (redo) {
+    // the bound is too far above this row: two passes relative to its own maximum
+    const int src = __ffs(redo) - 1, rw = i0 + src;
+    redo &= redo - 1;
+    float m = -INFINITY;
+    for (int k = lane; k <= rw; k += 32) m = fmaxf(m, a[k] + r[rw - k]);
+    m = warp_max(m);
+    float s0 = 0.0f;
+    for (int k = lane; k <= rw; k += 32) s0 += __expf(a[k] + r[rw - k] - m);
+    double u = static_cast<double>(s0);
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-      float s0 = 0.0f;
-      for (int k = lane; k <= row; k += 32) s0 += __expf(a[k] + r[row - k] - m);
-      t = static_cast<double>(s0);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    for (int o = 16; o > 0; o >>= 1) u += __shfl_xor_sync(0xffffffffu, u, o);
+    if (lane == src) {
+      t = u;
       ref = m;
     }
-    if (lane == 0) z[row] = static_cast<float>(static_cast<double>(ref) + log(t));
   }
+  const float zv = valid ? static_cast<float>(static_cast<double>(ref) + log(t)) : INFINITY;
+  if (valid) z[row] = zv;
   if (consts == nullptr) return;
-  __threadfence();
-  __syncthreads();
-  if (tid == 0) last = atomicInc(counters + h, gridDim.x - 1) == gridDim.x - 1;
-  __syncthreads();
-  if (!last) return;
-  __threadfence();
-  float mz = -INFINITY;
-  ma = mr = -INFINITY;
-  for (int t = tid; t < Tp; t += 256) {
-    ma = fmaxf(ma, a[t]);
-    mr = fmaxf(mr, r[t]);
-    mz = fmaxf(mz, -__ldcg(z + t));
-  }
-  ma = block_max(ma, red);
-  mr = block_max(mr, red);
-  mz = block_max(mz, red);
-  if (tid == 0) {
-    consts[2 * h] = ma;
-    consts[2 * h + 1] = mr;
-    const float wmax = ma + mr + mz;
-    fast_ok[h] = (wmax <= 9.0f && wmax > -1e30f && ma < 1e30f && mr < 1e30f) ? 1 : 0;
+  // constants: the block of the last rows has seen all of alpha and rho; the smallest normaliser through an atomic
+  // (ordered encoding: larger key = smaller z, 0 = none yet)
+  const float mz = warp_max(-zv);
+  if (lane == 0) {
+    if (iend == Tp) {
+      consts[2 * h] = ma;
+      consts[2 * h + 1] = mr;
+    }
+    unsigned* key = counters + 2 * h + 1;
+    const unsigned u = __float_as_uint(mz);
+    atomicMax(key, (u & 0x80000000u) ? ~u : (u | 0x80000000u));
+    __threadfence();
+    if (atomicInc(counters + 2 * h, gridDim.x - 1) == gridDim.x - 1) {
+      __threadfence();
+      const unsigned k = atomicExch(key, 0u);
+      const float ca = __ldcg(consts + 2 * h), cr = __ldcg(consts + 2 * h + 1);
+      const float wmax = ca + cr + __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);
+      fast_ok[h] = (wmax <= 9.0f && wmax > -1e30f && ca < 1e30f && cr < 1e30f) ? 1 : 0;
+    }
   }
 }
 
