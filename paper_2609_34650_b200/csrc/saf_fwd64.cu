@@ -104,7 +104,7 @@ constexpr int RING_END = -1;
 __device__ __forceinline__ bool ring_take(const int4* ring, uint64_t* ring_full, uint64_t* ring_empty, uint32_t n,
                                           const WaitCtx& wc, ItemView64& v) {
   const uint32_t slot = n % Fwd64Cfg::NRING;
-  if (!mbar_wait_warp(ring_full + slot, (n / Fwd64Cfg::NRING) & 1, wc, F_RING_FULL)) return false;
+  if (!mbar_wait_warp_compact(ring_full + slot, (n / Fwd64Cfg::NRING) & 1, wc, F_RING_FULL)) return false;
   const int4 raw = ring[slot];
   warp_arrive(ring_empty + slot);
   v.w = WorkItem{raw.x, raw.y, raw.z, raw.w < 0 ? RING_END : (raw.w & 0xff)};
@@ -201,7 +201,7 @@ saf_fwd64_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
       for (uint32_t nclaim = 0; ok; ++nclaim) {
         // claim the next item of the queue and publish it to the other roles
         const uint32_t slot = nclaim % C::NRING;
-        ok = mbar_wait(ring_empty + slot, ((nclaim / C::NRING) & 1) ^ 1, wc, F_RING_EMPTY);
+        ok = mbar_wait_compact(ring_empty + slot, ((nclaim / C::NRING) & 1) ^ 1, wc, F_RING_EMPTY);
         if (!ok) break;
         // (a CTA's first item is its own number; a grid of one item per CTA does not touch the queue)
         const int grid = static_cast<int>(gridDim.x);
@@ -225,10 +225,10 @@ saf_fwd64_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
           if (!fz_open) {
             // the last tiles that went through those stages must have been consumed
             for (uint32_t n = nk > C::NS ? nk - C::NS : 0; n < nk && ok; ++n)
-              ok = mbar_wait(k_empty + n % C::NS, (n / C::NS) & 1, wc, F_K_EMPTY);
+              ok = mbar_wait_compact(k_empty + n % C::NS, (n / C::NS) & 1, wc, F_K_EMPTY);
             for (uint32_t n = nv > C::NS ? nv - C::NS : 0; n < nv && ok; ++n)
-              ok = mbar_wait(v_empty + n % C::NS, (n / C::NS) & 1, wc, F_V_EMPTY);
-            if (ok && nq > 0) ok = mbar_wait(q_empty, (nq - 1) & 1, wc, F_Q_EMPTY);
+              ok = mbar_wait_compact(v_empty + n % C::NS, (n / C::NS) & 1, wc, F_V_EMPTY);
+            if (ok && nq > 0) ok = mbar_wait_compact(q_empty, (nq - 1) & 1, wc, F_Q_EMPTY);
             if (!ok) break;
             fz_open = true;
           }
@@ -236,7 +236,7 @@ saf_fwd64_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
           const uint8_t* bands = static_cast<const uint8_t*>(p.band_f) + static_cast<size_t>(w.h) * p.nblkp * 4096;
           for (int j = 0; j < ntiles; ++j) {
             const uint32_t k = nfz % C::NFZ;
-            ok = mbar_wait(fz_empty + k, ((nfz / C::NFZ) & 1) ^ 1, wc, F_V_EMPTY);
+            ok = mbar_wait_compact(fz_empty + k, ((nfz / C::NFZ) & 1) ^ 1, wc, F_V_EMPTY);
             if (!ok) break;
             mbar_expect_tx(fz_full + k, C::TILE_BYTES + 4096);
             bulk_load(smem + C::fz_band(k), bands + static_cast<size_t>(w.blk - j) * 4096, 4096, fz_full + k);
@@ -248,14 +248,14 @@ saf_fwd64_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
         if (fz_open) {
           // back to the ordinary stages: the frozen ring's tiles in flight must have been consumed
           for (uint32_t n = nfz > C::NFZ ? nfz - C::NFZ : 0; n < nfz && ok; ++n)
-            ok = mbar_wait(fz_empty + n % C::NFZ, (n / C::NFZ) & 1, wc, F_V_EMPTY);
+            ok = mbar_wait_compact(fz_empty + n % C::NFZ, (n / C::NFZ) & 1, wc, F_V_EMPTY);
           if (!ok) break;
           fz_open = false;
         }
         const bool ord = w.kind == KIND_ORDINARY;
         const int kh = !ord ? 0 : (p.qslot ? p.qslot[w.h] : w.h / p.kv_group);   // head index in the K tensor
         if (ord) {
-          ok = mbar_wait(q_empty, (nq & 1) ^ 1, wc, F_Q_EMPTY);
+          ok = mbar_wait_compact(q_empty, (nq & 1) ^ 1, wc, F_Q_EMPTY);
           if (!ok) break;
           mbar_expect_tx(q_full, C::TILE_BYTES);
           tma_load_4d(smem + C::OFF_Q, &mq, q_full, 0, w.blk * BLK, p.qslot ? p.qslot[w.h] : w.h, w.b);
@@ -264,7 +264,7 @@ saf_fwd64_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
         for (int j = 0; j < ntiles && ok; ++j) {
           if (ord) {
             const int s = nk % C::NS;
-            ok = mbar_wait(k_empty + s, ((nk / C::NS) & 1) ^ 1, wc, F_K_EMPTY);
+            ok = mbar_wait_compact(k_empty + s, ((nk / C::NS) & 1) ^ 1, wc, F_K_EMPTY);
             if (!ok) break;
             if (!drop_load) {
               mbar_expect_tx(k_full + s, C::TILE_BYTES);
@@ -274,7 +274,7 @@ saf_fwd64_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
             ++nk;
           }
           const int s = nv % C::NS;
-          ok = mbar_wait(v_empty + s, ((nv / C::NS) & 1) ^ 1, wc, F_V_EMPTY);
+          ok = mbar_wait_compact(v_empty + s, ((nv / C::NS) & 1) ^ 1, wc, F_V_EMPTY);
           if (!ok) break;
           mbar_expect_tx(v_full + s, C::TILE_BYTES);
           tma_load_4d(smem + C::OFF_V + s * C::TILE_BYTES, &mv, v_full + s, 0, j * BLK, w.h / p.kv_group, w.b);
@@ -313,11 +313,11 @@ saf_fwd64_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
       if (fast) {
         for (int j = 0; j < ntiles && ok; ++j) {
           const uint32_t k = nfz % C::NFZ;
-          ok = mbar_wait_warp(fz_full + k, (nfz / C::NFZ) & 1, wc, F_V_FULL);
+          ok = mbar_wait_warp_compact(fz_full + k, (nfz / C::NFZ) & 1, wc, F_V_FULL);
           if (!ok) break;
           ++nfz;
           if (j == 0) {
-            ok = mbar_wait_warp(o_free, (nitem & 1) ^ 1, wc, F_O_FREE);
+            ok = mbar_wait_warp_compact(o_free, (nitem & 1) ^ 1, wc, F_O_FREE);
             if (!ok) break;
           }
           tc_fence_after();
@@ -360,12 +360,12 @@ saf_fwd64_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
           }
           __syncwarp();
         };
-        ok = mbar_wait_warp(q_full, nq & 1, wc, F_Q_FULL);
+        ok = mbar_wait_warp_compact(q_full, nq & 1, wc, F_Q_FULL);
         if (!ok) break;
         ++nq;
         {
           const uint32_t s = nk % C::NS;
-          ok = mbar_wait_warp(k_full + s, (nk / C::NS) & 1, wc, F_K_FULL);
+          ok = mbar_wait_warp_compact(k_full + s, (nk / C::NS) & 1, wc, F_K_FULL);
           if (!ok) break;
           ++nk;
           tc_fence_after();
@@ -382,26 +382,26 @@ saf_fwd64_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
           // ---- group 0
           // the tiles' loads land long before P is ready: test their barriers first, so that only one test
           // stands between "P is ready" and the MMAs that wait for it
-          ok = mbar_wait_warp(v_full + sv, (nv / C::NS) & 1, wc, F_V_FULL);
+          ok = mbar_wait_warp_compact(v_full + sv, (nv / C::NS) & 1, wc, F_V_FULL);
           if (!ok) break;
           ++nv;
           if (more) {
-            ok = mbar_wait_warp(k_full + sk, (nk / C::NS) & 1, wc, F_K_FULL);
+            ok = mbar_wait_warp_compact(k_full + sk, (nk / C::NS) & 1, wc, F_K_FULL);
             if (!ok) break;
             ++nk;
           }
           if (j == 0) {
-            ok = mbar_wait_warp(o_free, (nitem & 1) ^ 1, wc, F_O_FREE);
+            ok = mbar_wait_warp_compact(o_free, (nitem & 1) ^ 1, wc, F_O_FREE);
             if (!ok) break;
           }
-          ok = mbar_wait_warp(p_full, np0 & 1, wc, F_P_FULL);
+          ok = mbar_wait_warp_compact(p_full, np0 & 1, wc, F_P_FULL);
           if (!ok) break;
           ++np0;
           tc_fence_after();
           issue_pv(0, sv, acc0);
           if (more) issue_qk(0, sk);                      // executes after P V_0: same thread, in order
           // ---- group 1
-          ok = mbar_wait_warp(p_full + 1, np1 & 1, wc, F_P_FULL);
+          ok = mbar_wait_warp_compact(p_full + 1, np1 & 1, wc, F_P_FULL);
           if (!ok) break;
           ++np1;
           tc_fence_after();
@@ -425,20 +425,20 @@ saf_fwd64_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
       // generic frozen item: P^ halves written by the groups, one P V MMA per group and tile
       for (int j = 0; j < ntiles && ok; ++j) {
         const uint32_t sv = nv % C::NS;
-        ok = mbar_wait_warp(v_full + sv, (nv / C::NS) & 1, wc, F_V_FULL);
+        ok = mbar_wait_warp_compact(v_full + sv, (nv / C::NS) & 1, wc, F_V_FULL);
         if (!ok) break;
         ++nv;
         if (j == 0) {
-          ok = mbar_wait_warp(o_free, (nitem & 1) ^ 1, wc, F_O_FREE);
+          ok = mbar_wait_warp_compact(o_free, (nitem & 1) ^ 1, wc, F_O_FREE);
           if (!ok) break;
         }
         const uint32_t acc0 = j > 0 ? 1u : 0u;
         for (uint32_t g = 0; g < 2 && ok; ++g) {
           if (g == 0) {
-            ok = mbar_wait_warp(p_full, np0 & 1, wc, F_P_FULL);
+            ok = mbar_wait_warp_compact(p_full, np0 & 1, wc, F_P_FULL);
             ++np0;
           } else {
-            ok = mbar_wait_warp(p_full + 1, np1 & 1, wc, F_P_FULL);
+            ok = mbar_wait_warp_compact(p_full + 1, np1 & 1, wc, F_P_FULL);
             ++np1;
           }
           if (!ok) break;
@@ -505,7 +505,7 @@ saf_fwd64_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
         for (int j = 0; j < ntiles; ++j) {
           if (q4 == 0) TRF(trr, 11);
           // (the completion of this score MMA also covers the group's previous P V MMA, issued before it)
-          if (!mbar_wait_warp(s_full + g, ns & 1, wc, F_S_FULL)) ok = false;
+          if (!mbar_wait_warp_compact(s_full + g, ns & 1, wc, F_S_FULL)) ok = false;
           ++ns;
           tc_fence_after();
           if (q4 == 0) TRF(trr, 12);
@@ -642,8 +642,8 @@ saf_fwd64_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
           if (j > 0) {
             // previous P^ tile consumed (both halves: a thread follows every phase of both barriers, so that
             // the parity it waits for in the epilogue can never be one phase pair behind)
-            if (!mbar_wait_warp(pv_done, npv & 1, wc, F_PV_DONE)) ok = false;
-            if (!mbar_wait_warp(pv_done + 1, npv & 1, wc, F_PV_DONE)) ok = false;
+            if (!mbar_wait_warp_compact(pv_done, npv & 1, wc, F_PV_DONE)) ok = false;
+            if (!mbar_wait_warp_compact(pv_done + 1, npv & 1, wc, F_PV_DONE)) ok = false;
             ++npv;
             tc_fence_after();
           }
@@ -684,8 +684,8 @@ saf_fwd64_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
       // ---------------- epilogue: wait for the last P V of both groups, merge, scale, store 32 columns each
       {
         const uint32_t par = npv & 1;
-        if (!mbar_wait_warp(pv_done, par, wc, F_PV_DONE)) ok = false;
-        if (!mbar_wait_warp(pv_done + 1, par, wc, F_PV_DONE)) ok = false;
+        if (!mbar_wait_warp_compact(pv_done, par, wc, F_PV_DONE)) ok = false;
+        if (!mbar_wait_warp_compact(pv_done + 1, par, wc, F_PV_DONE)) ok = false;
         ++npv;
       }
       tc_fence_after();
