@@ -1297,11 +1297,7 @@ int saf_calib_accumulate(saf_ctx* ctx, const saf_problem* p, const void* Q, cons
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   ctx->last_stream = st;
   const int kvg = kv_group_of(p);
-  if (!accumulate) {
-    const size_t hb = static_cast<size_t>(p->H) * sizeof(double);
-    if (cudaMemsetAsync(sumsq, 0, hb, st) != cudaSuccess || cudaMemsetAsync(sum_plogp, 0, hb, st) != cudaSuccess)
-      return SAF_ERR_CUDA;
-  }
+  if (!accumulate && launch_calib_zero(sumsq, sum_plogp, p->H, st) != cudaSuccess) return SAF_ERR_CUDA;
   CUtensorMap mq, mk;
   int rc;
   if ((rc = make_map(ctx, &mq, Q, p, p->q_strides, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, p->H))) return rc;
@@ -1353,8 +1349,11 @@ int saf_calib_finalize(saf_ctx* ctx, int32_t H, int32_t T, int64_t n_total, floa
   if (!g.ok) return SAF_ERR_CUDA;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   ctx->last_stream = st;
+  const size_t tmp_before = ctx->calib_tmp.bytes;
   int rc = ensure(ctx->calib_tmp, static_cast<size_t>(H) * 2 * sizeof(double));
   if (rc) return rc;
+  if (ctx->calib_tmp.bytes != tmp_before && cudaMemsetAsync(ctx->calib_tmp.ptr, 0, ctx->calib_tmp.bytes, st) != cudaSuccess)
+    return SAF_ERR_CUDA;
   ScopedTimer timer(ctx, SAF_KERNEL_CALIB_FINALIZE, st);
   if (launch_calib_finalize(mean_inout, sumsq, sum_plogp, static_cast<double*>(ctx->calib_tmp.ptr), H, T,
                             static_cast<double>(n_total), s_var_out, s_kl_out, ctx->num_sms, st) != cudaSuccess)

@@ -253,6 +253,7 @@ struct CalibParams {
 };
 cudaError_t launch_calib(int D, const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mm,
                          const CalibParams& p, int grid, cudaStream_t st);
+cudaError_t launch_calib_zero(double* a, double* b, int n, cudaStream_t st);
 cudaError_t launch_calib_finalize(float* mean, const double* sumsq, const double* sum_plogp, double* tmp, int H, int T,
                                   double n_total, double* s_var, double* s_kl, int num_sms, cudaStream_t st);
 
