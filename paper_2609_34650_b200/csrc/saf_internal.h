@@ -20,19 +20,19 @@ inline bool pdl_enabled() {
   }();
   return on;
 }
-// Which kernels are launched that way (SAF_PDL_MASK: bit 0 staging kernels, 1 forward, 2 backward preparation,
-// 3 backward, 4 the 128-wide forward).  Measured on the 124M-shaped step (fwd + bwd back to back, no events in between): only the backward
-// gains (-0.5 %); an early forward grid costs 3 %, because its CTAs then land on SMs in the order these become
-// free and the pairing of a light and a heavy CTA per SM that the scheduler's work lists assume is lost.  (That is the
-// D = 64 forward; the 128-wide one runs one CTA per SM and starts under the staging kernel.)
+// Which kernels are launched that way (SAF_PDL_MASK: bit 0 staging kernels, 1 D = 64 forward, 2 backward preparation,
+// 3 backward, 4 the 128-wide forward, 5 backward preparation of small layers).  All but the preparation of large layers:
+// its blocks then fill the SMs under the forward's tail, where the layer is long enough for that to cost more than the
+// launch gap (8x12x4096x64: pass +2 %, 8x12x2048x128 +3 %; 3x12x1537x64 -1 %, 4x12x1024x64 -3 %, 1x4x256x64 -5 %).
+// The others gain or are neutral: staging 1x32x333x128 -6 %, D = 64 forward 3x12x1537x64 -4 %, 8x12x2048x64 -1 %.
 inline int pdl_mask() {
   static const int m = [] {
     const char* e = std::getenv("SAF_PDL_MASK");
-    return e ? std::atoi(e) : 8 + 16;
+    return e ? std::atoi(e) : 1 + 2 + 8 + 16 + 32;
   }();
   return m;
 }
-enum { PDL_STAGE = 1, PDL_FWD = 2, PDL_PREP = 4, PDL_BWD = 8, PDL_FWD128 = 16 };
+enum { PDL_STAGE = 1, PDL_FWD = 2, PDL_PREP = 4, PDL_BWD = 8, PDL_FWD128 = 16, PDL_PREP_SMALL = 32 };
 template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl(int which, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
   cudaLaunchConfig_t cfg = {};

@@ -465,8 +465,10 @@ cudaError_t launch_bwd_prep(const void* O, int o_f32, const void* dO, const floa
 #define SAF_PREP_ARGS                                                                                                  \
   O, static_cast<const __nv_bfloat16*>(dO), LSE, os[0], os[1], os[2], mask_dev, static_cast<uint8_t*>(q_ext),          \
       static_cast<uint8_t*>(do_ext), inv_scale, dQacc, dK, dV, grad_f32, kv_group, qslot, n_ord, fz, B, H, T
+  // (small: at most ~14 blocks per SM, less than two waves)
+  const int which = grid <= 2048 ? PDL_PREP_SMALL : PDL_PREP;
 #define SAF_PREP_LAUNCH(DD, TT, FF) \
-  launch_pdl(PDL_PREP, saf_bwd_prep_kernel<DD, TT, FF>, dim3(grid), dim3(256), 0, st, SAF_PREP_ARGS)
+  launch_pdl(which, saf_bwd_prep_kernel<DD, TT, FF>, dim3(grid), dim3(256), 0, st, SAF_PREP_ARGS)
   cudaError_t e;
   if (D == 64) e = o_f32 ? SAF_PREP_LAUNCH(64, 8, true) : SAF_PREP_LAUNCH(64, 8, false);
   else if (D == 96) e = o_f32 ? SAF_PREP_LAUNCH(96, 16, true) : SAF_PREP_LAUNCH(96, 16, false);
