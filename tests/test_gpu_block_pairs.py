@@ -1,0 +1,83 @@
+"""GPU tests at the edges of the 128-wide kernels' work items (two query blocks per forward item, full 128-query tiles in
+the backward), of the normaliser kernel's chunks and of the calibration's mean pass."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2609_34650_b200 as saf
+import saf_inputs as si
+from oracle import saf_oracle as orc
+
+from gpu_util import Layer
+from test_gpu_parity import all_units, check_units
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("B,H,T,D,frozen", [
+    (1, 4, 128, 128, (1,)),             # one block, alone
+    (1, 3, 129, 96, (0,)),              # two blocks, one by one (fewer than the SMs)
+    (5, 10, 257, 128, (1, 4, 7)),       # 150 blocks: pairs, the first block of an odd count alone
+    (6, 13, 256, 128, (2, 3)),          # 156 blocks: one pair per unit
+    (4, 10, 512, 96, (0, 5, 9)),        # pairs of every length up to four tiles
+    (10, 16, 100, 128, (3,)),           # more one-block units than SMs: no pairs to form
+])
+def test_block_pairs(B, H, T, D, frozen):
+    inp = si.generate(si.Workload("pairs", B, H, T, D, frozen, -0.05, seed=T + D))
+    check_units(Layer(inp).run(), all_units(inp.wl))
+
+
+def test_running_maximum_far_above_the_first_tile():
+    """Scores that grow along the sequence: the rescaling of the accumulator between tiles, in both blocks of a pair."""
+    inp = si.generate(si.Workload("grow", 2, 2, 640, 128, (), -0.05, seed=9))
+    f = np.exp2(np.arange(640) // 128).astype(np.float32)          # exact in bf16
+    inp.k[...] = si.f32_to_bf16_bits(si.bf16_bits_to_f32(inp.k) * f[None, None, :, None])
+    L = Layer(inp, backward=False)
+    L.run(backward=False)
+    q, k, v = (si.bf16_bits_to_f64(x) for x in (inp.q, inp.k, inp.v))
+    want, _ = orc.hybrid_attn_fwd(q, k, v, inp.mask, inp.alpha, inp.rho)
+    got = L.O.float().cpu().numpy().astype(np.float64)
+    assert np.abs(got - want).max() <= 2e-2 and np.linalg.norm(got - want) <= 1e-2 * np.linalg.norm(want)
+
+
+@pytest.mark.parametrize("T", [1, 31, 33, 255, 4096, 4097, 8200])
+@pytest.mark.parametrize("spread", [1.0, 60.0])
+def test_normalisers_at_chunk_edges(T, spread):
+    """Rows around the 32-row blocks and the 4096-key chunks; `spread` 60 puts rows far below the common bound (a spike
+    late in alpha), which are then taken relative to their own maximum."""
+    rng = np.random.default_rng(T)
+    alpha = rng.standard_normal((2, T)).astype(np.float32)
+    alpha[:, -1] += 3.0 * spread
+    rho = (-0.01 * np.arange(T) + 0.1 * rng.standard_normal((2, T))).astype(np.float32)
+    mask = np.array([1, 1], dtype=np.uint8)
+    a, r = torch.from_numpy(alpha).cuda(), torch.from_numpy(rho).cuda()
+    z = torch.full((2, T), float("nan"), device="cuda")
+    saf.Context(0).saf_pattern_prepare(mask, a, r, z)
+    z = z.cpu().numpy().astype(np.float64)
+    # ex2 and sums 2e-6; alpha + rho is rounded once in fp32, and so is the result
+    big = np.abs(alpha).max() + np.abs(rho).max()
+    for h in range(2):
+        err = np.abs(z[h] - orc.pattern_logZ(alpha[h], rho[h], T))
+        assert err.max() <= 5e-6 + 2.0 ** -23 * big, err.max()
+
+
+@pytest.mark.parametrize("T", [4, 130, 1028, 1030])
+def test_calibration_mean_pass(T):
+    """Row lengths in whole 16-byte pieces and others; what lies above the diagonal stays as it was."""
+    rng = np.random.default_rng(T)
+    H, n = 3, 5
+    total = np.tril(rng.random((H, T, T))).astype(np.float32)
+    m = torch.from_numpy(total).cuda() + torch.triu(torch.full((H, T, T), 7.0, device="cuda"), diagonal=1)
+    zero = torch.zeros(H, device="cuda", dtype=torch.float64)
+    ctx = saf.Context(0)
+    for _ in range(2):                                             # (the second call starts from the same workspace)
+        mean, sq, pl = m.clone(), zero + 10.0 * T * T, zero + 1.0
+        var, kl = zero.clone(), zero.clone()
+        ctx.saf_calib_finalize(H, T, n, mean, sq, pl, var, kl)
+        got = mean.cpu().numpy().astype(np.float64)
+        want = total.astype(np.float64) / n
+        low = np.tril(np.ones((T, T), dtype=bool))
+        assert np.all(got[:, ~low] == 7.0)
+        assert np.abs(got[:, low] - want[:, low]).max() <= 2.0 ** -23    # two fp32 roundings of values below one
+        ref = (10.0 * T * T - n * (want ** 2).sum(axis=(1, 2))) / ((n - 1.0) * T * T)
+        assert np.abs(var.cpu().numpy() - ref).max() <= 1e-6 * np.abs(ref).max()
