@@ -26,10 +26,8 @@ struct WorklistEntry {
   std::vector<uint8_t> mask;
   std::vector<WorkItem> items_host;       // kept alive: the upload is asynchronous on the caller's stream
   std::vector<int> offsets_host;
-  WorkItem* items_dev = nullptr;
+  WorkItem* items_dev = nullptr;          // backward: grouped by CTA; forward: queue order
   int* offsets_dev = nullptr;
-  WorkItem* order_dev = nullptr;          // the same items in queue order (kernels that take work dynamically)
-  std::vector<WorkItem> order_host;
   int n_items = 0;
 };
 
@@ -70,10 +68,6 @@ struct saf_ctx {
   int frozen_weight_bwd_pct = 0;
   int item_overhead_pct = 0;
   int item_overhead_bwd_pct = 0;
-  // Forward grid = two CTAs per SM: the CTA that arrives second on an SM (block index >= grid / 2) runs slower
-  // than the first (measured 13 % at head dimension 64, 2 % on the 128-wide kernel; best settings 20 and 6) and gets that much less
-  // work.  -1 = the measured default; SAF_SECOND_WAVE_PCT overrides.
-  int second_wave_pct = -1;
   int call_counter = 0;                    // ids of the calls that stage fp16 operands (overflow marks)
   std::vector<WorklistEntry> worklists;
   DevBuf mask_buf, logz_buf, delta_buf, dqacc_buf, dkacc_buf, dvacc_buf, qslot_buf;
@@ -242,8 +236,8 @@ int upload_mask(saf_ctx* ctx, const uint8_t* mask, int H, cudaStream_t st) {
 // end, and each item goes to the CTA that becomes free first (list scheduling, which is what a dynamic
 // queue would do); only the last items are ordered longest-first so that the tail stays short.
 void build_worklist_host(int B, int H, int T, const uint8_t* mask, int backward, int n_ctas, int frozen_pct,
-                         int overhead_pct, int overhead_frozen_pct, int second_wave_pct, std::vector<WorkItem>& items,
-                         std::vector<int>& offsets, std::vector<WorkItem>* order = nullptr) {
+                         int overhead_pct, int overhead_frozen_pct, std::vector<WorkItem>* items,
+                         std::vector<int>* offsets, std::vector<WorkItem>* order) {
   const int nblk = (T + BLK - 1) / BLK;
   struct Cand { WorkItem w; long long cost; };
   std::vector<Cand> cand;
@@ -270,6 +264,7 @@ void build_worklist_host(int B, int H, int T, const uint8_t* mask, int backward,
     order->clear();
     for (const Cand& c : cand) order->push_back(c.w);
   }
+  if (!items) return;
   typedef std::pair<long long, int> Load;   // (load, cta)
   std::priority_queue<Load, std::vector<Load>, std::greater<Load>> heap;
   for (int c = 0; c < n_ctas; ++c) heap.push({0, c});
@@ -278,17 +273,15 @@ void build_worklist_host(int B, int H, int T, const uint8_t* mask, int backward,
     Load l = heap.top();
     heap.pop();
     per[l.second].push_back(c.w);
-    // CTAs of the second half of the grid (the second CTA of each SM when the grid is two per SM) run slower
-    const long long scaled = l.second >= n_ctas / 2 ? c.cost * (100 + second_wave_pct) : c.cost * 100;
-    heap.push({l.first + scaled, l.second});
+    heap.push({l.first + c.cost, l.second});
   }
-  items.clear();
-  offsets.assign(n_ctas + 1, 0);
+  items->clear();
+  offsets->assign(n_ctas + 1, 0);
   for (int c = 0; c < n_ctas; ++c) {
-    offsets[c] = static_cast<int>(items.size());
-    items.insert(items.end(), per[c].begin(), per[c].end());
+    (*offsets)[c] = static_cast<int>(items->size());
+    items->insert(items->end(), per[c].begin(), per[c].end());
   }
-  offsets[n_ctas] = static_cast<int>(items.size());
+  (*offsets)[n_ctas] = static_cast<int>(items->size());
 }
 
 // Work queue of the 128-wide forward, whose items are two consecutive query blocks of one (batch, head) unit (the first
@@ -346,11 +339,8 @@ int get_worklist(saf_ctx* ctx, int B, int H, int T, int D, const uint8_t* mask, 
     cudaStreamSynchronize(st);
     cudaFree(ctx->worklists.front().items_dev);
     cudaFree(ctx->worklists.front().offsets_dev);
-    cudaFree(ctx->worklists.front().order_dev);
     ctx->worklists.erase(ctx->worklists.begin());
   }
-  std::vector<WorkItem> items;
-  std::vector<int> offsets;
   const int wide = D != 64;
   int frozen_pct, overhead_pct, overhead_frozen_pct;
   sched_defaults(wide, backward, &frozen_pct, &overhead_pct, &overhead_frozen_pct);
@@ -358,38 +348,33 @@ int get_worklist(saf_ctx* ctx, int B, int H, int T, int D, const uint8_t* mask, 
   const int ov = backward ? ctx->item_overhead_bwd_pct : ctx->item_overhead_pct;
   if (fw > 0) frozen_pct = fw;
   if (ov > 0) overhead_pct = overhead_frozen_pct = ov;   // (the override sets both kinds)
-  const int second_wave = backward ? 0 : (ctx->second_wave_pct >= 0 ? ctx->second_wave_pct : (wide ? 6 : 20));
+  // backward: per-CTA lists; forward: a queue
   WorklistEntry e;
-  build_worklist_host(B, H, T, mask, backward, grid, frozen_pct, overhead_pct, overhead_frozen_pct, second_wave, items,
-                      offsets, &e.order_host);
-  if (wide && !backward) build_pair_order(B, H, T, D, mask, ctx->num_sms, e.order_host);
+  if (!backward && wide) {
+    build_pair_order(B, H, T, D, mask, ctx->num_sms, e.items_host);
+  } else {
+    build_worklist_host(B, H, T, mask, backward, grid, frozen_pct, overhead_pct, overhead_frozen_pct,
+                        backward ? &e.items_host : nullptr, &e.offsets_host, backward ? nullptr : &e.items_host);
+  }
   e.B = B; e.H = H; e.T = T; e.D = D; e.backward = backward; e.grid = grid;
   e.mask.assign(mask, mask + H);
-  e.n_items = static_cast<int>(e.order_host.size());
-  if (cudaMalloc(&e.items_dev, items.size() * sizeof(WorkItem)) != cudaSuccess) return SAF_ERR_NOMEM;
-  if (cudaMalloc(&e.offsets_dev, offsets.size() * sizeof(int)) != cudaSuccess) {
-    cudaFree(e.items_dev);
-    return SAF_ERR_NOMEM;
-  }
-  if (cudaMalloc(&e.order_dev, e.order_host.size() * sizeof(WorkItem)) != cudaSuccess) {
+  e.n_items = static_cast<int>(e.items_host.size());
+  auto give_up = [&](int code) {
     cudaFree(e.items_dev);
     cudaFree(e.offsets_dev);
-    return SAF_ERR_NOMEM;
-  }
+    return code;
+  };
   // uploaded on the stream the kernel will run on (a non-blocking stream does not order with the legacy stream);
   // the source vectors live as long as the entry
-  e.items_host = std::move(items);
-  e.offsets_host = std::move(offsets);
+  if (cudaMalloc(&e.items_dev, e.items_host.size() * sizeof(WorkItem)) != cudaSuccess) return give_up(SAF_ERR_NOMEM);
   if (cudaMemcpyAsync(e.items_dev, e.items_host.data(), e.items_host.size() * sizeof(WorkItem), cudaMemcpyHostToDevice,
-                      st) != cudaSuccess ||
-      cudaMemcpyAsync(e.offsets_dev, e.offsets_host.data(), e.offsets_host.size() * sizeof(int),
-                      cudaMemcpyHostToDevice, st) != cudaSuccess ||
-      cudaMemcpyAsync(e.order_dev, e.order_host.data(), e.order_host.size() * sizeof(WorkItem), cudaMemcpyHostToDevice,
-                      st) != cudaSuccess) {
-    cudaFree(e.order_dev);
-    cudaFree(e.items_dev);
-    cudaFree(e.offsets_dev);
-    return SAF_ERR_CUDA;
+                      st) != cudaSuccess)
+    return give_up(SAF_ERR_CUDA);
+  if (backward) {
+    if (cudaMalloc(&e.offsets_dev, e.offsets_host.size() * sizeof(int)) != cudaSuccess) return give_up(SAF_ERR_NOMEM);
+    if (cudaMemcpyAsync(e.offsets_dev, e.offsets_host.data(), e.offsets_host.size() * sizeof(int), cudaMemcpyHostToDevice,
+                        st) != cudaSuccess)
+      return give_up(SAF_ERR_CUDA);
   }
   ctx->worklists.push_back(std::move(e));
   *out = &ctx->worklists.back();
@@ -504,10 +489,6 @@ int saf_create(saf_ctx** out, int device) {
     long v = std::atol(e);
     if (v > 0 && v <= 400) ctx->frozen_weight_bwd_pct = static_cast<int>(v);
   }
-  if (const char* e = std::getenv("SAF_SECOND_WAVE_PCT")) {
-    long v = std::atol(e);
-    if (v >= 0 && v <= 100) ctx->second_wave_pct = static_cast<int>(v);
-  }
   if (const char* e = std::getenv("SAF_ITEM_OVERHEAD_PCT")) {
     long v = std::atol(e);
     if (v > 0 && v <= 2000) ctx->item_overhead_pct = static_cast<int>(v);
@@ -527,7 +508,6 @@ int saf_destroy(saf_ctx* ctx) {
   for (WorklistEntry& e : ctx->worklists) {
     cudaFree(e.items_dev);
     cudaFree(e.offsets_dev);
-    cudaFree(e.order_dev);
   }
   DevBuf* pbufs[] = {&ctx->pat_consts, &ctx->pat_ok, &ctx->pat_avec, &ctx->pat_wvec, &ctx->pat_bandf, &ctx->pat_bandb,
                      &ctx->pat_heads, &ctx->pat_snap, &ctx->pat_marks, &ctx->vt_buf, &ctx->dot_buf, &ctx->pg_hlist, &ctx->pg_delta, &ctx->pg_items, &ctx->pg_offsets, &ctx->fit_buf, &ctx->calib_tmp};
@@ -719,9 +699,7 @@ int saf_hybrid_attn_fwd(saf_ctx* ctx, const saf_problem* p, const void* Q, const
   fp.o_f32 = p->o_dtype == SAF_F32 ? 1 : 0;
   for (int i = 0; i < 3; ++i) fp.o_strides[i] = p->o_strides[i];
   fp.LSE = LSE;
-  fp.items = wl->items_dev;
-  fp.cta_offsets = wl->offsets_dev;
-  fp.order = wl->order_dev;
+  fp.order = wl->items_dev;
   fp.n_items = wl->n_items;
   fp.queue = ctx->queue_dev;
   fp.status = ctx->status_dev;
@@ -1417,7 +1395,8 @@ int saf_build_worklist(int32_t B, int32_t H, int32_t T, const uint8_t* frozen_ma
   std::vector<int> offsets;
   int fp_unused, ov, ovf;
   sched_defaults(0, backward ? 1 : 0, &fp_unused, &ov, &ovf);      // the 64-wide kernels' per-item overheads
-  build_worklist_host(B, H, T, frozen_mask_host, backward ? 1 : 0, n_ctas, frozen_weight_pct, ov, ovf, 0, items, offsets);
+  build_worklist_host(B, H, T, frozen_mask_host, backward ? 1 : 0, n_ctas, frozen_weight_pct, ov, ovf, &items, &offsets,
+                      nullptr);
   std::memcpy(items_out, items.data(), items.size() * sizeof(WorkItem));
   std::memcpy(offsets_out, offsets.data(), offsets.size() * sizeof(int));
   return SAF_OK;

@@ -79,8 +79,6 @@ struct FwdParams {
   const int* ovf;
   int call_id;
   int nblkp;
-  const WorkItem* items;            // grouped by CTA
-  const int* cta_offsets;           // [grid+1]
   // The items in queue order, claimed at run time.  queue[0] = next unclaimed item, queue[1] = CTAs
   // that have finished; the last CTA to finish sets both back to zero for the next launch.
   const WorkItem* order;
