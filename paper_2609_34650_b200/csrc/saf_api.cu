@@ -286,14 +286,17 @@ void build_worklist_host(int B, int H, int T, const uint8_t* mask, int backward,
 
 // Work queue of the 128-wide forward, whose items are two consecutive query blocks of one (batch, head) unit (the first
 // block of an odd count goes alone).  CTAs claim items in this order at run time, so longest-first within groups of
-// units keeps both the tail short and a group's K and V in L2 while its items run: a group is as many units as have
-// 32 MB of K and V together.  While the items would not fill the SMs, blocks go one by one: a pair takes longer than a
+// units keeps both the tail short and a group's K and V in L2 while its items run.  Groups are of equal size (a small last
+// group is a tail of long items: 2x16x8192x96 0.456 ms with groups of 10, 10, 10 and 2 units, 0.373 with two of 16) and
+// hold at most 64 MB of K and V (8x12x4096x128: 32 MB 0.335 ms, 64 MB 0.339, 128 MB 0.346; 1x16x16384x128: 0.778, 0.760,
+// 0.758).  While the items would not fill the SMs, blocks go one by one: a pair takes longer than a
 // single block and there are SMs to spare.
 void build_pair_order(int B, int H, int T, int D, const uint8_t* mask, int num_sms, std::vector<WorkItem>& order) {
   const int nblk = (T + BLK - 1) / BLK;
   const bool pair = static_cast<long long>(B) * H * nblk > num_sms;
   const long long unit_bytes = static_cast<long long>(T) * D * 4;
-  const int group = static_cast<int>(std::max<long long>(1, (32ll << 20) / unit_bytes));
+  const long long n_groups = std::max<long long>(1, (unit_bytes * B * H + (64ll << 20) - 1) / (64ll << 20));
+  const int group = static_cast<int>((static_cast<long long>(B) * H + n_groups - 1) / n_groups);
   order.clear();
   std::vector<std::pair<long long, WorkItem>> items;
   auto flush = [&] {
