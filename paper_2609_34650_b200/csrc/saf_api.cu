@@ -236,7 +236,7 @@ int upload_mask(saf_ctx* ctx, const uint8_t* mask, int H, cudaStream_t st) {
 // end, and each item goes to the CTA that becomes free first (list scheduling, which is what a dynamic
 // queue would do); only the last items are ordered longest-first so that the tail stays short.
 void build_worklist_host(int B, int H, int T, const uint8_t* mask, int backward, int n_ctas, int frozen_pct,
-                         int overhead_pct, int overhead_frozen_pct, std::vector<WorkItem>* items,
+                         int overhead_pct, int overhead_frozen_pct, int tail_per_cta, std::vector<WorkItem>* items,
                          std::vector<int>* offsets, std::vector<WorkItem>* order) {
   const int nblk = (T + BLK - 1) / BLK;
   struct Cand { WorkItem w; long long cost; };
@@ -256,8 +256,8 @@ void build_worklist_host(int B, int H, int T, const uint8_t* mask, int backward,
         cand.push_back({{b, h, k, kind}, cost});
       }
     }
-  // the tail (about two items per CTA) longest-first
-  const size_t tail = std::min(cand.size(), static_cast<size_t>(2) * n_ctas);
+  // the tail longest-first
+  const size_t tail = std::min(cand.size(), static_cast<size_t>(tail_per_cta) * n_ctas);
   std::stable_sort(cand.end() - tail, cand.end(), [](const Cand& a, const Cand& b) { return a.cost > b.cost; });
   if (order) {
     // the sequence itself is the work queue of the kernels that claim items at run time
@@ -356,7 +356,9 @@ int get_worklist(saf_ctx* ctx, int B, int H, int T, int D, const uint8_t* mask, 
   if (!backward && wide) {
     build_pair_order(B, H, T, D, mask, ctx->num_sms, e.items_host);
   } else {
-    build_worklist_host(B, H, T, mask, backward, grid, frozen_pct, overhead_pct, overhead_frozen_pct,
+    // (tail: two items per CTA; on the 128-wide backward four: -0.5 % on 8x12x4096x128, -1 % on 2x16x8192x96, -3 % on
+    // 1x16x8192x128 and on shared heads 3x8x3000x128; six and eight are no better)
+    build_worklist_host(B, H, T, mask, backward, grid, frozen_pct, overhead_pct, overhead_frozen_pct, wide ? 4 : 2,
                         backward ? &e.items_host : nullptr, &e.offsets_host, backward ? nullptr : &e.items_host);
   }
   e.B = B; e.H = H; e.T = T; e.D = D; e.backward = backward; e.grid = grid;
@@ -1398,7 +1400,7 @@ int saf_build_worklist(int32_t B, int32_t H, int32_t T, const uint8_t* frozen_ma
   std::vector<int> offsets;
   int fp_unused, ov, ovf;
   sched_defaults(0, backward ? 1 : 0, &fp_unused, &ov, &ovf);      // the 64-wide kernels' per-item overheads
-  build_worklist_host(B, H, T, frozen_mask_host, backward ? 1 : 0, n_ctas, frozen_weight_pct, ov, ovf, &items, &offsets,
+  build_worklist_host(B, H, T, frozen_mask_host, backward ? 1 : 0, n_ctas, frozen_weight_pct, ov, ovf, 2, &items, &offsets,
                       nullptr);
   std::memcpy(items_out, items.data(), items.size() * sizeof(WorkItem));
   std::memcpy(offsets_out, offsets.data(), offsets.size() * sizeof(int));
