@@ -21,12 +21,13 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
+enum { WL_QUEUE = 0, WL_BACKWARD = 1, WL_SHORT = 2 };   // forward queue, backward lists, lists of the short 128-wide forward
 struct WorklistEntry {
-  int B, H, T, D, backward, grid;
+  int B, H, T, D, kind, grid;
   std::vector<uint8_t> mask;
   std::vector<WorkItem> items_host;       // kept alive: the upload is asynchronous on the caller's stream
   std::vector<int> offsets_host;
-  WorkItem* items_dev = nullptr;          // backward: grouped by CTA; forward: queue order
+  WorkItem* items_dev = nullptr;          // WL_QUEUE: in queue order; else grouped by CTA
   int* offsets_dev = nullptr;
   int n_items = 0;
 };
@@ -318,6 +319,21 @@ void build_pair_order(int B, int H, int T, int D, const uint8_t* mask, int num_s
   flush();
 }
 
+// Whether a 128-wide forward goes to the kernel of short sequences (one query block per item, two CTAs per SM).  The line
+// lies where the two cross (us of back-to-back forwards, no frozen head; this kernel / the two-block kernel):
+//   up to two blocks a unit: 32x16x64x128 14.2 / 20.9, 12x16x256x128 16.6 / 20.9, 32x16x256x128 41.5 / 41.9
+//   three: up to about four (head dimension 96: eight) blocks per SM: 6x16x384x128 16.2 / 17.9, 16x16x384x128 36.5 / 33.3
+//   up to six: while the two-block items are one wave and a little: 6x16x512x128 20.4 / 25.0, 8x16x512x128 26.4 / 25.2
+//   up to ten: while the blocks are: 1x32x640x128, one forward waited for, 34.4 / 36.8
+bool fwd_is_short(int B, int H, int T, int D, int num_sms) {
+  const long long units = static_cast<long long>(B) * H, nblk = (T + BLK - 1) / BLK, blocks = units * nblk;
+  if (nblk <= 2) return true;
+  if (nblk == 3) return blocks <= (D == 96 ? 8LL : 4LL) * num_sms;
+  const long long items = units * ((nblk + 1) / 2);       // of the two-block kernel
+  if (nblk <= 6 && items > num_sms && 5 * items <= 8LL * num_sms) return true;
+  return nblk <= 10 && blocks > num_sms && 10 * blocks <= 13LL * num_sms;
+}
+
 // Measured cost-model defaults: `wide` = the 128-wide kernels (head dimension 96 or 128), else the 64-wide ones.
 void sched_defaults(int wide, int backward, int* frozen_pct, int* overhead_pct, int* overhead_frozen_pct) {
   if (backward) {
@@ -330,10 +346,10 @@ void sched_defaults(int wide, int backward, int* frozen_pct, int* overhead_pct, 
   }
 }
 
-int get_worklist(saf_ctx* ctx, int B, int H, int T, int D, const uint8_t* mask, int backward, int grid, cudaStream_t st,
+int get_worklist(saf_ctx* ctx, int B, int H, int T, int D, const uint8_t* mask, int kind, int grid, cudaStream_t st,
                  const WorklistEntry** out) {
   for (const WorklistEntry& e : ctx->worklists)
-    if (e.B == B && e.H == H && e.T == T && e.D == D && e.backward == backward && e.grid == grid &&
+    if (e.B == B && e.H == H && e.T == T && e.D == D && e.kind == kind && e.grid == grid &&
         std::memcmp(e.mask.data(), mask, H) == 0) {
       *out = &e;
       return SAF_OK;
@@ -344,24 +360,25 @@ int get_worklist(saf_ctx* ctx, int B, int H, int T, int D, const uint8_t* mask, 
     cudaFree(ctx->worklists.front().offsets_dev);
     ctx->worklists.erase(ctx->worklists.begin());
   }
-  const int wide = D != 64;
+  const int wide = D != 64, backward = kind == WL_BACKWARD ? 1 : 0;
   int frozen_pct, overhead_pct, overhead_frozen_pct;
   sched_defaults(wide, backward, &frozen_pct, &overhead_pct, &overhead_frozen_pct);
   const int fw = backward ? ctx->frozen_weight_bwd_pct : ctx->frozen_weight_pct;
   const int ov = backward ? ctx->item_overhead_bwd_pct : ctx->item_overhead_pct;
   if (fw > 0) frozen_pct = fw;
   if (ov > 0) overhead_pct = overhead_frozen_pct = ov;   // (the override sets both kinds)
-  // backward: per-CTA lists; forward: a queue
+  const bool lists = kind != WL_QUEUE;
   WorklistEntry e;
-  if (!backward && wide) {
+  if (!lists && wide) {
     build_pair_order(B, H, T, D, mask, ctx->num_sms, e.items_host);
   } else {
     // (tail: two items per CTA; on the 128-wide backward four: -0.5 % on 8x12x4096x128, -1 % on 2x16x8192x96, -3 % on
     // 1x16x8192x128 and on shared heads 3x8x3000x128; six and eight are no better)
-    build_worklist_host(B, H, T, mask, backward, grid, frozen_pct, overhead_pct, overhead_frozen_pct, wide ? 4 : 2,
-                        backward ? &e.items_host : nullptr, &e.offsets_host, backward ? nullptr : &e.items_host);
+    build_worklist_host(B, H, T, mask, backward, grid, frozen_pct, overhead_pct, overhead_frozen_pct,
+                        wide && backward ? 4 : 2, lists ? &e.items_host : nullptr, &e.offsets_host,
+                        lists ? nullptr : &e.items_host);
   }
-  e.B = B; e.H = H; e.T = T; e.D = D; e.backward = backward; e.grid = grid;
+  e.B = B; e.H = H; e.T = T; e.D = D; e.kind = kind; e.grid = grid;
   e.mask.assign(mask, mask + H);
   e.n_items = static_cast<int>(e.items_host.size());
   auto give_up = [&](int code) {
@@ -375,7 +392,7 @@ int get_worklist(saf_ctx* ctx, int B, int H, int T, int D, const uint8_t* mask, 
   if (cudaMemcpyAsync(e.items_dev, e.items_host.data(), e.items_host.size() * sizeof(WorkItem), cudaMemcpyHostToDevice,
                       st) != cudaSuccess)
     return give_up(SAF_ERR_CUDA);
-  if (backward) {
+  if (lists) {
     if (cudaMalloc(&e.offsets_dev, e.offsets_host.size() * sizeof(int)) != cudaSuccess) return give_up(SAF_ERR_NOMEM);
     if (cudaMemcpyAsync(e.offsets_dev, e.offsets_host.data(), e.offsets_host.size() * sizeof(int), cudaMemcpyHostToDevice,
                         st) != cudaSuccess)
@@ -646,10 +663,11 @@ int saf_hybrid_attn_fwd(saf_ctx* ctx, const saf_problem* p, const void* Q, const
   }
   const int nblk = (p->T + BLK - 1) / BLK;
   const long long n_items = static_cast<long long>(p->B) * p->H * nblk;
-  // (head dimension 64: two CTAs per SM; the 128-wide kernel: one)
-  const int grid = static_cast<int>(std::min<long long>((p->D == 64 ? 2LL : 1LL) * ctx->num_sms, n_items));
+  const bool is_short = p->D != 64 && fwd_is_short(p->B, p->H, p->T, p->D, ctx->num_sms);
+  // (head dimension 64 and the short 128-wide kernel: two CTAs per SM; the other 128-wide kernel: one)
+  const int grid = static_cast<int>(std::min<long long>((p->D == 64 || is_short ? 2LL : 1LL) * ctx->num_sms, n_items));
   const WorklistEntry* wl = nullptr;
-  rc = get_worklist(ctx, p->B, p->H, p->T, p->D, frozen_mask_host, 0, grid, st, &wl);
+  rc = get_worklist(ctx, p->B, p->H, p->T, p->D, frozen_mask_host, is_short ? WL_SHORT : WL_QUEUE, grid, st, &wl);
   if (rc) return rc;
 
   CUtensorMap mq, mk, mv;
@@ -704,7 +722,8 @@ int saf_hybrid_attn_fwd(saf_ctx* ctx, const saf_problem* p, const void* Q, const
   fp.o_f32 = p->o_dtype == SAF_F32 ? 1 : 0;
   for (int i = 0; i < 3; ++i) fp.o_strides[i] = p->o_strides[i];
   fp.LSE = LSE;
-  fp.order = wl->items_dev;
+  fp.items = wl->items_dev;
+  fp.cta_offsets = wl->offsets_dev;
   fp.n_items = wl->n_items;
   fp.queue = ctx->queue_dev;
   fp.status = ctx->status_dev;
@@ -718,6 +737,7 @@ int saf_hybrid_attn_fwd(saf_ctx* ctx, const saf_problem* p, const void* Q, const
   CUtensorMap mo;
   rc = make_map(ctx, &mo, O, p, p->o_strides);
   if (rc) return rc;
+  if (is_short) return launch_fwd_short(mq, mk, mv, mvt, fp, grid, st) == cudaSuccess ? SAF_OK : SAF_ERR_CUDA;
   if (launch_fwd(p->D == 96 ? 128 : p->D, mq, mk, mv, mvt, mo, fp, grid, st) != cudaSuccess) return SAF_ERR_CUDA;
   return SAF_OK;
 }
@@ -817,7 +837,7 @@ int saf_hybrid_attn_bwd(saf_ctx* ctx, const saf_problem* p, const void* Q, const
   const long long n_items = static_cast<long long>(p->B) * p->H * nblk;
   const int grid = static_cast<int>(std::min<long long>(ctx->num_sms, n_items));
   const WorklistEntry* wl = nullptr;
-  rc = get_worklist(ctx, p->B, p->H, p->T, p->D, frozen_mask_host, 1, grid, st, &wl);
+  rc = get_worklist(ctx, p->B, p->H, p->T, p->D, frozen_mask_host, WL_BACKWARD, grid, st, &wl);
   if (rc) return rc;
 
   CUtensorMap mq, mk, mv, mdo;

@@ -200,7 +200,7 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
           const int idx = nclaim == 1 ? static_cast<int>(blockIdx.x) : p.n_items <= grid ? p.n_items : grid + atomicAdd(p.queue, 1);
           next = make_int4(0, 0, 0, RING_END);
           if (idx < p.n_items) {
-            next = __ldg(reinterpret_cast<const int4*>(p.order + idx));
+            next = __ldg(reinterpret_cast<const int4*>(p.items + idx));
             if ((next.w & 0x7f) != KIND_ORDINARY && p.band_f != nullptr && __ldg(p.fast_ok + next.y) != 0 &&
                 __ldg(p.ovf + next.y) != p.call_id)
               next.w |= RING_FAST;

@@ -209,7 +209,7 @@ saf_fwd64_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
         int4 rec = make_int4(0, 0, 0, RING_END);
         bool fast = false;
         if (idx < p.n_items) {
-          rec = __ldg(reinterpret_cast<const int4*>(p.order + idx));
+          rec = __ldg(reinterpret_cast<const int4*>(p.items + idx));
           fast = rec.w != KIND_ORDINARY && p.band_f != nullptr && __ldg(p.fast_ok + rec.y) != 0 &&
                  __ldg(p.ovf + rec.y) != p.call_id;
           if (fast) rec.w |= RING_FAST;

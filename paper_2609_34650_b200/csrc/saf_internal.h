@@ -79,9 +79,11 @@ struct FwdParams {
   const int* ovf;
   int call_id;
   int nblkp;
-  // The items in queue order, claimed at run time.  queue[0] = next unclaimed item, queue[1] = CTAs
-  // that have finished; the last CTA to finish sets both back to zero for the next launch.
-  const WorkItem* order;
+  // The items: in queue order and claimed at run time (queue[0] = next unclaimed item, queue[1] = CTAs that have finished;
+  // the last CTA to finish sets both back to zero for the next launch); in the short 128-wide kernel grouped by CTA,
+  // cta_offsets[grid + 1].
+  const WorkItem* items;
+  const int* cta_offsets;
   int n_items;
   int* queue;
   int* status;                      // device status word
@@ -208,6 +210,9 @@ cudaError_t launch_bwd_finalize(const float* dQacc, void* dQ, size_t n, cudaStre
 cudaError_t launch_fwd64(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv, const CUtensorMap& mvt,
                          const CUtensorMap& mo, const FwdParams& p, int grid, cudaStream_t st);
 int fwd64_smem_bytes();
+// head dimension 128 / 96, short sequences (saf_fwd_short.cu)
+cudaError_t launch_fwd_short(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv, const CUtensorMap& mvt,
+                             const FwdParams& p, int grid, cudaStream_t st);
 // head dimension 128 / 96 (saf_bwd128.cu): mdot as in launch_bwd, mdq the fp32 dQ accumulator [B][Hq][T][D] in boxes of 32
 // rows; q_ext / do_ext of the parameters are fp32 vectors [B][H][128 nblk] (-LSE log2 e, -delta); dK / dV are written with
 // plain stores (reduce-adds for shared heads)

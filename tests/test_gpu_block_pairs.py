@@ -1,5 +1,5 @@
-"""GPU tests at the edges of the 128-wide kernels' work items (two query blocks per forward item, full 128-query tiles in
-the backward), of the normaliser kernel's chunks and of the calibration's mean pass."""
+"""GPU tests at the edges of the 128-wide kernels' work items (one or two query blocks per forward item, full 128-query tiles
+in the backward), of the normaliser kernel's chunks and of the calibration's mean pass."""
 import numpy as np
 import pytest
 import torch
@@ -9,28 +9,41 @@ import saf_inputs as si
 from oracle import saf_oracle as orc
 
 from gpu_util import Layer
-from test_gpu_parity import all_units, check_units
+from test_gpu_parity import all_units, check_units, sampled_units
 
 pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("B,H,T,D,frozen", [
-    (1, 4, 128, 128, (1,)),             # one block, alone
-    (1, 3, 129, 96, (0,)),              # two blocks, one by one (fewer than the SMs)
-    (5, 10, 257, 128, (1, 4, 7)),       # 150 blocks: pairs, the first block of an odd count alone
-    (6, 13, 256, 128, (2, 3)),          # 156 blocks: one pair per unit
-    (4, 10, 512, 96, (0, 5, 9)),        # pairs of every length up to four tiles
-    (10, 16, 100, 128, (3,)),           # more one-block units than SMs: no pairs to form
+    # one query block per item, two CTAs per SM
+    (1, 4, 128, 128, (1,)),             # one block
+    (1, 3, 129, 96, (0,)),              # two blocks
+    (5, 10, 257, 128, (1, 4, 7)),       # three blocks, 150 items
+    (10, 16, 100, 128, (3,)),           # 160 one-block units
+    (16, 12, 300, 128, (2, 3)),         # the most three-block units that go there (576 blocks on 148 SMs)
+    (12, 8, 512, 96, (0, 5)),           # four blocks: 192 two-block items would be a wave and a little
+    (1, 32, 640, 128, (7,)),            # 160 blocks
+    # two query blocks per item, one CTA per SM
+    (1, 4, 520, 128, (1,)),             # five blocks, one by one (fewer than the SMs)
+    (4, 10, 520, 96, (0, 5, 9)),        # 200 blocks: pairs, the first block of an odd count alone
+    (17, 12, 300, 128, (1, 4)),         # one more batch entry than above: a pair and a single block per unit
+    (4, 10, 768, 128, (2, 3)),          # pairs of every length up to six tiles
 ])
-def test_block_pairs(B, H, T, D, frozen):
-    inp = si.generate(si.Workload("pairs", B, H, T, D, frozen, -0.05, seed=T + D))
-    check_units(Layer(inp).run(), all_units(inp.wl))
+def test_item_shapes_of_the_wide_forward(B, H, T, D, frozen):
+    """Both kernels of head dimensions 96 and 128 on either side of the line between them."""
+    inp = si.generate(si.Workload("items", B, H, T, D, frozen, -0.05, seed=T + D))
+    units = all_units(inp.wl)
+    check_units(Layer(inp).run(), units if len(units) <= 50 else sampled_units(inp.wl, 24, seed=5))
 
 
-def test_running_maximum_far_above_the_first_tile():
-    """Scores that grow along the sequence: the rescaling of the accumulator between tiles, in both blocks of a pair."""
-    inp = si.generate(si.Workload("grow", 2, 2, 640, 128, (), -0.05, seed=9))
-    f = np.exp2(np.arange(640) // 128).astype(np.float32)          # exact in bf16
+@pytest.mark.parametrize("B,H,T", [(2, 2, 384), (4, 12, 640)])
+def test_running_maximum_far_above_the_first_tile(B, H, T):
+    """Scores that grow along the sequence: the rescaling of the accumulator between tiles, in the one-block kernel and in
+    both blocks of a pair (240 blocks: more than the one-block items that are tried first, so they are paired)."""
+    n_sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert T == 384 or B * H * (T // 128) > 1.3 * n_sms
+    inp = si.generate(si.Workload("grow", B, H, T, 128, (), -0.05, seed=9))
+    f = np.exp2(np.arange(T) // 128).astype(np.float32)            # exact in bf16
     inp.k[...] = si.f32_to_bf16_bits(si.bf16_bits_to_f32(inp.k) * f[None, None, :, None])
     L = Layer(inp, backward=False)
     L.run(backward=False)
@@ -38,6 +51,22 @@ def test_running_maximum_far_above_the_first_tile():
     want, _ = orc.hybrid_attn_fwd(q, k, v, inp.mask, inp.alpha, inp.rho)
     got = L.O.float().cpu().numpy().astype(np.float64)
     assert np.abs(got - want).max() <= 2e-2 and np.linalg.norm(got - want) <= 1e-2 * np.linalg.norm(want)
+
+
+@pytest.mark.parametrize("D", [96, 128])
+@pytest.mark.parametrize("B,H,T", [(16, 12, 300), (8, 8, 1200)])
+def test_item_kinds_alternate_at_the_wide_head_dimensions(B, H, T, D):
+    """Ordinary heads, frozen heads in the tensor-core form and frozen heads in the general form follow one another in the
+    one-block items of the short forward (576 blocks), in the paired items of the long one (640 blocks) and in the
+    backward's lists, several to a CTA."""
+    frozen = (0, 2, 3, 5, 6)
+    inp = si.generate(si.Workload("kinds", B, H, T, D, frozen, -0.05, seed=23 + D))
+    for h in (2, 5):                                               # far outside the range of the tensor-core form
+        inp.alpha[h] = (inp.alpha[h] + 25.0 * np.sin(0.37 * np.arange(T))).astype(np.float32)
+    # (rows whose mass sits on a few keys: see the same test at head dimension 64)
+    inp.do[...] = si.f32_to_bf16_bits(si.bf16_bits_to_f32(inp.do) / 16.0)
+    L = Layer(inp).run()
+    check_units(L, [(0, 0), (0, 2), (1, 1), (2, 5), (3, 3), (4, 4), (5, 6), (6, 7), (7, 2), (B - 1, H - 1)])
 
 
 @pytest.mark.parametrize("T", [1, 31, 33, 255, 4096, 4097, 8200])
