@@ -789,19 +789,19 @@ saf_fwd64_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
 
 int fwd64_smem_bytes() { return Fwd64Cfg::SMEM; }
 
+// Early launch (under the tail of the kernel before): the CTAs then land on the SMs in the order in which these become free,
+// so that long items meet on one SM.  Where a CTA gets one or two items in all, that costs more than the launch gap
+// (forwards back to back, early / not: 1x12x3072x64 45.3 / 36.2 us, 1x8x4096x64 54.4 / 44.2, 2x12x2048x64 33.2 / 29.2);
+// with several items per CTA it gains (1x32x2048x64 34.8 / 37.9, 4x12x2048x64 46.4 / 49.0).  Behind the staging kernel, which
+// lets go of its dependents when everything before it is done, one item per CTA gains as well (1x12x3072x64, three frozen
+// heads, 36.2 / 38.2; 1x8x1024x64, one forward waited for, 33.4 / 36.0).
 cudaError_t launch_fwd64(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv, const CUtensorMap& mvt,
                          const CUtensorMap& mo, const FwdParams& p, int grid, cudaStream_t st) {
-  cudaError_t e;
-  if (p.o_f32) {
-    e = cudaFuncSetAttribute(saf_fwd64_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, Fwd64Cfg::SMEM);
-    if (e != cudaSuccess) return e;
-    return launch_pdl(PDL_FWD, saf_fwd64_kernel<true>, dim3(grid), dim3(Fwd64Cfg::NTHREADS), Fwd64Cfg::SMEM, st, mq, mk, mv,
-                      mvt, mo, p);
-  }
-  e = cudaFuncSetAttribute(saf_fwd64_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, Fwd64Cfg::SMEM);
+  const bool early = 2 * p.n_items >= 5 * grid || (p.band_f != nullptr && p.n_items <= grid);
+  auto kern = p.o_f32 ? saf_fwd64_kernel<true> : saf_fwd64_kernel<false>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Fwd64Cfg::SMEM);
   if (e != cudaSuccess) return e;
-  return launch_pdl(PDL_FWD, saf_fwd64_kernel<false>, dim3(grid), dim3(Fwd64Cfg::NTHREADS), Fwd64Cfg::SMEM, st, mq, mk, mv,
-                    mvt, mo, p);
+  return launch_pdl(early ? PDL_FWD : 0, kern, dim3(grid), dim3(Fwd64Cfg::NTHREADS), Fwd64Cfg::SMEM, st, mq, mk, mv, mvt, mo, p);
 }
 
 }  // namespace saf

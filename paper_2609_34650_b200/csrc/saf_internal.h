@@ -20,11 +20,11 @@ inline bool pdl_enabled() {
   }();
   return on;
 }
-// Which kernels are launched that way (SAF_PDL_MASK: bit 0 staging kernels, 1 D = 64 forward, 2 backward preparation,
-// 3 backward, 4 the 128-wide forward, 5 backward preparation of small layers).  All but the preparation of large layers:
-// its blocks then fill the SMs under the forward's tail, where the layer is long enough for that to cost more than the
-// launch gap (8x12x4096x64: pass +2 %, 8x12x2048x128 +3 %; 3x12x1537x64 -1 %, 4x12x1024x64 -3 %, 1x4x256x64 -5 %).
-// The others gain or are neutral: staging 1x32x333x128 -6 %, D = 64 forward 3x12x1537x64 -4 %, 8x12x2048x64 -1 %.
+// Which kernels are launched that way (SAF_PDL_MASK: bit 0 staging kernels, 1 D = 64 forward where launch_fwd64 asks for
+// it, 2 backward preparation, 3 backward, 4 the 128-wide forwards, 5 backward preparation of small layers).  All but the
+// preparation of larger layers: its blocks then fill the SMs under the forward's tail, where the layer is long enough for
+// that to cost more than the launch gap (8x12x4096x64: pass +2 %, 8x12x2048x128 +3 %).
+// The others gain or are neutral: staging 1x32x333x128 -6 %.
 inline int pdl_mask() {
   static const int m = [] {
     const char* e = std::getenv("SAF_PDL_MASK");

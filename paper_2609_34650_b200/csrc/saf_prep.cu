@@ -249,8 +249,11 @@ __global__ void __launch_bounds__(256) saf_scale_rows_kernel(const __nv_bfloat16
                                                              int call_id, __half* __restrict__ dst, int B, int Hf,
                                                              int T, int src_group, const PatternCheck chk) {
   constexpr int TPR = D / 8;
-  pdl_launch_dependents();
-  pdl_wait();                                      // (launched with programmatic stream serialization)
+  // (launched with programmatic stream serialization.  Head dimension 64: the forward behind this kernel may start its CTAs
+  // only when everything earlier is done, see launch_fwd64)
+  if constexpr (D != 64) pdl_launch_dependents();
+  pdl_wait();
+  if constexpr (D == 64) pdl_launch_dependents();
   const long long gid = static_cast<long long>(blockIdx.x) * 256 + threadIdx.x;
   const long long rowid = gid / TPR;               // over [B][Hf][T]: frozen heads only
   const int part = static_cast<int>(gid % TPR);
