@@ -468,8 +468,10 @@ cudaError_t launch_bwd_prep(const void* O, int o_f32, const void* dO, const floa
 #define SAF_PREP_ARGS                                                                                                  \
   O, static_cast<const __nv_bfloat16*>(dO), LSE, os[0], os[1], os[2], mask_dev, static_cast<uint8_t*>(q_ext),          \
       static_cast<uint8_t*>(do_ext), inv_scale, dQacc, dK, dV, grad_f32, kv_group, qslot, n_ord, fz, B, H, T
-  // (small: at most ~14 blocks per SM, less than two waves)
-  const int which = grid <= 2048 ? PDL_PREP_SMALL : PDL_PREP;
+  // (early where that gains: with some two blocks per SM (passes of 1x4x1024x64 -1 %, 1x12x500x64 -2 %, 1x4x256x128 -2 %), and
+  // at head dimension 64 with 8 to 14 (one full wave and more: 8x12x512 -3 %, 2x12x2048 -2 %).  In between, and at the wider
+  // ones, blocks under the forward's tail cost more than the launch gap: 1x12x1500x64 +3 %, 2x12x640x64 +2 %, 1x8x1024x128 +4 %)
+  const int which = grid <= 400 || (D == 64 && grid >= 1184 && grid <= 2048) ? PDL_PREP_SMALL : PDL_PREP;
 #define SAF_PREP_LAUNCH(DD, TT, FF) \
   launch_pdl(which, saf_bwd_prep_kernel<DD, TT, FF>, dim3(grid), dim3(256), 0, st, SAF_PREP_ARGS)
   cudaError_t e;
