@@ -588,8 +588,8 @@ int saf_pattern_prepare(saf_ctx* ctx, int32_t H, int32_t Tp, const uint8_t* froz
       (rc = ensure(ctx->pat_bandb, bandb)) || (rc = ensure(ctx->pat_heads, 2 * hb)) || (rc = ensure(ctx->pat_snap, 3 * vecb)) ||
       (rc = ensure(ctx->pat_marks, 4 * hb)))
     return rc;
-  // A new buffer starts at zero: per-head overflow marks of the forward / backward staging kernels (a mark is the id of the
-  // call that set it, ids only grow) and the counters of the normaliser kernel (which returns them to zero).
+  // A new buffer starts at zero: the counters of the normaliser kernel (which returns them to zero) and the per-head overflow
+  // marks of the forward / backward staging kernels (the id of the call that set one; the table kernel clears them).
   if (ctx->pat_heads.bytes != heads_before) ctx->pat_heads_host.clear();
   if (ctx->pat_marks.bytes != marks_before) {
     if (cudaMemsetAsync(ctx->pat_marks.ptr, 0, ctx->pat_marks.bytes, st) != cudaSuccess) return SAF_ERR_CUDA;
@@ -620,7 +620,7 @@ int saf_pattern_prepare(saf_ctx* ctx, int32_t H, int32_t Tp, const uint8_t* froz
         launch_pattern_tables(alpha_dev, rho_dev, logZ_dev_out, static_cast<const uint8_t*>(ctx->mask_buf.ptr), H, Tp, consts,
                               static_cast<float*>(ctx->pat_avec.ptr), static_cast<float*>(ctx->pat_wvec.ptr),
                               ctx->pat_bandf.ptr, ctx->pat_bandb.ptr, static_cast<uint32_t*>(ctx->pat_snap.ptr),
-                              st) != cudaSuccess)
+                              ctx->pat_mark(0), ctx->pat_mark(1), st) != cudaSuccess)
       return SAF_ERR_CUDA;
   }
   ctx->pat.valid = true;

@@ -173,7 +173,8 @@ cudaError_t launch_logz(const float* alpha, const float* rho, float* logZ, const
                         float* consts, int* fast_ok, unsigned* counters, cudaStream_t st);
 cudaError_t launch_pattern_tables(const float* alpha, const float* rho, const float* logZ, const uint8_t* mask_dev,
                                   int H, int Tp, const float* consts, float* avec, float* wvec, void* band_f,
-                                  void* band_b, uint32_t* snap, cudaStream_t st);
+                                  void* band_b, uint32_t* snap, int* ovf_fwd, int* ovf_bwd,
+                                  cudaStream_t st);   // ovf_*: the overflow marks, cleared
 cudaError_t launch_scale_rows(const void* src, const int64_t* strides, const float* vec, float extra, int Tp,
                               const int* hlist, const int* pat_ok, int* ovf, int call_id, void* dst, int B, int Hf,
                               int T, int D, int src_group, const PatternCheck& chk, cudaStream_t st);   // src head = h / src_group

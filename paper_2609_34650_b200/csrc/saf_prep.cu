@@ -190,8 +190,11 @@ __global__ void __launch_bounds__(256) saf_pattern_tables_kernel(const float* __
                                                                  float* __restrict__ avec, float* __restrict__ wvec,
                                                                  __half* __restrict__ band_f,
                                                                  __half* __restrict__ band_b, uint32_t* __restrict__ snap,
+                                                                 int* __restrict__ ovf_fwd, int* __restrict__ ovf_bwd,
                                                                  int nblkp) {
   const int h = blockIdx.y, dblk = blockIdx.x;
+  // marks of earlier calls end here: a call recorded into a CUDA graph keeps its id over all replays
+  if (dblk == 0 && threadIdx.x == 0) ovf_fwd[h] = ovf_bwd[h] = 0;
   if (!mask[h]) return;
   const float ca = consts[2 * h], cr = consts[2 * h + 1];
   const size_t row = static_cast<size_t>(h) * Tp;
@@ -221,18 +224,19 @@ __global__ void __launch_bounds__(256) saf_pattern_tables_kernel(const float* __
 
 cudaError_t launch_pattern_tables(const float* alpha, const float* rho, const float* logZ, const uint8_t* mask_dev, int H,
                                   int Tp, const float* consts, float* avec, float* wvec, void* band_f, void* band_b,
-                                  uint32_t* snap, cudaStream_t st) {
+                                  uint32_t* snap, int* ovf_fwd, int* ovf_bwd, cudaStream_t st) {
   const int nblkp = (Tp + 127) / 128;
   saf_pattern_tables_kernel<<<dim3(nblkp, H), 256, 0, st>>>(alpha, rho, logZ, mask_dev, Tp, consts, avec, wvec,
                                                             static_cast<__half*>(band_f),
-                                                            static_cast<__half*>(band_b), snap, nblkp);
+                                                            static_cast<__half*>(band_b), snap, ovf_fwd, ovf_bwd, nblkp);
   return cudaGetLastError();
 }
 
 // dst[b][ord][t][:] = fp16(extra * vec[h][t] * src[b][h][t][:]), h = hlist[ord], for the frozen heads whose tensor-core form is
 // enabled (V scaled by a, or dO scaled by w).  Eight features per thread.  A product that leaves fp16's range
 // marks the head (ovf[h] = call_id), which sends it down the general path in the kernel that follows; the
-// mark of an earlier call has another id and needs no reset.  The same mark is raised when alpha, rho or logZ of the
+// mark of an earlier call has another id.  (The replays of a recorded call share theirs, so a mark holds for the later
+// replays too, until the next preparation clears it.)  The same mark is raised when alpha, rho or logZ of the
 // head no longer hold the bits the tables were built from (another call may have rewritten the vectors in place):
 // the threads of batch entry 0 compare their row's three values with the snapshot taken at preparation.
 __device__ __forceinline__ bool pattern_row_changed(const PatternCheck& c, size_t i) {

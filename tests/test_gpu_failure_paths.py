@@ -62,3 +62,38 @@ def test_vectors_rewritten_in_place_do_not_meet_stale_tables():
     # after a new preparation the tables are used again and agree as well
     L.run(prepare=True)
     check_units(L, all_units(wl))
+
+
+@pytest.mark.parametrize("D", [64, 128])
+def test_a_preparation_ends_the_overflow_marks_of_recorded_calls(D):
+    """A replay of a recorded forward and backward meets values that leave fp16's range, so the head takes the general form.
+    The replays share the recorded call's id; with the inputs restored and the pattern prepared again they must be back at
+    the tensor-core form, bit for bit."""
+    wl = si.Workload("marks", 2, 3, 300, D, (1,), -0.05, seed=91)
+    L = Layer(si.generate(wl))
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(s):
+        L.run()
+        want = [L.O[:, 1].clone(), L.grads[2][:, 1].clone()]
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s):
+            L.ctx.saf_hybrid_attn_fwd(L.prob, L.Q, L.K, L.V, L.mask, L.alpha, L.rho, L.logZ, L.O, L.LSE)
+            L.ctx.saf_hybrid_attn_bwd(L.prob, L.Q, L.K, L.V, L.O, L.dO, L.LSE, L.mask, L.alpha, L.rho, L.logZ, *L.grads)
+
+        def replay():
+            for t in (L.O, L.grads[2]):
+                t.fill_(float("nan"))
+            g.replay()
+            s.synchronize()
+            return [torch.equal(L.O[:, 1], want[0]), torch.equal(L.grads[2][:, 1], want[1])]
+
+        assert all(replay())
+        keep = L.V.clone(), L.dO.clone()
+        L.V[0, 1, 5, 3] = L.dO[0, 1, 5, 3] = 1e30                # (its own unit only; the range is checked per head)
+        replay()
+        assert torch.isfinite(L.O[1]).all()
+        L.V.copy_(keep[0])
+        L.dO.copy_(keep[1])
+        L.ctx.saf_pattern_prepare(L.mask, L.alpha, L.rho, L.logZ)
+        assert all(replay())
