@@ -14,10 +14,13 @@ namespace saf {
 // logZ[h][i] = log sum_{k<=i} exp(alpha[h][k] + rho[h][i-k])   (Eq. "compact-prior", the normaliser Z(i)).
 // A block takes 32 consecutive rows (lane = row) and its eight warps take slices of the keys in turn; alpha and rho pass
 // through shared memory in chunks (alpha[k] is the same for a warp, rho[i-k] contiguous over its lanes), -inf where the
-// causal range ends.  The exponentials are taken relative to max alpha[0..] + max rho[0..] over the block's range, an upper
-// bound that needs no pass of its own; a row whose sum is then too small for fp32 (every term 2^-100 below the bound) is
-// done again relative to its own maximum.  fp32 sums of 32 terms, fp64 from there.  Bound: one ex2 per causal pair.
-// (One warp per row with two passes over global memory: 19.4 us for 6 heads x 2048, now see the launcher.)
+// causal range ends.  The exponentials of a row are taken relative to its largest term among its nearest 32 keys, which
+// needs no pass of its own.  Where a larger term turns up further away (a sink under steep decay; beyond e^6 the differences
+// would carry more rounding than the sums alpha + rho themselves, and in the end overflow), the block goes over its range
+// once more, relative to the rows' own maxima.  fp32 sums of 32 terms, fp64 from there.
+// Bound: one ex2 per causal pair.
+// (6 heads x 2048: one warp per row with two passes over global memory 20.6 us with the launch gap, this one 16.6; with a sink of 90 on key 0,
+// where most rows are taken again, 19.5; 8 heads x 8192: 217 and 103)
 // The last block of a head to finish also forms the head's constants (consts != NULL): max alpha, max rho, and
 // whether the tensor-core form's range holds (see below); counters (two per head) return to zero.
 constexpr int LZ_KC = 4096;
@@ -31,7 +34,7 @@ __global__ void __launch_bounds__(256) saf_logz_kernel(const float* __restrict__
                                                        float* consts, int* __restrict__ fast_ok,
                                                        unsigned* __restrict__ counters) {
   __shared__ __align__(16) float sa[LZ_KC];
-  __shared__ float sr[LZ_KC + 32], red[2][8];
+  __shared__ float sr[LZ_KC + 32], red[2][8], near_max[8][32];
   __shared__ double part[8][32];
   const int h = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (!mask[h]) {
@@ -46,92 +49,105 @@ __global__ void __launch_bounds__(256) saf_logz_kernel(const float* __restrict__
   float* z = logZ + static_cast<size_t>(h) * Tp;
   const float L2E = 1.4426950408889634f;
   float ma = -INFINITY, mr = -INFINITY;
-  if (iend > LZ_KC) {                                   // (up to LZ_KC the maxima come out of the staging below)
-#pragma unroll 4
-    for (int k = tid; k < iend; k += 256) {
-      ma = fmaxf(ma, a[k]);
-      mr = fmaxf(mr, r[k]);
-    }
-  }
-  float bound = 0.0f, nb = 0.0f;
-  double s = 0.0;
-  for (int k0 = 0; k0 < iend; k0 += LZ_KC) {
-    const int n = (min(LZ_KC, iend - k0) + 31) / 32 * 32;      // keys of this chunk, in whole groups of 32
-    __syncthreads();
-    // sa[x] = alpha[k0 + x], sr[x] = rho[i0 + x - (k0 + n - 1)]
-#pragma unroll 4
-    for (int x = tid; x < n; x += 256) {
-      const bool in = k0 + x < iend;
-      const float v = in ? a[k0 + x] : 0.0f;
-      sa[x] = v;
-      ma = fmaxf(ma, in ? v : -INFINITY);
-    }
-#pragma unroll 4
-    for (int x = tid; x < n + 31; x += 256) {
-      const int d = i0 + x - (k0 + n - 1);
-      const float v = d >= 0 && d < iend ? r[d] : -INFINITY;
-      sr[x] = v;
-      mr = fmaxf(mr, v);
-    }
-    if (k0 == 0) {
-      ma = warp_max(ma);
-      mr = warp_max(mr);
-      if (lane == 0) {
-        red[0][warp] = ma;
-        red[1][warp] = mr;
-      }
-    }
-    __syncthreads();
-    if (k0 == 0) {
-#pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        ma = fmaxf(ma, red[0][k]);
-        mr = fmaxf(mr, red[1][k]);
-      }
-      bound = ma + mr;
-      nb = -bound * L2E;
-    }
-    for (int kb = 32 * warp; kb < n; kb += 256) {       // groups of 32 keys, in turn over the warps
-      const float* rp = sr + lane + n - 1 - kb;         // rp[-e] = rho[i0 + lane - (k0 + kb + e)]
-      float p[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-#pragma unroll
-      for (int e = 0; e < 32; e += 4) {
-        const float4 a4 = *reinterpret_cast<const float4*>(sa + kb + e);
-        p[0] += ex2_approx(fmaf(a4.x + rp[-e], L2E, nb));
-        p[1] += ex2_approx(fmaf(a4.y + rp[-e - 1], L2E, nb));
-        p[2] += ex2_approx(fmaf(a4.z + rp[-e - 2], L2E, nb));
-        p[3] += ex2_approx(fmaf(a4.w + rp[-e - 3], L2E, nb));
-      }
-      s += static_cast<double>((p[0] + p[1]) + (p[2] + p[3]));
-    }
-  }
-  part[warp][lane] = s;
-  __syncthreads();
-  if (warp != 0) return;
-  double t = 0.0;
-#pragma unroll
-  for (int k = 0; k < 8; ++k) t += part[k][lane];
+  float ref = 0.0f;                                     // what this lane's exponentials are relative to
   const int row = i0 + lane;
   const bool valid = row < Tp;
-  float ref = bound;
-  unsigned redo = __ballot_sync(0xffffffffu, valid && !(t > 1e-30));
-  while (redo) {
-    // the bound is too far above this row: two passes relative to its own maximum
-    const int src = __ffs(redo) - 1, rw = i0 + src;
-    redo &= redo - 1;
-    float m = -INFINITY;
-    for (int k = lane; k <= rw; k += 32) m = fmaxf(m, a[k] + r[rw - k]);
-    m = warp_max(m);
-    float s0 = 0.0f;
-    for (int k = lane; k <= rw; k += 32) s0 += __expf(a[k] + r[rw - k] - m);
-    double u = static_cast<double>(s0);
+  const int last = (iend - 1) / LZ_KC * LZ_KC;          // the chunk that holds the rows' own keys is taken first
+  double t = 0.0;
+  // pass 0: sums relative to the near maximum and, by the way, the rows' own maxima; 1, if one row needs it: relative to those
+  for (int pass = 0; pass < 2; ++pass) {
+    double s = 0.0;
+    float m = -INFINITY, top = 0.0f;
+    for (int k0 = last; k0 >= 0; k0 -= LZ_KC) {
+      const int n = (min(LZ_KC, iend - k0) + 31) / 32 * 32;    // keys of this chunk, in whole groups of 32
+      if (pass == 0 || last > 0) {                      // (a range of one chunk is still there)
+        __syncthreads();
+        // sa[x] = alpha[k0 + x], sr[x] = rho[i0 + x - (k0 + n - 1)]
+#pragma unroll 4
+        for (int x = tid; x < n; x += 256) {
+          const bool in = k0 + x < iend;
+          const float v = in ? a[k0 + x] : 0.0f;
+          sa[x] = v;
+          ma = fmaxf(ma, in ? v : -INFINITY);
+        }
+#pragma unroll 4
+        for (int x = tid; x < n + 31; x += 256) {
+          const int d = i0 + x - (k0 + n - 1);
+          const float v = d >= 0 && d < iend ? r[d] : -INFINITY;
+          sr[x] = v;
+          mr = fmaxf(mr, v);
+        }
+        __syncthreads();
+        if (pass == 0 && k0 == last) {                  // near maxima
+          float c = -INFINITY;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) u += __shfl_xor_sync(0xffffffffu, u, o);
-    if (lane == src) {
-      t = u;
-      ref = m;
+          for (int d = 4 * warp; d < 4 * warp + 4; ++d) {
+            const int x = row - d - k0;
+            if (x >= 0) c = fmaxf(c, sa[x] + sr[d + k0 + n - 1 - i0]);
+          }
+          near_max[warp][lane] = c;
+          __syncthreads();
+          ref = near_max[0][lane];
+#pragma unroll
+          for (int k = 1; k < 8; ++k) ref = fmaxf(ref, near_max[k][lane]);
+          __syncthreads();
+        }
+      }
+      for (int kb = 32 * warp; kb < n; kb += 256) {     // groups of 32 keys, in turn over the warps
+        const float* rp = sr + lane + n - 1 - kb;       // rp[-e] = rho[i0 + lane - (k0 + kb + e)]
+        float p[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        if (pass == 0) {
+#pragma unroll
+          for (int e = 0; e < 32; e += 4) {
+            const float4 a4 = *reinterpret_cast<const float4*>(sa + kb + e);
+            const float y0 = a4.x + rp[-e], y1 = a4.y + rp[-e - 1], y2 = a4.z + rp[-e - 2], y3 = a4.w + rp[-e - 3];
+            m = max3(max3(m, y0, y1), y2, y3);
+            p[0] += ex2_approx((y0 - ref) * L2E);
+            p[1] += ex2_approx((y1 - ref) * L2E);
+            p[2] += ex2_approx((y2 - ref) * L2E);
+            p[3] += ex2_approx((y3 - ref) * L2E);
+          }
+        } else {
+          // (what lies outside the row's range stays out, whatever alpha holds there)
+#pragma unroll 8
+          for (int e = 0; e < 32; ++e) {
+            const float w = rp[-e];
+            p[e & 3] += w == -INFINITY ? 0.0f : ex2_approx((sa[kb + e] + w - ref) * L2E);
+          }
+        }
+        const float g = (p[0] + p[1]) + (p[2] + p[3]);
+        top = fmaxf(top, g);
+        // (the nearest keys make up most of a decaying row: their four sums are not added in fp32 first)
+        s += kb + 64 >= n ? (static_cast<double>(p[0]) + p[1]) + (static_cast<double>(p[2]) + p[3]) : static_cast<double>(g);
+      }
+    }
+    part[warp][lane] = s;
+    near_max[warp][lane] = m;
+    const int again = __syncthreads_or(pass == 0 && valid && !(top < 512.0f && s >= 0.0));   // (or a NaN)
+    t = 0.0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) t += part[k][lane];
+    if (!again) break;
+    ref = near_max[0][lane];
+#pragma unroll
+    for (int k = 1; k < 8; ++k) ref = fmaxf(ref, near_max[k][lane]);
+    __syncthreads();                                    // (the sums of pass 0 have been read)
+  }
+  if (consts != nullptr && iend == Tp) {                // (this block has seen all of alpha and rho)
+    ma = warp_max(ma);
+    mr = warp_max(mr);
+    if (lane == 0) {
+      red[0][warp] = ma;
+      red[1][warp] = mr;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      ma = fmaxf(ma, red[0][k]);
+      mr = fmaxf(mr, red[1][k]);
     }
   }
+  if (warp != 0) return;
   const float zv = valid ? static_cast<float>(static_cast<double>(ref) + log(t)) : INFINITY;
   if (valid) z[row] = zv;
   if (consts == nullptr) return;

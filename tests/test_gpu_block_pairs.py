@@ -90,6 +90,62 @@ def test_normalisers_at_chunk_edges(T, spread):
         assert err.max() <= 5e-6 + 2.0 ** -23 * big, err.max()
 
 
+def test_normalisers_of_ordinary_patterns_are_rounded_once():
+    """Terms near the common bound: rms error at the rounding of the result (an fp32 unit of 2.4e-7 at |log Z| in [2, 4):
+    6.9e-8) and of alpha + rho (under 5e-8 over the few terms that make up a row's sum)."""
+    rng = np.random.default_rng(8)
+    T, H = 2048, 4
+    alpha = rng.standard_normal((H, T)).astype(np.float32)
+    rho = (-0.05 * np.arange(T) + 0.1 * rng.standard_normal((H, T))).astype(np.float32)
+    a, r, z = torch.from_numpy(alpha).cuda(), torch.from_numpy(rho).cuda(), torch.zeros(H, T, device="cuda")
+    saf.Context(0).saf_pattern_prepare(np.ones(H, dtype=np.uint8), a, r, z)
+    want = np.stack([orc.pattern_logZ(alpha[h], rho[h], T) for h in range(H)])
+    assert np.abs(want).max() < 8.0
+    assert np.sqrt(np.mean((z.cpu().numpy().astype(np.float64) - want) ** 2)) <= 1e-7
+
+
+@pytest.mark.parametrize("T", [70, 4200])
+def test_normalisers_ignore_what_a_row_does_not_see(T):
+    """Keys and distances beyond a row's causal range may hold anything, in its own 32-row block too; minus infinity switches
+    single keys off, the nearest ones among them."""
+    rng = np.random.default_rng(T)
+    alpha = rng.standard_normal((3, T)).astype(np.float32)
+    rho = (-0.01 * np.arange(T) + 0.1 * rng.standard_normal((3, T))).astype(np.float32)
+    alpha[0, T - 9] = np.inf
+    alpha[1, T - 9] = np.nan
+    alpha[2, T - 45:] = -np.inf
+    a, r, z = torch.from_numpy(alpha).cuda(), torch.from_numpy(rho).cuda(), torch.zeros(3, T, device="cuda")
+    saf.Context(0).saf_pattern_prepare(np.ones(3, dtype=np.uint8), a, r, z)
+    z = z.cpu().numpy().astype(np.float64)
+    assert not np.isfinite(z[:2, T - 9:]).any()
+    for h, n in ((0, T - 9), (1, T - 9), (2, T)):
+        finite = np.where(np.isneginf(alpha[h, :n]), -1e4, alpha[h, :n]).astype(np.float64)
+        assert np.abs(z[h, :n] - orc.pattern_logZ(finite, rho[h, :n], n)).max() <= 5e-6
+
+
+def test_rows_whose_largest_term_is_far_away_cost_two_more_passes():
+    """A sink of 90 on key 0 and decaying rho: every row is taken again relative to its own maximum, by the whole block."""
+    T, H = 4096, 3
+    mask, ctx = np.ones(H, dtype=np.uint8), saf.Context(0)
+    g = torch.Generator(device="cuda").manual_seed(1)
+    alpha = torch.randn((H, T), generator=g, device="cuda")
+    rho = -0.05 * torch.arange(T, device="cuda", dtype=torch.float32) + 0.1 * torch.randn((H, T), generator=g, device="cuda")
+    sink = alpha.clone()
+    sink[:, 0] += 90.0
+    z = torch.zeros(H, T, device="cuda")
+    us = {}
+    for name, a in (("flat", alpha), ("sink", sink)) * 3:
+        ctx.saf_pattern_prepare(mask, a, rho, z)
+        ctx.saf_set_profiling(1)
+        for _ in range(20):
+            ctx.saf_pattern_prepare(mask, a, rho, z)
+        torch.cuda.synchronize()
+        ms, n = ctx.saf_get_kernel_time(saf.SAF_KERNEL_LOGZ)
+        ctx.saf_set_profiling(0)
+        us[name] = min(us.get(name, 1e9), ms * 1e3 / n)
+    assert us["sink"] <= 4.0 * us["flat"], us            # (three passes instead of one)
+
+
 @pytest.mark.parametrize("T", [4, 130, 1028, 1030])
 def test_calibration_mean_pass(T):
     """Row lengths in whole 16-byte pieces and others; what lies above the diagonal stays as it was."""
