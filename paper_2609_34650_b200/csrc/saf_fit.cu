@@ -162,6 +162,7 @@ saf_fit_marginals_kernel(const float* __restrict__ Abar, float floor_v, double* 
 
 // ------------------------------------------------------------------------------------------------ Fit
 constexpr int FX = 256;            // x values of a block: 8 consecutive ones per lane
+constexpr int FPIECE = 64;         // terms of a chain of fp32 additions
 constexpr int FPAD = 288;          // floats kept neutral in front of A and behind A, R and W
 // Bounds (log2) inside which the product form is used: every factor and product of two stays within 2^+-120, sums of
 // 16384 of them below 2^127, so nothing overflows and nothing is flushed.
@@ -186,11 +187,9 @@ __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// 2^x of an fp64 exponent: the integer part goes into the exponent field, so the fp32 exponential sees |f| <= 1/2.
-__device__ __forceinline__ float exp2_split(double x) {
-  const double k = rint(x);
-  return ldexpf(ex2f(static_cast<float>(x - k)), static_cast<int>(k));
-}
+// 2^x of an fp64 exponent, rounded to fp32 once.  (The same A(j) and R(d) enter a whole row, column or diagonal of terms,
+// so that their own rounding does not average out: with ex2.approx of the fraction the loss was off by 1e-8.)
+__device__ __forceinline__ float exp2_f32(double x) { return static_cast<float>(exp2(x)); }
 
 // Layout of a vector in shared memory.  A lane reads 8 consecutive values plus a sliding window in 16-byte pieces, so
 // lanes are 32 bytes apart: PADDED inserts 16 bytes after every 32, which makes those reads conflict-free (lanes 48
@@ -221,9 +220,9 @@ __device__ __forceinline__ void fit_accumulate(const float* __restrict__ u0, con
     ld4(wp + fit_off<PADDED>(4), MODE == 0 ? win + 20 : win + 4);
   }
   for (int ye = y0; ye < y1;) {
-    // (pieces of 512 values of y are summed on their own, so that no chain of fp32 additions gets long)
+    // (pieces of FPIECE values of y are summed on their own, so that no chain of fp32 additions gets long)
     const int yb = ye;
-    ye = min(y1, yb + 512);
+    ye = min(y1, yb + FPIECE);
     float s0[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f}, s1[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll 2
     for (int y = yb; y < ye; y += 16) {
@@ -378,7 +377,7 @@ saf_fit_kernel(FitState s, int steps, const double* __restrict__ plogp, float* _
     const float r2 = static_cast<float>(r * LOG2E_D);
     mx = fmaxf(mx, r2);
     if (!(r2 >= R_LO && r2 <= R_HI)) bad = true;
-    R[d] = exp2_split(r * LOG2E_D);
+    R[d] = exp2_f32(r * LOG2E_D);
     A[fit_phys<PADDED>(d)] = 1.0f;
     // (each block's state is written and later read by its owner in pass B only, except for the fp64 parameters)
     const int k = d / FX, kr = k / static_cast<int>(cs), ki = k % static_cast<int>(cs);
@@ -434,7 +433,7 @@ saf_fit_kernel(FitState s, int steps, const double* __restrict__ plogp, float* _
       for (int q = tid; q < nb * FX; q += NT) {
         const int b = q / FX, i = i0 + b, x = p.xb[i] * FX + (q & (FX - 1));
         if (x >= T) continue;
-        float S = 0.0f;
+        double S = 0.0;
 #pragma unroll 4
         for (int w = p.lo[i]; w <= p.hi[i]; ++w) S += part[(w + b) * 2 * FX + (q & (FX - 1))];
         float* slot = W + fit_phys<PADDED>(x);
@@ -442,12 +441,12 @@ saf_fit_kernel(FitState s, int steps, const double* __restrict__ plogp, float* _
         double lz;
         bool in = true;
         if (slow) {
-          out = *slot - __log2f(S);
+          out = *slot - __log2f(static_cast<float>(S));
           lz = -static_cast<double>(out) * LN2_D;
         } else {
           in = S >= Z_LO && S <= Z_HI;
-          out = 1.0f / S;
-          lz = last ? log(static_cast<double>(S)) : 0.0;
+          out = static_cast<float>(1.0 / S);
+          lz = last ? log(S) : 0.0;
         }
         if (in) {
           const uint32_t a = smem_addr(slot);
@@ -529,11 +528,11 @@ saf_fit_kernel(FitState s, int steps, const double* __restrict__ plogp, float* _
         double* vv = (is_rho ? s.v_r : s.v_a) + o + x;
         const double eta = (is_rho ? s.eta_rel : s.eta_abs)[o + x];
         const double m0 = *mm, v0 = *vv, x_old = *par;
-        float S = 0.0f;
+        double S = 0.0;
 #pragma unroll 4
         for (int w = p.lo[i]; w <= p.hi[i]; ++w) S += part[(w + b) * 2 * FX + (q & (2 * FX - 1))];
         if (!slow) S *= is_rho ? R[x] : A[fit_phys<PADDED>(x)];
-        const double g = (static_cast<double>(S) - eta) * iT;
+        const double g = (S - eta) * iT;
         const double m = 0.9 * m0 + 0.1 * g;
         const double v = 0.999 * v0 + 0.001 * g * g;
         *mm = m;
@@ -541,7 +540,7 @@ saf_fit_kernel(FitState s, int steps, const double* __restrict__ plogp, float* _
         const double pnew = x_old - s.lr * (m * ib1) / (sqrt(v * ib2) + 1e-8);
         *par = pnew;
         const double e = pnew * LOG2E_D;
-        (is_rho ? s.r2 : s.a2)[o + x] = slow ? static_cast<float>(e) : exp2_split(e);
+        (is_rho ? s.r2 : s.a2)[o + x] = slow ? static_cast<float>(e) : exp2_f32(e);
         if (!slow && !(e >= (is_rho ? R_LO : A_LO) && e <= (is_rho ? R_HI : A_HI))) raise_flag(&out_par);
       }
     }
@@ -552,7 +551,10 @@ saf_fit_kernel(FitState s, int steps, const double* __restrict__ plogp, float* _
   const size_t oo = static_cast<size_t>(h) * static_cast<size_t>(out_stride);
   for (int k = static_cast<int>(rank) * NT + tid; k < T; k += static_cast<int>(cs) * NT) {
     const double a = __ldcg(s.alpha + o + k), r = __ldcg(s.rho + o + k);
-    acc -= s.eta_abs[o + k] * a + s.eta_rel[o + k] * r;
+    // L at the parameters as the sums saw them, to fp32: first-order in that rounding, log Z and the linear terms cancel
+    const float a32 = A[fit_phys<PADDED>(k)], r32 = R[k];
+    acc -= s.eta_abs[o + k] * (slow ? a32 * LN2_D : log(static_cast<double>(a32))) +
+           s.eta_rel[o + k] * (slow ? r32 * LN2_D : log(static_cast<double>(r32)));
     alpha_out[oo + k] = static_cast<float>(a);
     rho_out[oo + k] = static_cast<float>(r);
   }
