@@ -1,8 +1,10 @@
 """GPU parity of the compact-pattern fitter (target marginals, Fit, acceptance statistic) against the fp64 oracle.
 
-Tolerances.  The kernels take the exponentials in fp32 (ex2.approx: relative error about 2^-22 on top of an argument
-rounded at magnitudes up to ~60, i.e. a few 1e-6 relative per term) and accumulate what feeds Adam, and Adam itself,
-in fp64.  Marginals and normalisers are sums of positive terms, so they inherit that relative error: 2e-5 relative is
+Tolerances.  The kernels round the factors exp(alpha) and exp(rho) to fp32 once per step (2^-25 relative) and sum their
+products in fp32: chains of 64 terms, then the pieces of a warp (each chain of n positive terms rounds off up to n 2^-25,
+typically sqrt(n) times less), the warps' parts and Adam in fp64; heads that leave the product's range take one ex2.approx
+per term instead (2^-22, on an argument rounded at magnitudes up to ~60).  That is up to a few 1e-6 relative per
+sum.  Marginals and normalisers are sums of positive terms, so they inherit that relative error: 2e-5 relative is
 asserted.  Over the Adam steps the difference in the gradients (about 1e-6 relative) moves the parameters by far less
 than one step (0.05) each time; the asserted bound on alpha, rho after J steps is 2e-3 absolute for J <= 50 and
 2e-2 after 400 steps, with the quantities that do not depend on the path (loss, kappa: 1e-4 absolute) held tighter,
@@ -126,7 +128,7 @@ def test_fit_parity(T, steps, tol):
 
 
 def test_fit_long_sequence_two_steps():
-    """T beyond 4096: the pass kernels stage more than 48 KB of operands per CTA."""
+    """T beyond 4096, not a multiple of a block of 256 positions."""
     T = 5000
     A = si.mean_attention_maps(1, T, 31)
     P, ea, er, pl = _oracle_stats(A)
@@ -271,3 +273,23 @@ def test_fit_leaves_the_product_range(T, steps):
         want_z, _ = fo._logZ_and_P(a[h], r[h])
         assert np.max(np.abs(z[h] - want_z)) < 5e-4
         assert abs(loss[h] - fo.fit_objective(a[h], r[h], ea[h], er[h])) < 5e-4 * max(1.0, abs(loss[h]))
+
+
+def test_first_step_and_loss_keep_the_accuracy_of_their_terms():
+    """The first Adam step moves alpha by lr sign(g) / (1 + 1e-8 / |g|), so that small gradients show the rounding of the
+    column sums; at 40 heads a warp's chains are longest.  The loss at the returned parameters averages T normalisers, where
+    only what is common to them would remain.  Chains of 64 terms round off about sqrt(64/3) 2^-25 = 1.4e-7 of a sum (measured
+    3.7e-7 in alpha; 1.9e-6 with chains of 512); the loss is asserted at a quarter of the rounding 2^-25 that one fp32 factor
+    common to all rows would leave (measured 3e-9; 2e-8 with the factors' own rounding in it)."""
+    T, Hf = 4096, 40
+    base = si.mean_attention_maps(1, T, 40 + T)
+    P, ea, er, pl = _oracle_stats(base)
+    rep = lambda v: _dev(np.repeat(v, Hf, axis=0))
+    a, r, z, loss, kl = _gpu_fit(_ctx(), rep(ea), rep(er), rep(pl), 1)
+    wa, wr, wz = fo.fit_compact(ea[0], er[0], steps=1)
+    assert np.linalg.norm(a[0] - wa) <= 1e-6 * np.linalg.norm(wa)
+    A = si.mean_attention_maps(6, 512, 9)
+    P, ea, er, pl = _oracle_stats(A)
+    a, r, z, loss, kl = _gpu_fit(_ctx(), _dev(ea), _dev(er), _dev(pl), 400)
+    err = [loss[h] / fo.fit_objective(a[h], r[h], ea[h], er[h]) - 1.0 for h in range(6)]
+    assert np.sqrt(np.mean(np.square(err))) <= 2.0 ** -27, err
