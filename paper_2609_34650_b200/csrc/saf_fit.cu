@@ -280,9 +280,9 @@ struct FitPlan {
 };
 
 // One cluster = one head.  A head's x blocks go to the cluster's CTAs in snake order by descending work.  Bound: fp32
-// multiply-adds (128 per clock and SM), 1.5 T^2 per head and step.  Measured (36 heads, T = 4096, 400 steps): 22.3 ms =
-// 55 us per step on 108 SMs, against 100.2 ms for one exponential per pair and sum in two launches per step; the inner
-// loops run at 76 % of the multiply-add peak (148 heads: 64 % over everything).  One head of 256 positions: 5.4 us per
+// multiply-adds (128 per clock and SM), 1.5 T^2 per head and step.  Measured (36 heads, T = 4096, 400 steps): 23.4 ms =
+// 58 us per step on 108 SMs, against 100.2 ms for one exponential per pair and sum in two launches per step; the inner
+// loops run at 76 % of the multiply-add peak (148 heads: 64 % over everything).  One head of 256 positions: 6.0 us per
 // step (two cluster barriers, L2 round trips of the parameters, fp64 Adam).
 template <int NW, bool PADDED, int RB>
 __global__ void __launch_bounds__(NW * 32, 1)
@@ -626,6 +626,7 @@ cudaError_t launch_fit_clusters(const FitState& s, int Hf, cudaStream_t st, Args
   const size_t smem = fit_smem<NW, PADDED, RB>(s.T);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;
+  if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.blockDim = dim3(NW * 32);
   cfg.dynamicSmemBytes = smem;
@@ -637,12 +638,13 @@ cudaError_t launch_fit_clusters(const FitState& s, int Hf, cudaStream_t st, Args
   cfg.numAttrs = 1;
   // Cluster size: the shortest of (waves of clusters) x (a head's multiply-adds over its CTAs + a fixed cost per step).
   // Clusters stay inside a GPC, so fewer than 148 / size fit at once (measured with one CTA per SM: 74 of two, 45 of
-  // three, 33 of four, 26 of five, 22 of six, 15 of eight): 36 heads run faster on three CTAs each, in one wave, than
-  // on four.
+  // three, 33 of four, 26 of five, 22 of six, 15 of eight, 9 of ten, 7 of 12 to 16): 36 heads run faster on three CTAs each,
+  // in one wave, than on four.  Sizes above the portable eight are for few heads and long sequences: one head of 8192
+  // 44 us a step on 16 CTAs, 80 on 8 (51 with one exponential per pair on all SMs); of 16384 154 and 305.
   const int nxb = (s.T + FX - 1) / FX;
   double best = 0.0;
   int best_cs = 0;
-  for (int cs = 1; cs <= std::min(8, nxb); ++cs) {
+  for (int cs = 1; cs <= std::min(16, nxb); ++cs) {
     attr[0].val.clusterDim.x = cs;
     cfg.gridDim = dim3(static_cast<unsigned>(Hf) * cs);
     int n = 0;
@@ -667,11 +669,13 @@ cudaError_t launch_fit_clusters(const FitState& s, int Hf, cudaStream_t st, Args
 
 cudaError_t launch_fit(const FitState& s, int Hf, int steps, const double* plogp, float* alpha_out, float* rho_out,
                        float* logZ_out, long long out_stride, double* loss_out, double* kl_out, cudaStream_t st) {
-  // up to 8192 positions the padded vectors fit beside the partial sums of 16 warps; the longest sequences keep them
-  // unpadded (two-way bank conflicts on the window reads) and run 8 warps
+  // up to 8192 positions the padded vectors fit beside the partial sums of 16 warps, up to 12288 beside those of 12; the
+  // longest sequences keep them unpadded (two-way bank conflicts on the window reads)
   if (s.T <= 8192)
     return launch_fit_clusters<16, true, 16>(s, Hf, st, steps, plogp, alpha_out, rho_out, logZ_out, out_stride, loss_out, kl_out);
-  return launch_fit_clusters<8, false, 4>(s, Hf, st, steps, plogp, alpha_out, rho_out, logZ_out, out_stride, loss_out, kl_out);
+  if (s.T <= 12288)
+    return launch_fit_clusters<12, true, 2>(s, Hf, st, steps, plogp, alpha_out, rho_out, logZ_out, out_stride, loss_out, kl_out);
+  return launch_fit_clusters<12, false, 2>(s, Hf, st, steps, plogp, alpha_out, rho_out, logZ_out, out_stride, loss_out, kl_out);
 }
 
 }  // namespace saf

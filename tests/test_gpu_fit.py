@@ -246,8 +246,10 @@ def test_fit_no_heads_and_bad_arguments():
 
 
 # One launch per call: a cluster of CTAs per head.  Edges: blocks of 256 positions (one, two, a partial one), more heads
-# than clusters fit at once, the longest sequences (vectors kept unpadded), two to eight CTAs per cluster.
-@pytest.mark.parametrize("Hf,T,steps", [(1, 255, 3), (2, 257, 3), (1, 2304, 2), (150, 272, 2), (40, 300, 2), (1, 10300, 1)])
+# than clusters fit at once, two to sixteen CTAs per cluster, and the longest sequences (12 warps instead of 16 beyond 8192
+# positions, vectors kept unpadded beyond 12288).
+@pytest.mark.parametrize("Hf,T,steps", [(1, 255, 3), (2, 257, 3), (1, 2304, 2), (150, 272, 2), (40, 300, 2), (1, 10300, 1),
+                                        (1, 12289, 1), (16, 1500, 2)])
 def test_fit_cluster_edges(Hf, T, steps):
     base = si.mean_attention_maps(1, T, 40 + T)
     P, ea, er, pl = _oracle_stats(base)
@@ -293,3 +295,23 @@ def test_first_step_and_loss_keep_the_accuracy_of_their_terms():
     a, r, z, loss, kl = _gpu_fit(_ctx(), _dev(ea), _dev(er), _dev(pl), 400)
     err = [loss[h] / fo.fit_objective(a[h], r[h], ea[h], er[h]) - 1.0 for h in range(6)]
     assert np.sqrt(np.mean(np.square(err))) <= 2.0 ** -27, err
+
+
+def test_a_single_long_head_spreads_over_more_than_eight_sms():
+    """Twice the length is four times the multiply-adds beside the fixed costs of a step; on eight CTAs, the largest portable
+    cluster, they take over (a factor of 3.2 from 4096 to 8192 positions), on sixteen not yet."""
+    us = {}
+    for T in (4096, 8192):
+        g = torch.Generator(device="cuda").manual_seed(T)
+        eta = torch.rand((1, T), generator=g, device="cuda", dtype=torch.float64) * 2.0
+        o = [torch.empty((1, T), device="cuda") for _ in range(3)]
+        one = torch.zeros(1, device="cuda", dtype=torch.float64)
+        ctx = saf.Context(0)
+        for _ in range(4):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            ctx.saf_fit_compact(1, T, eta, eta, one, 50, 0.05, *o, T, one.clone(), one.clone())
+            b.record()
+            torch.cuda.synchronize()
+            us[T] = min(us.get(T, 1e9), a.elapsed_time(b) * 20.0)
+    assert us[8192] <= 2.5 * us[4096], us                # measured 22.8 and 44.4 us a step; on eight SMs 25.4 and 80.4
