@@ -183,6 +183,7 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
         uint32_t n = 0;                            // ring position
         uint32_t nq0 = 0, nq1 = 0;                 // uses of the two Q areas
         bool ok = true;
+        bool drop_load = p.selftest_drop_load != 0;   // (see FwdParams)
         // Claim the next item of the queue and publish it to the other roles.  Claimed CLAIM_AHEAD tiles before the current
         // item's last, but behind the loads of its first two: the claim's global round trips and the loads of Q_0 and K_0
         // behind it then fit under the tiles that are left (claimed behind the item's last load they cost ~13000 clk an item).
@@ -227,10 +228,14 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
             const uint32_t s = n % C::NS;
             ok = mbar_wait_compact(kv_empty + s, ((n / C::NS) & 1) ^ 1, wc, SITE_KV_EMPTY);
             if (!ok) return;
+            ++n;
+            if (drop_load) {
+              drop_load = false;
+              return;
+            }
             mbar_expect_tx(kv_full + s, C::TILE_BYTES);
             for (int pn = 0; pn < C::NPANEL; ++pn)
               tma_load_4d(smem + C::OFF_KV + s * C::TILE_BYTES + pn * C::PANEL_BYTES, m, kv_full + s, pn * 64, j * BLK, head, b);
-            ++n;
           };
           if (fast) {
             // tensor-core form: per tile the scaled V tile and the Hankel bands of distance blocks q1 - J, q1 - 1 - J
@@ -292,6 +297,7 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
             ++nq1;
             for (int j = 0; j < n1 && ok; ++j) load_kv(&mv, j, hv);
           }
+          if (!ok) break;                            // (a given-up item is the last: its tile sequence is broken)
         }
       }
     } else if (warp == 13) {

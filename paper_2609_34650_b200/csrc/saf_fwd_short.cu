@@ -118,6 +118,7 @@ saf_fwd_short_kernel(const __grid_constant__ CUtensorMap mq, const __grid_consta
       tma_prefetch_desc(&mvt);
       uint32_t nq = 0, nk = 0, nv = 0;
       bool ok = true;
+      bool drop_load = p.selftest_drop_load != 0;   // (see FwdParams)
       for (int it = it_begin; it < it_end && ok; ++it) {
         const WorkItem w = p.items[it];
         const int ntiles = w.blk + 1;
@@ -153,10 +154,13 @@ saf_fwd_short_kernel(const __grid_constant__ CUtensorMap mq, const __grid_consta
           if (w.kind == KIND_ORDINARY) {
             ok = mbar_wait(k_empty, (nk & 1) ^ 1, wc, SITE_K_EMPTY);
             if (!ok) break;
-            mbar_expect_tx(k_full, C::TILE_BYTES);
-            for (int pn = 0; pn < C::NPANEL; ++pn)
-              tma_load_4d(smem + C::OFF_K + pn * C::PANEL_BYTES, &mk, k_full, pn * 64,
-                          j * BLK, p.qslot ? p.qslot[w.h] : w.h / p.kv_group, w.b);
+            if (!drop_load) {
+              mbar_expect_tx(k_full, C::TILE_BYTES);
+              for (int pn = 0; pn < C::NPANEL; ++pn)
+                tma_load_4d(smem + C::OFF_K + pn * C::PANEL_BYTES, &mk, k_full, pn * 64, j * BLK,
+                            p.qslot ? p.qslot[w.h] : w.h / p.kv_group, w.b);
+            }
+            drop_load = false;
             ++nk;
           }
           ok = mbar_wait(v_empty, (nv & 1) ^ 1, wc, SITE_V_EMPTY);

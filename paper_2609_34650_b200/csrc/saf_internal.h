@@ -88,8 +88,8 @@ struct FwdParams {
   int* queue;
   int* status;                      // device status word
   unsigned long long wait_limit_ns;
-  // Self-test of the give-up path (0 in normal use): the producer of the D = 64 forward leaves out the load of the
-  // first key tile of its first ordinary item, so that the waits for it run out.  Set by saf_create from
+  // Self-test of the give-up path (0 in normal use): the producer leaves out the load of the first key tile of its first
+  // ordinary item, so that the waits for it run out.  Set by saf_create from
   // SAF_SELFTEST_DROP_LOAD, and only for grids of at most 16 CTAs with a wait limit of at most 50 ms.
   int selftest_drop_load;
 };

@@ -43,6 +43,33 @@ def test_a_wait_that_runs_out_is_reported_and_the_context_stays_usable(monkeypat
     check_units(fresh, all_units(inp.wl))
 
 
+@pytest.mark.parametrize("D,H,T,sites", [
+    (128, 4, 256, range(101, 111)),      # one query block per item (8 items)
+    (96, 3, 520, range(1, 12)),          # the kernel of the longer sequences (15 items of up to five tiles: the producer's
+    (128, 3, 520, range(1, 12)),         # ring runs full, so its own wait gives up as well)
+])
+def test_a_wait_that_runs_out_in_the_wide_forwards(monkeypatch, D, H, T, sites):
+    """The same at head dimensions 96 and 128, in both kernels."""
+    monkeypatch.setenv("SAF_WAIT_LIMIT_MS", "20")
+    monkeypatch.setenv("SAF_SELFTEST_DROP_LOAD", "1")
+    ctx = saf.Context(0)
+    monkeypatch.delenv("SAF_SELFTEST_DROP_LOAD")
+    monkeypatch.delenv("SAF_WAIT_LIMIT_MS")
+    inp = si.generate(si.Workload("drop", 1, H, T, D, (1,), -0.05, seed=D + T))
+    L = Layer(inp, ctx=ctx, backward=False)
+    ctx.saf_pattern_prepare(L.mask, L.alpha, L.rho, L.logZ)
+    ctx.saf_hybrid_attn_fwd(L.prob, L.Q, L.K, L.V, L.mask, L.alpha, L.rho, L.logZ, L.O, L.LSE)
+    torch.cuda.synchronize()
+    code, detail = ctx.saf_last_device_status()
+    assert code == saf.SAF_ERR_DEVICE_TIMEOUT, (code, hex(detail))
+    assert (detail >> 24) & 0xFF == DEV_TIMEOUT and (detail >> 16) & 0xFF in sites, hex(detail)
+    assert (detail & 0xFFFF) < 16
+    code, detail = ctx.saf_last_device_status()
+    assert code == saf.SAF_OK and detail == 0
+    fresh = Layer(inp).run()
+    check_units(fresh, all_units(inp.wl))
+
+
 def test_vectors_rewritten_in_place_do_not_meet_stale_tables():
     """saf_pattern_prepare builds tensor-core tables and remembers the device pointers.  When alpha is then changed in
     place and only the normalisers are refreshed (by the entry point that has no context), the next layer call gets the
