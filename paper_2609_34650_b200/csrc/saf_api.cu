@@ -35,6 +35,7 @@ struct WorklistEntry {
 struct DevBuf {
   void* ptr = nullptr;
   size_t bytes = 0;
+  bool fresh = false;       // allocated (or left in doubt) and not yet initialised by whoever relies on its contents
 };
 
 // Which (alpha, rho, logZ) the context's tensor-core pattern tables were built from.
@@ -114,6 +115,14 @@ int ensure(DevBuf& b, size_t bytes) {
     return SAF_ERR_NOMEM;
   }
   b.bytes = bytes;
+  b.fresh = true;
+  return SAF_OK;
+}
+// Buffers that kernels expect at zero and leave at zero.
+int zero_if_fresh(DevBuf& b, cudaStream_t st) {
+  if (!b.fresh) return SAF_OK;
+  if (cudaMemsetAsync(b.ptr, 0, b.bytes, st) != cudaSuccess) return SAF_ERR_CUDA;
+  b.fresh = false;
   return SAF_OK;
 }
 void release(DevBuf& b) {
@@ -582,7 +591,6 @@ int saf_pattern_prepare(saf_ctx* ctx, int32_t H, int32_t Tp, const uint8_t* froz
   const size_t vecb = static_cast<size_t>(H) * Tp * sizeof(float);
   const size_t bandb = static_cast<size_t>(H) * nblkp * 4096;
   const size_t hb = static_cast<size_t>(std::max(H, 64)) * sizeof(int);
-  const size_t marks_before = ctx->pat_marks.bytes, heads_before = ctx->pat_heads.bytes;
   if ((rc = ensure(ctx->pat_consts, 2 * hb)) || (rc = ensure(ctx->pat_ok, hb)) || (rc = ensure(ctx->pat_avec, vecb)) ||
       (rc = ensure(ctx->pat_wvec, vecb)) || (rc = ensure(ctx->pat_bandf, bandb)) ||
       (rc = ensure(ctx->pat_bandb, bandb)) || (rc = ensure(ctx->pat_heads, 2 * hb)) || (rc = ensure(ctx->pat_snap, 3 * vecb)) ||
@@ -590,10 +598,7 @@ int saf_pattern_prepare(saf_ctx* ctx, int32_t H, int32_t Tp, const uint8_t* froz
     return rc;
   // A new buffer starts at zero: the counters of the normaliser kernel (which returns them to zero) and the per-head overflow
   // marks of the forward / backward staging kernels (the id of the call that set one; the table kernel clears them).
-  if (ctx->pat_heads.bytes != heads_before) ctx->pat_heads_host.clear();
-  if (ctx->pat_marks.bytes != marks_before) {
-    if (cudaMemsetAsync(ctx->pat_marks.ptr, 0, ctx->pat_marks.bytes, st) != cudaSuccess) return SAF_ERR_CUDA;
-  }
+  if ((rc = zero_if_fresh(ctx->pat_marks, st))) return rc;
   // ordinals of the frozen heads, uploaded when the mask (or the stream) is another one: hord[H], then hlist
   std::vector<int> heads(2 * static_cast<size_t>(H), 0);
   for (int h = 0, ord = 0; h < H; ++h) {
@@ -603,14 +608,15 @@ int saf_pattern_prepare(saf_ctx* ctx, int32_t H, int32_t Tp, const uint8_t* froz
       heads[h] = ord++;
     }
   }
-  if (heads != ctx->pat_heads_host || ctx->pat_heads_stream != st) {
+  // (or the buffer is a new one, possibly since a call that then failed to get another buffer)
+  if (ctx->pat_heads.fresh || heads != ctx->pat_heads_host || ctx->pat_heads_stream != st) {
+    ctx->pat_heads.fresh = true;
     ctx->pat_heads_host = heads;
     ctx->pat_heads_stream = st;
     if (cudaMemcpyAsync(ctx->pat_heads.ptr, ctx->pat_heads_host.data(), heads.size() * sizeof(int), cudaMemcpyHostToDevice,
-                        st) != cudaSuccess) {
-      ctx->pat_heads_host.clear();
+                        st) != cudaSuccess)
       return SAF_ERR_CUDA;
-    }
+    ctx->pat_heads.fresh = false;
   }
   {
     ScopedTimer timer(ctx, SAF_KERNEL_LOGZ, st);
@@ -620,8 +626,10 @@ int saf_pattern_prepare(saf_ctx* ctx, int32_t H, int32_t Tp, const uint8_t* froz
         launch_pattern_tables(alpha_dev, rho_dev, logZ_dev_out, static_cast<const uint8_t*>(ctx->mask_buf.ptr), H, Tp, consts,
                               static_cast<float*>(ctx->pat_avec.ptr), static_cast<float*>(ctx->pat_wvec.ptr),
                               ctx->pat_bandf.ptr, ctx->pat_bandb.ptr, static_cast<uint32_t*>(ctx->pat_snap.ptr),
-                              ctx->pat_mark(0), ctx->pat_mark(1), st) != cudaSuccess)
+                              ctx->pat_mark(0), ctx->pat_mark(1), st) != cudaSuccess) {
+      ctx->pat_marks.fresh = true;
       return SAF_ERR_CUDA;
+    }
   }
   ctx->pat.valid = true;
   ctx->pat.alpha = alpha_dev;
@@ -1351,15 +1359,14 @@ int saf_calib_finalize(saf_ctx* ctx, int32_t H, int32_t T, int64_t n_total, floa
   if (!g.ok) return SAF_ERR_CUDA;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   ctx->last_stream = st;
-  const size_t tmp_before = ctx->calib_tmp.bytes;
   int rc = ensure(ctx->calib_tmp, static_cast<size_t>(H) * 2 * sizeof(double));
-  if (rc) return rc;
-  if (ctx->calib_tmp.bytes != tmp_before && cudaMemsetAsync(ctx->calib_tmp.ptr, 0, ctx->calib_tmp.bytes, st) != cudaSuccess)
-    return SAF_ERR_CUDA;
+  if (rc || (rc = zero_if_fresh(ctx->calib_tmp, st))) return rc;
   ScopedTimer timer(ctx, SAF_KERNEL_CALIB_FINALIZE, st);
   if (launch_calib_finalize(mean_inout, sumsq, sum_plogp, static_cast<double*>(ctx->calib_tmp.ptr), H, T,
-                            static_cast<double>(n_total), s_var_out, s_kl_out, ctx->num_sms, st) != cudaSuccess)
+                            static_cast<double>(n_total), s_var_out, s_kl_out, ctx->num_sms, st) != cudaSuccess) {
+    ctx->calib_tmp.fresh = true;
     return SAF_ERR_CUDA;
+  }
   return SAF_OK;
 }
 

@@ -124,3 +124,24 @@ def test_a_preparation_ends_the_overflow_marks_of_recorded_calls(D):
         L.dO.copy_(keep[1])
         L.ctx.saf_pattern_prepare(L.mask, L.alpha, L.rho, L.logZ)
         assert all(replay())
+
+
+def test_a_preparation_that_runs_out_of_memory_leaves_the_context_usable():
+    """Larger tables are asked for while the device is full: some buffers are new by then and hold nothing.  Going back to
+    the earlier pattern has to fill them again."""
+    inp = si.generate(si.Workload("oom", 1, 4, 300, 64, (1, 2), -0.05, seed=5))
+    L = Layer(inp).run()
+    H, Tp = 2048, 4096                                   # 32 MB a vector: 600 MB of tables before the last 96 MB
+    big = [torch.zeros((H, Tp), device="cuda") for _ in range(3)]
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    hold = torch.empty(torch.cuda.mem_get_info()[0] - (650 << 20), device="cuda", dtype=torch.uint8)
+    with pytest.raises(saf.SafError) as e:
+        L.ctx.saf_pattern_prepare(np.ones(H, dtype=np.uint8), *big)
+    assert e.value.code == saf.SAF_ERR_NOMEM
+    del hold, big
+    torch.cuda.empty_cache()
+    for t in (L.O, L.LSE, *L.grads):
+        t.fill_(float("nan"))
+    L.run()
+    check_units(L, all_units(inp.wl))
