@@ -296,36 +296,34 @@ void build_worklist_host(int B, int H, int T, const uint8_t* mask, int backward,
 
 // Work queue of the 128-wide forward, whose items are two consecutive query blocks of one (batch, head) unit (the first
 // block of an odd count goes alone).  CTAs claim items in this order at run time, so longest-first within groups of
-// units keeps both the tail short and a group's K and V in L2 while its items run.  Groups are of equal size (a small last
-// group is a tail of long items: 2x16x8192x96 0.456 ms with groups of 10, 10, 10 and 2 units, 0.373 with two of 16) and
-// hold at most 64 MB of K and V (8x12x4096x128: 32 MB 0.335 ms, 64 MB 0.339, 128 MB 0.346; 1x16x16384x128: 0.778, 0.760,
-// 0.758).  While the items would not fill the SMs, blocks go one by one: a pair takes longer than a
-// single block and there are SMs to spare.
-void build_pair_order(int B, int H, int T, int D, const uint8_t* mask, int num_sms, std::vector<WorkItem>& order) {
+// units keeps both the tail short and a group's K and V in L2 while its items run.  Group sizes differ by at most one unit (a
+// small last group is a tail of long items: 2x16x8192x96 0.456 ms with groups of 10, 10, 10 and 2 units, 0.373 with two of 16),
+// as many groups as hold 64 MB of K and V each (8x12x4096x128: 32 MB 0.335 ms, 64 MB 0.339, 128 MB 0.346; 1x16x16384x128:
+// 0.778, 0.760, 0.758), K and V counted per query head where heads share them.  While the items would not fill the SMs,
+// blocks go one by one: a pair takes longer than a single block and there are SMs to spare.  An item's fixed cost does not
+// change the order; a frozen tile counts frozen_pct percent of an ordinary one.
+void build_pair_order(int B, int H, int T, int D, const uint8_t* mask, int num_sms, int frozen_pct, std::vector<WorkItem>& order) {
   const int nblk = (T + BLK - 1) / BLK;
-  const bool pair = static_cast<long long>(B) * H * nblk > num_sms;
-  const long long unit_bytes = static_cast<long long>(T) * D * 4;
-  const long long n_groups = std::max<long long>(1, (unit_bytes * B * H + (64ll << 20) - 1) / (64ll << 20));
-  const int group = static_cast<int>((static_cast<long long>(B) * H + n_groups - 1) / n_groups);
+  const long long units = static_cast<long long>(B) * H;
+  const bool pair = units * nblk > num_sms;
+  const long long n_groups = std::min(units, std::max<long long>(1, (static_cast<long long>(T) * D * 4 * units + (64ll << 20) - 1) / (64ll << 20)));
   order.clear();
   std::vector<std::pair<long long, WorkItem>> items;
-  auto flush = [&] {
-    std::stable_sort(items.begin(), items.end(),
-                     [](const std::pair<long long, WorkItem>& a, const std::pair<long long, WorkItem>& b) { return a.first > b.first; });
-    for (const auto& it : items) order.push_back(it.second);
+  for (long long g = 0; g < n_groups; ++g) {
     items.clear();
-  };
-  for (int u = 0; u < B * H; ++u) {
-    const int b = u / H, h = u % H;
-    const int kind = mask[h] ? KIND_FROZEN : KIND_ORDINARY;
-    for (int q = nblk - 1; q >= 0; q -= pair ? 2 : 1) {
-      const bool two = pair && q > 0;
-      const long long tiles = two ? 2 * q + 1 : q + 1;
-      items.push_back({(mask[h] ? 50 : 100) * tiles + 100, WorkItem{b, h, q, kind | (two ? KIND_PAIR : 0)}});
+    for (long long u = units * g / n_groups; u < units * (g + 1) / n_groups; ++u) {
+      const int b = static_cast<int>(u / H), h = static_cast<int>(u % H);
+      const int kind = mask[h] ? KIND_FROZEN : KIND_ORDINARY;
+      for (int q = nblk - 1; q >= 0; q -= pair ? 2 : 1) {
+        const bool two = pair && q > 0;
+        const long long tiles = two ? 2 * q + 1 : q + 1;
+        items.push_back({(mask[h] ? frozen_pct : 100) * tiles, WorkItem{b, h, q, kind | (two ? KIND_PAIR : 0)}});
+      }
     }
-    if ((u + 1) % group == 0) flush();
+    std::stable_sort(items.begin(), items.end(),
+                     [](const std::pair<long long, WorkItem>& x, const std::pair<long long, WorkItem>& y) { return x.first > y.first; });
+    for (const auto& it : items) order.push_back(it.second);
   }
-  flush();
 }
 
 // Whether a 128-wide forward goes to the kernel of short sequences (one query block per item, two CTAs per SM).  The line
@@ -379,7 +377,7 @@ int get_worklist(saf_ctx* ctx, int B, int H, int T, int D, const uint8_t* mask, 
   const bool lists = kind != WL_QUEUE;
   WorklistEntry e;
   if (!lists && wide) {
-    build_pair_order(B, H, T, D, mask, ctx->num_sms, e.items_host);
+    build_pair_order(B, H, T, D, mask, ctx->num_sms, frozen_pct, e.items_host);
   } else {
     // (tail: two items per CTA; on the 128-wide backward four: -0.5 % on 8x12x4096x128, -1 % on 2x16x8192x96, -3 % on
     // 1x16x8192x128 and on shared heads 3x8x3000x128; six and eight are no better)
