@@ -921,8 +921,6 @@ saf_bwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
   if (warp == 21) tmem_dealloc(tmem, C::TMEM_COLS);
 }
 
-int bwd_smem_bytes(int) { return BwdCfg::SMEM; }
-
 cudaError_t launch_bwd(int D, const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv,
                        const CUtensorMap& mdo, const CUtensorMap& mdq, const CUtensorMap& mdot, const CUtensorMap& mdk,
                        const CUtensorMap& mdv, const BwdParams& p, int grid, cudaStream_t st) {

@@ -648,8 +648,6 @@ saf_bwd128_kernel(const __grid_constant__ CUtensorMap mk, const __grid_constant_
   if (warp == 25) tmem_dealloc(tmem, C::TMEM_COLS);
 }
 
-int bwd128_smem_bytes() { return W128::SMEM; }
-
 cudaError_t launch_bwd128(const CUtensorMap& mk, const CUtensorMap& mv, const CUtensorMap& mq, const CUtensorMap& mdo,
                           const CUtensorMap& mdot, const CUtensorMap& mdq, const BwdParams& p, int grid,
                           cudaStream_t st) {

@@ -412,7 +412,6 @@ __global__ void saf_calib_scores_kernel(const double* __restrict__ sumsq, const 
 
 }  // namespace
 
-int calib_smem_bytes(int D) { return D == 64 ? CalCfg<64>::SMEM : CalCfg<128>::SMEM; }
 
 template <int D, bool ACC>
 static cudaError_t launch_calib_t(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mm,

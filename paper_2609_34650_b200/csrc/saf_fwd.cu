@@ -53,8 +53,8 @@ namespace {
 constexpr float LOG2E_F = 1.4426950408889634f;
 constexpr float LN2_F = 0.6931471805599453f;
 
-template <int D>
 struct FwdCfg {
+  static constexpr int D = 128;                         // (96 runs here with features 96..127 zero-filled by TMA)
   static constexpr int NPANEL = D / 64;                 // 64-column bf16 panels: 128-byte rows, one swizzle atom
   static constexpr int PANEL_BYTES = 128 * 64 * 2;      // 16 KB
   static constexpr int TILE_BYTES = NPANEL * PANEL_BYTES;
@@ -87,11 +87,10 @@ struct ItemView {
   bool fast;
 };
 
-template <int NRING>
 __device__ __forceinline__ bool ring_take(const int4* ring, uint64_t* ring_full, uint64_t* ring_empty, uint32_t n,
                                           const WaitCtx& wc, ItemView& v) {
-  const uint32_t slot = n % NRING;
-  if (!mbar_wait_warp_compact(ring_full + slot, (n / NRING) & 1, wc, SITE_RING_FULL)) return false;
+  const uint32_t slot = n % FwdCfg::NRING;
+  if (!mbar_wait_warp_compact(ring_full + slot, (n / FwdCfg::NRING) & 1, wc, SITE_RING_FULL)) return false;
   const int4 raw = ring[slot];
   warp_arrive(ring_empty + slot);
   v.b = raw.x;
@@ -106,11 +105,11 @@ __device__ __forceinline__ bool ring_take(const int4* ring, uint64_t* ring_full,
 
 }  // namespace
 
-template <int D>
-__global__ void __launch_bounds__(512, 1)
+__global__ void __launch_bounds__(FwdCfg::NTHREADS, 1)
 saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ CUtensorMap mk,
                const __grid_constant__ CUtensorMap mv, const __grid_constant__ CUtensorMap mvt, const FwdParams p) {
-  using C = FwdCfg<D>;
+  using C = FwdCfg;
+  constexpr int D = C::D;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::OFF_BAR);
@@ -358,7 +357,7 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
       };
       bool early = false;                          // block 0's first scores of `cur` are already issued
       ItemView cur;
-      bool ok = ring_take<C::NRING>(ring, ring_full, ring_empty, nrec++, wc, cur);
+      bool ok = ring_take(ring, ring_full, ring_empty, nrec++, wc, cur);
       while (ok && cur.kind != RING_END) {
         ItemView nxt;
         bool have_next = false;
@@ -434,7 +433,7 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
                 __syncwarp();
                 if (ord && t == 0) {
                   // block 0 is through: its first scores of the next item go out now
-                  ok = ring_take<C::NRING>(ring, ring_full, ring_empty, nrec++, wc, nxt);
+                  ok = ring_take(ring, ring_full, ring_empty, nrec++, wc, nxt);
                   if (!ok) break;
                   have_next = true;
                   if (nxt.kind == KIND_ORDINARY && nxt.n0 > 0) {
@@ -465,7 +464,7 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
         }
         if (!ok) break;
         if (have_next) cur = nxt;
-        else ok = ring_take<C::NRING>(ring, ring_full, ring_empty, nrec++, wc, cur);
+        else ok = ring_take(ring, ring_full, ring_empty, nrec++, wc, cur);
       }
     }
   } else if (warp < 8) {
@@ -483,7 +482,7 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
     // agreement barrier, where its four leave together; none is ever left alone at a barrier.
     for (uint32_t nrec = 0;; ++nrec) {
       ItemView w;
-      if (!ring_take<C::NRING>(ring, ring_full, ring_empty, nrec, wc, w)) {
+      if (!ring_take(ring, ring_full, ring_empty, nrec, wc, w)) {
         ok = false;
         w.kind = KIND_ORDINARY; w.n0 = w.n1 = 0; w.fast = false; w.b = w.h = w.blk = 0;
       }
@@ -701,7 +700,7 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
     bool ok = true;
     for (uint32_t nrec = 0; ok; ++nrec) {
       ItemView w;
-      ok = ring_take<C::NRING>(ring, ring_full, ring_empty, nrec, wc, w);
+      ok = ring_take(ring, ring_full, ring_empty, nrec, wc, w);
       if (!ok || w.kind == RING_END) break;
 #pragma unroll 1
       for (int t = 0; t < 2 && ok; ++t) {
@@ -782,14 +781,12 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
   }
 }
 
-int fwd_smem_bytes(int D) { return D == 64 ? fwd64_smem_bytes() : FwdCfg<128>::SMEM; }
-
 cudaError_t launch_fwd(int D, const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv,
                        const CUtensorMap& mvt, const CUtensorMap& mo, const FwdParams& p, int grid, cudaStream_t st) {
   if (D == 64) return launch_fwd64(mq, mk, mv, mvt, mo, p, grid, st);   // head dimension 64 has its own kernel
-  cudaError_t e = cudaFuncSetAttribute(saf_fwd_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdCfg<128>::SMEM);
+  cudaError_t e = cudaFuncSetAttribute(saf_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdCfg::SMEM);
   if (e != cudaSuccess) return e;
-  return launch_pdl(PDL_FWD128, saf_fwd_kernel<128>, dim3(grid), dim3(FwdCfg<128>::NTHREADS), FwdCfg<128>::SMEM, st, mq, mk, mv,
+  return launch_pdl(PDL_FWD128, saf_fwd_kernel, dim3(grid), dim3(FwdCfg::NTHREADS), FwdCfg::SMEM, st, mq, mk, mv,
                     mvt, p);
 }
 

@@ -787,8 +787,6 @@ saf_fwd64_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
   }
 }
 
-int fwd64_smem_bytes() { return Fwd64Cfg::SMEM; }
-
 // Early launch (under the tail of the kernel before): the CTAs then land on the SMs in the order in which these become free,
 // so that long items meet on one SM.  Where a CTA gets one or two items in all, that costs more than the launch gap
 // (forwards back to back, early / not: 1x12x3072x64 45.3 / 36.2 us, 1x8x4096x64 54.4 / 44.2, 2x12x2048x64 33.2 / 29.2);

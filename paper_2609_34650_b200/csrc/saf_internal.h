@@ -210,7 +210,6 @@ cudaError_t launch_bwd_finalize(const float* dQacc, void* dQ, size_t n, cudaStre
 // head dimension 64 (saf_fwd64.cu); launch_fwd dispatches to it
 cudaError_t launch_fwd64(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv, const CUtensorMap& mvt,
                          const CUtensorMap& mo, const FwdParams& p, int grid, cudaStream_t st);
-int fwd64_smem_bytes();
 // head dimension 128 / 96, short sequences (saf_fwd_short.cu)
 cudaError_t launch_fwd_short(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv, const CUtensorMap& mvt,
                              const FwdParams& p, int grid, cudaStream_t st);
@@ -220,9 +219,6 @@ cudaError_t launch_fwd_short(const CUtensorMap& mq, const CUtensorMap& mk, const
 cudaError_t launch_bwd128(const CUtensorMap& mk, const CUtensorMap& mv, const CUtensorMap& mq, const CUtensorMap& mdo,
                           const CUtensorMap& mdot, const CUtensorMap& mdq, const BwdParams& p, int grid,
                           cudaStream_t st);
-int bwd128_smem_bytes();
-int fwd_smem_bytes(int D);
-int bwd_smem_bytes(int D);
 
 // compact-pattern fitter (saf_fit.cu): per-head state of Fit, all arrays [Hf, T]
 struct FitState {
