@@ -334,11 +334,12 @@ void build_pair_order(int B, int H, int T, int D, const uint8_t* mask, int num_s
 //   up to ten: while the blocks are: 1x32x640x128, one forward waited for, 34.4 / 36.8
 bool fwd_is_short(int B, int H, int T, int D, int num_sms) {
   const long long units = static_cast<long long>(B) * H, nblk = (T + BLK - 1) / BLK, blocks = units * nblk;
+  if (blocks <= num_sms) return false;                    // (one block per CTA and SM either way, and the same time)
   if (nblk <= 2) return true;
   if (nblk == 3) return blocks <= (D == 96 ? 8LL : 4LL) * num_sms;
   const long long items = units * ((nblk + 1) / 2);       // of the two-block kernel
   if (nblk <= 6 && items > num_sms && 5 * items <= 8LL * num_sms) return true;
-  return nblk <= 10 && blocks > num_sms && 10 * blocks <= 13LL * num_sms;
+  return nblk <= 10 && 10 * blocks <= 13LL * num_sms;
 }
 
 // Measured cost-model defaults: `wide` = the 128-wide kernels (head dimension 96 or 128), else the 64-wide ones.

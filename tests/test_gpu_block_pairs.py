@@ -15,28 +15,30 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("B,H,T,D,frozen", [
-    # one query block per item, two CTAs per SM
+    # at most one block per SM: one query block per item, one CTA per SM
     (1, 4, 128, 128, (1,)),             # one block
     (1, 3, 129, 96, (0,)),              # two blocks
-    (5, 10, 257, 128, (1, 4, 7)),       # three blocks, 150 items
+    (1, 4, 520, 128, (1,)),             # five blocks
+    # one query block per item, two CTAs per SM
     (10, 16, 100, 128, (3,)),           # 160 one-block units
+    (10, 9, 200, 96, (1, 4)),           # two blocks, 180 items
+    (5, 10, 257, 128, (1, 4, 7)),       # three blocks, 150 items
     (16, 12, 300, 128, (2, 3)),         # the most three-block units that go there (576 blocks on 148 SMs)
     (12, 8, 512, 96, (0, 5)),           # four blocks: 192 two-block items would be a wave and a little
     (1, 32, 640, 128, (7,)),            # 160 blocks
     # two query blocks per item, one CTA per SM
-    (1, 4, 520, 128, (1,)),             # five blocks, one by one (fewer than the SMs)
     (4, 10, 520, 96, (0, 5, 9)),        # 200 blocks: pairs, the first block of an odd count alone
     (17, 12, 300, 128, (1, 4)),         # one more batch entry than above: a pair and a single block per unit
     (4, 10, 768, 128, (2, 3)),          # pairs of every length up to six tiles
 ])
 def test_item_shapes_of_the_wide_forward(B, H, T, D, frozen):
-    """Both kernels of head dimensions 96 and 128 on either side of the line between them."""
+    """Both kernels of head dimensions 96 and 128 on either side of the lines between them."""
     inp = si.generate(si.Workload("items", B, H, T, D, frozen, -0.05, seed=T + D))
     units = all_units(inp.wl)
     check_units(Layer(inp).run(), units if len(units) <= 50 else sampled_units(inp.wl, 24, seed=5))
 
 
-@pytest.mark.parametrize("B,H,T", [(2, 2, 384), (4, 12, 640)])
+@pytest.mark.parametrize("B,H,T", [(4, 13, 384), (4, 12, 640)])
 def test_running_maximum_far_above_the_first_tile(B, H, T):
     """Scores that grow along the sequence: the rescaling of the accumulator between tiles, in the one-block kernel and in
     both blocks of a pair (240 blocks: more than the one-block items that are tried first, so they are paired)."""
