@@ -788,14 +788,18 @@ saf_fwd64_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
 }
 
 // Early launch (under the tail of the kernel before): the CTAs then land on the SMs in the order in which these become free,
-// so that long items meet on one SM.  Where a CTA gets one or two items in all, that costs more than the launch gap
-// (forwards back to back, early / not: 1x12x3072x64 45.3 / 36.2 us, 1x8x4096x64 54.4 / 44.2, 2x12x2048x64 33.2 / 29.2);
-// with several items per CTA it gains (1x32x2048x64 34.8 / 37.9, 4x12x2048x64 46.4 / 49.0).  Behind the staging kernel, which
-// lets go of its dependents when everything before it is done, one item per CTA gains as well (1x12x3072x64, three frozen
-// heads, 36.2 / 38.2; 1x8x1024x64, one forward waited for, 33.4 / 36.0).
+// so that long items meet on one SM.  Where a CTA gets one long item, or two, that costs more than the launch gap (forwards
+// back to back, early / not: 1x12x3072x64 45.3 / 36.2 us, 1x8x4096x64 54.4 / 44.2, 2x12x2048x64 33.2 / 29.2); with more per CTA
+// (1x32x2048x64 34.8 / 37.9, 3x12x1537x64 28.5 / 31.1) and with short ones (8x12x512x64 14.7 / 16.7; updates of 9x8x300x64
+// 30.3 / 32.8, but of 1x16x900x64 44.0 / 41.3) it gains.  Behind the staging kernel, which lets go of its dependents when
+// everything before it is done, one item per CTA gains whatever its length (1x12x3072x64, three frozen heads, 36.2 / 38.2), two
+// if they are short (8x12x512x64, three frozen heads, 16.9 / 20.1; an update of packed 3x12x1537x64 with six 78.1 / 81.4; but
+// 1x16x4096x64 with eight 59.3 / 52.4).
 cudaError_t launch_fwd64(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv, const CUtensorMap& mvt,
                          const CUtensorMap& mo, const FwdParams& p, int grid, cudaStream_t st) {
-  const bool early = 2 * p.n_items >= 5 * grid || (p.band_f != nullptr && p.n_items <= grid);
+  const bool early = p.band_f != nullptr
+                         ? p.n_items <= grid || p.T <= 13 * BLK || 2 * p.n_items >= 5 * grid
+                         : p.T <= 3 * BLK || (p.T <= 8 * BLK && p.n_items > grid) || 2 * p.n_items >= 3 * grid;
   auto kern = p.o_f32 ? saf_fwd64_kernel<true> : saf_fwd64_kernel<false>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Fwd64Cfg::SMEM);
   if (e != cudaSuccess) return e;
