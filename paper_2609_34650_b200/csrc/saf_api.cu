@@ -735,7 +735,7 @@ int saf_hybrid_attn_fwd(saf_ctx* ctx, const saf_problem* p, const void* Q, const
   fp.queue = ctx->queue_dev;
   fp.status = ctx->status_dev;
   fp.wait_limit_ns = ctx->wait_limit_ns;
-  fp.selftest_drop_load = (ctx->selftest_drop_load && grid <= 16 && ctx->wait_limit_ns <= 50000000ull) ? 1 : 0;
+  fp.selftest_drop_load = (ctx->selftest_drop_load && (grid <= 16 || is_short) && ctx->wait_limit_ns <= 50000000ull) ? 1 : 0;
   ScopedTimer timer(ctx, SAF_KERNEL_FWD, st);
   // head dimension 96 runs on the 128-wide kernel: TMA zero-fills features 96..127 of every operand tile
   // bf16 O leaves the D = 64 kernel as whole tiles by TMA stores (rows beyond T are clipped by the map); with fp32 O

@@ -90,7 +90,8 @@ struct FwdParams {
   unsigned long long wait_limit_ns;
   // Self-test of the give-up path (0 in normal use): the producer leaves out the load of the first key tile of its first
   // ordinary item, so that the waits for it run out.  Set by saf_create from
-  // SAF_SELFTEST_DROP_LOAD, and only for grids of at most 16 CTAs with a wait limit of at most 50 ms.
+  // SAF_SELFTEST_DROP_LOAD, and only with a wait limit of at most 50 ms, for grids of at most 16 CTAs or, in the 128-wide
+  // kernel of short sequences (which never has so few), in its first 16 CTAs.
   int selftest_drop_load;
 };
 

@@ -44,7 +44,7 @@ def test_a_wait_that_runs_out_is_reported_and_the_context_stays_usable(monkeypat
 
 
 @pytest.mark.parametrize("D,H,T,sites", [
-    (128, 4, 256, range(101, 111)),      # one query block per item (8 items)
+    (128, 80, 256, range(101, 111)),     # one query block per item (160 items: more than one per SM)
     (96, 3, 520, range(1, 12)),          # the kernel of the longer sequences (15 items of up to five tiles: the producer's
     (128, 3, 520, range(1, 12)),         # ring runs full, so its own wait gives up as well)
 ])
