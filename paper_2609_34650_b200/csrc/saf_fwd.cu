@@ -73,6 +73,8 @@ struct FwdCfg {
   static constexpr int COL_S = 0, COL_O = 256;          // + 128 t, + D t
   static constexpr int NTHREADS = 512;
 };
+constexpr int TAB_FLOATS = 784;                         // one tile's tables of the general frozen form (two buffers)
+static_assert(2 * TAB_FLOATS * 4 <= FwdCfg::TILE_BYTES, "the tables fit into a query tile");
 
 enum FwdSite { SITE_Q_EMPTY = 1, SITE_KV_EMPTY, SITE_Q_FULL, SITE_KV_FULL, SITE_P_FULL, SITE_O_FREE, SITE_S_FULL,
                SITE_O_FULL, SITE_L_FULL, SITE_RING_EMPTY, SITE_RING_FULL };
@@ -599,43 +601,48 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
           p.LSE[(static_cast<size_t>(w.b) * p.H + w.h) * p.T + row] = (m_ref + log2f(l)) * LN2_F;
       } else {
         // ---------------- frozen head, general form: generate P^ tiles
-        float* tab = reinterpret_cast<float*>(smem + C::OFF_Q + t * C::TILE_BYTES);
-        float* aJ = tab;                               // [128] a of the tile's keys
-        float* rband = tab + 128;                      // [256] r of the tile's distances
-        float* a2raw = tab + 384;                      // [128]
-        float* r2raw = tab + 512;                      // [256]
-        float* red = tab + 768;                        // [8]
         const int wt = tid & 127;
         const float* alpha_h = p.alpha + static_cast<size_t>(w.h) * p.Tp;
         const float* rho_h = p.rho + static_cast<size_t>(w.h) * p.Tp;
         const float z2 = (row < p.T) ? p.logZ[static_cast<size_t>(w.h) * p.Tp + row] * LOG2E_F : INFINITY;
-        bool leave = false;
-        for (int j = 0; j < nt; ++j) {
-          // previous P^ tile consumed (first tile: everything issued before this item has completed)
+        // A tile's table entries are fetched one tile ahead and its tables are made while the previous tile's P^ V is
+        // still running: with one table buffer, filled behind that wait, a tile was one serial chain (head dimension
+        // 128, 4 heads x 8192, one of them of this form, so that its last item sets the time: 184 us, 154 with the fetch ahead, 142 with both).
+        float a_next = 0.0f, r_next[2] = {0.0f, 0.0f};
+        auto fetch = [&](int j) {
+          const int key = j * BLK + wt;
+          a_next = key < p.T ? alpha_h[key] : -INFINITY;
+#pragma unroll
+          for (int k = 0; k < 2; ++k) {
+            const int x = wt + 128 * k, d = (blk - j) * BLK - 127 + x;     // band covers distances d0 .. d0+254
+            r_next[k] = x < 255 && d >= 0 && d < p.T ? rho_h[d] : -INFINITY;
+          }
+        };
+        // P^ buffer free (first tile: everything issued before this item has completed, which also frees the tables'
+        // memory); the four warps agree whether to go on.  Past the agreement of tile j every reader of tile j - 1's
+        // tables is done with them, so two buffers suffice.
+        auto p_free = [&]() {
           if (!mbar_wait_warp_compact(s_full + t, ns & 1, wc, SITE_S_FULL)) ok = false;
           ++ns;
           tc_fence_after();
-          // previous tile's table readers are done; the four warps also agree whether to go on
-          if (named_bar_or(wg_bar, 128, !ok)) {
-            ok = false;
-            leave = true;
-            break;
-          }
-          const int d0 = (blk - j) * BLK - 127;        // band covers distances d0 .. d0+254
-          float ma = -INFINITY, mr = -INFINITY, a2 = -INFINITY, r2[2];
-          {
-            const int key = j * BLK + wt;
-            if (key < p.T) a2 = alpha_h[key] * LOG2E_F;
-            a2raw[wt] = a2;
-            ma = a2;
-          }
-#pragma unroll
-          for (int k = 0; k < 2; ++k) {
-            const int x = wt + 128 * k, d = d0 + x;
-            r2[k] = (x < 255 && d >= 0 && d < p.T) ? rho_h[d] * LOG2E_F : -INFINITY;
-            r2raw[x] = r2[k];
-            mr = fmaxf(mr, r2[k]);
-          }
+          if (named_bar_or(wg_bar, 128, !ok)) ok = false;
+          return ok;
+        };
+        fetch(0);
+        bool stay = p_free();
+        for (int j = 0; j < nt && stay; ++j) {
+          float* tab = reinterpret_cast<float*>(smem + C::OFF_Q + t * C::TILE_BYTES) + (j & 1) * TAB_FLOATS;
+          float* aJ = tab;                             // [128] a of the tile's keys
+          float* rband = tab + 128;                    // [256] r of the tile's distances
+          float* a2raw = tab + 384;                    // [128]
+          float* r2raw = tab + 512;                    // [256]
+          float* red = tab + 768;                      // [8]
+          const float a2 = a_next * LOG2E_F, r2[2] = {r_next[0] * LOG2E_F, r_next[1] * LOG2E_F};
+          a2raw[wt] = a2;
+          r2raw[wt] = r2[0];
+          r2raw[wt + 128] = r2[1];
+          float ma = a2, mr = fmaxf(r2[0], r2[1]);
+          if (j + 1 < nt) fetch(j + 1);
 #pragma unroll
           for (int o = 16; o > 0; o >>= 1) {
             ma = fmaxf(ma, __shfl_xor_sync(0xffffffffu, ma, o));
@@ -654,6 +661,7 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
           rband[wt + 128] = ex2_approx(r2[1] - mr);
           // (agreement on the form: the factorised one would overflow or flush for some row)
           const bool exact = named_bar_or(wg_bar2, 128, ew > 100.0f);
+          if (j > 0 && !(stay = p_free())) break;
 #pragma unroll 1
           for (int cc = 0; cc < 4; ++cc) {
             uint32_t pk[16];
@@ -686,7 +694,7 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
           fence_proxy_async_smem();                    // the tables' memory is a TMA destination of a later item
           warp_arrive(p_full + t);
         }
-        if (leave) break;
+        if (!stay) break;
       }
       ++nof;
     }

@@ -71,6 +71,21 @@ def test_item_kinds_alternate_at_the_wide_head_dimensions(B, H, T, D):
     check_units(L, [(0, 0), (0, 2), (1, 1), (2, 5), (3, 3), (4, 4), (5, 6), (6, 7), (7, 2), (B - 1, H - 1)])
 
 
+@pytest.mark.parametrize("D", [96, 128])
+@pytest.mark.parametrize("B,H,T", [(4, 10, 520), (2, 6, 2050)])
+def test_patterns_without_prepared_tables_in_paired_items(B, H, T, D):
+    """Frozen heads whose normalisers come from the entry point without a context take the general form throughout: two table
+    buffers per query block in turn, over odd and even tile counts and a last tile of a few rows; head 1 has keys switched
+    off, head 2 leaves the range of the factorised exponential in some tiles."""
+    inp = si.generate(si.Workload("general", B, H, T, D, tuple(range(H)), -0.05, seed=31 + D))
+    inp.alpha[1, 40:60] = -1e30
+    inp.alpha[2] = (inp.alpha[2] + 25.0 * np.sin(0.37 * np.arange(T))).astype(np.float32)
+    L = Layer(inp, backward=False)
+    saf.saf_pattern_logz_static(0, L.mask, L.alpha, L.rho, L.logZ)
+    L.run(backward=False, prepare=False)
+    check_units(L, [(0, 0), (0, 1), (1, 2), (B - 1, 3), (B - 1, H - 1)], backward=False)
+
+
 @pytest.mark.parametrize("T", [1, 31, 33, 255, 4096, 4097, 8200])
 @pytest.mark.parametrize("spread", [1.0, 60.0])
 def test_normalisers_at_chunk_edges(T, spread):
