@@ -281,8 +281,8 @@ struct FitPlan {
 
 // One cluster = one head.  A head's x blocks go to the cluster's CTAs in snake order by descending work.  Bound: fp32
 // multiply-adds (128 per clock and SM), 1.5 T^2 per head and step.  Measured (36 heads, T = 4096, 400 steps): 23.4 ms =
-// 58 us per step on 108 SMs, against 100.2 ms for one exponential per pair and sum in two launches per step; the inner
-// loops run at 76 % of the multiply-add peak (148 heads: 64 % over everything).  One head of 256 positions: 6.0 us per
+// 58 us per step on 108 SMs, against 100.2 ms for one exponential per pair and sum in two launches per step; 57 % of those
+// SMs' multiply-add peak over everything.  One head of 256 positions: 6.0 us per
 // step (two cluster barriers, L2 round trips of the parameters, fp64 Adam).
 template <int NW, bool PADDED, int RB>
 __global__ void __launch_bounds__(NW * 32, 1)

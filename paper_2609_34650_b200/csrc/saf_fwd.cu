@@ -606,8 +606,8 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
         const float* rho_h = p.rho + static_cast<size_t>(w.h) * p.Tp;
         const float z2 = (row < p.T) ? p.logZ[static_cast<size_t>(w.h) * p.Tp + row] * LOG2E_F : INFINITY;
         // A tile's table entries are fetched one tile ahead and its tables are made while the previous tile's P^ V is
-        // still running: with one table buffer, filled behind that wait, a tile was one serial chain (head dimension
-        // 128, 4 heads x 8192, one of them of this form, so that its last item sets the time: 184 us, 154 with the fetch ahead, 142 with both).
+        // still running.  Fetched and filled behind that wait, a tile was one serial chain (4 heads x 8192 x 128, one
+        // head of this form, so that its last item sets the time: 184 us, 154 with the fetch ahead, 142 with both).
         float a_next = 0.0f, r_next[2] = {0.0f, 0.0f};
         auto fetch = [&](int j) {
           const int key = j * BLK + wt;

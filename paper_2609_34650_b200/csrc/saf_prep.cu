@@ -19,8 +19,8 @@ namespace saf {
 // would carry more rounding than the sums alpha + rho themselves, and in the end overflow), the block goes over its range
 // once more, relative to the rows' own maxima.  fp32 sums of 32 terms, fp64 from there.
 // Bound: one ex2 per causal pair.
-// (6 heads x 2048: one warp per row with two passes over global memory 20.6 us with the launch gap, this one 16.6; with a sink of 90 on key 0,
-// where most rows are taken again, 19.5; 8 heads x 8192: 217 and 103)
+// (6 heads x 2048: one warp per row with two passes over global memory 20.6 us with the launch gap, this one 16.6; with a
+// sink of 90 on key 0, where most rows are taken again, 19.5; 8 heads x 8192: 217 and 103)
 // The last block of a head to finish also forms the head's constants (consts != NULL): max alpha, max rho, and
 // whether the tensor-core form's range holds (see below); counters (two per head) return to zero.
 constexpr int LZ_KC = 4096;
