@@ -183,7 +183,7 @@ int saf_fit_marginals(saf_ctx* ctx, int32_t Hf, int32_t T, const float* mean_att
  * and installation": alpha = 0, rho(d) = log max(eta_rel(d)/(T-d), 1e-9), then `steps` Adam steps (beta1 0.9,
  * beta2 0.999, eps 1e-8, bias-corrected) at learning rate `lr` on
  * L = (1/T)[sum_i log Z(i) - sum_j eta_abs(j) alpha(j) - sum_d eta_rel(d) rho(d)]; the paper uses 400 steps at 0.05).
- * All heads are fitted together; nothing of size T x T is allocated (state: 56 bytes per head and position, held by
+ * All heads are fitted together; nothing of size T x T is allocated (state: 108 bytes per head and position, held by
  * the context and reused).  Exponentials and the terms of the sums are fp32, Adam and its state fp64.
  *   eta_abs, eta_rel : device float64 [Hf, T] (from saf_fit_marginals, or accumulated by the caller)
  *   plogp            : device float64 [Hf] or NULL if kl_out is NULL
@@ -244,7 +244,7 @@ enum {
   SAF_KERNEL_LOGZ = 4,         /* pattern normalisers and tables (saf_pattern_prepare) */
   SAF_KERNEL_SCALE = 5,        /* per-call row scaling of the frozen heads' V (forward) / dO (backward) */
   SAF_KERNEL_PGRAD = 6,        /* pattern-gradient kernel (saf_pattern_grad) */
-  SAF_KERNEL_FIT = 7,          /* the launch of saf_fit_compact */
+  SAF_KERNEL_FIT = 7,          /* the launches of saf_fit_compact */
   SAF_KERNEL_FIT_MARGINALS = 8,/* target marginals (saf_fit_marginals) */
   SAF_KERNEL_CALIB = 9,        /* calibration statistics kernel (saf_calib_accumulate) */
   SAF_KERNEL_CALIB_FINALIZE = 10, /* mean and scores (saf_calib_finalize) */

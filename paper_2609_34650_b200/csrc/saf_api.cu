@@ -1274,9 +1274,9 @@ int saf_fit_compact(saf_ctx* ctx, int32_t Hf, int32_t T, const double* eta_abs, 
   if (!g.ok) return SAF_ERR_CUDA;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   ctx->last_stream = st;
-  // state: 6 fp64 and 2 fp32 arrays of [Hf, T]
+  // state: two copies of 6 fp64 arrays and 3 fp32 arrays of [Hf, T], one int per head
   const size_t n = static_cast<size_t>(Hf) * T;
-  int rc = ensure(ctx->fit_buf, n * (6 * sizeof(double) + 2 * sizeof(float)));
+  int rc = ensure(ctx->fit_buf, n * (12 * sizeof(double) + 3 * sizeof(float)) + static_cast<size_t>(Hf) * sizeof(int));
   if (rc) return rc;
   FitState s;
   s.T = T;
@@ -1285,8 +1285,11 @@ int saf_fit_compact(saf_ctx* ctx, int32_t Hf, int32_t T, const double* eta_abs, 
   s.eta_rel = eta_rel;
   double* d = static_cast<double*>(ctx->fit_buf.ptr);
   s.alpha = d; s.rho = d + n; s.m_a = d + 2 * n; s.v_a = d + 3 * n; s.m_r = d + 4 * n; s.v_r = d + 5 * n;
-  float* f = reinterpret_cast<float*>(d + 6 * n);
+  s.second = 6 * n;
+  float* f = reinterpret_cast<float*>(d + 12 * n);
   s.a2 = f; s.r2 = f + n;
+  s.wref = f + 2 * n;
+  s.resume = reinterpret_cast<int*>(f + 3 * n);
   ScopedTimer timer(ctx, SAF_KERNEL_FIT, st);
   if (launch_fit(s, Hf, steps, plogp, alpha_out, rho_out, logZ_out, out_stride, loss_out, kl_out, st) != cudaSuccess)
     return SAF_ERR_CUDA;

@@ -8,8 +8,9 @@
 //              (fitted marginal - target marginal)/T
 //   accept     kappa = mean row KL(P || P^) = L + (1/T) sum P log P   (rows of P sum to one)
 //
-// Nothing of size T x T is formed after the target has been read once.  The whole fit is ONE launch: a thread-block
-// cluster per head runs all Adam steps, exchanging vectors of length T through distributed shared memory (normalisers)
+// Nothing of size T x T is formed after the target has been read once.  Beyond 128 positions the Adam steps run in
+// saf_fit_fft.cu, where the three sums of a step are fp64 transforms; the kernel here serves the shortest sequences and goes
+// on with the heads that leave the transforms' bounds.  A thread-block cluster per head runs all Adam steps in one launch, exchanging vectors of length T through distributed shared memory (normalisers)
 // and L2 (parameters), with two cluster barriers per step:
 //   pass A   rows:      Z(i) = sum_{d<=i} R(d) A(i-d),  W(i) = 1 / Z(i)
 //   pass B   marginals: c(j) = A(j) sum_d R(d) W(j+d)  and  g(d) = R(d) sum_j A(j) W(j+d),
@@ -311,6 +312,10 @@ saf_fit_kernel(FitState s, int steps, const double* __restrict__ plogp, float* _
   float* part = R + Tr + FPAD;                   // [NW + RB][2][FX] partial sums
   const int nxb = (T + FX - 1) / FX;
   bool slow = false;
+  // a head that the transform form has finished, or the step at which it handed it over (1: nothing done yet)
+  const int t0 = s.resume ? s.resume[h] : 1;
+  if (t0 < 0) return;
+  const bool fresh = t0 <= 1;
 
   if (tid < 2) {                                 // plan[0]: pass A, plan[1]: pass B
     FitPlan& p = plan[tid];
@@ -373,12 +378,15 @@ saf_fit_kernel(FitState s, int steps, const double* __restrict__ plogp, float* _
   float mx = -INFINITY;
   bool bad = false;
   for (int d = tid; d < T; d += NT) {
-    const double r = log(fmax(s.eta_rel[o + d] / static_cast<double>(T - d), 1e-9));
-    const float r2 = static_cast<float>(r * LOG2E_D);
+    const double r = fresh ? log(fmax(s.eta_rel[o + d] / static_cast<double>(T - d), 1e-9)) : s.rho[o + d];
+    const double a = fresh ? 0.0 : s.alpha[o + d];
+    const float r2 = static_cast<float>(r * LOG2E_D), a2 = static_cast<float>(a * LOG2E_D);
     mx = fmaxf(mx, r2);
-    if (!(r2 >= R_LO && r2 <= R_HI)) bad = true;
+    if (!(r2 >= R_LO && r2 <= R_HI && a2 >= A_LO && a2 <= A_HI)) bad = true;
+    if (!fresh && !(fabsf(s.wref[o + d]) <= A_HI)) bad = true;
     R[d] = exp2_f32(r * LOG2E_D);
-    A[fit_phys<PADDED>(d)] = 1.0f;
+    A[fit_phys<PADDED>(d)] = exp2_f32(a * LOG2E_D);
+    if (!fresh) continue;
     // (each block's state is written and later read by its owner in pass B only, except for the fp64 parameters)
     const int k = d / FX, kr = k / static_cast<int>(cs), ki = k % static_cast<int>(cs);
     if (((kr & 1) ? static_cast<int>(cs) - 1 - ki : ki) == static_cast<int>(rank)) {
@@ -395,11 +403,12 @@ saf_fit_kernel(FitState s, int steps, const double* __restrict__ plogp, float* _
 #pragma unroll
   for (int w = 1; w < NW; ++w) mx = fmaxf(mx, redf[w]);
   fill_pads(0.0f);
-  for (int i = tid; i < T; i += NT) W[fit_phys<PADDED>(i)] = bad ? -mx : ex2f(-mx);
+  auto wstart = [&](int i) { return fresh ? -mx : s.wref[o + i]; };
+  for (int i = tid; i < T; i += NT) W[fit_phys<PADDED>(i)] = bad ? wstart(i) : ex2f(wstart(i));
   cluster_sync_all();
   if (bad) {                                     // (the same decision in every CTA of the cluster)
     go_slow();
-    for (int i = tid; i < T; i += NT) W[fit_phys<PADDED>(i)] = -mx;
+    for (int i = tid; i < T; i += NT) W[fit_phys<PADDED>(i)] = wstart(i);
     cluster_sync_all();
   }
 
@@ -464,9 +473,13 @@ saf_fit_kernel(FitState s, int steps, const double* __restrict__ plogp, float* _
   };
 
   double p1 = 1.0, p2 = 1.0;
-  for (int t = 1; t <= steps + 1; ++t) {
+  for (int t = 1; t < t0; ++t) {
+    p1 *= 0.9;
+    p2 *= 0.999;
+  }
+  for (int t = max(t0, 1); t <= steps + 1; ++t) {
     const bool last = t == steps + 1;
-    if (t > 1) {
+    if (t > max(t0, 1)) {
       // the parameters of this step, from the owners of their blocks
       if (!slow && out_par) {
         go_slow();
@@ -667,8 +680,15 @@ cudaError_t launch_fit_clusters(const FitState& s, int Hf, cudaStream_t st, Args
 
 }  // namespace
 
-cudaError_t launch_fit(const FitState& s, int Hf, int steps, const double* plogp, float* alpha_out, float* rho_out,
+cudaError_t launch_fit(FitState s, int Hf, int steps, const double* plogp, float* alpha_out, float* rho_out,
                        float* logZ_out, long long out_stride, double* loss_out, double* kl_out, cudaStream_t st) {
+  // Up to 128 positions the direct sums are the shorter of two serial chains (us a step of one head, direct / transforms: 64
+  // 5.2 / 4.8, 100 5.1 / 5.2, 256 5.9 / 5.1, 1024 9.1 / 7.5, 4096 22.8 / 10.1)
+  s.resume = s.T > 128 ? s.resume : nullptr;
+  if (s.resume) {
+    const cudaError_t e = launch_fit_fft(s, Hf, steps, plogp, alpha_out, rho_out, logZ_out, out_stride, loss_out, kl_out, st);
+    if (e != cudaSuccess) return e;
+  }
   // up to 8192 positions the padded vectors fit beside the partial sums of 16 warps, up to 12288 beside those of 12; the
   // longest sequences keep them unpadded (two-way bank conflicts on the window reads)
   if (s.T <= 8192)

@@ -230,11 +230,17 @@ struct FitState {
   double* alpha; double* rho;          // fp64 parameters
   double* m_a; double* v_a; double* m_r; double* v_r;   // Adam moments
   float* a2; float* r2;                // exp (in the log form: log2e-scaled copy) of the current parameters
+  // The transform form writes parameters and moments to two copies in turn (the second one `second` elements further on) and
+  // hands to the others, per head, the step to go on with (-1: done) and log2 of nearby reciprocal normalisers.
+  size_t second;
+  int* resume; float* wref;
 };
 int fit_max_T();
 cudaError_t launch_fit_marginals(const float* Abar, float floor_v, double* eta_abs, double* eta_rel, double* plogp,
                                  int Hf, int T, int num_sms, cudaStream_t st);
-cudaError_t launch_fit(const FitState& s, int Hf, int steps, const double* plogp, float* alpha_out, float* rho_out,
+cudaError_t launch_fit_fft(const FitState& s, int Hf, int steps, const double* plogp, float* alpha_out, float* rho_out,
+                           float* logZ_out, long long out_stride, double* loss_out, double* kl_out, cudaStream_t st);
+cudaError_t launch_fit(FitState s, int Hf, int steps, const double* plogp, float* alpha_out, float* rho_out,
                        float* logZ_out, long long out_stride, double* loss_out, double* kl_out, cudaStream_t st);
 
 // calibration statistics (saf_calib.cu)

@@ -315,3 +315,40 @@ def test_a_single_long_head_spreads_over_more_than_eight_sms():
             torch.cuda.synchronize()
             us[T] = min(us.get(T, 1e9), a.elapsed_time(b) * 20.0)
     assert us[8192] <= 2.5 * us[4096], us                # measured 22.8 and 44.4 us a step; on eight SMs 25.4 and 80.4
+
+
+# ------------------------------------------------------------------------------------------------ the transform form
+# Transforms of 256, 512 points in one CTA, 1024, 2048, 4096 in two, four, eight CTAs of 512, 8192 and 16384 in eight of 1024
+# and 2048; lengths at and beside the powers of two; 50 heads of 4096 positions run in clusters of four.  The sums are exact
+# to about 1e-9 relative, so what is left of the parameters' error is their rounding to fp32 (2^-24 of up to 32) and an Adam step's
+# response to its gradient's error, lr |dg| / |g| with |g| down to 1e-3 of the marginals: 1e-6.
+@pytest.mark.parametrize("Hf,T,steps", [(2, 129, 4), (1, 256, 3), (2, 257, 3), (1, 512, 3), (2, 513, 3), (1, 1024, 3), (1, 1025, 3),
+                                        (1, 2048, 2), (1, 2049, 2), (1, 4096, 2), (50, 4095, 2), (1, 4097, 2), (1, 8193, 1)])
+def test_fit_transform_lengths(Hf, T, steps):
+    base = si.mean_attention_maps(1, T, 60 + T)
+    P, ea, er, pl = _oracle_stats(base)
+    rep = lambda v: _dev(np.repeat(v, Hf, axis=0))
+    a, r, z, loss, kl = _gpu_fit(_ctx(), rep(ea), rep(er), rep(pl), steps)
+    for x in (a, r, z, loss, kl):
+        assert np.array_equal(x, np.broadcast_to(x[:1], x.shape))
+    wa, wr, wz = fo.fit_compact(ea[0], er[0], steps=steps)
+    tol = 1e-6 + 2.0 ** -24 * np.abs(wr).max()
+    assert np.max(np.abs(a[0] - wa)) < tol and np.max(np.abs(r[0] - wr)) < tol and np.max(np.abs(z[0] - wz)) < tol
+    assert abs(loss[0] - fo.fit_objective(wa, wr, ea[0], er[0])) < 1e-9 * max(1.0, abs(loss[0]))
+
+
+# Steps of 3 and 10 nats take heads out of the transforms' bounds after a few steps, so that both parities of the step at which
+# they are handed on occur; what was done before must not be lost: the parameters after few steps against the oracle (the direct
+# sums' bounds above), the normalisers at the returned parameters always.
+@pytest.mark.parametrize("T,lr,steps", [(200, 3.0, 6), (300, 10.0, 3), (300, 10.0, 4), (300, 10.0, 7), (700, 10.0, 5), (1500, 10.0, 6)])
+def test_fit_heads_handed_on(T, lr, steps):
+    A = si.mean_attention_maps(2, T, 70 + T)
+    P, ea, er, pl = _oracle_stats(A)
+    a, r, z, loss, kl = _gpu_fit(_ctx(), _dev(ea), _dev(er), _dev(pl), steps, lr=lr)
+    for h in range(2):
+        want_z, _ = fo._logZ_and_P(a[h], r[h])
+        assert np.max(np.abs(z[h] - want_z)) < 5e-4
+        assert abs(loss[h] - fo.fit_objective(a[h], r[h], ea[h], er[h])) < 5e-4 * max(1.0, abs(loss[h]))
+        wa, wr, wz = fo.fit_compact(ea[h], er[h], steps=steps, lr=lr)
+        # a gradient that nearly cancels may take the other sign in one element: most elements, not all
+        assert np.mean(np.abs(a[h] - wa) < 1e-2 * lr) > 0.97 and np.mean(np.abs(r[h] - wr) < 1e-2 * lr) > 0.97
