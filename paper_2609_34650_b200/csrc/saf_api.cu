@@ -1340,10 +1340,8 @@ int saf_calib_accumulate(saf_ctx* ctx, const saf_problem* p, const void* Q, cons
   cp.sumsq = sumsq;
   cp.sum_plogp = sum_plogp;
   cp.accumulate = accumulate ? 1 : 0;
-  cp.npairs = nblk * (nblk + 1) / 2;
-  const long long n_items = static_cast<long long>(p->H) * cp.npairs;
+  const long long n_items = static_cast<long long>(p->H) * (nblk * (nblk + 1LL) / 2);
   if (n_items > 0x7fffffffLL) return SAF_ERR_INVALID_ARG;
-  cp.n_items = static_cast<int>(n_items);
   cp.status = ctx->status_dev;
   cp.wait_limit_ns = ctx->wait_limit_ns;
   const int grid = static_cast<int>(std::min<long long>(ctx->num_sms, n_items));

@@ -10,14 +10,17 @@
 // No A^(n) is ever stored.  The row normalisers come from the attention forward of the same sequences (its LSE
 // output), so a tile of probabilities is exp2(s c - lse') straight from the score tile.
 //
-// One persistent kernel, item = (head, query block I, key block J <= I), all items cost the same.  Per item a loop
+// One persistent kernel, item = (head, query block I, key block J <= I).  Per item a loop
 // over the N sequences: S = Q_I K_J^T on the tensor core (tcgen05, both operands K-major in 128B-swizzled smem via
 // TMA, score tiles in four TMEM buffers), then per element in registers p = exp2(s c - lse'), acc += p,
 // sq += p^2, ent += p log2 p; the 128 x 128 fp32 accumulator tile lives in the registers of the 16 compute warps
 // (thread = query row x 32 keys) and leaves once per item through shared memory as four TMA stores into the dense
 // accumulator, which drain while the next item computes; in the calls that add to earlier ones the old tile is
 // fetched by TMA into the same boxes during the item and summed there (TMA reduce-adds measured 1.2 TB/s, half of
-// what the plain load + store path reaches).
+// what the plain load + store path reaches).  Rows that TMA cannot describe (T no multiple of 4) go the same way with
+// four-byte asynchronous copies in and coalesced stores out, a warp on its own 32 rows.
+// A CTA takes its share of the items below the diagonal, then of the diagonal ones.  Two fp64 sums of
+// a thread stay in shared memory until the head changes.
 // CTA = 576 threads: warps 0-15 compute (TMEM lane = query row; warp >> 2 picks the 32-key column group), warp 16
 // TMA producer, warp 17 tcgen05 issuer and TMEM owner.  Every wait is bounded.
 #include <cuda_bf16.h>
@@ -41,7 +44,8 @@ struct CalCfg {
   static constexpr int STAGE_BYTES = 2 * TILE_BYTES;    // Q tile then K tile
   static constexpr int OFF_OUT = NS * STAGE_BYTES;      // 4 boxes of 128 rows x 32 fp32 (128-byte rows, swizzled): 64 KB
   static constexpr int OUT_BOX_BYTES = 128 * 128;
-  static constexpr int OFF_BAR = OFF_OUT + 4 * OUT_BOX_BYTES;
+  static constexpr int OFF_SUMS = OFF_OUT + 4 * OUT_BOX_BYTES;          // two fp64 sums of every compute thread
+  static constexpr int OFF_BAR = OFF_SUMS + 512 * 16;
   static constexpr int NSB = 4;                         // score buffers in TMEM (128 fp32 columns each)
   static constexpr int NBAR = 2 * NS + 2 * NSB + 4;
   static constexpr int SMEM = OFF_BAR + NBAR * 8 + 16 + 1024;
@@ -51,20 +55,52 @@ struct CalCfg {
 
 enum CalSite { C_QK_EMPTY = 71, C_QK_FULL, C_S_FREE, C_S_FULL, C_OLD_FULL };
 
-// item index -> (h, I, J) with J <= I; pairs are numbered row by row: q = I (I+1)/2 + J
-__device__ __forceinline__ void decode_item(int idx, int npairs, int& h, int& I, int& J) {
-  h = idx / npairs;
-  const int q = idx - h * npairs;
-  int i = static_cast<int>((sqrtf(8.0f * static_cast<float>(q) + 1.0f) - 1.0f) * 0.5f);
-  while ((i + 1) * (i + 2) / 2 <= q) ++i;
-  while (i * (i + 1) / 2 > q) --i;
-  I = i;
-  J = q - i * (i + 1) / 2;
+// The items of one CTA: of the n_off = H nblk (nblk-1)/2 ones below the diagonal (numbered head by head, row by row: q =
+// I (I-1)/2 + J) every grid-th run of four, then every grid-th of the rest, then every grid-th diagonal one, from the CTAs on that
+// have one item fewer.  Runs keep a thread's sums on one head; all CTAs together stay on a few heads, whose Q and K fit the L2
+// (one long run per CTA: 8x12x4096x64 348 us, 329 with single items).
+struct CalItems {
+  int nblk, pairs, n_off, n_diag, runs, run, diag0, cta, step;
+  __device__ __forceinline__ CalItems(int H, int T, int cta_, int grid) {
+    nblk = (T + BLK - 1) / BLK;
+    pairs = nblk * (nblk - 1) / 2;
+    n_off = H * pairs;
+    n_diag = H * nblk;
+    const int q = n_off / grid, r = n_off - q * grid;
+    runs = q & ~3;
+    run = q + (cta_ < r);
+    diag0 = cta_ < r ? cta_ - r + grid : cta_ - r;
+    cta = cta_;
+    step = grid;
+  }
+  // item k of the CTA; false behind the last one
+  __device__ __forceinline__ bool get(int k, int& h, int& I, int& J) const {
+    if (k < run) {
+      const int idx = k < runs ? ((k & ~3) * step + 4 * cta + (k & 3)) : k * step + cta;
+      h = idx / pairs;
+      const int q = idx - h * pairs;
+      int i = static_cast<int>((sqrtf(8.0f * static_cast<float>(q) + 1.0f) + 1.0f) * 0.5f);
+      while (i * (i + 1) / 2 <= q) ++i;
+      while (i * (i - 1) / 2 > q) --i;
+      I = i;
+      J = q - i * (i - 1) / 2;
+      return true;
+    }
+    const int d = diag0 + (k - run) * step;
+    if (d >= n_diag) return false;
+    h = d / nblk;
+    I = J = d - h * nblk;
+    return true;
+  }
+};
+
+__device__ __forceinline__ void cp_async4(uint32_t dst, const float* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
 }
 
 }  // namespace
 
-template <int D, bool ACC>
+template <int D, bool ACC, bool TMA>
 __global__ void __launch_bounds__(576, 1)
 saf_calib_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ CUtensorMap mk,
                  const __grid_constant__ CUtensorMap mm, const CalibParams p) {
@@ -112,9 +148,7 @@ saf_calib_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
       tma_prefetch_desc(&mk);
       uint32_t nl = 0;
       bool ok = true;
-      for (int idx = blockIdx.x; idx < p.n_items && ok; idx += gridDim.x) {
-        int h, I, J;
-        decode_item(idx, p.npairs, h, I, J);
+      for (int it = 0, h, I, J; ok && CalItems(p.H, p.T, blockIdx.x, gridDim.x).get(it, h, I, J); ++it) {
         for (int n = 0; n < p.B; ++n, ++nl) {
           const int s = nl % C::NS;
           ok = mbar_wait(qk_empty + s, ((nl / C::NS) & 1) ^ 1, wc, C_QK_EMPTY);
@@ -137,7 +171,7 @@ saf_calib_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
     const uint32_t lo_k = desc_lo(d_k), hi_k = desc_hi(d_k);
     uint32_t nl = 0;
     bool ok = true;
-    for (int idx = blockIdx.x; idx < p.n_items && ok; idx += gridDim.x) {
+    for (int it = 0, h, I, J; ok && CalItems(p.H, p.T, blockIdx.x, gridDim.x).get(it, h, I, J); ++it) {
       for (int n = 0; n < p.B && ok; ++n, ++nl) {
         const uint32_t s = nl % C::NS, gb = nl % C::NSB;
         ok = mbar_wait_warp(qk_full + s, (nl / C::NS) & 1, wc, C_QK_FULL);
@@ -170,32 +204,62 @@ saf_calib_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
     const size_t lse_step = static_cast<size_t>(p.H) * p.T;
     // first normaliser of an item: its load passes under the hand-over of the item before
     int hn = 0, In = 0, Jn = 0;
-    auto first_lse = [&](int idx) {
-      if (idx >= p.n_items) return 0.0f;
-      decode_item(idx, p.npairs, hn, In, Jn);
+    bool more = true;
+    auto first_lse = [&](int it) {
+      more = CalItems(p.H, p.T, blockIdx.x, gridDim.x).get(it, hn, In, Jn);
       const int q = In * BLK + rowl;
-      return q < p.T ? __ldg(p.LSE + static_cast<size_t>(hn) * p.T + q) : 0.0f;
+      return more && q < p.T ? __ldg(p.LSE + static_cast<size_t>(hn) * p.T + q) : 0.0f;
     };
-    float lse_first = first_lse(blockIdx.x);
-    for (int idx = blockIdx.x; idx < p.n_items; idx += gridDim.x) {
+    float lse_first = first_lse(0);
+    double2* const sums = reinterpret_cast<double2*>(smem + C::OFF_SUMS) + tid;   // sum p^2, sum p log2 p of head h_sum
+    *sums = make_double2(0.0, 0.0);
+    int h_sum = hn;
+    auto flush = [&]() {
+      double sq_sum = sums->x, ent_sum = sums->y;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        sq_sum += __shfl_xor_sync(0xffffffffu, sq_sum, o);
+        ent_sum += __shfl_xor_sync(0xffffffffu, ent_sum, o);
+      }
+      if (lane == 0) {
+        atomicAdd(p.sumsq + h_sum, sq_sum);
+        atomicAdd(p.sum_plogp + h_sum, ent_sum * LN2_C);
+      }
+      *sums = make_double2(0.0, 0.0);
+    };
+    for (int it = 0; more; ++it) {
       const int h = hn, I = In, J = Jn;
+      if (h != h_sum) {
+        flush();
+        h_sum = h;
+      }
       const int qi = I * BLK + rowl;
       const int k0 = J * BLK + 32 * cq;                // first key of this thread's 32 columns
-      const bool diag = (I == J) || (J * BLK + BLK > p.T);   // tiles that need the per-element mask
+      // (tiles that need the per-element mask; leaving out the warps whose keys all lie above their rows costs 5 % at every
+      // other tile, 8x12x4096x64)
+      const bool diag = I == J && cq >= q4;
       const float* lse_h = p.LSE + static_cast<size_t>(h) * p.T + qi;
       // The four 32-column groups of compute warps hand their output box over independently of one another
       // (thread 128 cq leads group cq): a barrier over all 16 warps would put them back in lockstep at every item.
       const bool box_ok = J * BLK + 32 * cq < p.T;     // the group's box lies inside the matrix
       const bool lead = (tid == 128 * cq);
       uint8_t* const box = smem + C::OFF_OUT + cq * C::OUT_BOX_BYTES;
-      if (ACC && p.use_tma && lead) {
-        // what earlier calls left in this box is fetched while the sequences are processed (the previous item's
-        // store has finished reading the box first)
+      const uint32_t box_a = smem_u32(box);
+      float* const old = p.mean_sum + (static_cast<size_t>(h) * p.T + I * BLK + 32 * q4) * p.T + k0 + lane;   // row 32 q4, column lane
+      const int rows = k0 + lane < p.T ? min(32, p.T - I * BLK - 32 * q4) : 0;
+      auto box_addr = [&](int r) {                     // of row 32 q4 + r, column lane
+        return box_a + (32 * q4 + r) * 128 + (((lane >> 2) ^ (r & 7)) << 4) + ((lane & 3) << 2);
+      };
+      // what earlier calls left in this box is fetched while the sequences are processed (the previous item's
+      // store has finished reading the box first)
+      if (ACC && TMA && lead) {
         bulk_wait_group_read0();
         if (box_ok) {
           mbar_expect_tx(old_full + cq, C::OUT_BOX_BYTES);
           tma_load_4d(box, &mm, old_full + cq, J * BLK + 32 * cq, I * BLK, h, 0);
         }
+      } else if (ACC && !TMA) {
+        for (int r = 0; r < rows; ++r) cp_async4(box_addr(r), old + static_cast<size_t>(r) * p.T);
       }
       uint64_t acc2[16];                               // the thread's 32 accumulators as packed pairs
 #pragma unroll
@@ -205,6 +269,7 @@ saf_calib_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
       // the normaliser of sequence n+1 is loaded while sequence n is processed and first touched one round later
       // (a use right after the load would stall the warp for the whole memory latency in front of the wait below)
       const bool row_ok = qi < p.T;
+      const uint64_t c2p = pk2(c2, c2);
       float lse_raw = lse_first;
       for (int n = 0; n < p.B; ++n, ++nl) {
         float lse_raw_next = 0.0f;
@@ -214,17 +279,17 @@ saf_calib_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
         if (!ok) continue;                             // (keeps the loop counters in step; nothing is read)
         const float lse2 = row_ok ? lse_raw * LOG2E_C : INFINITY;
         lse_raw = lse_raw_next;
+        const uint64_t nlse = pk2(-lse2, -lse2);
+        // p log2 p = p (s c - lse'): the first part is summed per element as p s, the second needs no tile at
+        // all because a row of probabilities sums to one: the threads of key block 0, column group 0 add lse'
+        // once per row and sequence.
+        if (J == 0 && cq == 0 && row_ok) lsum += lse2;
         tc_fence_after();
         uint32_t r[32];
         tmem_ld32(tmem + lane_base + 128 * gb + 32 * cq, r);
         tmem_wait_ld();
         tc_fence_before();
         warp_arrive(s_free + gb);                      // the tensor core may overwrite this buffer
-        // p log2 p = p (s c - lse'): the first part is summed per element as p s, the second needs no tile at
-        // all because a row of probabilities sums to one: the threads of key block 0, column group 0 add lse'
-        // once per row and sequence.
-        if (J == 0 && cq == 0 && row_ok) lsum += lse2;
-        const uint64_t c2p = pk2(c2, c2), nlse = pk2(-lse2, -lse2);
         if (diag) {
 #pragma unroll
           for (int k = 0; k < 16; ++k) {
@@ -251,39 +316,43 @@ saf_calib_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
           }
         }
       }
-      lse_first = first_lse(idx + gridDim.x);
+      lse_first = first_lse(it + 1);
       float acc[32];
 #pragma unroll
       for (int k = 0; k < 16; ++k) upk2(acc2[k], acc[2 * k], acc[2 * k + 1]);
-      float sq, ps;
       {
         float x0, x1;
         upk2(sq2, x0, x1);
-        sq = x0 + x1;
+        const double sq = static_cast<double>(x0 + x1);
         upk2(ps2, x0, x1);
-        ps = x0 + x1;
+        // (sum of p log2 p of this thread's part of the item)
+        *sums = make_double2(sums->x + sq, sums->y + static_cast<double>(fmaf(x0 + x1, c2, -lsum)));
       }
-      float ent = fmaf(ps, c2, -lsum);                 // sum of p log2 p of this thread's part of the item
-      // the item's tile of sum_n A^(n): written, or added to what earlier calls left
-      if (p.use_tma) {
-        // through shared memory and one TMA store per 32-column box: coalesced, and it drains while the next item
-        // computes.  The previous item's box has been read out before it is overwritten; the four warps of the
-        // group also agree here whether a wait has been abandoned.
+      // The item's tile of sum_n A^(n), written, or added to what earlier calls left, goes through shared memory.  By TMA: one store
+      // per 32-column box, which drains while the next item computes.  The previous item's box has been read out before it is
+      // overwritten; the four warps of the group also agree here whether a wait has been abandoned.
+      if (TMA) {
         if (!ACC && lead) bulk_wait_group_read0();
         if (ACC && box_ok) {
           if (ok && !mbar_wait_warp(old_full + cq, nold & 1, wc, C_OLD_FULL)) ok = false;
           ++nold;
         }
         if (named_bar_or(1 + cq, 128, !ok)) break;
-        const uint32_t stage_row = smem_u32(box) + rowl * 128;
+      } else {
+        if (!ok) break;
+        if (ACC) asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncwarp();
+      }
+      const uint32_t stage_row = box_a + rowl * 128;
 #pragma unroll
-        for (int g = 0; g < 8; ++g) {
-          const uint32_t chunk = static_cast<uint32_t>(g ^ (rowl & 7)) * 16;
-          float o0 = 0.0f, o1 = 0.0f, o2 = 0.0f, o3 = 0.0f;
-          if (ACC) ld_shared_v4f(stage_row + chunk, o0, o1, o2, o3);
-          st_shared_v4w(stage_row + chunk, __float_as_uint(acc[4 * g] + o0), __float_as_uint(acc[4 * g + 1] + o1),
-                        __float_as_uint(acc[4 * g + 2] + o2), __float_as_uint(acc[4 * g + 3] + o3));
-        }
+      for (int g = 0; g < 8; ++g) {
+        const uint32_t chunk = static_cast<uint32_t>(g ^ (rowl & 7)) * 16;
+        float o0 = 0.0f, o1 = 0.0f, o2 = 0.0f, o3 = 0.0f;
+        if (ACC) ld_shared_v4f(stage_row + chunk, o0, o1, o2, o3);
+        st_shared_v4w(stage_row + chunk, __float_as_uint(acc[4 * g] + o0), __float_as_uint(acc[4 * g + 1] + o1),
+                      __float_as_uint(acc[4 * g + 2] + o2), __float_as_uint(acc[4 * g + 3] + o3));
+      }
+      if (TMA) {
         fence_proxy_async_smem();
         named_bar_sync(5 + cq, 128);
         if (lead && box_ok) {
@@ -291,25 +360,13 @@ saf_calib_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
           bulk_commit_group();
         }
       } else {
-        // row lengths that are no multiple of four floats cannot be described to TMA: plain loads and stores
-        if (!ok) break;
-        if (qi < p.T) {
-          float* dst = p.mean_sum + (static_cast<size_t>(h) * p.T + qi) * p.T + k0;
-#pragma unroll
-          for (int e = 0; e < 32; ++e)
-            if (k0 + e < p.T) dst[e] = ACC ? dst[e] + acc[e] : acc[e];
-        }
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        sq += __shfl_xor_sync(0xffffffffu, sq, o);
-        ent += __shfl_xor_sync(0xffffffffu, ent, o);
-      }
-      if (lane == 0) {
-        atomicAdd(p.sumsq + h, static_cast<double>(sq));
-        atomicAdd(p.sum_plogp + h, static_cast<double>(ent) * LN2_C);
+        __syncwarp();
+#pragma unroll 8
+        for (int r = 0; r < rows; ++r) old[static_cast<size_t>(r) * p.T] = *reinterpret_cast<const float*>(box + (box_addr(r) - box_a));
+        __syncwarp();
       }
     }
+    flush();
     if ((tid & 127) == 0) bulk_wait_group0();          // every store has landed before the kernel ends
   }
 
@@ -413,22 +470,24 @@ __global__ void saf_calib_scores_kernel(const double* __restrict__ sumsq, const 
 }  // namespace
 
 
-template <int D, bool ACC>
+template <int D, bool ACC, bool TMA>
 static cudaError_t launch_calib_t(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mm,
                                   const CalibParams& p, int grid, cudaStream_t st) {
-  cudaError_t e = cudaFuncSetAttribute(saf_calib_kernel<D, ACC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  cudaError_t e = cudaFuncSetAttribute(saf_calib_kernel<D, ACC, TMA>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        CalCfg<D>::SMEM);
   if (e != cudaSuccess) return e;
-  saf_calib_kernel<D, ACC><<<grid, CalCfg<D>::NTHREADS, CalCfg<D>::SMEM, st>>>(mq, mk, mm, p);
+  saf_calib_kernel<D, ACC, TMA><<<grid, CalCfg<D>::NTHREADS, CalCfg<D>::SMEM, st>>>(mq, mk, mm, p);
   return cudaGetLastError();
 }
 
 cudaError_t launch_calib(int D, const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mm,
                          const CalibParams& p, int grid, cudaStream_t st) {
-  if (D == 64) return p.accumulate ? launch_calib_t<64, true>(mq, mk, mm, p, grid, st)
-                                   : launch_calib_t<64, false>(mq, mk, mm, p, grid, st);
-  return p.accumulate ? launch_calib_t<128, true>(mq, mk, mm, p, grid, st)
-                      : launch_calib_t<128, false>(mq, mk, mm, p, grid, st);
+#define SAF_CALIB(DD) (p.accumulate ? p.use_tma ? launch_calib_t<DD, true, true>(mq, mk, mm, p, grid, st)         \
+                                                : launch_calib_t<DD, true, false>(mq, mk, mm, p, grid, st)        \
+                                    : p.use_tma ? launch_calib_t<DD, false, true>(mq, mk, mm, p, grid, st)        \
+                                                : launch_calib_t<DD, false, false>(mq, mk, mm, p, grid, st))
+  return D == 64 ? SAF_CALIB(64) : SAF_CALIB(128);
+#undef SAF_CALIB
 }
 
 // Two vectors of n doubles to zero (one launch instead of two memsets).

@@ -254,7 +254,6 @@ struct CalibParams {
   double* sum_plogp;                // [H] += sum_n sum A_n log A_n
   int accumulate;                   // 0: overwrite mean_sum tiles, 1: add to them
   int use_tma;                      // T % 4 == 0: tiles leave by TMA; else plain loads / stores
-  int n_items, npairs;              // items = H x npairs, npairs = nblk (nblk+1)/2
   int* status;
   unsigned long long wait_limit_ns;
 };

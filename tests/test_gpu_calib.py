@@ -149,3 +149,12 @@ def test_invalid_arguments():
         with pytest.raises(saf.SafError) as e:
             call()
         assert e.value.code == saf.SAF_ERR_INVALID_ARG
+
+
+# Five heads of 17 blocks: 680 tiles below the diagonal, 4.6 a CTA, so that runs of four, single tiles and diagonal ones occur; rows
+# that TMA describes (2052) and not (2049, 2050), ragged last blocks of 1, 2 and 4.
+@pytest.mark.parametrize("T", [2049, 2050, 2052])
+def test_runs_singles_and_diagonal_items_in_adding_calls(T):
+    wl = _workload(3, 5, T, 64, seed=T)
+    L = Layer(si.generate(wl), backward=False)
+    _check(L, *_run(L, splits=2), heads=(0, 4))
