@@ -46,7 +46,7 @@ def load_library() -> C.CDLL:
     if not os.path.exists(LIB_PATH):
         raise FileNotFoundError(f"{LIB_PATH} not built; run `python -m paper_2609_34650_b200.build`")
     lib = C.CDLL(LIB_PATH)
-    vp, i32, u8p, f32p = C.c_void_p, C.c_int32, C.c_char_p, C.c_void_p
+    vp, i32, u8p, f32p = C.c_void_p, C.c_int32, C.c_void_p, C.c_void_p
     pp = C.POINTER(SafProblem)
     lib.saf_version.restype = C.c_int
     lib.saf_status_string.restype = C.c_char_p
