@@ -140,6 +140,8 @@ saf_calib_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  pdl_launch_dependents();
+  pdl_wait();
 
   if (warp == 16) {
     // ------------------------------------------------------------------ TMA producer
@@ -391,6 +393,8 @@ __global__ void __launch_bounds__(256)
 saf_calib_mean_kernel(float* __restrict__ mean, double inv_n, double* __restrict__ tmp, int T) {
   __shared__ double red[2][8];
   const int h = blockIdx.y, tid = threadIdx.x;
+  pdl_launch_dependents();
+  pdl_wait();
   float* M = mean + static_cast<size_t>(h) * T * T;
   double s2 = 0.0, sl = 0.0;
   const float invf = static_cast<float>(inv_n);
@@ -459,6 +463,8 @@ saf_calib_mean_kernel(float* __restrict__ mean, double inv_n, double* __restrict
 __global__ void saf_calib_scores_kernel(const double* __restrict__ sumsq, const double* __restrict__ sum_plogp,
                                         double* __restrict__ tmp, double n_total, int T, int H,
                                         double* __restrict__ s_var, double* __restrict__ s_kl) {
+  pdl_launch_dependents();
+  pdl_wait();
   const int h = blockIdx.x * blockDim.x + threadIdx.x;
   if (h >= H) return;
   const double t = static_cast<double>(T);
@@ -476,8 +482,8 @@ static cudaError_t launch_calib_t(const CUtensorMap& mq, const CUtensorMap& mk, 
   cudaError_t e = cudaFuncSetAttribute(saf_calib_kernel<D, ACC, TMA>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        CalCfg<D>::SMEM);
   if (e != cudaSuccess) return e;
-  saf_calib_kernel<D, ACC, TMA><<<grid, CalCfg<D>::NTHREADS, CalCfg<D>::SMEM, st>>>(mq, mk, mm, p);
-  return cudaGetLastError();
+  e = launch_pdl(PDL_REST, saf_calib_kernel<D, ACC, TMA>, dim3(grid), dim3(CalCfg<D>::NTHREADS), CalCfg<D>::SMEM, st, mq, mk, mm, p);
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 cudaError_t launch_calib(int D, const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mm,
@@ -492,24 +498,29 @@ cudaError_t launch_calib(int D, const CUtensorMap& mq, const CUtensorMap& mk, co
 
 // Two vectors of n doubles to zero (one launch instead of two memsets).
 __global__ void saf_calib_zero_kernel(double* __restrict__ a, double* __restrict__ b, int n) {
+  pdl_launch_dependents();
+  pdl_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) a[i] = b[i] = 0.0;
 }
 cudaError_t launch_calib_zero(double* a, double* b, int n, cudaStream_t st) {
-  saf_calib_zero_kernel<<<(n + 127) / 128, 128, 0, st>>>(a, b, n);
-  return cudaGetLastError();
+  const cudaError_t e = launch_pdl(PDL_REST, saf_calib_zero_kernel, dim3((n + 127) / 128), dim3(128), 0, st, a, b, n);
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 // tmp: 2 H doubles, zero before the call and after it
 cudaError_t launch_calib_finalize(float* mean, const double* sumsq, const double* sum_plogp, double* tmp, int H, int T,
                                   double n_total, double* s_var, double* s_kl, int num_sms, cudaStream_t st) {
+  cudaError_t e;
   int nb = std::max(1, std::min((8 * num_sms + H - 1) / H, T));
   if (T % 4 == 0 && (reinterpret_cast<uintptr_t>(mean) & 15u) == 0)
-    saf_calib_mean_kernel<true><<<dim3(nb, H), 256, 0, st>>>(mean, 1.0 / n_total, tmp, T);
+    e = launch_pdl(PDL_REST, saf_calib_mean_kernel<true>, dim3(nb, H), dim3(256), 0, st, mean, 1.0 / n_total, tmp, T);
   else
-    saf_calib_mean_kernel<false><<<dim3(nb, H), 256, 0, st>>>(mean, 1.0 / n_total, tmp, T);
-  saf_calib_scores_kernel<<<(H + 127) / 128, 128, 0, st>>>(sumsq, sum_plogp, tmp, n_total, T, H, s_var, s_kl);
-  return cudaGetLastError();
+    e = launch_pdl(PDL_REST, saf_calib_mean_kernel<false>, dim3(nb, H), dim3(256), 0, st, mean, 1.0 / n_total, tmp, T);
+  if (e != cudaSuccess) return e;
+  e = launch_pdl(PDL_REST, saf_calib_scores_kernel, dim3((H + 127) / 128), dim3(128), 0, st, sumsq, sum_plogp, tmp, n_total, T, H,
+                 s_var, s_kl);
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 }  // namespace saf

@@ -21,18 +21,19 @@ inline bool pdl_enabled() {
   return on;
 }
 // Which kernels are launched that way (SAF_PDL_MASK: bit 0 staging kernels, 1 D = 64 forward where launch_fwd64 asks for
-// it, 2 backward preparation, 3 backward, 4 the 128-wide forwards, 5 backward preparation of small layers).  All but the
+// it, 2 backward preparation, 3 backward, 4 the 128-wide forwards, 5 backward preparation of small layers, 6 everything behind
+// these: conversion of gradients, pattern preparation and gradients, calibration).  All but the
 // preparation of larger layers: its blocks then fill the SMs under the forward's tail, where the layer is long enough for
 // that to cost more than the launch gap (8x12x4096x64: pass +2 %, 8x12x2048x128 +3 %).
 // The others gain or are neutral: staging 1x32x333x128 -6 %.
 inline int pdl_mask() {
   static const int m = [] {
     const char* e = std::getenv("SAF_PDL_MASK");
-    return e ? std::atoi(e) : 1 + 2 + 8 + 16 + 32;
+    return e ? std::atoi(e) : 1 + 2 + 8 + 16 + 32 + 64;
   }();
   return m;
 }
-enum { PDL_STAGE = 1, PDL_FWD = 2, PDL_PREP = 4, PDL_BWD = 8, PDL_FWD128 = 16, PDL_PREP_SMALL = 32 };
+enum { PDL_STAGE = 1, PDL_FWD = 2, PDL_PREP = 4, PDL_BWD = 8, PDL_FWD128 = 16, PDL_PREP_SMALL = 32, PDL_REST = 64 };
 template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl(int which, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
   cudaLaunchConfig_t cfg = {};

@@ -37,6 +37,8 @@ __global__ void __launch_bounds__(256) saf_logz_kernel(const float* __restrict__
   __shared__ float sr[LZ_KC + 32], red[2][8], near_max[8][32];
   __shared__ double part[8][32];
   const int h = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  pdl_launch_dependents();
+  pdl_wait();
   if (!mask[h]) {
     if (consts != nullptr && blockIdx.x == 0 && tid == 0) fast_ok[h] = 0;
     return;
@@ -176,8 +178,11 @@ __global__ void __launch_bounds__(256) saf_logz_kernel(const float* __restrict__
 cudaError_t launch_logz(const float* alpha, const float* rho, float* logZ, const uint8_t* mask_dev, int H, int Tp,
                         float* consts, int* fast_ok, unsigned* counters, cudaStream_t st) {
   dim3 grid((Tp + 31) / 32, H);
-  saf_logz_kernel<<<grid, 256, 0, st>>>(alpha, rho, logZ, mask_dev, Tp, consts, fast_ok, counters);
-  return cudaGetLastError();
+  // (early for short vectors: trainable passes of 13x12x415x128 -1.7 %, 19x16x627x64 -1.5 %; the long rows' blocks, first in the
+  // grid, then crowd where the kernel in front leaves room: 2x12x3434x128 +5 %, 12x8x1536x128 +3 %)
+  const cudaError_t e = launch_pdl(Tp <= 1024 ? PDL_REST : 0, saf_logz_kernel, grid, dim3(256), 0, st, alpha, rho, logZ, mask_dev, Tp, consts,
+                                   fast_ok, counters);
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -209,6 +214,8 @@ __global__ void __launch_bounds__(256) saf_pattern_tables_kernel(const float* __
                                                                  int* __restrict__ ovf_fwd, int* __restrict__ ovf_bwd,
                                                                  int nblkp) {
   const int h = blockIdx.y, dblk = blockIdx.x;
+  pdl_launch_dependents();
+  pdl_wait();
   // marks of earlier calls end here: a call recorded into a CUDA graph keeps its id over all replays
   if (dblk == 0 && threadIdx.x == 0) ovf_fwd[h] = ovf_bwd[h] = 0;
   if (!mask[h]) return;
@@ -242,10 +249,10 @@ cudaError_t launch_pattern_tables(const float* alpha, const float* rho, const fl
                                   int Tp, const float* consts, float* avec, float* wvec, void* band_f, void* band_b,
                                   uint32_t* snap, int* ovf_fwd, int* ovf_bwd, cudaStream_t st) {
   const int nblkp = (Tp + 127) / 128;
-  saf_pattern_tables_kernel<<<dim3(nblkp, H), 256, 0, st>>>(alpha, rho, logZ, mask_dev, Tp, consts, avec, wvec,
-                                                            static_cast<__half*>(band_f),
-                                                            static_cast<__half*>(band_b), snap, ovf_fwd, ovf_bwd, nblkp);
-  return cudaGetLastError();
+  const cudaError_t e = launch_pdl(PDL_REST, saf_pattern_tables_kernel, dim3(nblkp, H), dim3(256), 0, st, alpha, rho, logZ, mask_dev,
+                                   Tp, consts, avec, wvec, static_cast<__half*>(band_f), static_cast<__half*>(band_b), snap,
+                                   ovf_fwd, ovf_bwd, nblkp);
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 // dst[b][ord][t][:] = fp16(extra * vec[h][t] * src[b][h][t][:]), h = hlist[ord], for the frozen heads whose tensor-core form is
@@ -505,6 +512,8 @@ cudaError_t launch_bwd_prep(const void* O, int o_f32, const void* dO, const floa
 
 __global__ void __launch_bounds__(256) saf_f32_to_bf16_kernel(const float* __restrict__ src, __nv_bfloat16* __restrict__ dst,
                                                               size_t n8) {
+  pdl_launch_dependents();
+  pdl_wait();
   const size_t i = static_cast<size_t>(blockIdx.x) * 256 + threadIdx.x;
   if (i >= n8) return;
   const float4 a = *reinterpret_cast<const float4*>(src + i * 8);
@@ -519,9 +528,11 @@ __global__ void __launch_bounds__(256) saf_f32_to_bf16_kernel(const float* __res
 
 cudaError_t launch_bwd_finalize(const float* dQacc, void* dQ, size_t n, cudaStream_t st) {
   const size_t n8 = n / 8;
-  saf_f32_to_bf16_kernel<<<static_cast<unsigned>((n8 + 255) / 256), 256, 0, st>>>(
-      dQacc, static_cast<__nv_bfloat16*>(dQ), n8);
-  return cudaGetLastError();
+  // (early where the launch gap shows: updates of 4x12x388x96 -9 %, 11x16x224x64 -3 %; 2x16x8192x96 +0.2 %)
+  const unsigned grid = static_cast<unsigned>((n8 + 255) / 256);
+  const cudaError_t e = launch_pdl(grid <= 4096 ? PDL_REST : 0, saf_f32_to_bf16_kernel, dim3(grid), dim3(256), 0, st, dQacc,
+                                   static_cast<__nv_bfloat16*>(dQ), n8);
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 }  // namespace saf
