@@ -30,6 +30,7 @@ struct WorklistEntry {
   WorkItem* items_dev = nullptr;          // WL_QUEUE: in queue order; else grouped by CTA
   int* offsets_dev = nullptr;
   int n_items = 0;
+  bool split = false;                     // some items are KIND_SPLIT
 };
 
 struct DevBuf {
@@ -294,18 +295,24 @@ void build_worklist_host(int B, int H, int T, const uint8_t* mask, int backward,
   (*offsets)[n_ctas] = static_cast<int>(items->size());
 }
 
-// Work queue of the 128-wide forward, whose items are two consecutive query blocks of one (batch, head) unit (the first
-// block of an odd count goes alone).  CTAs claim items in this order at run time, so longest-first within groups of
+// Work queue of the 128-wide forward.  An item is two consecutive query blocks of one (batch, head) unit (the first
+// block of an odd count goes alone), which share every K and V tile, or one block: of an ordinary head split over the
+// kernel's two chains (even and odd key tiles), of a frozen head in one.  Single blocks halve the longest items where these would
+// set the time, at the cost of twice the loads and item ends; which blocks go alone is decided by build_pair_order.
+// CTAs claim items in this order at run time, so longest-first within groups of
 // units keeps both the tail short and a group's K and V in L2 while its items run.  Group sizes differ by at most one unit (a
 // small last group is a tail of long items: 2x16x8192x96 0.456 ms with groups of 10, 10, 10 and 2 units, 0.373 with two of 16),
 // as many groups as hold 64 MB of K and V each (8x12x4096x128: 32 MB 0.335 ms, 64 MB 0.339, 128 MB 0.346; 1x16x16384x128:
-// 0.778, 0.760, 0.758), K and V counted per query head where heads share them.  While the items would not fill the SMs,
-// blocks go one by one: a pair takes longer than a single block and there are SMs to spare.  An item's fixed cost does not
+// 0.778, 0.760, 0.758), K and V counted per query head where heads share them.  An item's fixed cost does not
 // change the order; a frozen tile counts frozen_pct percent of an ordinary one.
-void build_pair_order(int B, int H, int T, int D, const uint8_t* mask, int num_sms, int frozen_pct, std::vector<WorkItem>& order) {
+// cap: a pair that takes longer (in ns, by pair_item_ns) is dissolved.
+long long pair_item_ns(int tiles, bool pair, bool ordinary) {     // tiles: of the item's later block
+  if (!ordinary) return (pair ? 2 * tiles - 1 : tiles) * 550LL + 2500;
+  return (pair ? tiles * 2100LL : (tiles + 1) / 2 * 2400LL) + 3000;
+}
+void build_pair_order(int B, int H, int T, int D, const uint8_t* mask, int frozen_pct, long long cap, std::vector<WorkItem>& order) {
   const int nblk = (T + BLK - 1) / BLK;
   const long long units = static_cast<long long>(B) * H;
-  const bool pair = units * nblk > num_sms;
   const long long n_groups = std::min(units, std::max<long long>(1, (static_cast<long long>(T) * D * 4 * units + (64ll << 20) - 1) / (64ll << 20)));
   order.clear();
   std::vector<std::pair<long long, WorkItem>> items;
@@ -314,10 +321,12 @@ void build_pair_order(int B, int H, int T, int D, const uint8_t* mask, int num_s
     for (long long u = units * g / n_groups; u < units * (g + 1) / n_groups; ++u) {
       const int b = static_cast<int>(u / H), h = static_cast<int>(u % H);
       const int kind = mask[h] ? KIND_FROZEN : KIND_ORDINARY;
-      for (int q = nblk - 1; q >= 0; q -= pair ? 2 : 1) {
-        const bool two = pair && q > 0;
-        const long long tiles = two ? 2 * q + 1 : q + 1;
-        items.push_back({(mask[h] ? frozen_pct : 100) * tiles, WorkItem{b, h, q, kind | (two ? KIND_PAIR : 0)}});
+      for (int q = nblk - 1; q >= 0;) {
+        const bool two = q > 0 && pair_item_ns(q + 1, true, !mask[h]) <= cap, split = !two && q > 0 && !mask[h];
+        // (half tiles: a split block takes half the time of a pair of the same length)
+        const long long half = two ? 2 * (2 * q + 1) : split ? q + 1 : 2 * (q + 1);
+        items.push_back({(mask[h] ? frozen_pct : 100) * half, WorkItem{b, h, q, kind | (two ? KIND_PAIR : split ? KIND_SPLIT : 0)}});
+        q -= two ? 2 : 1;
       }
     }
     std::stable_sort(items.begin(), items.end(),
@@ -325,21 +334,57 @@ void build_pair_order(int B, int H, int T, int D, const uint8_t* mask, int num_s
     for (const auto& it : items) order.push_back(it.second);
   }
 }
+// The order whose simulated run on num_sms CTAs ends first, over a few caps between "all blocks alone" and "all in pairs", while
+// there are up to three blocks per SM (beyond, the pairs' tail is short and the longer loads of single blocks count: 1x16x8192x128
+// 247 us in pairs, 268 alone).  us of back-to-back forwards without frozen heads, pairs (blocks alone and in one chain up to
+// one per SM) / this: 1x32x333x128 12.2 / 11.7, 1x8x1024x128 20.0 / 16.1, 1x8x2048x128 34.5 / 25.6, 1x16x1300x128 29.4 / 21.2,
+// 1x8x4096x128 70.7 / 43.6, 1x4x8192x128 132 / 76, 1x12x4096x128 72.7 / 68.3, 4x12x900x128 28.2 / 28.2.
+void build_wide_order(int B, int H, int T, int D, const uint8_t* mask, int num_sms, int frozen_pct, std::vector<WorkItem>& order) {
+  const int nblk = (T + BLK - 1) / BLK;
+  const long long forever = 1LL << 60;
+  const long long blocks = static_cast<long long>(B) * H * nblk;
+  if (blocks <= num_sms) return build_pair_order(B, H, T, D, mask, frozen_pct, 0, order);
+  if (blocks > 3LL * num_sms) return build_pair_order(B, H, T, D, mask, frozen_pct, forever, order);
+  std::vector<WorkItem> trial;
+  long long work = 0, best = -1;
+  build_pair_order(B, H, T, D, mask, frozen_pct, forever, trial);
+  auto ns = [](const WorkItem& w) {
+    return pair_item_ns(w.blk + 1, (w.kind & KIND_PAIR) != 0, (w.kind & 0x7f) == KIND_ORDINARY);
+  };
+  for (const WorkItem& w : trial) work += ns(w);
+  for (int k = 8; k >= 0; --k) {                      // caps in quarters of the mean load, from none to twice; first: all pairs
+    build_pair_order(B, H, T, D, mask, frozen_pct, k == 8 ? forever : work / num_sms * k / 4, trial);
+    std::priority_queue<long long, std::vector<long long>, std::greater<long long>> free_at;
+    for (int c = 0; c < num_sms; ++c) free_at.push(0);
+    long long end = 0;
+    for (const WorkItem& w : trial) {
+      const long long t = free_at.top() + ns(w);
+      free_at.pop();
+      free_at.push(t);
+      end = std::max(end, t);
+    }
+    if (k == 8) end = end * 97 / 100;                 // (pairs unless the gain is clear)
+    if (best < 0 || end < best) {
+      best = end;
+      order.swap(trial);
+    }
+  }
+}
 
 // Whether a 128-wide forward goes to the kernel of short sequences (one query block per item, two CTAs per SM).  The line
 // lies where the two cross (us of back-to-back forwards, no frozen head; this kernel / the two-block kernel):
 //   up to two blocks a unit: 32x16x64x128 14.2 / 20.9, 12x16x256x128 16.6 / 20.9, 32x16x256x128 41.5 / 41.9
 //   three: up to about four (head dimension 96: eight) blocks per SM: 6x16x384x128 16.2 / 17.9, 16x16x384x128 36.5 / 33.3
-//   up to six: while the two-block items are one wave and a little: 6x16x512x128 20.4 / 25.0, 8x16x512x128 26.4 / 25.2
-//   up to ten: while the blocks are: 1x32x640x128, one forward waited for, 34.4 / 36.8
+//   up to six: while the two-block items are one wave and a little: 6x16x512x128 20.4 / 25.4, 8x16x512x128 26.4 / 25.2
+//   (where these are less than a wave, the other kernel's split blocks are faster: 4x12x500x128 17.6 / 15.5, 1x32x640x128
+//   19.0 / 15.6, 2x12x1000x128 26.8 / 19.1)
 bool fwd_is_short(int B, int H, int T, int D, int num_sms) {
   const long long units = static_cast<long long>(B) * H, nblk = (T + BLK - 1) / BLK, blocks = units * nblk;
-  if (blocks <= num_sms) return false;                    // (one block per CTA and SM either way, and the same time)
+  if (blocks <= num_sms) return false;                    // (one block per CTA and SM either way)
   if (nblk <= 2) return true;
   if (nblk == 3) return blocks <= (D == 96 ? 8LL : 4LL) * num_sms;
   const long long items = units * ((nblk + 1) / 2);       // of the two-block kernel
-  if (nblk <= 6 && items > num_sms && 5 * items <= 8LL * num_sms) return true;
-  return nblk <= 10 && 10 * blocks <= 13LL * num_sms;
+  return nblk <= 6 && items > num_sms && 5 * items <= 8LL * num_sms;
 }
 
 // Measured cost-model defaults: `wide` = the 128-wide kernels (head dimension 96 or 128), else the 64-wide ones.
@@ -378,7 +423,7 @@ int get_worklist(saf_ctx* ctx, int B, int H, int T, int D, const uint8_t* mask, 
   const bool lists = kind != WL_QUEUE;
   WorklistEntry e;
   if (!lists && wide) {
-    build_pair_order(B, H, T, D, mask, ctx->num_sms, frozen_pct, e.items_host);
+    build_wide_order(B, H, T, D, mask, ctx->num_sms, frozen_pct, e.items_host);
   } else {
     // (tail: two items per CTA; on the 128-wide backward four: -0.5 % on 8x12x4096x128, -1 % on 2x16x8192x96, -3 % on
     // 1x16x8192x128 and on shared heads 3x8x3000x128; six and eight are no better)
@@ -389,6 +434,7 @@ int get_worklist(saf_ctx* ctx, int B, int H, int T, int D, const uint8_t* mask, 
   e.B = B; e.H = H; e.T = T; e.D = D; e.kind = kind; e.grid = grid;
   e.mask.assign(mask, mask + H);
   e.n_items = static_cast<int>(e.items_host.size());
+  for (const WorkItem& w : e.items_host) e.split |= (w.kind & KIND_SPLIT) != 0;
   auto give_up = [&](int code) {
     cudaFree(e.items_dev);
     cudaFree(e.offsets_dev);
@@ -732,6 +778,7 @@ int saf_hybrid_attn_fwd(saf_ctx* ctx, const saf_problem* p, const void* Q, const
   fp.items = wl->items_dev;
   fp.cta_offsets = wl->offsets_dev;
   fp.n_items = wl->n_items;
+  fp.split = wl->split;
   fp.queue = ctx->queue_dev;
   fp.status = ctx->status_dev;
   fp.wait_limit_ns = ctx->wait_limit_ns;

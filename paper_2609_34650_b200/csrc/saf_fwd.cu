@@ -1,4 +1,4 @@
-// Forward of the hybrid causal attention layer on sm_100a, two query blocks per work item: one persistent kernel for
+// Forward of the hybrid causal attention layer on sm_100a, two chains of tiles per work item: one persistent kernel for
 // ordinary (flash-style online softmax) and frozen (pattern rebuilt from alpha/rho/logZ) heads.
 //
 // One CTA per SM, 512 threads: warps 0-3 softmax of query block 0 of the item, warps 4-7 of query block 1 (one thread
@@ -16,6 +16,10 @@
 //   row sum in registers, P_t -> TMEM as bf16 over S_t, O_t += P_t V_J; the next score MMA of a block is queued
 //   directly behind the MMA that consumes its P (MMAs of one thread execute in order).  The first scores of the next
 //   item go out as soon as block 0 of this one has its last P V MMA, so no softmax warp idles between items.
+// Split item: one query block, its even key tiles in the first chain and the odd ones in the second, each with running
+//   maximum, row sum and accumulator of its own; chain 1 hands maximum and sum to chain 0, which forms the factors
+//   with which the epilogue adds the two accumulators.  It takes half the time of a pair of its length (a pair of tiles 2.2 us
+//   either way) but loads every K and V tile for one block: for grids whose longest items would set the time.
 // Frozen item, tensor-core form (pattern tables prepared and the head's flag set): with global maxima,
 //   O = diag(w) R (diag(a) V), R(i,j) = r(i-j).  A tile of R with reversed rows is a Hankel matrix that the tensor
 //   core reads straight from a 4 KB band table (no-swizzle descriptor, both strides 128 bytes), so a tile is two bulk
@@ -63,10 +67,11 @@ struct FwdCfg {
   static constexpr int OFF_KV = 2 * TILE_BYTES;
   static constexpr int OFF_BAND = OFF_KV + NS * TILE_BYTES;   // 2 x 4 KB of Hankel bands per ring stage
   static constexpr int OFF_LINV = OFF_BAND + NS * 8192;       // [2][128] 1 / row sum
-  static constexpr int OFF_BAR = OFF_LINV + 2 * 128 * 4;
+  static constexpr int OFF_XM = OFF_LINV + 2 * 128 * 4;       // [128] split items: chain 1's reference
+  static constexpr int OFF_BAR = OFF_XM + 128 * 4;
   static constexpr int NRING = 4;                       // work-item records in flight
   static constexpr int CLAIM_AHEAD = 4;
-  static constexpr int NBAR = 2 * NS + 14 + 2 * NRING;
+  static constexpr int NBAR = 2 * NS + 15 + 2 * NRING;
   static constexpr int OFF_RING = (OFF_BAR + NBAR * 8 + 16 + 15) / 16 * 16;
   static constexpr int SMEM = OFF_RING + NRING * 16 + 1024;   // + slack for 1024-byte alignment
   static constexpr int TMEM_COLS = 512;
@@ -77,18 +82,20 @@ constexpr int TAB_FLOATS = 784;                         // one tile's tables of 
 static_assert(2 * TAB_FLOATS * 4 <= FwdCfg::TILE_BYTES, "the tables fit into a query tile");
 
 enum FwdSite { SITE_Q_EMPTY = 1, SITE_KV_EMPTY, SITE_Q_FULL, SITE_KV_FULL, SITE_P_FULL, SITE_O_FREE, SITE_S_FULL,
-               SITE_O_FULL, SITE_L_FULL, SITE_RING_EMPTY, SITE_RING_FULL };
+               SITE_O_FULL, SITE_L_FULL, SITE_RING_EMPTY, SITE_RING_FULL, SITE_X_FULL };
 
 constexpr int RING_FAST = 1 << 8;
 constexpr int RING_END = -1;
 
-// A work item as the roles see it.  n1 = key tiles of query block `blk` (tile 1), n0 = key tiles of query block blk - 1
-// (tile 0; 0: the item has one query block).
+// A work item as the roles see it: two chains of score MMA, softmax and P V MMA.  n1 = key tiles of query block `blk`
+// (chain 1), n0 = key tiles of query block blk - 1 (chain 0; 0: the item has one query block).  Split: both chains work on
+// block `blk`, chain 0 on its even key tiles and chain 1 on the odd ones.  tiles = key tiles loaded.
 struct ItemView {
-  int b, h, blk, kind, n0, n1;
-  bool fast;
+  int b, h, blk, kind, n0, n1, tiles;
+  bool fast, split;
 };
 
+template <bool SPLIT>
 __device__ __forceinline__ bool ring_take(const int4* ring, uint64_t* ring_full, uint64_t* ring_empty, uint32_t n,
                                           const WaitCtx& wc, ItemView& v) {
   const uint32_t slot = n % FwdCfg::NRING;
@@ -100,13 +107,17 @@ __device__ __forceinline__ bool ring_take(const int4* ring, uint64_t* ring_full,
   v.blk = raw.z;
   v.kind = raw.w < 0 ? RING_END : (raw.w & 0x7f);
   v.fast = raw.w >= 0 && (raw.w & RING_FAST) != 0;
-  v.n1 = raw.z + 1;
-  v.n0 = (raw.w & KIND_PAIR) ? raw.z : 0;
+  v.split = SPLIT && raw.w >= 0 && (raw.w & KIND_SPLIT) != 0;
+  v.tiles = raw.z + 1;
+  v.n1 = v.split ? v.tiles >> 1 : v.tiles;
+  v.n0 = v.split ? v.tiles - v.n1 : (raw.w & KIND_PAIR) ? raw.z : 0;
   return true;
 }
 
 }  // namespace
 
+// SPLIT: the list holds split items (the issuer's extra conditions cost lists without them 1.6 %, 4x32x4096x128 on shared heads)
+template <bool SPLIT>
 __global__ void __launch_bounds__(FwdCfg::NTHREADS, 1)
 saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ CUtensorMap mk,
                const __grid_constant__ CUtensorMap mv, const __grid_constant__ CUtensorMap mvt, const FwdParams p) {
@@ -124,12 +135,14 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
   uint64_t* o_full = p_full + 2;                 // [2] last MMA into O_t has completed
   uint64_t* o_free = o_full + 2;                 // [2] epilogue has read O_t (4 warp arrivals)
   uint64_t* l_full = o_free + 2;                 // [2] 1 / row sum of block t written (4 warp arrivals)
-  uint64_t* ring_full = l_full + 2;              // [NRING] record n has been published by the producer
+  uint64_t* x_full = l_full + 2;                 // split items: row sums and references of chain 1 written (4 warp arrivals)
+  uint64_t* ring_full = x_full + 1;              // [NRING] record n has been published by the producer
   uint64_t* ring_empty = ring_full + C::NRING;   // [NRING] issuer + 8 softmax warps + 4 epilogue warps have copied it
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(ring_empty + C::NRING);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   int4* ring = reinterpret_cast<int4*>(smem + C::OFF_RING);
   float* linv = reinterpret_cast<float*>(smem + C::OFF_LINV);
+  float* xm = reinterpret_cast<float*>(smem + C::OFF_XM);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const WaitCtx wc{abort_flag, p.status, p.wait_limit_ns};
@@ -153,6 +166,7 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
       mbar_init(o_free + t, 4);
       mbar_init(l_full + t, 4);
     }
+    mbar_init(x_full, 4);
     for (int k = 0; k < C::NRING; ++k) {
       mbar_init(ring_full + k, 1);
       mbar_init(ring_empty + k, 13);
@@ -264,13 +278,15 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
           const int hv = h / p.kv_group;
           if ((rec.w & 0x7f) == KIND_ORDINARY) {
             const int hq = p.qslot ? p.qslot[h] : h, hk = p.qslot ? hq : hv;
-            // Q_0 and K_0 first: block 0's first scores are issued before this item's predecessor has finished with Q_1
-            if (pair) {
+            // Q_0 and K_0 first: chain 0's first scores are issued before this item's predecessor has finished with Q_1
+            // (a split item has its block's Q in both areas)
+            const bool split = SPLIT && (rec.w & KIND_SPLIT) != 0;
+            if (pair || split) {
               ok = mbar_wait_compact(q_empty, (nq0 & 1) ^ 1, wc, SITE_Q_EMPTY);
               if (!ok) break;
               mbar_expect_tx(q_full, C::TILE_BYTES);
               for (int pn = 0; pn < C::NPANEL; ++pn)
-                tma_load_4d(smem + C::OFF_Q + pn * C::PANEL_BYTES, &mq, q_full, pn * 64, (rec.z - 1) * BLK, hq, b);
+                tma_load_4d(smem + C::OFF_Q + pn * C::PANEL_BYTES, &mq, q_full, pn * 64, (split ? rec.z : rec.z - 1) * BLK, hq, b);
               ++nq0;
             }
             load_kv(&mk, 0, hk);
@@ -281,13 +297,16 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
             for (int pn = 0; pn < C::NPANEL; ++pn)
               tma_load_4d(smem + C::OFF_Q + C::TILE_BYTES + pn * C::PANEL_BYTES, &mq, q_full + 1, pn * 64, rec.z * BLK, hq, b);
             ++nq1;
-            load_kv(&mv, 0, hv);
-            for (int j = 1;; ++j) {
+            // K_0 V_0 K_1 V_1 ...; split: K_0 K_1 V_0 K_2 V_1 ... V_last, in the order of the two chains
+            load_kv(split ? &mk : &mv, split ? 1 : 0, split ? hk : hv);
+            for (int j = split ? 2 : 1;; ++j) {
+              if (ok && split) load_kv(&mv, j - 2, hv);
               if (ok && !claimed && j + C::CLAIM_AHEAD > n1 && (j > 1 || j == n1)) claim();
               if (j == n1 || !ok) break;
               load_kv(&mk, j, hk);
-              if (ok) load_kv(&mv, j, hv);
+              if (ok && !split) load_kv(&mv, j, hv);
             }
+            if (ok && split) load_kv(&mv, n1 - 1, hv);
           } else {
             // general frozen form: the Q areas hold the tables of the softmax warps; an area counts as used by this item
             if (pair) {
@@ -359,11 +378,12 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
       };
       bool early = false;                          // block 0's first scores of `cur` are already issued
       ItemView cur;
-      bool ok = ring_take(ring, ring_full, ring_empty, nrec++, wc, cur);
+      bool ok = ring_take<SPLIT>(ring, ring_full, ring_empty, nrec++, wc, cur);
       while (ok && cur.kind != RING_END) {
         ItemView nxt;
         bool have_next = false;
-        const int n0 = cur.n0, n1 = cur.n1;
+        const int n0 = cur.n0, n1 = cur.n1, tiles = cur.tiles;
+        const bool split = SPLIT && cur.split;
         if (cur.fast) {
           for (int j = 0; j < n1 && ok; ++j, ++n) {
             ok = kv_wait(n);
@@ -394,13 +414,17 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
             // first scores
 #pragma unroll 1
             for (uint32_t t = n0 > 0 && !early ? 0 : 1; t < 2 && ok; ++t) {
-              ok = wait_t(q_full, ph_q, t, SITE_Q_FULL) && kv_wait(n);
+              const uint32_t k0 = split ? n + t : n;
+              ok = wait_t(q_full, ph_q, t, SITE_Q_FULL) && kv_wait(k0);
               if (!ok) break;
               tc_fence_after();
-              issue_qk(t, n);
+              issue_qk(t, k0);
               if (leader && (t ? n1 : n0) == 1) umma_commit(q_empty + t);
             }
-            if (leader) umma_commit(kv_empty + n % C::NS);
+            if (leader) {
+              umma_commit(kv_empty + n % C::NS);
+              if (split) umma_commit(kv_empty + (n + 1) % C::NS);
+            }
             early = false;
           } else if (leader) {
             // general frozen form: P^ written by the softmax warps, one P V per block and tile; s_full says that a
@@ -409,22 +433,31 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
             umma_commit(s_full + 1);
           }
           __syncwarp();
-          for (int j = 0; j < n1 && ok; ++j) {
-            const uint32_t pv = ord ? n + 2 * j + 1 : n + j;       // ring position of V_j; K_{j+1} follows
+          const int steps = split ? n0 : n1;                        // (split: chain 0 has the odd tile, or as many)
+          for (int j = 0; j < steps && ok; ++j) {
+            uint32_t pv = ord ? n + 2 * j + 1 : n + j;             // ring position of V_j; K_{j+1} follows
             const uint32_t acc0 = j > 0 ? 1u : 0u;
             // the tiles' loads land long before P is ready: test their barriers first, so that only one test
             // stands between "P is ready" and the MMAs that wait for it
-            ok = kv_wait(pv) && (!ord || j + 1 == n1 || kv_wait(pv + 1));
+            if (!split) ok = kv_wait(pv) && (!ord || j + 1 == n1 || kv_wait(pv + 1));
 #pragma unroll 1
             for (uint32_t t = j < n0 ? 0 : 1; t < 2 && ok; ++t) {
               const int nt = t ? n1 : n0;
+              if (split) {
+                // tile J = 2 j + t of the block: V_J, followed by K_{J+2}
+                if (j == nt) break;
+                const int J = 2 * j + static_cast<int>(t);
+                pv = J + 1 < tiles ? n + 2 + 2 * J : n + 2 * tiles - 1;
+                ok = kv_wait(pv) && (j + 1 == nt || kv_wait(pv + 1));
+                if (!ok) break;
+              }
               if (j == 0) ok = wait_t(o_free, ph_o, t, SITE_O_FREE);
               if (ok) ok = wait_t(p_full, ph_p, t, SITE_P_FULL);
               if (!ok) break;
               tc_fence_after();
               TRF(0, 2 + 2 * t);
               issue_pv(t, pv, acc0);
-              if (leader && t == 1) umma_commit(kv_empty + pv % C::NS);
+              if (leader && (t == 1 || split)) umma_commit(kv_empty + pv % C::NS);
               uint32_t pos = pv + 1;
               bool qk = ord && j + 1 < nt, last_qk = j + 2 == nt;
               if (j + 1 == nt) {
@@ -435,11 +468,11 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
                 __syncwarp();
                 if (ord && t == 0) {
                   // block 0 is through: its first scores of the next item go out now
-                  ok = ring_take(ring, ring_full, ring_empty, nrec++, wc, nxt);
+                  ok = ring_take<SPLIT>(ring, ring_full, ring_empty, nrec++, wc, nxt);
                   if (!ok) break;
                   have_next = true;
                   if (nxt.kind == KIND_ORDINARY && nxt.n0 > 0) {
-                    pos = n + 2 * n1;
+                    pos = n + 2 * tiles;
                     ok = wait_t(q_full, ph_q, 0, SITE_Q_FULL) && kv_wait(pos);
                     if (!ok) break;
                     tc_fence_after();
@@ -454,7 +487,7 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
               if (qk) {
                 issue_qk(t, pos);                        // executes after P V: same thread, in order
                 if (leader) {
-                  if (t == 1) umma_commit(kv_empty + pos % C::NS);
+                  if ((t == 1 || split) && !(j + 1 == nt)) umma_commit(kv_empty + pos % C::NS);
                   if (last_qk) umma_commit(q_empty + t);
                 }
               }
@@ -462,11 +495,11 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
               TRF(0, 3 + 2 * t);
             }
           }
-          n += ord ? 2 * n1 : n1;
+          n += ord ? 2 * tiles : tiles;
         }
         if (!ok) break;
         if (have_next) cur = nxt;
-        else ok = ring_take(ring, ring_full, ring_empty, nrec++, wc, cur);
+        else ok = ring_take<SPLIT>(ring, ring_full, ring_empty, nrec++, wc, cur);
       }
     }
   } else if (warp < 8) {
@@ -478,20 +511,20 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
     const uint32_t t_s = tmem + lane_base + C::COL_S + 128 * t;       // scores, then bf16 pairs of P in the first 64
     const uint32_t t_o = tmem + lane_base + C::COL_O + D * t;
     const int wg_bar = 1 + t, wg_bar2 = 3 + t;
-    uint32_t ns = 0, nof = 0;                          // phases of s_full[t]; items of this block so far
+    uint32_t ns = 0, nof = 0, nx = 0;                  // phases of s_full[t]; items of this chain so far; split ones
     bool ok = true;
     // A softmax warp whose wait was abandoned keeps walking (without storing) until the next
     // agreement barrier, where its four leave together; none is ever left alone at a barrier.
     for (uint32_t nrec = 0;; ++nrec) {
       ItemView w;
-      if (!ring_take(ring, ring_full, ring_empty, nrec, wc, w)) {
+      if (!ring_take<SPLIT>(ring, ring_full, ring_empty, nrec, wc, w)) {
         ok = false;
-        w.kind = KIND_ORDINARY; w.n0 = w.n1 = 0; w.fast = false; w.b = w.h = w.blk = 0;
+        w.kind = KIND_ORDINARY; w.n0 = w.n1 = w.tiles = 0; w.fast = w.split = false; w.b = w.h = w.blk = 0;
       }
       if (named_bar_or(wg_bar, 128, !ok) || w.kind == RING_END) break;
       const int nt = t == 0 ? w.n0 : w.n1;
       if (nt == 0) continue;
-      const int blk = nt - 1;
+      const int blk = SPLIT && w.split ? w.blk : nt - 1;
       const int row = blk * BLK + rowl;
       if (w.fast) {
         ++nof;
@@ -502,6 +535,7 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
         uint64_t l2a = 0, l2b = 0;                     // packed pairs of partial row sums
         const float c = p.scale_log2;
         const uint64_t c2 = pk2(c, c);
+        const int j_diag = !(SPLIT && w.split) ? blk : (blk & 1) == t ? blk >> 1 : -1;   // this chain's tile on the diagonal
         for (int j = 0; j < nt; ++j) {
           if (q4 == 0) TRF(1 + t, 11);
           // (the completion of this score MMA also covers the block's previous P V MMA, issued before it)
@@ -515,7 +549,7 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
           tmem_wait_ld();
           tmem_ld32(t_s + 64, r[2]);
           tmem_ld32(t_s + 96, r[3]);
-          if (j == blk) {
+          if (j == j_diag) {
 #pragma unroll
             for (int e = 0; e < 64; ++e)
               if (e > rowl) r[e >> 5][e & 31] = 0xff800000u;          // -inf above the diagonal
@@ -533,7 +567,7 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
             for (int k = 0; k < 4; ++k)
               mx[k] = max3(mx[k], __uint_as_float(r[k >> 1][e + 2 * (k & 1)]), __uint_as_float(r[k >> 1][e + 2 * (k & 1) + 1]));
           tmem_wait_ld();
-          if (j == blk) {
+          if (j == j_diag) {
 #pragma unroll
             for (int e = 64; e < 128; ++e)
               if (e > rowl) r[e >> 5][e & 31] = 0xff800000u;
@@ -595,10 +629,27 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
         const float l = (la + lb) + (lc + ld);
         // the epilogue has read the previous item's row sums once it has released O_t
         if (nof > 0 && !mbar_wait_warp_compact(o_free + t, (nof - 1) & 1, wc, SITE_O_FREE)) ok = false;
-        linv[t * 128 + rowl] = 1.0f / l;
-        warp_arrive(l_full + t);
-        if (p.LSE != nullptr && row < p.T && ok)
-          p.LSE[(static_cast<size_t>(w.b) * p.H + w.h) * p.T + row] = (m_ref + log2f(l)) * LN2_F;
+        float m_all = m_ref, l_all = l;
+        if (!SPLIT || !w.split) {
+          linv[t * 128 + rowl] = 1.0f / l;
+          warp_arrive(l_full + t);
+        } else if (t == 1) {
+          // chain 1 hands its row sums and references to chain 0, which forms the two accumulators' factors
+          linv[128 + rowl] = l;
+          xm[rowl] = m_ref;
+          warp_arrive(x_full);
+        } else {
+          if (!mbar_wait_warp_compact(x_full, nx++ & 1, wc, SITE_X_FULL)) ok = false;
+          const float l1 = linv[128 + rowl], m1 = xm[rowl];
+          m_all = fmaxf(m_ref, m1);
+          const float f0 = ex2_approx(m_ref - m_all), f1 = ex2_approx(m1 - m_all);
+          l_all = fmaf(f0, l, f1 * l1);
+          linv[rowl] = f0 / l_all;
+          linv[128 + rowl] = f1 / l_all;
+          warp_arrive(l_full);
+        }
+        if (p.LSE != nullptr && row < p.T && ok && !(SPLIT && w.split && t == 1))
+          p.LSE[(static_cast<size_t>(w.b) * p.H + w.h) * p.T + row] = (m_all + log2f(l_all)) * LN2_F;
       } else {
         // ---------------- frozen head, general form: generate P^ tiles
         const int wt = tid & 127;
@@ -708,8 +759,53 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
     bool ok = true;
     for (uint32_t nrec = 0; ok; ++nrec) {
       ItemView w;
-      ok = ring_take(ring, ring_full, ring_empty, nrec, wc, w);
+      ok = ring_take<SPLIT>(ring, ring_full, ring_empty, nrec, wc, w);
       if (!ok || w.kind == RING_END) break;
+      if (SPLIT && w.split) {
+        // both accumulators of the block, each times its factor
+        ok = mbar_wait_warp_compact(l_full, nl0++ & 1, wc, SITE_L_FULL);
+        if (!ok) break;
+        const float f0 = linv[rowl], f1 = linv[128 + rowl];
+        ok = mbar_wait_warp_compact(o_full, nof0++ & 1, wc, SITE_O_FULL) && mbar_wait_warp_compact(o_full + 1, nof1++ & 1, wc, SITE_O_FULL);
+        if (!ok) break;
+        tc_fence_after();
+        const uint32_t t_o = tmem + lane_base + C::COL_O;
+        const int row = w.blk * BLK + rowl;
+        const int64_t off = w.b * p.o_strides[0] + w.h * p.o_strides[1] + static_cast<int64_t>(row) * p.o_strides[2];
+#pragma unroll 1
+        for (int cc = 0; cc < D / 16; ++cc) {
+          uint32_t r0[16], r1[16];
+          tmem_ld16(t_o + 16 * cc, r0);
+          tmem_ld16(t_o + D + 16 * cc, r1);
+          tmem_wait_ld();
+          if (cc == D / 16 - 1) {
+            tc_fence_before();
+            warp_arrive(o_free);
+            warp_arrive(o_free + 1);
+          }
+          if (row < p.T && 16 * cc < p.d_real) {
+#pragma unroll
+            for (int e = 0; e < 16; ++e) r0[e] = __float_as_uint(fmaf(__uint_as_float(r0[e]), f0, __uint_as_float(r1[e]) * f1));
+            if (p.o_f32) {
+              uint4* orow = reinterpret_cast<uint4*>(static_cast<float*>(p.O) + off + 16 * cc);
+#pragma unroll
+              for (int g = 0; g < 4; ++g) orow[g] = make_uint4(r0[4 * g], r0[4 * g + 1], r0[4 * g + 2], r0[4 * g + 3]);
+            } else {
+              uint4* orow = reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(p.O) + off + 16 * cc);
+#pragma unroll
+              for (int g = 0; g < 2; ++g) {
+                uint4 o;
+                o.x = pack_bf16x2(__uint_as_float(r0[8 * g + 0]), __uint_as_float(r0[8 * g + 1]));
+                o.y = pack_bf16x2(__uint_as_float(r0[8 * g + 2]), __uint_as_float(r0[8 * g + 3]));
+                o.z = pack_bf16x2(__uint_as_float(r0[8 * g + 4]), __uint_as_float(r0[8 * g + 5]));
+                o.w = pack_bf16x2(__uint_as_float(r0[8 * g + 6]), __uint_as_float(r0[8 * g + 7]));
+                orow[g] = o;
+              }
+            }
+          }
+        }
+        continue;
+      }
 #pragma unroll 1
       for (int t = 0; t < 2 && ok; ++t) {
         const int nt = t == 0 ? w.n0 : w.n1;
@@ -792,9 +888,10 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
 cudaError_t launch_fwd(int D, const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv,
                        const CUtensorMap& mvt, const CUtensorMap& mo, const FwdParams& p, int grid, cudaStream_t st) {
   if (D == 64) return launch_fwd64(mq, mk, mv, mvt, mo, p, grid, st);   // head dimension 64 has its own kernel
-  cudaError_t e = cudaFuncSetAttribute(saf_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdCfg::SMEM);
+  auto kern = p.split ? saf_fwd_kernel<true> : saf_fwd_kernel<false>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdCfg::SMEM);
   if (e != cudaSuccess) return e;
-  return launch_pdl(PDL_FWD128, saf_fwd_kernel, dim3(grid), dim3(FwdCfg::NTHREADS), FwdCfg::SMEM, st, mq, mk, mv,
+  return launch_pdl(PDL_FWD128, kern, dim3(grid), dim3(FwdCfg::NTHREADS), FwdCfg::SMEM, st, mq, mk, mv,
                     mvt, p);
 }
 

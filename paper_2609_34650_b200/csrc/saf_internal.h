@@ -53,6 +53,7 @@ constexpr int BLK = 128;            // query rows per item and keys per tile
 constexpr int KIND_ORDINARY = 0;
 constexpr int KIND_FROZEN = 1;
 constexpr int KIND_PAIR = 1 << 7;   // 128-wide forward: the item is query blocks blk - 1 and blk
+constexpr int KIND_SPLIT = 1 << 9;  // 128-wide forward: one query block, its even and odd key tiles in two chains
 
 struct WorkItem { int32_t b, h, blk, kind; };
 
@@ -86,6 +87,7 @@ struct FwdParams {
   const WorkItem* items;
   const int* cta_offsets;
   int n_items;
+  int split;                        // 128-wide kernel: some items are KIND_SPLIT
   int* queue;
   int* status;                      // device status word
   unsigned long long wait_limit_ns;

@@ -183,3 +183,31 @@ def test_calibration_mean_pass(T):
         assert np.abs(got[:, low] - want[:, low]).max() <= 2.0 ** -23    # two fp32 roundings of values below one
         ref = (10.0 * T * T - n * (want ** 2).sum(axis=(1, 2))) / ((n - 1.0) * T * T)
         assert np.abs(var.cpu().numpy() - ref).max() <= 1e-6 * np.abs(ref).max()
+
+
+# Query blocks whose even and odd key tiles run in two chains: two tiles, odd and even counts, ragged ends, a row whose second chain
+# sees the diagonal tile only; 12 units of 13 blocks and 32 of 9 mix them with pairs.  fp32 output.
+@pytest.mark.parametrize("B,H,T,D,frozen,o_f32", [
+    (1, 4, 256, 128, (), False), (1, 3, 257, 96, (1,), True), (1, 4, 385, 128, (0,), False), (2, 4, 1025, 128, (3,), True),
+    (1, 12, 1664, 128, (3, 7), False), (2, 16, 1152, 96, (0, 5), False)])
+def test_split_blocks_of_the_wide_forward(B, H, T, D, frozen, o_f32):
+    inp = si.generate(si.Workload("split", B, H, T, D, frozen, -0.05, seed=T + D))
+    units = all_units(inp.wl)
+    check_units(Layer(inp, o_f32=o_f32).run(), units if len(units) <= 12 else sampled_units(inp.wl, 12, seed=5))
+
+
+@pytest.mark.parametrize("B,H,T", [(1, 8, 640), (8, 12, 640)])
+def test_running_maximum_far_above_the_first_tile_in_split_and_paired_blocks(B, H, T):
+    """Scores that grow along the sequence: the chains of a split block (40 blocks) rescale at different tiles and meet with
+    references far apart; 480 blocks are paired (more than three per SM)."""
+    n_sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert B == 1 or B * H * (T // 128) > 3 * n_sms
+    inp = si.generate(si.Workload("grow", B, H, T, 128, (), -0.05, seed=9))
+    f = np.exp2(np.arange(T) // 128).astype(np.float32)            # exact in bf16
+    inp.k[...] = si.f32_to_bf16_bits(si.bf16_bits_to_f32(inp.k) * f[None, None, :, None])
+    L = Layer(inp, backward=False)
+    L.run(backward=False)
+    q, k, v = (si.bf16_bits_to_f64(x) for x in (inp.q, inp.k, inp.v))
+    want, _ = orc.hybrid_attn_fwd(q, k, v, inp.mask, inp.alpha, inp.rho)
+    got = L.O.float().cpu().numpy().astype(np.float64)
+    assert np.abs(got - want).max() <= 2e-2 and np.linalg.norm(got - want) <= 1e-2 * np.linalg.norm(want)
