@@ -23,7 +23,7 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
 
 enum { WL_QUEUE = 0, WL_BACKWARD = 1, WL_SHORT = 2 };   // forward queue, backward lists, lists of the short 128-wide forward
 struct WorklistEntry {
-  int B, H, T, D, kind, grid;
+  int B, H, T, D, kind, grid, plan_batch;
   std::vector<uint8_t> mask;
   std::vector<WorkItem> items_host;       // kept alive: the upload is asynchronous on the caller's stream
   std::vector<int> offsets_host;
@@ -71,6 +71,9 @@ struct saf_ctx {
   int frozen_weight_bwd_pct = 0;
   int item_overhead_pct = 0;
   int item_overhead_bwd_pct = 0;
+  // Batch size that the 128-wide forward chooses its kernel and items for (0: that of the call).  The host-buffer step sets it for its
+  // chunks, whose O and LSE are then those of one call, bit for bit: a block's key tiles in one chain or in two round differently.
+  int plan_batch = 0;
   int call_counter = 0;                    // ids of the calls that stage fp16 operands (overflow marks)
   std::vector<WorklistEntry> worklists;
   DevBuf mask_buf, logz_buf, delta_buf, dqacc_buf, dkacc_buf, dvacc_buf, qslot_buf;
@@ -334,26 +337,27 @@ void build_pair_order(int B, int H, int T, int D, const uint8_t* mask, int froze
     for (const auto& it : items) order.push_back(it.second);
   }
 }
-// The order whose simulated run on num_sms CTAs ends first, over a few caps between "all blocks alone" and "all in pairs", while
+// The cap whose order ends first in a simulated run on num_sms CTAs, over a few caps between "all blocks alone" and "all in pairs", while
 // there are up to three blocks per SM (beyond, the pairs' tail is short and the longer loads of single blocks count: 1x16x8192x128
 // 247 us in pairs, 268 alone).  us of back-to-back forwards without frozen heads, pairs (blocks alone and in one chain up to
 // one per SM) / this: 1x32x333x128 12.2 / 11.7, 1x8x1024x128 20.0 / 16.1, 1x8x2048x128 34.5 / 25.6, 1x16x1300x128 29.4 / 21.2,
 // 1x8x4096x128 70.7 / 43.6, 1x4x8192x128 132 / 76, 1x12x4096x128 72.7 / 68.3, 4x12x900x128 28.2 / 28.2.
-void build_wide_order(int B, int H, int T, int D, const uint8_t* mask, int num_sms, int frozen_pct, std::vector<WorkItem>& order) {
+long long choose_pair_cap(int B, int H, int T, int D, const uint8_t* mask, int num_sms, int frozen_pct) {
   const int nblk = (T + BLK - 1) / BLK;
   const long long forever = 1LL << 60;
   const long long blocks = static_cast<long long>(B) * H * nblk;
-  if (blocks <= num_sms) return build_pair_order(B, H, T, D, mask, frozen_pct, 0, order);
-  if (blocks > 3LL * num_sms) return build_pair_order(B, H, T, D, mask, frozen_pct, forever, order);
+  if (blocks <= num_sms) return 0;
+  if (blocks > 3LL * num_sms) return forever;
   std::vector<WorkItem> trial;
-  long long work = 0, best = -1;
+  long long work = 0, best = -1, best_cap = forever;
   build_pair_order(B, H, T, D, mask, frozen_pct, forever, trial);
   auto ns = [](const WorkItem& w) {
     return pair_item_ns(w.blk + 1, (w.kind & KIND_PAIR) != 0, (w.kind & 0x7f) == KIND_ORDINARY);
   };
   for (const WorkItem& w : trial) work += ns(w);
   for (int k = 8; k >= 0; --k) {                      // caps in quarters of the mean load, from none to twice; first: all pairs
-    build_pair_order(B, H, T, D, mask, frozen_pct, k == 8 ? forever : work / num_sms * k / 4, trial);
+    const long long cap = k == 8 ? forever : work / num_sms * k / 4;
+    build_pair_order(B, H, T, D, mask, frozen_pct, cap, trial);
     std::priority_queue<long long, std::vector<long long>, std::greater<long long>> free_at;
     for (int c = 0; c < num_sms; ++c) free_at.push(0);
     long long end = 0;
@@ -366,9 +370,10 @@ void build_wide_order(int B, int H, int T, int D, const uint8_t* mask, int num_s
     if (k == 8) end = end * 97 / 100;                 // (pairs unless the gain is clear)
     if (best < 0 || end < best) {
       best = end;
-      order.swap(trial);
+      best_cap = cap;
     }
   }
+  return best_cap;
 }
 
 // Whether a 128-wide forward goes to the kernel of short sequences (one query block per item, two CTAs per SM).  The line
@@ -399,10 +404,11 @@ void sched_defaults(int wide, int backward, int* frozen_pct, int* overhead_pct, 
   }
 }
 
-int get_worklist(saf_ctx* ctx, int B, int H, int T, int D, const uint8_t* mask, int kind, int grid, cudaStream_t st,
+// plan_batch: the batch size that the forms of the 128-wide forward's items are chosen for (saf_ctx::plan_batch)
+int get_worklist(saf_ctx* ctx, int B, int H, int T, int D, const uint8_t* mask, int kind, int grid, int plan_batch, cudaStream_t st,
                  const WorklistEntry** out) {
   for (const WorklistEntry& e : ctx->worklists)
-    if (e.B == B && e.H == H && e.T == T && e.D == D && e.kind == kind && e.grid == grid &&
+    if (e.B == B && e.H == H && e.T == T && e.D == D && e.kind == kind && e.grid == grid && e.plan_batch == plan_batch &&
         std::memcmp(e.mask.data(), mask, H) == 0) {
       *out = &e;
       return SAF_OK;
@@ -423,7 +429,7 @@ int get_worklist(saf_ctx* ctx, int B, int H, int T, int D, const uint8_t* mask, 
   const bool lists = kind != WL_QUEUE;
   WorklistEntry e;
   if (!lists && wide) {
-    build_wide_order(B, H, T, D, mask, ctx->num_sms, frozen_pct, e.items_host);
+    build_pair_order(B, H, T, D, mask, frozen_pct, choose_pair_cap(plan_batch, H, T, D, mask, ctx->num_sms, frozen_pct), e.items_host);
   } else {
     // (tail: two items per CTA; on the 128-wide backward four: -0.5 % on 8x12x4096x128, -1 % on 2x16x8192x96, -3 % on
     // 1x16x8192x128 and on shared heads 3x8x3000x128; six and eight are no better)
@@ -431,7 +437,7 @@ int get_worklist(saf_ctx* ctx, int B, int H, int T, int D, const uint8_t* mask, 
                         wide && backward ? 4 : 2, lists ? &e.items_host : nullptr, &e.offsets_host,
                         lists ? nullptr : &e.items_host);
   }
-  e.B = B; e.H = H; e.T = T; e.D = D; e.kind = kind; e.grid = grid;
+  e.B = B; e.H = H; e.T = T; e.D = D; e.kind = kind; e.grid = grid; e.plan_batch = plan_batch;
   e.mask.assign(mask, mask + H);
   e.n_items = static_cast<int>(e.items_host.size());
   for (const WorkItem& w : e.items_host) e.split |= (w.kind & KIND_SPLIT) != 0;
@@ -716,11 +722,12 @@ int saf_hybrid_attn_fwd(saf_ctx* ctx, const saf_problem* p, const void* Q, const
   }
   const int nblk = (p->T + BLK - 1) / BLK;
   const long long n_items = static_cast<long long>(p->B) * p->H * nblk;
-  const bool is_short = p->D != 64 && fwd_is_short(p->B, p->H, p->T, p->D, ctx->num_sms);
+  const int plan_batch = ctx->plan_batch > 0 ? ctx->plan_batch : p->B;
+  const bool is_short = p->D != 64 && fwd_is_short(plan_batch, p->H, p->T, p->D, ctx->num_sms);
   // (head dimension 64 and the short 128-wide kernel: two CTAs per SM; the other 128-wide kernel: one)
   const int grid = static_cast<int>(std::min<long long>((p->D == 64 || is_short ? 2LL : 1LL) * ctx->num_sms, n_items));
   const WorklistEntry* wl = nullptr;
-  rc = get_worklist(ctx, p->B, p->H, p->T, p->D, frozen_mask_host, is_short ? WL_SHORT : WL_QUEUE, grid, st, &wl);
+  rc = get_worklist(ctx, p->B, p->H, p->T, p->D, frozen_mask_host, is_short ? WL_SHORT : WL_QUEUE, grid, plan_batch, st, &wl);
   if (rc) return rc;
 
   CUtensorMap mq, mk, mv;
@@ -890,7 +897,7 @@ int saf_hybrid_attn_bwd(saf_ctx* ctx, const saf_problem* p, const void* Q, const
   const long long n_items = static_cast<long long>(p->B) * p->H * nblk;
   const int grid = static_cast<int>(std::min<long long>(ctx->num_sms, n_items));
   const WorklistEntry* wl = nullptr;
-  rc = get_worklist(ctx, p->B, p->H, p->T, p->D, frozen_mask_host, WL_BACKWARD, grid, st, &wl);
+  rc = get_worklist(ctx, p->B, p->H, p->T, p->D, frozen_mask_host, WL_BACKWARD, grid, p->B, st, &wl);
   if (rc) return rc;
 
   CUtensorMap mq, mk, mv, mdo;
@@ -1097,6 +1104,11 @@ int saf_hybrid_attn_step_host(saf_ctx* ctx, const saf_problem* p, const void* Q_
   const size_t per_b_lse = static_cast<size_t>(p->H) * p->T;
   auto off = [](const void* base, size_t bytes) { return static_cast<const char*>(base) + bytes; };
   auto offw = [](void* base, size_t bytes) { return static_cast<char*>(base) + bytes; };
+  struct PlanBatch {
+    saf_ctx* ctx;
+    PlanBatch(saf_ctx* c, int b) : ctx(c) { ctx->plan_batch = b; }
+    ~PlanBatch() { ctx->plan_batch = 0; }
+  } plan(ctx, p->B);
   int ci = 0;
   for (int b0 = 0; b0 < p->B; b0 += bc_max, ++ci) {
     const int bc = std::min(bc_max, p->B - b0);

@@ -211,3 +211,18 @@ def test_running_maximum_far_above_the_first_tile_in_split_and_paired_blocks(B, 
     want, _ = orc.hybrid_attn_fwd(q, k, v, inp.mask, inp.alpha, inp.rho)
     got = L.O.float().cpu().numpy().astype(np.float64)
     assert np.abs(got - want).max() <= 2e-2 and np.linalg.norm(got - want) <= 1e-2 * np.linalg.norm(want)
+
+
+def test_chunks_of_the_host_step_take_the_forms_of_the_whole_batch():
+    """8 x 4 heads x 12 blocks = 384: some blocks split, some paired; chunks of one batch entry (48 blocks) alone would all be
+    split."""
+    wl = si.Workload("host-split", 8, 4, 1536, 128, (1,), -0.05, seed=34)
+    inp = si.generate(wl)
+    Dv = Layer(inp, backward=False)
+    Dv.run(backward=False)
+    Q, K, V = (t.cpu().contiguous().pin_memory() for t in (Dv.Q, Dv.K, Dv.V))
+    alpha, rho = torch.from_numpy(inp.alpha), torch.from_numpy(inp.rho)
+    O, LSE = torch.empty_like(Q), torch.empty(wl.B, wl.H, wl.T)
+    prob = saf.make_problem(Q, wl.stored_len, k_like=K, v_like=V, o_like=O, H=wl.H)
+    saf.Context(0).saf_hybrid_attn_step_host(prob, Q, K, V, None, inp.mask, alpha, rho, 1, O, LSE, None, None, None)
+    assert torch.equal(O, Dv.O.cpu()) and torch.equal(LSE, Dv.LSE.cpu())
