@@ -900,6 +900,15 @@ int saf_hybrid_attn_bwd(saf_ctx* ctx, const saf_problem* p, const void* Q, const
   rc = get_worklist(ctx, p->B, p->H, p->T, p->D, frozen_mask_host, WL_BACKWARD, grid, p->B, st, &wl);
   if (rc) return rc;
 
+  auto finalize = [&]() -> int {
+    if (grad_f32) return SAF_OK;
+    ScopedTimer timer(ctx, SAF_KERNEL_BWD_FINALIZE, st);
+    const F32ToBf16 g = {{dqacc, kv_acc ? static_cast<const float*>(dK_k) : nullptr, kv_acc ? static_cast<const float*>(dV_k) : nullptr},
+                         {dQ, dK, dV},
+                         {nelem / 8, kv_acc ? nkv / 8 : 0, kv_acc ? nkv / 8 : 0}};
+    return launch_bwd_finalize(g, st) == cudaSuccess ? SAF_OK : SAF_ERR_CUDA;
+  };
+
   CUtensorMap mq, mk, mv, mdo;
   rc = make_map(ctx, &mdo, dO, p, p->o_strides);
   if (rc) return rc;
@@ -959,14 +968,7 @@ int saf_hybrid_attn_bwd(saf_ctx* ctx, const saf_problem* p, const void* Q, const
       ScopedTimer timer(ctx, SAF_KERNEL_BWD, st);
       if (launch_bwd128(mk, mv, mq, mdo, mdot, mdq128, bp, grid, st) != cudaSuccess) return SAF_ERR_CUDA;
     }
-    if (!grad_f32) {
-      ScopedTimer timer(ctx, SAF_KERNEL_BWD_FINALIZE, st);
-      if (nelem > 0 && launch_bwd_finalize(dqacc, dQ, nelem, st) != cudaSuccess) return SAF_ERR_CUDA;
-      if (kv_acc && (launch_bwd_finalize(static_cast<const float*>(dK_k), dK, nkv, st) != cudaSuccess ||
-                     launch_bwd_finalize(static_cast<const float*>(dV_k), dV, nkv, st) != cudaSuccess))
-        return SAF_ERR_CUDA;
-    }
-    return SAF_OK;
+    return finalize();
   }
   // fp32 dQ accumulator [B][H][T][64] as a 4-D tensor for tiled reduce-adds: box = 32 floats x 128 rows
   // (dK and dV get maps of the same shape for the tiled stores of the fp32 epilogue)
@@ -1030,14 +1032,7 @@ int saf_hybrid_attn_bwd(saf_ctx* ctx, const saf_problem* p, const void* Q, const
     ScopedTimer timer(ctx, SAF_KERNEL_BWD, st);
     if (launch_bwd(p->D, mq, mk, mv, mdo, mdq, mdot, mdk, mdv, bp, grid, st) != cudaSuccess) return SAF_ERR_CUDA;
   }
-  if (!grad_f32) {
-    ScopedTimer timer(ctx, SAF_KERNEL_BWD_FINALIZE, st);
-    if (nelem > 0 && launch_bwd_finalize(dqacc, dQ, nelem, st) != cudaSuccess) return SAF_ERR_CUDA;
-    if (kv_acc && (launch_bwd_finalize(static_cast<const float*>(dK_k), dK, nkv, st) != cudaSuccess ||
-                   launch_bwd_finalize(static_cast<const float*>(dV_k), dV, nkv, st) != cudaSuccess))
-      return SAF_ERR_CUDA;
-  }
-  return SAF_OK;
+  return finalize();
 }
 
 int saf_hybrid_attn_step_host(saf_ctx* ctx, const saf_problem* p, const void* Q_host, const void* K_host,

@@ -210,7 +210,8 @@ cudaError_t launch_bwd_prep(const void* O, int o_f32, const void* dO, const floa
                             void* dV, int grad_f32, int kv_group, const int* qslot, int n_ord, const PrepFrozen& fz, int B,
                             int H, int T, int D, cudaStream_t st);   // kv_group > 1: zeroes all of dK and dV (fp32) instead
 // dQ (grad dtype) = scale-free copy/convert of dQacc (fp32) for the bf16-gradient case.
-cudaError_t launch_bwd_finalize(const float* dQacc, void* dQ, size_t n, cudaStream_t st);
+struct F32ToBf16 { const float* src[3]; void* dst[3]; size_t n8[3]; };
+cudaError_t launch_bwd_finalize(const F32ToBf16& g, cudaStream_t st);
 // head dimension 64 (saf_fwd64.cu); launch_fwd dispatches to it
 cudaError_t launch_fwd64(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv, const CUtensorMap& mvt,
                          const CUtensorMap& mo, const FwdParams& p, int grid, cudaStream_t st);

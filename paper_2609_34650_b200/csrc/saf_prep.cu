@@ -510,12 +510,23 @@ cudaError_t launch_bwd_prep(const void* O, int o_f32, const void* dO, const floa
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-__global__ void __launch_bounds__(256) saf_f32_to_bf16_kernel(const float* __restrict__ src, __nv_bfloat16* __restrict__ dst,
-                                                              size_t n8) {
+// Up to three accumulated gradients to bf16, eight elements per thread.
+__global__ void __launch_bounds__(256) saf_f32_to_bf16_kernel(const F32ToBf16 g) {
   pdl_launch_dependents();
   pdl_wait();
-  const size_t i = static_cast<size_t>(blockIdx.x) * 256 + threadIdx.x;
-  if (i >= n8) return;
+  size_t i = static_cast<size_t>(blockIdx.x) * 256 + threadIdx.x, n = g.n8[0];
+  const float* src = g.src[0];
+  void* out = g.dst[0];
+#pragma unroll
+  for (int k = 1; k < 3; ++k)
+    if (i >= n) {
+      i -= n;
+      n = g.n8[k];
+      src = g.src[k];
+      out = g.dst[k];
+    }
+  if (i >= n) return;
+  __nv_bfloat16* dst = static_cast<__nv_bfloat16*>(out);
   const float4 a = *reinterpret_cast<const float4*>(src + i * 8);
   const float4 b = *reinterpret_cast<const float4*>(src + i * 8 + 4);
   __nv_bfloat162 r[4];
@@ -526,12 +537,12 @@ __global__ void __launch_bounds__(256) saf_f32_to_bf16_kernel(const float* __res
   *reinterpret_cast<uint4*>(dst + i * 8) = *reinterpret_cast<uint4*>(r);
 }
 
-cudaError_t launch_bwd_finalize(const float* dQacc, void* dQ, size_t n, cudaStream_t st) {
-  const size_t n8 = n / 8;
+cudaError_t launch_bwd_finalize(const F32ToBf16& g, cudaStream_t st) {
   // (early where the launch gap shows: updates of 4x12x388x96 -9 %, 11x16x224x64 -3 %; 2x16x8192x96 +0.2 %)
+  const size_t n8 = g.n8[0] + g.n8[1] + g.n8[2];
+  if (n8 == 0) return cudaSuccess;
   const unsigned grid = static_cast<unsigned>((n8 + 255) / 256);
-  const cudaError_t e = launch_pdl(grid <= 4096 ? PDL_REST : 0, saf_f32_to_bf16_kernel, dim3(grid), dim3(256), 0, st, dQacc,
-                                   static_cast<__nv_bfloat16*>(dQ), n8);
+  const cudaError_t e = launch_pdl(grid <= 4096 ? PDL_REST : 0, saf_f32_to_bf16_kernel, dim3(grid), dim3(256), 0, st, g);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
