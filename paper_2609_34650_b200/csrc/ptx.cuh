@@ -23,8 +23,13 @@ __device__ __forceinline__ uint64_t globaltimer_ns() {
 // ------------------------------------------------------------------ programmatic dependent launch
 // A kernel launched with the programmatic-stream-serialization attribute may start while the kernel before it in
 // the stream is still running.  pdl_wait() blocks until that kernel has completed and its memory operations are
-// visible; everything that reads or writes global memory must come after it.  pdl_launch_dependents() lets the
+// visible; everything that reads or writes global memory must come after it, but for reads of what no kernel writes: the
+// tensor maps (kernel parameters) and the work lists, which the host copies in on the stream (a copy between two kernels
+// waits for the first and is waited for by the second as a whole, early launch or not).  pdl_launch_dependents() lets the
 // next kernel's CTAs be scheduled as soon as this grid leaves room (its own pdl_wait() still orders the data).
+// Maps and lists fetched ahead of the wait (the 64-wide forward, the short forward, both backwards, the pattern gradients;
+// updates 1x16x395x128 57.5 -> 56.3 us, 26x16x256x64 61.7 -> 60.6, 3x12x1537x64 72.6 -> 72.1); the wide forward spilled
+// more for it (1x16x20721x128 +0.4 %) and the calibration gained nothing, so those two fetch them behind it.
 // Both are no-ops in a kernel launched the ordinary way.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
@@ -150,6 +155,7 @@ __device__ __forceinline__ uint32_t elect_one() {
 __device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap* map) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");
 }
+__device__ __forceinline__ void prefetch_l1(const void* ptr) { asm volatile("prefetch.global.L1 [%0];" ::"l"(ptr)); }
 // 4-D tiled load global -> shared, completion counted in bytes on `bar`.
 // Coordinate c0 (innermost) times the element size must be a multiple of 16 bytes.
 __device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* map, uint64_t* bar, int c0, int c1,

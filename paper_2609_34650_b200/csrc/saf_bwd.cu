@@ -191,6 +191,7 @@ saf_bwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
     }
     reinterpret_cast<uint4*>(smem + C::OFF_ONES)[i] = v;
   }
+  const int it_begin = p.cta_offsets[blockIdx.x], it_end = p.cta_offsets[blockIdx.x + 1];
   if (warp == 21) {
     tmem_alloc(tmem_slot, C::TMEM_COLS);
     tmem_relinquish();
@@ -199,20 +200,23 @@ saf_bwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  if (warp == 20 && lane == 0) {
+    tma_prefetch_desc(&mk);
+    tma_prefetch_desc(&mv);
+    tma_prefetch_desc(&mq);
+    tma_prefetch_desc(&mdo);
+    tma_prefetch_desc(&mdot);
+    if (it_begin < it_end) prefetch_l1(p.items + it_begin);
+  }
   const uint32_t tmem = *tmem_slot;
-  // the prologue above overlapped the previous kernel's tail; global memory is touched only from here on
+  // The prologue above overlapped the previous kernel's tail.  Of global memory it touches only what no kernel writes, the
+  // tensor maps and the work list (pdl_wait in ptx.cuh): their first use would otherwise miss behind the wait.
   pdl_launch_dependents();
   pdl_wait();
-  const int it_begin = p.cta_offsets[blockIdx.x], it_end = p.cta_offsets[blockIdx.x + 1];
 
   if (warp == 20) {
     // ------------------------------------------------------------------ TMA producer
     if (lane == 0) {
-      tma_prefetch_desc(&mq);
-      tma_prefetch_desc(&mk);
-      tma_prefetch_desc(&mv);
-      tma_prefetch_desc(&mdo);
-      tma_prefetch_desc(&mdot);
       uint32_t nkv = 0, nqdo = 0, nfz = 0;
       bool ok = true, fz_open = false;
 #ifdef SAF_TRACE

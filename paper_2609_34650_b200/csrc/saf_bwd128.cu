@@ -154,6 +154,7 @@ saf_bwd128_kernel(const __grid_constant__ CUtensorMap mk, const __grid_constant_
     mbar_init(pfree, 1);
     mbar_fence_init();
   }
+  const int it_begin = p.cta_offsets[blockIdx.x], it_end = p.cta_offsets[blockIdx.x + 1];
   if (warp == 25) {
     tmem_alloc(tmem_slot, C::TMEM_COLS);
     tmem_relinquish();
@@ -161,22 +162,25 @@ saf_bwd128_kernel(const __grid_constant__ CUtensorMap mk, const __grid_constant_
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  if (warp == 24 && lane == 0) {
+    tma_prefetch_desc(&mk);
+    tma_prefetch_desc(&mv);
+    tma_prefetch_desc(&mq);
+    tma_prefetch_desc(&mdo);
+    tma_prefetch_desc(&mdot);
+    if (it_begin < it_end) prefetch_l1(p.items + it_begin);
+  }
   const uint32_t tmem = *tmem_slot;
-  // the prologue above overlapped the previous kernel's tail; global memory is touched only from here on
+  // The prologue above overlapped the previous kernel's tail.  Of global memory it touches only what no kernel writes, the
+  // tensor maps and the work list (pdl_wait in ptx.cuh): their first use would otherwise miss behind the wait.
   pdl_launch_dependents();
   pdl_wait();
-  const int it_begin = p.cta_offsets[blockIdx.x], it_end = p.cta_offsets[blockIdx.x + 1];
 
   if (warp >= 24) {
     reg_dec<40>();
     if (warp == 24) {
       // ---------------------------------------------------------------- TMA producer
       if (lane == 0) {
-        tma_prefetch_desc(&mk);
-        tma_prefetch_desc(&mv);
-        tma_prefetch_desc(&mq);
-        tma_prefetch_desc(&mdo);
-        tma_prefetch_desc(&mdot);
         uint32_t nkv = 0, nq = 0, ndo = 0;
         bool ok = true, bands_open = false;
         ItemW nxt = load_item_w(p, it_begin, it_end);

@@ -183,18 +183,22 @@ saf_fwd64_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  if (warp == 8 && lane == 0) {
+    tma_prefetch_desc(&mq);
+    tma_prefetch_desc(&mk);
+    tma_prefetch_desc(&mv);
+    tma_prefetch_desc(&mvt);
+    if (static_cast<int>(blockIdx.x) < p.n_items) prefetch_l1(p.items + blockIdx.x);
+  }
   const uint32_t tmem = *tmem_slot;
-  // the prologue above overlapped the previous kernel's tail; global memory is touched only from here on
+  // The prologue above overlapped the previous kernel's tail.  Of global memory it touches only what no kernel writes, the
+  // tensor maps and the work list (pdl_wait in ptx.cuh): their first use would otherwise miss behind the wait.
   pdl_launch_dependents();
   pdl_wait();
 
   if (warp == 8) {
     // ------------------------------------------------------------------ TMA producer
     if (lane == 0) {
-      tma_prefetch_desc(&mq);
-      tma_prefetch_desc(&mk);
-      tma_prefetch_desc(&mv);
-      tma_prefetch_desc(&mvt);
       uint32_t nq = 0, nk = 0, nv = 0, nfz = 0;
       bool ok = true, fz_open = false;
       bool drop_load = p.selftest_drop_load != 0;        // self-test of the give-up path: see FwdParams

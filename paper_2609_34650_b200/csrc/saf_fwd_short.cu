@@ -95,6 +95,7 @@ saf_fwd_short_kernel(const __grid_constant__ CUtensorMap mq, const __grid_consta
     mbar_init(o_free, 8);
     mbar_fence_init();
   }
+  const int it_begin = p.cta_offsets[blockIdx.x], it_end = p.cta_offsets[blockIdx.x + 1];
   if (warp == 9) {
     tmem_alloc(tmem_slot, C::TMEM_COLS);
     tmem_relinquish();
@@ -102,20 +103,22 @@ saf_fwd_short_kernel(const __grid_constant__ CUtensorMap mq, const __grid_consta
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  if (warp == 8 && lane == 0) {
+    tma_prefetch_desc(&mq);
+    tma_prefetch_desc(&mk);
+    tma_prefetch_desc(&mv);
+    tma_prefetch_desc(&mvt);
+    if (it_begin < it_end) prefetch_l1(p.items + it_begin);
+  }
   const uint32_t tmem = *tmem_slot;
-  // the prologue above overlapped the previous kernel's tail; global memory is touched only from here on
+  // The prologue above overlapped the previous kernel's tail.  Of global memory it touches only what no kernel writes, the
+  // tensor maps and the work list (pdl_wait in ptx.cuh): their first use would otherwise miss behind the wait.
   pdl_launch_dependents();
   pdl_wait();
-
-  const int it_begin = p.cta_offsets[blockIdx.x], it_end = p.cta_offsets[blockIdx.x + 1];
 
   if (warp == 8) {
     // ------------------------------------------------------------------ TMA producer
     if (lane == 0) {
-      tma_prefetch_desc(&mq);
-      tma_prefetch_desc(&mk);
-      tma_prefetch_desc(&mv);
-      tma_prefetch_desc(&mvt);
       uint32_t nq = 0, nk = 0, nv = 0;
       bool ok = true;
       bool drop_load = p.selftest_drop_load != 0 && blockIdx.x < 16;   // (see FwdParams)

@@ -11,7 +11,7 @@ namespace saf {
 // Launch with the programmatic-stream-serialization attribute: the kernel may be scheduled while the kernel
 // before it in the stream drains, runs its prologue (barrier set-up, TMEM allocation, descriptor prefetch) and
 // then blocks in pdl_wait() until that kernel has completed.  Every kernel launched this way calls pdl_wait()
-// before it touches global memory, so completion of a kernel still implies completion of all earlier ones.
+// before it touches global memory that a kernel may write, so completion of a kernel still implies completion of all earlier ones.
 // SAF_DISABLE_PDL=1 launches the ordinary way.
 inline bool pdl_enabled() {
   static const bool on = [] {

@@ -95,6 +95,8 @@ saf_pgrad_kernel(const __grid_constant__ CUtensorMap mv, const __grid_constant__
     }
     mbar_fence_init();
   }
+  // the tensor maps and the work list may be read ahead of pdl_wait (ptx.cuh)
+  const int it_begin = p.cta_offsets[blockIdx.x], it_end = p.cta_offsets[blockIdx.x + 1];
   if (warp == C::NCW + 1) {
     tmem_alloc(tmem_slot, C::TMEM_COLS);
     tmem_relinquish();
@@ -102,16 +104,18 @@ saf_pgrad_kernel(const __grid_constant__ CUtensorMap mv, const __grid_constant__
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  if (warp == C::NCW && lane == 0) {
+    tma_prefetch_desc(&mv);
+    tma_prefetch_desc(&mdo);
+    if (it_begin < it_end) prefetch_l1(p.items + it_begin);
+  }
   const uint32_t tmem = *tmem_slot;
   pdl_launch_dependents();
   pdl_wait();
-  const int it_begin = p.cta_offsets[blockIdx.x], it_end = p.cta_offsets[blockIdx.x + 1];
 
   if (warp == C::NCW) {
     // ------------------------------------------------------------------ TMA producer
     if (lane == 0) {
-      tma_prefetch_desc(&mv);
-      tma_prefetch_desc(&mdo);
       uint32_t nv = 0, ndo = 0;
       bool ok = true;
       for (int it = it_begin; it < it_end && ok; ++it) {
