@@ -28,7 +28,7 @@ __device__ __forceinline__ uint64_t globaltimer_ns() {
 // waits for the first and is waited for by the second as a whole, early launch or not).  pdl_launch_dependents() lets the
 // next kernel's CTAs be scheduled as soon as this grid leaves room (its own pdl_wait() still orders the data).
 // Maps and lists fetched ahead of the wait (the 64-wide forward, the short forward, both backwards, the pattern gradients;
-// updates 1x16x395x128 57.5 -> 56.3 us, 26x16x256x64 61.7 -> 60.6, 3x12x1537x64 72.6 -> 72.1); the wide forward spilled
+// updates 5x16x395x128 57.5 -> 56.3 us, 26x16x256x64 61.7 -> 60.6, 3x12x1537x64 72.6 -> 72.1); the wide forward spilled
 // more for it (1x16x20721x128 +0.4 %) and the calibration gained nothing, so those two fetch them behind it.
 // Both are no-ops in a kernel launched the ordinary way.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }

@@ -19,8 +19,12 @@
 // sub-transform lies inside a warp.  16-byte pads behind every 8 points keep all passes free of bank conflicts.
 //
 // Bound: latency.  One warp per scheduler works through chains of dependent fp64 operations (the fp64 pipe is 30 % busy for one
-// warp alone), barriers and exchanges.  36 heads of 4096 positions, 400 steps: 14.8 us a step against 59.3 with the
-// direct fp32 sums on 108 SMs; one head: 10.1 against 22.8.
+// warp alone), barriers and exchanges.  36 heads of 4096 positions, 400 steps: 13.9 us a step against 59.3 with the
+// direct fp32 sums on 108 SMs; one head: 9.3 against 22.8.  Registers decide much of it: the kernel of eight-CTA clusters
+// spilled 160 bytes a thread and thrashed L1 with them (with less L1 it lost another 12 %); with the owner twiddles in shared
+// memory, the references of the normalisers written out and the peers' addresses computed where they are used, 28 bytes are
+// left (36 x 4096: 6.29 -> 5.91 ms for the whole fit, 1 x 8192: 7.61 -> 6.59, 36 x 8192: 19.6 -> 17.8).  Clusters of up to four
+// keep all of these in registers (with them moved out they measured 1-6 % slower).
 //
 // Accuracy.  An output's error is up to about 4.5 2^-53 of the 2-norms of its two factors, whatever its own size (measured, T =
 // 4096).  The pattern does not change under alpha(j) -> alpha(j) - k j, rho(d) -> rho(d) - k d, Z(i) -> e^{-k i} Z(i), and
@@ -208,9 +212,12 @@ __device__ __forceinline__ void bf_last(cd* x) {
 }
 
 __device__ __forceinline__ uint32_t smem_a(const void* p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
+// FRESH: computed at each use, not hoisted out of the steps' loop and held
+template <bool FRESH>
 __device__ __forceinline__ uint32_t peer(uint32_t addr, uint32_t rank) {
   uint32_t r;
-  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  if (FRESH) asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  else asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
   return r;
 }
 __device__ __forceinline__ void st_peer(uint32_t a, cd v) {
@@ -245,15 +252,15 @@ struct FftCfg {
   static constexpr int UN = SPLIT ? 1 : 4 / C;                         // n2 of a thread (and vector)
   static constexpr int NV = SPLIT ? 1 : 2;                             // vectors of a thread
   static constexpr int BUF = L + L / 8;                                // padded points
-  static constexpr int NTW = LOGL / 3 * 3 * G;                         // twiddle bases
-  static constexpr int SMEM = (3 * BUF + 2 * L + NTW) * 16;
+  static constexpr int NTW = (LOGL - 1) / 3 * 3 * G;                   // twiddle bases (none for a pass of sub-length 8)
+  static constexpr int SMEM = (3 * BUF + 2 * L + NTW + (SPLIT ? 2 * N2 : 0)) * 16;
 };
 
 // Twiddle bases in shared memory: w, w^2, w^4 of thread t and pass q (sub-length N = L / 8^q, w = e^{-2 pi i p / N}) at
 // [3 q + e][t].  (In registers they push the kernel into spills.)
 template <int LOGL, int G>
 __device__ __forceinline__ void twiddle_init(cd* tab, int tid) {
-  for (int i = tid; i < LOGL / 3 * 3 * G; i += 2 * G) {
+  for (int i = tid; i < (LOGL - 1) / 3 * 3 * G; i += 2 * G) {
     const int e = i / G, q = e / 3, n = (1 << LOGL) >> (3 * q), t = i - e * G;
     double sn, cs;
     sincospi(-2.0 * static_cast<double>((t & (n / 8 - 1)) << (e - 3 * q)) / n, &sn, &cs);
@@ -349,10 +356,23 @@ saf_fit_fft_kernel(FitState s, int steps, const double* __restrict__ plogp, floa
   cd* const TZ = FW + F::BUF;                    // [C][N2] back at the owners: Z, later c
   cd* const TG = TZ + L;                         // g
   cd* const tw = TG + L;                         // twiddle bases
+  cd* const own = tw + F::NTW;                   // owner twiddles [2][N2] (registers where a thread has both vectors)
   __shared__ float nrm[4][8 * NW];               // partial |A|^2, |R|^2, |W|^2, slope of log Z of every warp of the cluster
   __shared__ double lossp[8 * NW];
   __shared__ int flag[2];                        // raised between barriers 2 and 3, 4 and 1
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, T = s.T;
+  // Where half of the threads own alpha and the normalisers, that half has twice the other's fp64 work (and the first
+  // warps always sit on the same schedulers): every second CTA of an SM, by its hardware warp slots, swaps the halves
+  // (36 x 4096 -2.4 %, one head -5 %; the values do not depend on it).
+  __shared__ int swapped;
+  if (F::SPLIT) {
+    if (threadIdx.x == 0) {
+      uint32_t slot;
+      asm volatile("mov.u32 %0, %%warpid;" : "=r"(slot));
+      swapped = slot / NW & 1;
+    }
+    __syncthreads();
+  }
+  const int tid = F::SPLIT && swapped ? threadIdx.x ^ G : threadIdx.x, lane = tid & 31, warp = tid >> 5, T = s.T;
   uint32_t rank = 0;
   if (C > 1) asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
   const int h = blockIdx.x / C;
@@ -365,19 +385,20 @@ saf_fit_fft_kernel(FitState s, int steps, const double* __restrict__ plogp, floa
   auto n2l = [&](int u) { return F::SPLIT ? tid - my_vec * N2 : tid + u * NT; };
   auto pos = [&](int u, int n1) { return static_cast<int>(rank) * N2 + n2l(u) + L * n1; };
   // owner twiddles e^{-2 pi i n2 (k1 + 1/4) / M}: of k1 = 0, and the factor from one k1 to the next
-  cd ow[UN], ows[UN];
+  cd owr[2 * UN];
 #pragma unroll
-  for (int u = 0; u < UN; ++u) {
+  for (int k = 0; k < 2 * UN; ++k) {
+    const int u = k % UN;
     double sn, cs;
-    sincospi(-0.5 * pos(u, 0) / (static_cast<double>(L) * C), &sn, &cs);
-    ow[u] = make_double2(cs, sn);
-    sincospi(-2.0 * pos(u, 0) / (static_cast<double>(L) * C), &sn, &cs);
-    ows[u] = make_double2(cs, sn);
+    sincospi((k < UN ? -0.5 : -2.0) * pos(u, 0) / (static_cast<double>(L) * C), &sn, &cs);
+    owr[k] = make_double2(cs, sn);
+    if (F::SPLIT) own[k * N2 + n2l(u)] = owr[k];
   }
   // C-point sum of an owner's real values, twiddled, to the CTAs of the residues
   auto send = [&](cd* buf, const double* x, int u) {
     const int slot = pad8(static_cast<int>(rank) * N2 + n2l(u));
-    cd f = ow[u], y[C];
+    const cd fs = F::SPLIT ? own[N2 + n2l(u)] : owr[UN + u];
+    cd f = F::SPLIT ? own[n2l(u)] : owr[u], y[C];
     if constexpr (C == 8) {                                // e^{-2 pi i n / 32}, then an 8-point DFT
 #pragma unroll
       for (int n = 0; n < C; ++n) y[n] = make_double2(x[n] * cos32(n), -x[n] * sin32(n));
@@ -397,18 +418,19 @@ saf_fit_fft_kernel(FitState s, int steps, const double* __restrict__ plogp, floa
 #pragma unroll
     for (int k = 0; k < C; ++k) {
       const cd v = cmul(y[C == 8 ? rev8(k) : k], f);
-      if (k + 1 < C) f = cmul(f, ows[u]);
+      if (k + 1 < C) f = cmul(f, fs);
       if (C == 1) buf[slot] = v;
-      else st_peer(peer(smem_a(buf + slot), k), v);
+      else st_peer(peer<F::SPLIT>(smem_a(buf + slot), k), v);
     }
   };
   // and back: real parts of the inverse at the owner's positions (scaled by 1 / M)
   auto receive = [&](const cd* buf, double* x, int u) {
-    cd f = ow[u], y[C];
+    const cd fs = F::SPLIT ? own[N2 + n2l(u)] : owr[UN + u];
+    cd f = F::SPLIT ? own[n2l(u)] : owr[u], y[C];
 #pragma unroll
     for (int k = 0; k < C; ++k) {
       y[C == 8 ? rev8(k) : k] = cmulc(buf[k * N2 + n2l(u)], f);
-      if (k + 1 < C) f = cmul(f, ows[u]);
+      if (k + 1 < C) f = cmul(f, fs);
     }
     if constexpr (C == 8) {
       bf8_inv(y);
@@ -434,20 +456,20 @@ saf_fit_fft_kernel(FitState s, int steps, const double* __restrict__ plogp, floa
       const int i = t + G * k, q = i / N2;
       cd* dst = buf + static_cast<int>(rank) * N2 + (i - q * N2);
       if (C == 1) *dst = x[k];
-      else st_peer(peer(smem_a(dst), q), x[k]);
+      else st_peer(peer<F::SPLIT>(smem_a(dst), q), x[k]);
     }
   };
   auto raise = [&](int which) {
     if (C == 1) flag[which] = 1;
     else
-      for (int r = 0; r < C; ++r) st_peer(peer(smem_a(flag + which), r), 1);
+      for (int r = 0; r < C; ++r) st_peer(peer<F::SPLIT>(smem_a(flag + which), r), 1);
   };
   auto give_norm = [&](int which, float v) {               // v: this thread's part
     v = wsum(v);
     if (C == 1) {
       if (lane == 0) nrm[which][warp] = v;
     } else if (lane < C) {
-      st_peer(peer(smem_a(&nrm[which][rank * NW + warp]), lane), v);
+      st_peer(peer<F::SPLIT>(smem_a(&nrm[which][rank * NW + warp]), lane), v);
     }
   };
   auto norm2 = [&](int which) {
@@ -474,13 +496,13 @@ saf_fit_fft_kernel(FitState s, int steps, const double* __restrict__ plogp, floa
         (is_rho ? s.m_r : s.m_a)[o + i] = 0.0;
         (is_rho ? s.v_r : s.v_a)[o + i] = 0.0;
         val[v][u][n] = is_rho ? exp(x) : 1.0;
+        if (F::SPLIT && !is_rho) s.wref[o + i] = 0.0f;
       }
   double tilt = 0.0;                                       // k: A(j) = exp(alpha(j) - k j), R(d) = exp(rho(d) - k d)
-  float wlog[UN][C];                                       // log2 of the last normalisers' reciprocals (without tilt)
+  // log2 of the last normalisers' reciprocals, without tilt (straight to memory where registers are short)
+  float wlog[F::SPLIT ? 1 : UN * C];
 #pragma unroll
-  for (int u = 0; u < UN; ++u)
-#pragma unroll
-    for (int n = 0; n < C; ++n) wlog[u][n] = 0.0f;
+  for (int k = 0; k < (F::SPLIT ? 1 : UN * C); ++k) wlog[k] = 0.0f;
   all_sync<C>();
 
   double acc = 0.0;                                        // this thread's part of T * loss
@@ -553,10 +575,15 @@ saf_fit_fft_kernel(FitState s, int steps, const double* __restrict__ plogp, floa
           w[u][n] = in ? r : 0.0;
           const float lg = __log2f(static_cast<float>(z[n])), fi = static_cast<float>(pos(u, n));
           slope = fmaf(fi - 0.5f * (T - 1), lg, slope);    // (beyond T: log 1)
-          z[n] = in_bounds ? -lg - ft * fi : wlog[u][n];
+          z[n] = -lg - ft * fi;
         }
+        if (in_bounds) {
 #pragma unroll
-        for (int n = 0; n < C; ++n) wlog[u][n] = static_cast<float>(z[n]);
+          for (int n = 0; n < C; ++n) {
+            if (!F::SPLIT) wlog[F::SPLIT ? 0 : u * C + n] = static_cast<float>(z[n]);
+            else if (pos(u, n) < T) s.wref[o + pos(u, n)] = static_cast<float>(z[n]);
+          }
+        }
         ok = ok && in_bounds;
         if (!last) send(FW, w[u], u);
       }
@@ -660,12 +687,12 @@ saf_fit_fft_kernel(FitState s, int steps, const double* __restrict__ plogp, floa
 
   if (failed) {
     // the parameters are those before this step; a reference for the normalisers goes along (of this step or the last)
-    if (!F::SPLIT || my_vec == 0) {
+    if (!F::SPLIT) {
 #pragma unroll
       for (int u = 0; u < UN; ++u)
 #pragma unroll
         for (int n = 0; n < C; ++n)
-          if (pos(u, n) < T) s.wref[o + pos(u, n)] = wlog[u][n];
+          if (pos(u, n) < T) s.wref[o + pos(u, n)] = wlog[F::SPLIT ? 0 : u * C + n];
     }
     if (!(step & 1)) {                                     // the state before the step, from the second copy to the first
 #pragma unroll
@@ -700,7 +727,7 @@ saf_fit_fft_kernel(FitState s, int steps, const double* __restrict__ plogp, floa
   for (int k = 16; k > 0; k >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, k);
   if (lane == 0) {
     if (C == 1) lossp[warp] = acc;
-    else st_peer(peer(smem_a(lossp + rank * NW + warp), 0), acc);
+    else st_peer(peer<F::SPLIT>(smem_a(lossp + rank * NW + warp), 0), acc);
   }
   all_sync<C>();
   if (rank == 0 && tid == 0) {
@@ -746,7 +773,7 @@ cudaError_t fft_dispatch(int logl, int c, int* active, bool go, const FitState& 
 }  // namespace
 
 // One transform of 512 points (128 threads, three CTAs per SM) per CTA and as many CTAs as that takes, up to eight: us a step of
-// one head, clusters of 1 / 2 / 4 / 8: 1024 positions 9.2 / 7.5, 2048 14.8 / 11.4 / 8.4, 4096 - / 18.3 / 12.8 / 10.7.  With
+// one head, clusters of 1 / 2 / 4 / 8: 1024 positions 9.2 / 7.5, 2048 14.8 / 11.4 / 8.4, 4096 - / 18.3 / 12.8 / 9.9.  With
 // more heads of 4096 than fit at once (48 clusters of eight), 71 clusters of four do.
 cudaError_t launch_fit_fft(const FitState& s, int Hf, int steps, const double* plogp, float* alpha_out, float* rho_out,
                            float* logZ_out, long long out_stride, double* loss_out, double* kl_out, cudaStream_t st) {

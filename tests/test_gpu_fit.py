@@ -340,7 +340,8 @@ def test_fit_transform_lengths(Hf, T, steps):
 # Steps of 3 and 10 nats take heads out of the transforms' bounds after a few steps, so that both parities of the step at which
 # they are handed on occur; what was done before must not be lost: the parameters after few steps against the oracle (the direct
 # sums' bounds above), the normalisers at the returned parameters always.
-@pytest.mark.parametrize("T,lr,steps", [(200, 3.0, 6), (300, 10.0, 3), (300, 10.0, 4), (300, 10.0, 7), (700, 10.0, 5), (1500, 10.0, 6)])
+@pytest.mark.parametrize("T,lr,steps", [(200, 3.0, 6), (300, 10.0, 3), (300, 10.0, 4), (300, 10.0, 7), (700, 10.0, 5), (1500, 10.0, 6),
+                                        (2500, 10.0, 5), (2500, 10.0, 6)])
 def test_fit_heads_handed_on(T, lr, steps):
     A = si.mean_attention_maps(2, T, 70 + T)
     P, ea, er, pl = _oracle_stats(A)
