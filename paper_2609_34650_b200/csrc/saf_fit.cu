@@ -284,7 +284,8 @@ struct FitPlan {
 // multiply-adds (128 per clock and SM), 1.5 T^2 per head and step.  Measured (36 heads, T = 4096, 400 steps): 23.4 ms =
 // 58 us per step on 108 SMs, against 100.2 ms for one exponential per pair and sum in two launches per step; 57 % of those
 // SMs' multiply-add peak over everything.  One head of 256 positions: 6.0 us per
-// step (two cluster barriers, L2 round trips of the parameters, fp64 Adam).
+// step (two cluster barriers, L2 round trips of the parameters, fp64 Adam).  Heads of more than 128 positions start in
+// saf_fit_fft_kernel (13.9 us a step of the 36) and come here only from there.
 template <int NW, bool PADDED, int RB>
 __global__ void __launch_bounds__(NW * 32, 1)
 saf_fit_kernel(FitState s, int steps, const double* __restrict__ plogp, float* __restrict__ alpha_out,
