@@ -300,7 +300,9 @@ void build_worklist_host(int B, int H, int T, const uint8_t* mask, int backward,
 
 // Work queue of the 128-wide forward.  An item is two consecutive query blocks of one (batch, head) unit (the first
 // block of an odd count goes alone), which share every K and V tile, or one block: of an ordinary head split over the
-// kernel's two chains (even and odd key tiles), of a frozen head in one.  Single blocks halve the longest items where these would
+// kernel's two chains (even and odd key tiles), of a frozen head in one, as in units of up to three blocks (the merge then costs
+// about what the chains save: us split / not 1x32x256x96 10.4 / 9.9, 1x32x333x128 11.8 / 11.4, on shared heads 15.4 / 15.1,
+// 1x16x333x128 13.0 / 13.4; with four blocks 1x16x512x128 15.3 / 16.0).  Single blocks halve the longest items where these would
 // set the time, at the cost of twice the loads and item ends; which blocks go alone is decided by build_pair_order.
 // CTAs claim items in this order at run time, so longest-first within groups of
 // units keeps both the tail short and a group's K and V in L2 while its items run.  Group sizes differ by at most one unit (a
@@ -325,7 +327,7 @@ void build_pair_order(int B, int H, int T, int D, const uint8_t* mask, int froze
       const int b = static_cast<int>(u / H), h = static_cast<int>(u % H);
       const int kind = mask[h] ? KIND_FROZEN : KIND_ORDINARY;
       for (int q = nblk - 1; q >= 0;) {
-        const bool two = q > 0 && pair_item_ns(q + 1, true, !mask[h]) <= cap, split = !two && q > 0 && !mask[h];
+        const bool two = q > 0 && pair_item_ns(q + 1, true, !mask[h]) <= cap, split = !two && q > 0 && nblk > 3 && !mask[h];
         // (half tiles: a split block takes half the time of a pair of the same length)
         const long long half = two ? 2 * (2 * q + 1) : split ? q + 1 : 2 * (q + 1);
         items.push_back({(mask[h] ? frozen_pct : 100) * half, WorkItem{b, h, q, kind | (two ? KIND_PAIR : split ? KIND_SPLIT : 0)}});
@@ -340,7 +342,7 @@ void build_pair_order(int B, int H, int T, int D, const uint8_t* mask, int froze
 // The cap whose order ends first in a simulated run on num_sms CTAs, over a few caps between "all blocks alone" and "all in pairs", while
 // there are up to three blocks per SM (beyond, the pairs' tail is short and the longer loads of single blocks count: 1x16x8192x128
 // 247 us in pairs, 268 alone).  us of back-to-back forwards without frozen heads, pairs (blocks alone and in one chain up to
-// one per SM) / this: 1x32x333x128 12.2 / 11.7, 1x8x1024x128 20.0 / 16.1, 1x8x2048x128 34.5 / 25.6, 1x16x1300x128 29.4 / 21.2,
+// one per SM) / this: 1x8x1024x128 20.0 / 16.1, 1x8x2048x128 34.5 / 25.6, 1x16x1300x128 29.4 / 21.2,
 // 1x8x4096x128 70.7 / 43.6, 1x4x8192x128 132 / 76, 1x12x4096x128 72.7 / 68.3, 4x12x900x128 28.2 / 28.2.
 long long choose_pair_cap(int B, int H, int T, int D, const uint8_t* mask, int num_sms, int frozen_pct) {
   const int nblk = (T + BLK - 1) / BLK;
