@@ -182,8 +182,13 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   // the prologue above overlapped the previous kernel's tail; global memory is touched only from here on
-  pdl_launch_dependents();
+  // On a grid that fills much of the chip the next kernel is let in only once the one in front has ended: let in before, a queue of
+  // passes runs two kernels deep and its waiting CTAs hold back the one in front (1x32x333x128 on shared heads, 96 CTAs: 15.5 us
+  // a pass, 14.5 so; updates on few CTAs want it at once: 1x4x139x96 27.8 us, 28.6 so).
+  const bool at_once = gridDim.x <= 64;
+  if (at_once) pdl_launch_dependents();
   pdl_wait();
+  if (!at_once) pdl_launch_dependents();
 
   // (each warpgroup sets its register share at the top of its own branch)
   if (warp >= 12) {
