@@ -199,6 +199,10 @@ int saf_fit_compact(saf_ctx* ctx, int32_t Hf, int32_t T, const double* eta_abs, 
                     const double* plogp, int32_t steps, double lr, float* alpha_out, float* rho_out, float* logZ_out,
                     int64_t out_stride, double* loss_out, double* kl_out, void* stream);
 
+/* The fp64 functions that saf_fit_compact uses in place of the library's, for tests: y[i] = 1 / x[i] (`which` 0), sqrt(x[i]) (1)
+ * or exp(x[i]) (2), x and y device float64 [n].  SAF_ERR_INVALID_ARG for any other `which`.  Asynchronous on `stream`. */
+int saf_fit_math(int32_t device, int32_t which, int32_t n, const double* x, double* y, void* stream);
+
 /* Calibration statistics of one layer, streaming part (Sec. 3.1 "Calibration and head selection";
  * Eq. "variance-score", Eq. "forward-kl-score").  For the `problem->B` calibration sequences of this call and every
  * head, the attention maps A^(n) = softmax_causal(Q K^T scale) are formed tile by tile (never stored) and added up:

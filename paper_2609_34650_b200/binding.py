@@ -67,10 +67,11 @@ def load_library() -> C.CDLL:
     lib.saf_get_kernel_time.argtypes = [vp, i32, C.POINTER(C.c_float), C.POINTER(C.c_int32)]
     lib.saf_pattern_logz_static.argtypes = [i32, i32, i32, u8p, f32p, f32p, f32p, vp]
     lib.saf_pattern_logz_static.restype = C.c_int
+    lib.saf_fit_math.argtypes = [i32, i32, i32, vp, vp, vp]
     lib.saf_build_worklist.argtypes = [i32, i32, i32, u8p, i32, i32, i32, C.POINTER(C.c_int32), C.POINTER(C.c_int32)]
     for name in ("saf_create", "saf_destroy", "saf_pattern_prepare", "saf_hybrid_attn_fwd", "saf_hybrid_attn_bwd",
                  "saf_hybrid_attn_step_host", "saf_last_device_status", "saf_build_worklist", "saf_set_profiling",
-                 "saf_get_kernel_time", "saf_pattern_grad", "saf_fit_marginals", "saf_fit_compact", "saf_calib_accumulate", "saf_calib_finalize"):
+                 "saf_get_kernel_time", "saf_pattern_grad", "saf_fit_marginals", "saf_fit_compact", "saf_calib_accumulate", "saf_calib_finalize", "saf_fit_math"):
         getattr(lib, name).restype = C.c_int
     _lib = lib
     return lib
@@ -151,6 +152,11 @@ def make_problem(q_like, Tp, softmax_scale=0.0, grad_dtype=SAF_F32, k_like=None,
         arr = getattr(p, name)
         arr[0], arr[1], arr[2] = t.stride(0), t.stride(1), t.stride(2)
     return p
+
+
+def saf_fit_math(device, which, x, y):
+    """y = 1 / x (which = 0), sqrt(x) (1) or exp(x) (2) by the fitter's own fp64 functions."""
+    _check(load_library().saf_fit_math(device, which, x.numel(), _ptr(x), _ptr(y), _stream()), "saf_fit_math")
 
 
 class Context:

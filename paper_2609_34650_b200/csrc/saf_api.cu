@@ -1352,6 +1352,14 @@ int saf_fit_compact(saf_ctx* ctx, int32_t Hf, int32_t T, const double* eta_abs, 
   return SAF_OK;
 }
 
+int saf_fit_math(int32_t device, int32_t which, int32_t n, const double* x, double* y, void* stream) {
+  if (which < 0 || which > 2 || n < 0 || (n > 0 && (!x || !y))) return SAF_ERR_INVALID_ARG;
+  if (n == 0) return SAF_OK;
+  DeviceGuard g(device);
+  if (!g.ok) return SAF_ERR_CUDA;
+  return launch_fit_math(which, n, x, y, static_cast<cudaStream_t>(stream)) == cudaSuccess ? SAF_OK : SAF_ERR_CUDA;
+}
+
 int saf_calib_accumulate(saf_ctx* ctx, const saf_problem* p, const void* Q, const void* K, const float* LSE,
                          float* mean_sum, double* sumsq, double* sum_plogp, int32_t accumulate, void* stream) {
   if (!ctx || !p || !mean_sum || !sumsq || !sum_plogp) return SAF_ERR_INVALID_ARG;

@@ -38,6 +38,7 @@
 #include <cstdint>
 #include <cmath>
 #include <algorithm>
+#include "saf_fit_math.cuh"
 #include "saf_internal.h"
 
 namespace saf {
@@ -68,47 +69,6 @@ __device__ __forceinline__ cd cmulc(cd a, cd b) {                      // a conj
 }
 __device__ __forceinline__ cd cadd(cd a, cd b) { return make_double2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ cd csub(cd a, cd b) { return make_double2(a.x - b.x, a.y - b.y); }
-
-// Branch-free fp64 functions, so that a thread's elements overlap (the library's, with their special cases, took two thirds
-// of a step).  Seeds of about 20 bits from the special-function unit, then Newton / Halley steps; arguments are positive and
-// normal here.
-__device__ __forceinline__ double rcp64(double a) {
-  double x;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(x) : "d"(a));
-  const double e = fma(-a, x, 1.0);
-  x = fma(x, fma(e, e, e), x);
-  return fma(x, fma(-a, x, 1.0), x);
-}
-__device__ __forceinline__ double sqrt64(double a) {
-  double r;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
-  const double e = fma(-a * r, r, 1.0);
-  r = fma(r * e, fma(0.375, e, 0.5), r);
-  const double q = a * r;
-  return fma(0.5 * r, fma(-q, q, a), q);
-}
-// e^x = 2^n e^f, |f| <= ln 2 / 2, by the Taylor sum to f^13 (remainder 4e-18); x beyond +-700 saturates
-__device__ __forceinline__ double exp64(double x) {
-  x = fmin(fmax(x, -700.0), 700.0);
-  const double big = fma(x, 1.4426950408889634074, 6755399441055744.0);       // 1.5 * 2^52: n in the low bits
-  const double n = big - 6755399441055744.0;
-  const double f = fma(n, -2.3190468138462996e-17, fma(n, -LN2_D, x));          // ln 2 as two doubles
-  double p = 1.0 / 6227020800.0;
-  p = fma(p, f, 1.0 / 479001600.0);
-  p = fma(p, f, 1.0 / 39916800.0);
-  p = fma(p, f, 1.0 / 3628800.0);
-  p = fma(p, f, 1.0 / 362880.0);
-  p = fma(p, f, 1.0 / 40320.0);
-  p = fma(p, f, 1.0 / 5040.0);
-  p = fma(p, f, 1.0 / 720.0);
-  p = fma(p, f, 1.0 / 120.0);
-  p = fma(p, f, 1.0 / 24.0);
-  p = fma(p, f, 1.0 / 6.0);
-  p = fma(p, f, 0.5);
-  p = fma(p, f, 1.0);
-  p = fma(p, f, 1.0);
-  return __hiloint2double(__double2hiint(p) + (__double2loint(big) << 20), __double2loint(p));
-}
 
 template <bool INV>
 __device__ __forceinline__ cd rot90(cd a) {                            // times -i (INV: i)
@@ -558,9 +518,10 @@ saf_fit_fft_kernel(FitState s, int steps, const double* __restrict__ plogp, floa
 #pragma unroll
       for (int n = 0; n < C; ++n) w[u][n] = 0.0;
     if (!F::SPLIT || my_vec == 0) {
-      const double lim = static_cast<double>(GUARD) * na * nr;
+      // (1e-30 .. 1e30: rcp64 and the fp32 logarithm)
+      const double lim = fmax(static_cast<double>(GUARD) * na * nr, 1e-30);
       const float ft = static_cast<float>(tilt / LN2_D);
-      bool ok = lim > 0.0;
+      bool ok = na * nr > 0.0f;
 #pragma unroll
       for (int u = 0; u < UN; ++u) {
         double z[C];
@@ -672,7 +633,7 @@ saf_fit_fft_kernel(FitState s, int steps, const double* __restrict__ plogp, floa
         const double g = (fitted - st[half][e][3]) * iT;
         const double m = fma(0.9, st[half][e][1], 0.1 * g);
         const double q = fma(0.999, st[half][e][2], 0.001 * g * g);
-        const double pnew = fma(-s.lr * (m * ib1), rcp64(sqrt64(fmax(q * ib2, 1e-200)) + 1e-8), st[half][e][0]);
+        const double pnew = fma(-s.lr * (m * ib1), rcp64(sqrt64(q * ib2) + 1e-8), st[half][e][0]);
         const double ex = exp64(fma(-tilt, static_cast<double>(i), pnew));
         value = i < T ? ex : 0.0;
         if (i < T) {
@@ -770,7 +731,17 @@ cudaError_t fft_dispatch(int logl, int c, int* active, bool go, const FitState& 
   return cudaErrorInvalidValue;
 }
 
+__global__ void saf_fit_math_kernel(int which, int n, const double* __restrict__ x, double* __restrict__ y) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) y[i] = which == 0 ? rcp64(x[i]) : which == 1 ? sqrt64(x[i]) : exp64(x[i]);
+}
+
 }  // namespace
+
+cudaError_t launch_fit_math(int which, int n, const double* x, double* y, cudaStream_t st) {
+  saf_fit_math_kernel<<<(n + 255) / 256, 256, 0, st>>>(which, n, x, y);
+  return cudaGetLastError();
+}
 
 // One transform of 512 points (128 threads, three CTAs per SM) per CTA and as many CTAs as that takes, up to eight: us a step of
 // one head, clusters of 1 / 2 / 4 / 8: 1024 positions 9.2 / 7.5, 2048 14.8 / 11.4 / 8.4, 4096 - / 18.3 / 12.8 / 9.9.  With

@@ -244,6 +244,7 @@ cudaError_t launch_fit_marginals(const float* Abar, float floor_v, double* eta_a
                                  int Hf, int T, int num_sms, cudaStream_t st);
 cudaError_t launch_fit_fft(const FitState& s, int Hf, int steps, const double* plogp, float* alpha_out, float* rho_out,
                            float* logZ_out, long long out_stride, double* loss_out, double* kl_out, cudaStream_t st);
+cudaError_t launch_fit_math(int which, int n, const double* x, double* y, cudaStream_t st);
 cudaError_t launch_fit(FitState s, int Hf, int steps, const double* plogp, float* alpha_out, float* rho_out,
                        float* logZ_out, long long out_stride, double* loss_out, double* kl_out, cudaStream_t st);
 

@@ -353,3 +353,34 @@ def test_fit_heads_handed_on(T, lr, steps):
         wa, wr, wz = fo.fit_compact(ea[h], er[h], steps=steps, lr=lr)
         # a gradient that nearly cancels may take the other sign in one element: most elements, not all
         assert np.mean(np.abs(a[h] - wa) < 1e-2 * lr) > 0.97 and np.mean(np.abs(r[h] - wr) < 1e-2 * lr) > 0.97
+
+
+# Largest errors in units in the last place: a correctly rounded result has 0.5; the exponential's argument reduction and sum add a
+# quarter (0.76 over 2e7 arguments evaluated on a CPU with the same steps).  Ranges: normalisers and Adam's denominators, moments,
+# parameters.
+@pytest.mark.parametrize("which,lo,hi,ulps", [(0, 1e-30, 1e30, 0.51), (0, 1e-8, 1e150, 0.51), (1, 1e-199, 1e290, 0.51), (2, -690.0, 690.0, 0.8),
+                                              (2, -1.0, 1.0, 0.8)])
+def test_fit_math(which, lo, hi, ulps):
+    rng = np.random.default_rng(which)
+    n = 1 << 20
+    x = rng.uniform(lo, hi, n) if which == 2 else np.exp(rng.uniform(np.log(lo), np.log(hi), n))
+    x[:4] = [lo, hi, *((0.0, 0.5) if which == 2 else (1.0, 4.0))]
+    xd = torch.from_numpy(x).cuda()
+    y = torch.empty_like(xd)
+    saf.saf_fit_math(0, which, xd, y)
+    got = y.cpu().numpy()
+    assert np.finfo(np.longdouble).nmant >= 63
+    xl = x.astype(np.longdouble)
+    want = 1.0 / xl if which == 0 else np.sqrt(xl) if which == 1 else np.exp(xl)
+    err = np.abs(got.astype(np.longdouble) - want) / np.spacing(want.astype(np.float64))
+    assert err.max() <= ulps, (err.max(), x[err.argmax()])
+
+
+def test_fit_math_ends():
+    y = torch.empty(2, dtype=torch.float64, device="cuda")
+    saf.saf_fit_math(0, 1, torch.zeros(2, dtype=torch.float64, device="cuda"), y)
+    assert ((0.0 <= y) & (y <= 1e-99)).all()
+    saf.saf_fit_math(0, 2, torch.tensor([-1e9, 1e9], dtype=torch.float64, device="cuda"), y)
+    assert 0.0 < y[0] < 1e-300 and 1e300 < y[1] < float("inf")
+    with pytest.raises(saf.SafError):
+        saf.saf_fit_math(0, 3, y, y)
