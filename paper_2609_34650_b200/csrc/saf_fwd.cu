@@ -583,7 +583,7 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
             for (int k = 0; k < 4; ++k)
               mx[k] = max3(mx[k], __uint_as_float(r[2 + (k >> 1)][e + 2 * (k & 1)]), __uint_as_float(r[2 + (k >> 1)][e + 2 * (k & 1) + 1]));
           if (q4 == 0) TRF(1 + t, 13);
-          const float m_new = fmaxf(m_ref, fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * c);   // finite: key 0 is visible to every row
+          const float m_new = fmaxf(m_ref, fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * c);
           if (j == 0) {
             m_ref = m_new;
           } else {
@@ -604,7 +604,10 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
               }
             }
           }
-          const uint64_t nm2 = pk2(-m_ref, -m_ref);
+          // (the second chain of a split block does not start at key 0: all its scores of a row so far may be -inf, by overflow of
+          // Q K^T; they count zero then, and a finite maximum later scales sums and accumulator, zeros so far, by zero)
+          const float neg_m = SPLIT && m_ref == -INFINITY ? 0.0f : -m_ref;
+          const uint64_t nm2 = pk2(neg_m, neg_m);
 #pragma unroll
           for (int cc = 0; cc < 4; ++cc) {
             uint32_t pk[16];
@@ -647,7 +650,7 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
           if (!mbar_wait_warp_compact(x_full, nx++ & 1, wc, SITE_X_FULL)) ok = false;
           const float l1 = linv[128 + rowl], m1 = xm[rowl];
           m_all = fmaxf(m_ref, m1);
-          const float f0 = ex2_approx(m_ref - m_all), f1 = ex2_approx(m1 - m_all);
+          const float f0 = ex2_approx(m_ref - m_all), f1 = ex2_approx(m1 - m_all);   // (NaN where no chain has a finite score)
           l_all = fmaf(f0, l, f1 * l1);
           linv[rowl] = f0 / l_all;
           linv[128 + rowl] = f1 / l_all;

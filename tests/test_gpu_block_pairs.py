@@ -213,6 +213,29 @@ def test_running_maximum_far_above_the_first_tile_in_split_and_paired_blocks(B, 
     assert np.abs(got - want).max() <= 2e-2 and np.linalg.norm(got - want) <= 1e-2 * np.linalg.norm(want)
 
 
+@pytest.mark.parametrize("D,T,tiles", [(128, 640, (1,)), (96, 640, (1,)), (128, 1000, (1, 3, 5)), (128, 640, (2,))])
+def test_a_chain_of_a_split_block_whose_scores_overflow(D, T, tiles):
+    """Finite Q and K whose product is -inf throughout some key tiles: rows that see other keys as well are finite, wherever in
+    its chain the tile comes (tile 1 is the first of chain 1, and all of it for the block whose own tile it is)."""
+    inp = si.generate(si.Workload("overflow", 1, 4, T, D, (), -0.05, seed=T))
+    big = si.f32_to_bf16_bits(np.float32([1e20, -1e20, 0.0]))
+    inp.q[..., 0] = big[0]
+    inp.k[..., 0] = big[2]
+    for t in tiles:
+        inp.k[:, :, 128 * t:128 * (t + 1), 0] = big[1]
+    L = Layer(inp, backward=False)
+    c = L.ctx
+    c.saf_hybrid_attn_fwd(L.prob, L.Q, L.K, L.V, L.mask, None, None, None, L.O, L.LSE)
+    torch.cuda.synchronize()
+    assert c.saf_last_device_status()[0] == saf.SAF_OK
+    q, k, v = (si.bf16_bits_to_f64(x) for x in (inp.q, inp.k, inp.v))
+    want, lse = orc.hybrid_attn_fwd(q, k, v, inp.mask, inp.alpha, inp.rho)
+    got = L.O.float().cpu().numpy().astype(np.float64)
+    assert np.isfinite(got).all(), np.argwhere(~np.isfinite(got).all(axis=-1))[:3]
+    assert np.abs(got - want).max() <= 2e-2 and np.linalg.norm(got - want) <= 1e-2 * np.linalg.norm(want)
+    assert np.abs(L.LSE.cpu().numpy() - lse).max() <= 1e-4
+
+
 def test_chunks_of_the_host_step_take_the_forms_of_the_whole_batch():
     """8 x 4 heads x 12 blocks = 384: some blocks split, some paired; chunks of one batch entry (48 blocks) alone would all be
     split."""
