@@ -32,8 +32,8 @@
 // positions), so every step uses the k that makes the last step's log Z level (2^19 and 2^12).  A head stays here while every
 // Z is at least 2^-28 |A||R| and every marginal, or the target it is compared with, at least 2^-28 of A(j) |R||W| or R(d) |A||W|,
 // so that no error exceeds 1.5e-7 of these (the direct fp32 sums: 1.4e-7 in the mean, 8e-7 at most); a head that leaves the
-// bounds is handed to saf_fit_kernel, which has no such restriction, at the step it has reached.  Its state before that step
-// is still there: the steps write to two copies in turn.
+// bounds, or whose targets are not finite, is handed to saf_fit_kernel, which has no such restriction, at the step it has
+// reached.  Its state before that step is still there: the steps write to two copies in turn.
 #include <cuda_runtime.h>
 #include <cstdint>
 #include <cmath>
@@ -629,10 +629,11 @@ saf_fit_fft_kernel(FitState s, int steps, const double* __restrict__ plogp, floa
         const int u = F::SPLIT ? 0 : e / C, n = F::SPLIT ? 4 * half + e : e % C, i = pos(u, n);
         double& value = val[F::SPLIT ? 0 : half][u][n];
         const double fitted = S[u][n] * value;
-        ok = ok && fmax(fitted, st[half][e][3]) >= (is_rho ? lim_g : lim_c) * value;
         const double g = (fitted - st[half][e][3]) * iT;
         const double m = fma(0.9, st[half][e][1], 0.1 * g);
         const double q = fma(0.999, st[half][e][2], 0.001 * g * g);
+        // (fmax drops a NaN, which q holds: NaN and infinite targets go to the direct sums, which pass them on to the whole head)
+        ok = ok && fmax(fitted, st[half][e][3]) >= (is_rho ? lim_g : lim_c) * value && q < 1e300;
         const double pnew = fma(-s.lr * (m * ib1), rcp64(sqrt64(q * ib2) + 1e-8), st[half][e][0]);
         const double ex = exp64(fma(-tilt, static_cast<double>(i), pnew));
         value = i < T ? ex : 0.0;

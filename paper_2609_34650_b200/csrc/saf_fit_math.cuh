@@ -30,10 +30,10 @@ __device__ __forceinline__ double sqrt64(double a) {
   return g + fma(g, e * fma(e, fma(e, 0.3125, 0.375), 0.5), 0.5 * d);
 }
 
-// x beyond +-700 saturates
+// x beyond +-700 saturates, NaN stays
 __device__ __forceinline__ double exp64(double x) {
   constexpr double L2E = 1.4426950408889634074, L2E_LO = 2.0355273740931033e-17, LN2 = 0.6931471805599453094, LN2_LO = 2.3190468138462996e-17;
-  x = fmin(fmax(x, -700.0), 700.0);
+  x = x > 700.0 ? 700.0 : x < -700.0 ? -700.0 : x;
   const double h = x * L2E, l = fma(x, L2E_LO, fma(x, L2E, -h));
   const int n = __double2int_rn(h);
   const double r = (h - static_cast<double>(n)) + l;

@@ -382,5 +382,23 @@ def test_fit_math_ends():
     assert ((0.0 <= y) & (y <= 1e-99)).all()
     saf.saf_fit_math(0, 2, torch.tensor([-1e9, 1e9], dtype=torch.float64, device="cuda"), y)
     assert 0.0 < y[0] < 1e-300 and 1e300 < y[1] < float("inf")
+    for which in range(3):
+        saf.saf_fit_math(0, which, torch.full((2,), float("nan"), dtype=torch.float64, device="cuda"), y)
+        assert torch.isnan(y).all(), which
     with pytest.raises(saf.SafError):
         saf.saf_fit_math(0, 3, y, y)
+
+
+@pytest.mark.parametrize("T", [100, 300, 2500])
+@pytest.mark.parametrize("which,value", [(0, float("nan")), (1, float("nan")), (0, float("inf")), (1, float("inf"))])
+def test_a_target_that_is_not_finite_spoils_its_whole_head_and_no_other(T, which, value):
+    """One NaN or infinite element of eta_abs (0) or eta_rel (1): after two steps it is in every normaliser and gradient, so
+    that no caller installs a pattern from it by looking at one output alone."""
+    A = si.mean_attention_maps(2, T, 80 + T)
+    P, ea, er, pl = _oracle_stats(A)
+    clean = _gpu_fit(_ctx(), _dev(ea), _dev(er), _dev(pl), 4)
+    (ea, er)[which][0, 17] = value
+    got = _gpu_fit(_ctx(), _dev(ea), _dev(er), _dev(pl), 4)
+    for x, y in zip(got, clean):
+        assert np.array_equal(x[1], y[1])
+        assert not np.isfinite(x[0]).any()
