@@ -108,8 +108,9 @@ def _stream():
     global _raw_stream
     if _raw_stream is None:
         import torch
-        current_device, raw = torch.cuda.current_device, torch._C._cuda_getCurrentRawStream
-        _raw_stream = lambda: raw(current_device())
+        current_device, raw = torch.cuda.current_device, getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        # (the query behind the public one, which other torch releases need not have)
+        _raw_stream = (lambda: raw(current_device())) if raw else (lambda: torch.cuda.current_stream().cuda_stream)
     return _raw_stream()
 
 

@@ -67,6 +67,15 @@ def test_create_fails_loudly_without_a_gpu(lib):
         lib.Context(0)
 
 
+def test_the_stream_is_found_without_torchs_private_query(lib, monkeypatch):
+    import types
+    from paper_2609_34650_b200 import binding
+    monkeypatch.setattr(binding, "_raw_stream", None)
+    monkeypatch.delattr(torch._C, "_cuda_getCurrentRawStream", raising=False)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: types.SimpleNamespace(cuda_stream=0x1234))
+    assert binding._stream() == 0x1234
+
+
 # --------------------------------------------------------------------------- scheduler
 @pytest.mark.parametrize("backward", [0, 1])
 @pytest.mark.parametrize("B,H,T,frozen,ncta", [(8, 12, 4096, (1, 5, 7), 296), (1, 4, 256, (0,), 8),
