@@ -687,8 +687,10 @@ cudaError_t launch_fit(FitState s, int Hf, int steps, const double* plogp, float
   // 5.2 / 4.8, 100 5.1 / 5.2, 256 5.9 / 5.1, 1024 9.1 / 7.5, 4096 22.8 / 10.1)
   s.resume = s.T > 128 ? s.resume : nullptr;
   if (s.resume) {
-    const cudaError_t e = launch_fit_fft(s, Hf, steps, plogp, alpha_out, rho_out, logZ_out, out_stride, loss_out, kl_out, st);
+    bool launched = false;
+    const cudaError_t e = launch_fit_fft(s, Hf, steps, plogp, alpha_out, rho_out, logZ_out, out_stride, loss_out, kl_out, st, &launched);
     if (e != cudaSuccess) return e;
+    if (!launched) s.resume = nullptr;
   }
   // up to 8192 positions the padded vectors fit beside the partial sums of 16 warps, up to 12288 beside those of 12; the
   // longest sequences keep them unpadded (two-way bank conflicts on the window reads)

@@ -747,22 +747,33 @@ cudaError_t launch_fit_math(int which, int n, const double* x, double* y, cudaSt
 // One transform of 512 points (128 threads, three CTAs per SM) per CTA and as many CTAs as that takes, up to eight: us a step of
 // one head, clusters of 1 / 2 / 4 / 8: 1024 positions 9.2 / 7.5, 2048 14.8 / 11.4 / 8.4, 4096 - / 18.3 / 12.8 / 9.9.  With
 // more heads of 4096 than fit at once (48 clusters of eight), 71 clusters of four do.
+// *launched: false where no such cluster can be resident (then nothing was launched and the direct sums, which run in any
+// cluster size, serve all heads).
 cudaError_t launch_fit_fft(const FitState& s, int Hf, int steps, const double* plogp, float* alpha_out, float* rho_out,
-                           float* logZ_out, long long out_stride, double* loss_out, double* kl_out, cudaStream_t st) {
+                           float* logZ_out, long long out_stride, double* loss_out, double* kl_out, cudaStream_t st, bool* launched) {
   int logm = 8;
   while ((1 << logm) < s.T) ++logm;
   int lc = std::max(0, std::min(3, logm - 9));
-  auto dispatch = [&](int logl, int c, int* active) {
-    return fft_dispatch(logl, c, active, active == nullptr, s, Hf, st, steps, plogp, alpha_out, rho_out, logZ_out, out_stride,
+  auto dispatch = [&](int lc, int* active) {
+    return fft_dispatch(logm - lc, 1 << lc, active, active == nullptr, s, Hf, st, steps, plogp, alpha_out, rho_out, logZ_out, out_stride,
                         loss_out, kl_out);
   };
+  auto resident = [&](int lc) {
+    int n = 0;
+    if (dispatch(lc, &n) == cudaSuccess) return n;
+    cudaGetLastError();
+    return 0;
+  };
+  int n = resident(lc);
   if (logm == 12) {
-    int n8 = 0, n4 = 0;
-    if (dispatch(9, 8, &n8) != cudaSuccess || n8 < 1 ||
-        (Hf > n8 && dispatch(10, 4, &n4) == cudaSuccess && n4 > 0 && 18 * ((Hf + n4 - 1) / n4) < 15 * ((Hf + n8 - 1) / n8)))
+    const int n4 = resident(2);
+    if (n4 > 0 && (n < 1 || (Hf > n && 18 * ((Hf + n4 - 1) / n4) < 15 * ((Hf + n - 1) / n)))) {
       lc = 2;
+      n = n4;
+    }
   }
-  return dispatch(logm - lc, 1 << lc, nullptr);
+  *launched = n > 0;
+  return n > 0 ? dispatch(lc, nullptr) : cudaSuccess;
 }
 
 }  // namespace saf

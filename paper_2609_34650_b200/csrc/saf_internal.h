@@ -243,7 +243,7 @@ int fit_max_T();
 cudaError_t launch_fit_marginals(const float* Abar, float floor_v, double* eta_abs, double* eta_rel, double* plogp,
                                  int Hf, int T, int num_sms, cudaStream_t st);
 cudaError_t launch_fit_fft(const FitState& s, int Hf, int steps, const double* plogp, float* alpha_out, float* rho_out,
-                           float* logZ_out, long long out_stride, double* loss_out, double* kl_out, cudaStream_t st);
+                           float* logZ_out, long long out_stride, double* loss_out, double* kl_out, cudaStream_t st, bool* launched);
 cudaError_t launch_fit_math(int which, int n, const double* x, double* y, cudaStream_t st);
 cudaError_t launch_fit(FitState s, int Hf, int steps, const double* plogp, float* alpha_out, float* rho_out,
                        float* logZ_out, long long out_stride, double* loss_out, double* kl_out, cudaStream_t st);
