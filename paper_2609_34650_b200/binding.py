@@ -67,11 +67,13 @@ def load_library() -> C.CDLL:
     lib.saf_get_kernel_time.argtypes = [vp, i32, C.POINTER(C.c_float), C.POINTER(C.c_int32)]
     lib.saf_pattern_logz_static.argtypes = [i32, i32, i32, u8p, f32p, f32p, f32p, vp]
     lib.saf_pattern_logz_static.restype = C.c_int
+    lib.saf_fit_handover.argtypes = [vp, i32, C.POINTER(i32)]
     lib.saf_fit_math.argtypes = [i32, i32, i32, vp, vp, vp]
     lib.saf_build_worklist.argtypes = [i32, i32, i32, u8p, i32, i32, i32, C.POINTER(C.c_int32), C.POINTER(C.c_int32)]
     for name in ("saf_create", "saf_destroy", "saf_pattern_prepare", "saf_hybrid_attn_fwd", "saf_hybrid_attn_bwd",
                  "saf_hybrid_attn_step_host", "saf_last_device_status", "saf_build_worklist", "saf_set_profiling",
-                 "saf_get_kernel_time", "saf_pattern_grad", "saf_fit_marginals", "saf_fit_compact", "saf_calib_accumulate", "saf_calib_finalize", "saf_fit_math"):
+                 "saf_get_kernel_time", "saf_pattern_grad", "saf_fit_marginals", "saf_fit_compact", "saf_calib_accumulate", "saf_calib_finalize", "saf_fit_handover",
+                 "saf_fit_math"):
         getattr(lib, name).restype = C.c_int
     _lib = lib
     return lib
@@ -207,6 +209,12 @@ class Context:
         _check(self._lib.saf_fit_compact(self._h, int(Hf), int(T), _ptr(eta_abs), _ptr(eta_rel), _ptr(plogp),
                                          int(steps), float(lr), _ptr(alpha), _ptr(rho), _ptr(logZ), int(out_stride),
                                          _ptr(loss), _ptr(kl), _stream()), "saf_fit_compact")
+
+    def saf_fit_handover(self, Hf):
+        """Per head of the last fit: -1 transforms throughout, k >= 1 direct sums from step k on, 0 direct sums throughout."""
+        steps = np.zeros(Hf, dtype=np.int32)
+        _check(self._lib.saf_fit_handover(self._h, Hf, steps.ctypes.data_as(C.POINTER(C.c_int32))), "saf_fit_handover")
+        return steps
 
     def saf_calib_accumulate(self, prob, Q, K, LSE, mean_sum, sumsq, sum_plogp, accumulate):
         _check(self._lib.saf_calib_accumulate(self._h, C.byref(prob), _ptr(Q), _ptr(K), _ptr(LSE), _ptr(mean_sum),

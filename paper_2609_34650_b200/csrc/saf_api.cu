@@ -86,6 +86,9 @@ struct saf_ctx {
   std::vector<int> pat_heads_host;         // what pat_heads holds (and its upload source), and the stream that wrote it
   cudaStream_t pat_heads_stream = nullptr;
   bool tensor_pattern = true;              // SAF_DISABLE_TENSOR_PATTERN=1 turns the form off
+  bool fit_direct = false;                 // SAF_FIT_DIRECT=1: no fit starts in the transform form
+  int fit_heads = 0;                       // of the last fit, and its per-head hand-over steps (nullptr: direct sums throughout)
+  const int* fit_resume = nullptr;
   bool selftest_drop_load = false;         // SAF_SELFTEST_DROP_LOAD=1: see FwdParams::selftest_drop_load
   DevBuf pat_consts, pat_ok, pat_avec, pat_wvec, pat_bandf, pat_bandb, pat_heads, pat_snap, pat_marks, vt_buf, dot_buf, pg_hlist, pg_delta, pg_items, pg_offsets, fit_buf, calib_tmp;
   std::vector<int> pg_hlist_host, pg_offsets_host;   // host copies of the pattern-gradient tables (upload sources)
@@ -564,6 +567,7 @@ int saf_create(saf_ctx** out, int device) {
     if (v > 0) ctx->wait_limit_ns = static_cast<unsigned long long>(v) * 1000000ull;
   }
   if (const char* e = std::getenv("SAF_DISABLE_TENSOR_PATTERN")) ctx->tensor_pattern = std::atoi(e) == 0;
+  if (const char* e = std::getenv("SAF_FIT_DIRECT")) ctx->fit_direct = std::atoi(e) == 1;
   if (const char* e = std::getenv("SAF_SELFTEST_DROP_LOAD")) ctx->selftest_drop_load = std::atoi(e) == 1;
   if (const char* e = std::getenv("SAF_FROZEN_WEIGHT_PCT")) {
     long v = std::atol(e);
@@ -1345,9 +1349,24 @@ int saf_fit_compact(saf_ctx* ctx, int32_t Hf, int32_t T, const double* eta_abs, 
   float* f = reinterpret_cast<float*>(d + 12 * n);
   s.a2 = f; s.r2 = f + n;
   s.wref = f + 2 * n;
-  s.resume = reinterpret_cast<int*>(f + 3 * n);
+  s.resume = ctx->fit_direct ? nullptr : reinterpret_cast<int*>(f + 3 * n);
+  ctx->fit_heads = 0;
   ScopedTimer timer(ctx, SAF_KERNEL_FIT, st);
   if (launch_fit(s, Hf, steps, plogp, alpha_out, rho_out, logZ_out, out_stride, loss_out, kl_out, st) != cudaSuccess)
+    return SAF_ERR_CUDA;
+  ctx->fit_heads = Hf;
+  ctx->fit_resume = s.resume;
+  return SAF_OK;
+}
+
+int saf_fit_handover(saf_ctx* ctx, int32_t Hf, int32_t* steps_out) {
+  if (!ctx || !steps_out || Hf < 1 || Hf != ctx->fit_heads) return SAF_ERR_INVALID_ARG;
+  DeviceGuard g(ctx->device);
+  if (!g.ok) return SAF_ERR_CUDA;
+  std::fill(steps_out, steps_out + Hf, 0);
+  if (!ctx->fit_resume) return SAF_OK;
+  if (cudaStreamSynchronize(ctx->last_stream) != cudaSuccess ||
+      cudaMemcpy(steps_out, ctx->fit_resume, static_cast<size_t>(Hf) * sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
     return SAF_ERR_CUDA;
   return SAF_OK;
 }

@@ -681,7 +681,7 @@ cudaError_t launch_fit_clusters(const FitState& s, int Hf, cudaStream_t st, Args
 
 }  // namespace
 
-cudaError_t launch_fit(FitState s, int Hf, int steps, const double* plogp, float* alpha_out, float* rho_out,
+cudaError_t launch_fit(FitState& s, int Hf, int steps, const double* plogp, float* alpha_out, float* rho_out,
                        float* logZ_out, long long out_stride, double* loss_out, double* kl_out, cudaStream_t st) {
   // Up to 128 positions the direct sums are the shorter of two serial chains (us a step of one head, direct / transforms: 64
   // 5.2 / 4.8, 100 5.1 / 5.2, 256 5.9 / 5.1, 1024 9.1 / 7.5, 4096 22.8 / 10.1)

@@ -245,7 +245,8 @@ cudaError_t launch_fit_marginals(const float* Abar, float floor_v, double* eta_a
 cudaError_t launch_fit_fft(const FitState& s, int Hf, int steps, const double* plogp, float* alpha_out, float* rho_out,
                            float* logZ_out, long long out_stride, double* loss_out, double* kl_out, cudaStream_t st, bool* launched);
 cudaError_t launch_fit_math(int which, int n, const double* x, double* y, cudaStream_t st);
-cudaError_t launch_fit(FitState s, int Hf, int steps, const double* plogp, float* alpha_out, float* rho_out,
+// s.resume on entry: may use the transform form; on return: whether it does (else nullptr)
+cudaError_t launch_fit(FitState& s, int Hf, int steps, const double* plogp, float* alpha_out, float* rho_out,
                        float* logZ_out, long long out_stride, double* loss_out, double* kl_out, cudaStream_t st);
 
 // calibration statistics (saf_calib.cu)

@@ -24,6 +24,14 @@ def _ctx():
     return saf.Context(0)
 
 
+@pytest.fixture(params=["transforms", "direct"])
+def form(request, monkeypatch):
+    """A context whose fits beyond 128 positions start with the transforms, and one that takes the direct sums throughout."""
+    if request.param == "direct":
+        monkeypatch.setenv("SAF_FIT_DIRECT", "1")
+    return request.param, saf.Context(0)
+
+
 def _status(ctx):
     torch.cuda.synchronize()
     code, detail = ctx.saf_last_device_status()
@@ -245,16 +253,18 @@ def test_fit_no_heads_and_bad_arguments():
     _status(ctx)
 
 
-# One launch per call: a cluster of CTAs per head.  Edges: blocks of 256 positions (one, two, a partial one), more heads
+# The direct sums: a cluster of CTAs per head.  Edges: blocks of 256 positions (one, two, a partial one), more heads
 # than clusters fit at once, two to sixteen CTAs per cluster, and the longest sequences (12 warps instead of 16 beyond 8192
-# positions, vectors kept unpadded beyond 12288).
+# positions, vectors kept unpadded beyond 12288).  The transforms at the same sizes.
 @pytest.mark.parametrize("Hf,T,steps", [(1, 255, 3), (2, 257, 3), (1, 2304, 2), (150, 272, 2), (40, 300, 2), (1, 10300, 1),
                                         (1, 12289, 1), (16, 1500, 2)])
-def test_fit_cluster_edges(Hf, T, steps):
+def test_fit_cluster_edges(form, Hf, T, steps):
+    name, ctx = form
     base = si.mean_attention_maps(1, T, 40 + T)
     P, ea, er, pl = _oracle_stats(base)
     rep = lambda v: _dev(np.repeat(v, Hf, axis=0))
-    a, r, z, loss, kl = _gpu_fit(_ctx(), rep(ea), rep(er), rep(pl), steps)
+    a, r, z, loss, kl = _gpu_fit(ctx, rep(ea), rep(er), rep(pl), steps)
+    assert (ctx.saf_fit_handover(Hf) == (0 if name == "direct" else -1)).all()
     for x in (a, r, z, loss, kl):
         assert np.array_equal(x, np.broadcast_to(x[:1], x.shape))             # every head ran the same program
     wa, wr, wz = fo.fit_compact(ea[0], er[0], steps=steps)
@@ -266,10 +276,13 @@ def test_fit_cluster_edges(Hf, T, steps):
 # steps; magnitudes reach a few hundred nats, where an fp32 exponent argument carries 2^-24 * 2^9 = 3e-5 nats per
 # rounding, so 5e-4 is asserted on log Z (about ten roundings) against the fp64 normalisers at the returned parameters.
 @pytest.mark.parametrize("T,steps", [(100, 12), (700, 8)])
-def test_fit_leaves_the_product_range(T, steps):
+def test_fit_leaves_the_product_range(form, T, steps):
+    name, ctx = form
     A = si.mean_attention_maps(2, T, 50 + T)
     P, ea, er, pl = _oracle_stats(A)
-    a, r, z, loss, kl = _gpu_fit(_ctx(), _dev(ea), _dev(er), _dev(pl), steps, lr=10.0)
+    a, r, z, loss, kl = _gpu_fit(ctx, _dev(ea), _dev(er), _dev(pl), steps, lr=10.0)
+    at = ctx.saf_fit_handover(2)
+    assert (at == 0).all() if name == "direct" or T <= 128 else (at >= 1).all()
     assert max(np.abs(a).max(), np.abs(r).max()) > 50 * np.log(2)
     for h in range(2):
         want_z, _ = fo._logZ_and_P(a[h], r[h])
@@ -277,28 +290,29 @@ def test_fit_leaves_the_product_range(T, steps):
         assert abs(loss[h] - fo.fit_objective(a[h], r[h], ea[h], er[h])) < 5e-4 * max(1.0, abs(loss[h]))
 
 
-def test_first_step_and_loss_keep_the_accuracy_of_their_terms():
+def test_first_step_and_loss_keep_the_accuracy_of_their_terms(form):
     """The first Adam step moves alpha by lr sign(g) / (1 + 1e-8 / |g|), so that small gradients show the rounding of the
     column sums; at 40 heads a warp's chains are longest.  The loss at the returned parameters averages T normalisers, where
     only what is common to them would remain.  Chains of 64 terms round off about sqrt(64/3) 2^-25 = 1.4e-7 of a sum (measured
     3.7e-7 in alpha; 1.9e-6 with chains of 512); the loss is asserted at a quarter of the rounding 2^-25 that one fp32 factor
     common to all rows would leave (measured 3e-9; 2e-8 with the factors' own rounding in it)."""
+    ctx = form[1]
     T, Hf = 4096, 40
     base = si.mean_attention_maps(1, T, 40 + T)
     P, ea, er, pl = _oracle_stats(base)
     rep = lambda v: _dev(np.repeat(v, Hf, axis=0))
-    a, r, z, loss, kl = _gpu_fit(_ctx(), rep(ea), rep(er), rep(pl), 1)
+    a, r, z, loss, kl = _gpu_fit(ctx, rep(ea), rep(er), rep(pl), 1)
     wa, wr, wz = fo.fit_compact(ea[0], er[0], steps=1)
     assert np.linalg.norm(a[0] - wa) <= 1e-6 * np.linalg.norm(wa)
     A = si.mean_attention_maps(6, 512, 9)
     P, ea, er, pl = _oracle_stats(A)
-    a, r, z, loss, kl = _gpu_fit(_ctx(), _dev(ea), _dev(er), _dev(pl), 400)
+    a, r, z, loss, kl = _gpu_fit(ctx, _dev(ea), _dev(er), _dev(pl), 400)
     err = [loss[h] / fo.fit_objective(a[h], r[h], ea[h], er[h]) - 1.0 for h in range(6)]
     assert np.sqrt(np.mean(np.square(err))) <= 2.0 ** -27, err
 
 
-def test_a_single_long_head_spreads_over_more_than_eight_sms():
-    """Twice the length is four times the multiply-adds beside the fixed costs of a step; on eight CTAs, the largest portable
+def test_a_single_long_head_spreads_over_more_than_eight_sms(monkeypatch):
+    """The direct sums.  Twice the length is four times the multiply-adds beside the fixed costs of a step; on eight CTAs, the largest portable
     cluster, they take over (a factor of 3.2 from 4096 to 8192 positions), on sixteen not yet."""
     us = {}
     for T in (4096, 8192):
@@ -306,6 +320,7 @@ def test_a_single_long_head_spreads_over_more_than_eight_sms():
         eta = torch.rand((1, T), generator=g, device="cuda", dtype=torch.float64) * 2.0
         o = [torch.empty((1, T), device="cuda") for _ in range(3)]
         one = torch.zeros(1, device="cuda", dtype=torch.float64)
+        monkeypatch.setenv("SAF_FIT_DIRECT", "1")
         ctx = saf.Context(0)
         for _ in range(4):
             a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
@@ -337,15 +352,18 @@ def test_fit_transform_lengths(Hf, T, steps):
     assert abs(loss[0] - fo.fit_objective(wa, wr, ea[0], er[0])) < 1e-9 * max(1.0, abs(loss[0]))
 
 
-# Steps of 3 and 10 nats take heads out of the transforms' bounds after a few steps, so that both parities of the step at which
-# they are handed on occur; what was done before must not be lost: the parameters after few steps against the oracle (the direct
-# sums' bounds above), the normalisers at the returned parameters always.
+# Steps of 10 nats take heads out of the transforms' bounds behind the first one (steps of 3 nats do not here); what was done before
+# must not be lost: the parameters after few steps against the oracle (the direct sums' bounds above), the normalisers at the
+# returned parameters always.
 @pytest.mark.parametrize("T,lr,steps", [(200, 3.0, 6), (300, 10.0, 3), (300, 10.0, 4), (300, 10.0, 7), (700, 10.0, 5), (1500, 10.0, 6),
                                         (2500, 10.0, 5), (2500, 10.0, 6)])
 def test_fit_heads_handed_on(T, lr, steps):
     A = si.mean_attention_maps(2, T, 70 + T)
     P, ea, er, pl = _oracle_stats(A)
-    a, r, z, loss, kl = _gpu_fit(_ctx(), _dev(ea), _dev(er), _dev(pl), steps, lr=lr)
+    ctx = _ctx()
+    a, r, z, loss, kl = _gpu_fit(ctx, _dev(ea), _dev(er), _dev(pl), steps, lr=lr)
+    at = ctx.saf_fit_handover(2)
+    assert (at == (2 if lr == 10.0 else -1)).all(), at
     for h in range(2):
         want_z, _ = fo._logZ_and_P(a[h], r[h])
         assert np.max(np.abs(z[h] - want_z)) < 5e-4
@@ -387,6 +405,44 @@ def test_fit_math_ends():
         assert torch.isnan(y).all(), which
     with pytest.raises(saf.SafError):
         saf.saf_fit_math(0, 3, y, y)
+
+
+# A tiny eta_rel(0) puts the first normaliser, Z(0) = A(0) R(0), and then the last key's marginal ever further below the norms of
+# their factors: heads leave the transforms' bounds at the step named, by a normaliser (Z, in the middle of a step) or a marginal (M,
+# at its end).  The steps are those of a double-precision model of the bounds, with a factor of 1.2 to spare at least.  Lengths
+# for the direct kernel of 16 warps, of 12 (beyond 8192) and with unpadded vectors (beyond 12288).
+@pytest.mark.parametrize("T,log_r0,at,steps", [(300, -8.5, 1, 4), (300, -7.6, 1, 4), (300, -7.15, 2, 4), (300, -6.8, 2, 4), (300, -6.1, 3, 4),
+                                               (300, -5.3, 4, 5), (300, -4.4, 5, 5),
+                                               (1000, -8.5, 1, 4), (1000, -7.4, 1, 4), (1000, -6.95, 2, 4), (1000, -6.2, 2, 4),
+                                               (1000, -5.2, 3, 4), (2500, -8.5, 1, 3), (2500, -6.8, 2, 3), (2500, -6.0, 2, 2),
+                                               (5000, -7.2, 1, 2), (5000, -6.0, 2, 2), (9000, -8.5, 1, 2), (9000, -6.2, 2, 2),
+                                               (9000, -5.6, 2, 2), (12500, -7.0, 1, 2), (12500, -6.2, 2, 2), (12500, -5.6, 2, 2)])
+def test_fit_goes_on_where_it_was_handed_on(T, log_r0, at, steps):
+    lr, rng, d = 1.5, np.random.default_rng(1 + T), np.arange(T)
+    ea = np.exp(0.5 * rng.standard_normal(T))
+    er = (T - d) * (1.0 + d) ** -1.3 * np.exp(0.3 * rng.standard_normal(T))
+    ea, er = ea * T / ea.sum(), er * T / er.sum()
+    er[0], ea[0] = T * 10.0 ** log_r0, 0.5
+    ctx = _ctx()
+    a, r, z, loss, kl = _gpu_fit(ctx, _dev(ea[None]), _dev(er[None]), _dev(np.zeros(1)), steps, lr=lr)
+    assert ctx.saf_fit_handover(1)[0] == at
+    # An element moves by lr m / (sqrt(v) + 1e-8); an error of 2e-6 of its marginal in the gradients (direct sums of positive
+    # fp32 terms) moves it by lr 2e-6 / |g / marginal| a step.  Elements whose gradient is below 1e-3 of the marginal at some step: excepted.
+    x = np.concatenate(fo.fit_init(er))
+    m, v, ratio = np.zeros(2 * T), np.zeros(2 * T), np.full(2 * T, np.inf)
+    for t in range(1, steps + 1):
+        g = np.concatenate(fo.fit_gradient(x[:T], x[T:], ea, er))
+        target = np.concatenate([ea, er]) / T
+        ratio = np.minimum(ratio, np.abs(g) / np.maximum(target, g + target))
+        m, v = 0.9 * m + 0.1 * g, 0.999 * v + 0.001 * g * g
+        x = x - lr * (m / (1 - 0.9 ** t)) / (np.sqrt(v / (1 - 0.999 ** t)) + 1e-8)
+    clear = ratio > 1e-3
+    assert clear.mean() > 0.97
+    err = np.abs(np.concatenate([a[0], r[0]]) - x)[clear]
+    assert err.max() <= steps * lr * 2e-3, (err.max(), np.sort(err)[-5:])
+    want_z, _ = fo._logZ_and_P(a[0], r[0])
+    assert np.max(np.abs(z[0] - want_z)) < 1e-4
+    assert abs(loss[0] - fo.fit_objective(a[0], r[0], ea, er)) < 1e-4
 
 
 @pytest.mark.parametrize("T", [100, 300, 2500])
