@@ -201,8 +201,8 @@ int saf_fit_compact(saf_ctx* ctx, int32_t Hf, int32_t T, const double* eta_abs, 
 
 /* Where the heads of the context's last saf_fit_compact (of as many heads) ran: steps_out (host int32 [Hf]) is -1 for a head
  * whose steps were all taken with fp64 transforms, k >= 1 for one that left their bounds and whose steps from the k-th on were
- * taken with the direct sums, 0 where the direct sums took all (T <= 128, or SAF_FIT_DIRECT=1 when the context was
- * created).  Waits for the context's last stream. */
+ * taken with the direct sums, 0 where the direct sums took all (T <= 128, SAF_FIT_DIRECT=1 when the context was created, or no
+ * room on the device for the transforms' state).  Waits for the context's last stream. */
 int saf_fit_handover(saf_ctx* ctx, int32_t Hf, int32_t* steps_out);
 
 /* The fp64 functions that saf_fit_compact uses in place of the library's, for tests: y[i] = 1 / x[i] (`which` 0), sqrt(x[i]) (1)

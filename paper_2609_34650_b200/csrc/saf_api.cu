@@ -1334,9 +1334,16 @@ int saf_fit_compact(saf_ctx* ctx, int32_t Hf, int32_t T, const double* eta_abs, 
   if (!g.ok) return SAF_ERR_CUDA;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   ctx->last_stream = st;
-  // state: two copies of 6 fp64 arrays and 3 fp32 arrays of [Hf, T], one int per head
-  const size_t n = static_cast<size_t>(Hf) * T;
-  int rc = ensure(ctx->fit_buf, n * (12 * sizeof(double) + 3 * sizeof(float)) + static_cast<size_t>(Hf) * sizeof(int));
+  // State: 6 fp64 and 2 fp32 arrays of [Hf, T]; for the transform form also a second copy of the fp64 ones, another fp32 array and
+  // one int per head (where the device has no room for these, the direct sums do without)
+  const size_t n = static_cast<size_t>(Hf) * T, direct_bytes = n * (6 * sizeof(double) + 2 * sizeof(float));
+  bool transforms = !ctx->fit_direct && fit_has_transforms(T);
+  int rc = SAF_ERR_NOMEM;
+  if (transforms) {
+    rc = ensure(ctx->fit_buf, direct_bytes + n * (6 * sizeof(double) + sizeof(float)) + static_cast<size_t>(Hf) * sizeof(int));
+    transforms = rc == SAF_OK;
+  }
+  if (rc == SAF_ERR_NOMEM) rc = ensure(ctx->fit_buf, direct_bytes);
   if (rc) return rc;
   FitState s;
   s.T = T;
@@ -1345,11 +1352,11 @@ int saf_fit_compact(saf_ctx* ctx, int32_t Hf, int32_t T, const double* eta_abs, 
   s.eta_rel = eta_rel;
   double* d = static_cast<double*>(ctx->fit_buf.ptr);
   s.alpha = d; s.rho = d + n; s.m_a = d + 2 * n; s.v_a = d + 3 * n; s.m_r = d + 4 * n; s.v_r = d + 5 * n;
-  s.second = 6 * n;
-  float* f = reinterpret_cast<float*>(d + 12 * n);
-  s.a2 = f; s.r2 = f + n;
-  s.wref = f + 2 * n;
-  s.resume = ctx->fit_direct ? nullptr : reinterpret_cast<int*>(f + 3 * n);
+  s.a2 = reinterpret_cast<float*>(d + 6 * n);
+  s.r2 = s.a2 + n;
+  s.second = 7 * n;
+  s.wref = reinterpret_cast<float*>(d + 13 * n);
+  s.resume = transforms ? reinterpret_cast<int*>(s.wref + n) : nullptr;
   ctx->fit_heads = 0;
   ScopedTimer timer(ctx, SAF_KERNEL_FIT, st);
   if (launch_fit(s, Hf, steps, plogp, alpha_out, rho_out, logZ_out, out_stride, loss_out, kl_out, st) != cudaSuccess)

@@ -596,6 +596,10 @@ saf_fit_kernel(FitState s, int steps, const double* __restrict__ plogp, float* _
 // ------------------------------------------------------------------------------------------------ launchers
 int fit_max_T() { return 16384; }
 
+// Up to 128 positions the direct sums are the shorter of two serial chains (us a step of one head, direct / transforms: 64
+// 5.2 / 4.8, 100 5.1 / 5.2, 256 5.9 / 5.1, 1024 9.1 / 7.5, 4096 22.8 / 10.1)
+bool fit_has_transforms(int T) { return T > 128; }
+
 cudaError_t launch_fit_marginals(const float* Abar, float floor_v, double* eta_abs, double* eta_rel, double* plogp,
                                  int Hf, int T, int num_sms, cudaStream_t st) {
   // CTAs per head: one resident wave over all heads, but at least 32 rows each so that the final flush
@@ -683,9 +687,6 @@ cudaError_t launch_fit_clusters(const FitState& s, int Hf, cudaStream_t st, Args
 
 cudaError_t launch_fit(FitState& s, int Hf, int steps, const double* plogp, float* alpha_out, float* rho_out,
                        float* logZ_out, long long out_stride, double* loss_out, double* kl_out, cudaStream_t st) {
-  // Up to 128 positions the direct sums are the shorter of two serial chains (us a step of one head, direct / transforms: 64
-  // 5.2 / 4.8, 100 5.1 / 5.2, 256 5.9 / 5.1, 1024 9.1 / 7.5, 4096 22.8 / 10.1)
-  s.resume = s.T > 128 ? s.resume : nullptr;
   if (s.resume) {
     bool launched = false;
     const cudaError_t e = launch_fit_fft(s, Hf, steps, plogp, alpha_out, rho_out, logZ_out, out_stride, loss_out, kl_out, st, &launched);

@@ -240,12 +240,13 @@ struct FitState {
   int* resume; float* wref;
 };
 int fit_max_T();
+bool fit_has_transforms(int T);
 cudaError_t launch_fit_marginals(const float* Abar, float floor_v, double* eta_abs, double* eta_rel, double* plogp,
                                  int Hf, int T, int num_sms, cudaStream_t st);
 cudaError_t launch_fit_fft(const FitState& s, int Hf, int steps, const double* plogp, float* alpha_out, float* rho_out,
                            float* logZ_out, long long out_stride, double* loss_out, double* kl_out, cudaStream_t st, bool* launched);
 cudaError_t launch_fit_math(int which, int n, const double* x, double* y, cudaStream_t st);
-// s.resume on entry: may use the transform form; on return: whether it does (else nullptr)
+// s.resume: nullptr for the direct sums throughout, also on return where the transform form was not launched
 cudaError_t launch_fit(FitState& s, int Hf, int steps, const double* plogp, float* alpha_out, float* rho_out,
                        float* logZ_out, long long out_stride, double* loss_out, double* kl_out, cudaStream_t st);
 

@@ -445,6 +445,26 @@ def test_fit_goes_on_where_it_was_handed_on(T, log_r0, at, steps):
     assert abs(loss[0] - fo.fit_objective(a[0], r[0], ea, er)) < 1e-4
 
 
+def test_a_fit_for_which_only_the_direct_sums_have_room():
+    """36000 heads of 300 positions: 605 MB of state for the direct sums, 1166 MB with the transforms' second copy."""
+    Hf, T = 36000, 300
+    P, ea, er, pl = _oracle_stats(si.mean_attention_maps(1, T, 3))
+    ea_d, er_d = (_dev(x).expand(Hf, T).contiguous() for x in (ea, er))
+    out = [torch.empty((Hf, T), device="cuda") for _ in range(3)]
+    ctx = _ctx()
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    hold = torch.empty(torch.cuda.mem_get_info()[0] - (850 << 20), device="cuda", dtype=torch.uint8)
+    ctx.saf_fit_compact(Hf, T, ea_d, er_d, None, 2, 0.05, *out, T, None, None)
+    _status(ctx)
+    assert (ctx.saf_fit_handover(Hf) == 0).all()
+    del hold
+    torch.cuda.empty_cache()
+    want = fo.fit_compact(ea[0], er[0], steps=2)
+    for x, w in zip(out, want):
+        assert np.abs(x[0].cpu().numpy() - w).max() < 2e-4 and torch.equal(x, x[:1].expand(Hf, T))
+
+
 @pytest.mark.parametrize("T", [100, 300, 2500])
 @pytest.mark.parametrize("which,value", [(0, float("nan")), (1, float("nan")), (0, float("inf")), (1, float("inf"))])
 def test_a_target_that_is_not_finite_spoils_its_whole_head_and_no_other(T, which, value):
