@@ -353,6 +353,10 @@ long long choose_pair_cap(int B, int H, int T, int D, const uint8_t* mask, int n
   const long long blocks = static_cast<long long>(B) * H * nblk;
   if (blocks <= num_sms) return 0;
   if (blocks > 3LL * num_sms) return forever;
+  // Pairs unless the run promises 5 %, or 7 % among frozen heads (predicted gain; us in pairs / alone as far as it says: 3.9 %
+  // 2x8x3000x96 50.9 / 52.0, 6.0 % 1x12x4096x128 70.7 / 69.3; frozen 3.3 % 2x20x1300x96 33.6 / 36.2, 4.9 % 1x24x2048x128 45.1 / 46.6,
+  // 6.8 % 3x12x1100x96 30.5 / 31.4)
+  const int margin = std::any_of(mask, mask + H, [](uint8_t m) { return m != 0; }) ? 93 : 95;
   std::vector<WorkItem> trial;
   long long work = 0, best = -1, best_cap = forever;
   build_pair_order(B, H, T, D, mask, frozen_pct, forever, trial);
@@ -372,7 +376,7 @@ long long choose_pair_cap(int B, int H, int T, int D, const uint8_t* mask, int n
       free_at.push(t);
       end = std::max(end, t);
     }
-    if (k == 8) end = end * 97 / 100;                 // (pairs unless the gain is clear)
+    if (k == 8) end = end * margin / 100;
     if (best < 0 || end < best) {
       best = end;
       best_cap = cap;
