@@ -30,6 +30,7 @@ struct WorklistEntry {
   WorkItem* items_dev = nullptr;          // WL_QUEUE: in queue order; else grouped by CTA
   int* offsets_dev = nullptr;
   int n_items = 0;
+  bool general = false;                   // the items of frozen heads are ordered as of the general form
   bool split = false;                     // some items are KIND_SPLIT
 };
 
@@ -304,21 +305,30 @@ void build_worklist_host(int B, int H, int T, const uint8_t* mask, int backward,
 // Work queue of the 128-wide forward.  An item is two consecutive query blocks of one (batch, head) unit (the first
 // block of an odd count goes alone), which share every K and V tile, or one block: of an ordinary head split over the
 // kernel's two chains (even and odd key tiles), of a frozen head in one, as in units of up to three blocks (the merge then costs
-// about what the chains save: us split / not 1x32x256x96 10.4 / 9.9, 1x32x333x128 11.8 / 11.4, on shared heads 15.4 / 15.1,
-// 1x16x333x128 13.0 / 13.4; with four blocks 1x16x512x128 15.3 / 16.0).  Single blocks halve the longest items where these would
-// set the time, at the cost of twice the loads and item ends; which blocks go alone is decided by build_pair_order.
+// about what the chains save; us of back-to-back forwards, split / not: 1x32x333x128 10.9 / 11.3, 1x16x333x128 10.3 / 10.6,
+// 1x8x384x128 10.4 / 10.9, with 10 frozen heads 1x32x333x128 15.6 / 14.5, 1x32x200x96 10.2 / 9.2, 1x48x256x128 11.4 / 10.7,
+// 1x16x256x96 9.4 / 9.7).  Single blocks halve the longest items where these would
+// set the time, at the cost of twice the loads and item ends; which blocks go alone is decided by choose_pair_cap.
 // CTAs claim items in this order at run time, so longest-first within groups of
 // units keeps both the tail short and a group's K and V in L2 while its items run.  Group sizes differ by at most one unit (a
 // small last group is a tail of long items: 2x16x8192x96 0.456 ms with groups of 10, 10, 10 and 2 units, 0.373 with two of 16),
 // as many groups as hold 64 MB of K and V each (8x12x4096x128: 32 MB 0.335 ms, 64 MB 0.339, 128 MB 0.346; 1x16x16384x128:
 // 0.778, 0.760, 0.758), K and V counted per query head where heads share them.  An item's fixed cost does not
 // change the order; a frozen tile counts frozen_pct percent of an ordinary one.
+// general: no tables were prepared for the frozen heads, so their items are made by the softmax warps, a tile in the time of an
+// ordinary one (whether a single head of a prepared pattern takes that form is known on the device only).
 // cap: a pair that takes longer (in ns, by pair_item_ns) is dissolved.
-long long pair_item_ns(int tiles, bool pair, bool ordinary) {     // tiles: of the item's later block
-  if (!ordinary) return (pair ? 2 * tiles - 1 : tiles) * 550LL + 2500;
+// (times at head dimension 128; those at 96 are near enough: us in pairs / as chosen by them 1x8x2048x96 32.4 / 23.3, 1x4x8192x96
+// 118.7 / 72.1, 1x12x4096x96 65.4 / 63.7.  The general form, as of prepared tables / with its own times: 1x4x8192x128, one such
+// head, 136 / 106 (all pairs 140), 1x8x4096x128, two, 74.3 / 57.2 (73.5), 1x16x1300x96, four, 28.4 / 22.7 (28.3),
+// 2x16x4096x128, eight, 140.6 / 137.9 (141.5), 2x8x2048x128, all, 31.5 / 31.5 (39.7).)
+enum ItemForm { FORM_ORDINARY, FORM_TABLES, FORM_GENERAL };
+long long pair_item_ns(int tiles, bool pair, ItemForm form) {     // tiles: of the item's later block
+  if (form == FORM_TABLES) return (pair ? 2 * tiles - 1 : tiles) * 550LL + 2500;
+  if (form == FORM_GENERAL) return tiles * (pair ? 2250LL : 1550LL) + 3000;
   return (pair ? tiles * 2100LL : (tiles + 1) / 2 * 2400LL) + 3000;
 }
-void build_pair_order(int B, int H, int T, int D, const uint8_t* mask, int frozen_pct, long long cap, std::vector<WorkItem>& order) {
+void build_pair_order(int B, int H, int T, int D, const uint8_t* mask, bool general, int frozen_pct, long long cap, std::vector<WorkItem>& order) {
   const int nblk = (T + BLK - 1) / BLK;
   const long long units = static_cast<long long>(B) * H;
   const long long n_groups = std::min(units, std::max<long long>(1, (static_cast<long long>(T) * D * 4 * units + (64ll << 20) - 1) / (64ll << 20)));
@@ -330,9 +340,12 @@ void build_pair_order(int B, int H, int T, int D, const uint8_t* mask, int froze
       const int b = static_cast<int>(u / H), h = static_cast<int>(u % H);
       const int kind = mask[h] ? KIND_FROZEN : KIND_ORDINARY;
       for (int q = nblk - 1; q >= 0;) {
-        const bool two = q > 0 && pair_item_ns(q + 1, true, !mask[h]) <= cap, split = !two && q > 0 && nblk > 3 && !mask[h];
-        // (half tiles: a split block takes half the time of a pair of the same length)
-        const long long half = two ? 2 * (2 * q + 1) : split ? q + 1 : 2 * (q + 1);
+        const ItemForm form = !mask[h] ? FORM_ORDINARY : general ? FORM_GENERAL : FORM_TABLES;
+        const bool two = q > 0 && pair_item_ns(q + 1, true, form) <= cap, split = !two && q > 0 && nblk > 3 && !mask[h];
+        // (in half tiles, as pairs take them; a single block of the general form takes three quarters of a pair's time, a split one half.
+        // Split ones count a quarter all the same, so that pairs start first: us at a quarter / at a half 1x12x3500x128, three frozen,
+        // 52.0 / 55.4, 2x16x1300x96 29.5 / 30.6, 1x12x4096x128 68.8 / 65.6, 1x16x3000x128, four frozen, 53.9 / 52.2)
+        const long long half = two ? 2 * (2 * q + 1) : split ? q + 1 : (form == FORM_GENERAL ? 3 : 2) * (q + 1);
         items.push_back({(mask[h] ? frozen_pct : 100) * half, WorkItem{b, h, q, kind | (two ? KIND_PAIR : split ? KIND_SPLIT : 0)}});
         q -= two ? 2 : 1;
       }
@@ -347,7 +360,7 @@ void build_pair_order(int B, int H, int T, int D, const uint8_t* mask, int froze
 // 247 us in pairs, 268 alone).  us of back-to-back forwards without frozen heads, pairs (blocks alone and in one chain up to
 // one per SM) / this: 1x8x1024x128 20.0 / 16.1, 1x8x2048x128 34.5 / 25.6, 1x16x1300x128 29.4 / 21.2,
 // 1x8x4096x128 70.7 / 43.6, 1x4x8192x128 132 / 76, 1x12x4096x128 72.7 / 68.3, 4x12x900x128 28.2 / 28.2.
-long long choose_pair_cap(int B, int H, int T, int D, const uint8_t* mask, int num_sms, int frozen_pct) {
+long long choose_pair_cap(int B, int H, int T, int D, const uint8_t* mask, bool general, int num_sms, int frozen_pct) {
   const int nblk = (T + BLK - 1) / BLK;
   const long long forever = 1LL << 60;
   const long long blocks = static_cast<long long>(B) * H * nblk;
@@ -359,14 +372,14 @@ long long choose_pair_cap(int B, int H, int T, int D, const uint8_t* mask, int n
   const int margin = std::any_of(mask, mask + H, [](uint8_t m) { return m != 0; }) ? 93 : 95;
   std::vector<WorkItem> trial;
   long long work = 0, best = -1, best_cap = forever;
-  build_pair_order(B, H, T, D, mask, frozen_pct, forever, trial);
-  auto ns = [](const WorkItem& w) {
-    return pair_item_ns(w.blk + 1, (w.kind & KIND_PAIR) != 0, (w.kind & 0x7f) == KIND_ORDINARY);
+  build_pair_order(B, H, T, D, mask, general, frozen_pct, forever, trial);
+  auto ns = [&](const WorkItem& w) {
+    return pair_item_ns(w.blk + 1, (w.kind & KIND_PAIR) != 0, !mask[w.h] ? FORM_ORDINARY : general ? FORM_GENERAL : FORM_TABLES);
   };
   for (const WorkItem& w : trial) work += ns(w);
   for (int k = 8; k >= 0; --k) {                      // caps in quarters of the mean load, from none to twice; first: all pairs
     const long long cap = k == 8 ? forever : work / num_sms * k / 4;
-    build_pair_order(B, H, T, D, mask, frozen_pct, cap, trial);
+    build_pair_order(B, H, T, D, mask, general, frozen_pct, cap, trial);
     std::priority_queue<long long, std::vector<long long>, std::greater<long long>> free_at;
     for (int c = 0; c < num_sms; ++c) free_at.push(0);
     long long end = 0;
@@ -413,12 +426,13 @@ void sched_defaults(int wide, int backward, int* frozen_pct, int* overhead_pct, 
   }
 }
 
-// plan_batch: the batch size that the forms of the 128-wide forward's items are chosen for (saf_ctx::plan_batch)
-int get_worklist(saf_ctx* ctx, int B, int H, int T, int D, const uint8_t* mask, int kind, int grid, int plan_batch, cudaStream_t st,
-                 const WorklistEntry** out) {
+// plan_batch: the batch size that the forms of the 128-wide forward's items are chosen for (saf_ctx::plan_batch); general: see
+// build_pair_order
+int get_worklist(saf_ctx* ctx, int B, int H, int T, int D, const uint8_t* mask, int kind, int grid, int plan_batch, bool general,
+                 cudaStream_t st, const WorklistEntry** out) {
   for (const WorklistEntry& e : ctx->worklists)
     if (e.B == B && e.H == H && e.T == T && e.D == D && e.kind == kind && e.grid == grid && e.plan_batch == plan_batch &&
-        std::memcmp(e.mask.data(), mask, H) == 0) {
+        e.general == general && std::memcmp(e.mask.data(), mask, H) == 0) {
       *out = &e;
       return SAF_OK;
     }
@@ -438,7 +452,9 @@ int get_worklist(saf_ctx* ctx, int B, int H, int T, int D, const uint8_t* mask, 
   const bool lists = kind != WL_QUEUE;
   WorklistEntry e;
   if (!lists && wide) {
-    build_pair_order(B, H, T, D, mask, frozen_pct, choose_pair_cap(plan_batch, H, T, D, mask, ctx->num_sms, frozen_pct), e.items_host);
+    if (general && fw <= 0) frozen_pct = 100;
+    const long long cap = choose_pair_cap(plan_batch, H, T, D, mask, general, ctx->num_sms, frozen_pct);
+    build_pair_order(B, H, T, D, mask, general, frozen_pct, cap, e.items_host);
   } else {
     // (tail: two items per CTA; on the 128-wide backward four: -0.5 % on 8x12x4096x128, -1 % on 2x16x8192x96, -3 % on
     // 1x16x8192x128 and on shared heads 3x8x3000x128; six and eight are no better)
@@ -446,7 +462,7 @@ int get_worklist(saf_ctx* ctx, int B, int H, int T, int D, const uint8_t* mask, 
                         wide && backward ? 4 : 2, lists ? &e.items_host : nullptr, &e.offsets_host,
                         lists ? nullptr : &e.items_host);
   }
-  e.B = B; e.H = H; e.T = T; e.D = D; e.kind = kind; e.grid = grid; e.plan_batch = plan_batch;
+  e.B = B; e.H = H; e.T = T; e.D = D; e.kind = kind; e.grid = grid; e.plan_batch = plan_batch; e.general = general;
   e.mask.assign(mask, mask + H);
   e.n_items = static_cast<int>(e.items_host.size());
   for (const WorkItem& w : e.items_host) e.split |= (w.kind & KIND_SPLIT) != 0;
@@ -737,7 +753,9 @@ int saf_hybrid_attn_fwd(saf_ctx* ctx, const saf_problem* p, const void* Q, const
   // (head dimension 64 and the short 128-wide kernel: two CTAs per SM; the other 128-wide kernel: one)
   const int grid = static_cast<int>(std::min<long long>((p->D == 64 || is_short ? 2LL : 1LL) * ctx->num_sms, n_items));
   const WorklistEntry* wl = nullptr;
-  rc = get_worklist(ctx, p->B, p->H, p->T, p->D, frozen_mask_host, is_short ? WL_SHORT : WL_QUEUE, grid, plan_batch, st, &wl);
+  const bool tables = nf > 0 && pattern_matches(ctx, p, frozen_mask_host, alpha, rho, logZ);
+  const bool general = nf > 0 && !tables && p->D != 64 && !is_short;
+  rc = get_worklist(ctx, p->B, p->H, p->T, p->D, frozen_mask_host, is_short ? WL_SHORT : WL_QUEUE, grid, plan_batch, general, st, &wl);
   if (rc) return rc;
 
   CUtensorMap mq, mk, mv;
@@ -757,7 +775,7 @@ int saf_hybrid_attn_fwd(saf_ctx* ctx, const saf_problem* p, const void* Q, const
   FwdParams fp;
   CUtensorMap mvt = mv;
   fp.band_f = nullptr; fp.wvec = nullptr; fp.fast_ok = nullptr; fp.hord = nullptr; fp.ovf = nullptr; fp.call_id = 0; fp.nblkp = (p->Tp + 127) / 128;
-  if (nf > 0 && pattern_matches(ctx, p, frozen_mask_host, alpha, rho, logZ)) {
+  if (tables) {
     // tensor-core form: V of the frozen heads scaled by a(j) once per call
     const size_t vtb = static_cast<size_t>(p->B) * nf * p->T * p->D * 2;
     rc = ensure(ctx->vt_buf, vtb);
@@ -907,7 +925,7 @@ int saf_hybrid_attn_bwd(saf_ctx* ctx, const saf_problem* p, const void* Q, const
   const long long n_items = static_cast<long long>(p->B) * p->H * nblk;
   const int grid = static_cast<int>(std::min<long long>(ctx->num_sms, n_items));
   const WorklistEntry* wl = nullptr;
-  rc = get_worklist(ctx, p->B, p->H, p->T, p->D, frozen_mask_host, WL_BACKWARD, grid, p->B, st, &wl);
+  rc = get_worklist(ctx, p->B, p->H, p->T, p->D, frozen_mask_host, WL_BACKWARD, grid, p->B, false, st, &wl);
   if (rc) return rc;
 
   auto finalize = [&]() -> int {
