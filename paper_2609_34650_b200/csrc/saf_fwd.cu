@@ -183,9 +183,11 @@ saf_fwd_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ C
   const uint32_t tmem = *tmem_slot;
   // the prologue above overlapped the previous kernel's tail; global memory is touched only from here on
   // On a grid that fills much of the chip the next kernel is let in only once the one in front has ended: let in before, a queue of
-  // passes runs two kernels deep and its waiting CTAs hold back the one in front (1x32x333x128 on shared heads, 96 CTAs: 15.5 us
-  // a pass, 14.5 so; updates on few CTAs want it at once: 1x4x139x96 27.8 us, 28.6 so).
-  const bool at_once = gridDim.x <= 64;
+  // passes runs two kernels deep and its waiting CTAs hold back the one in front; updates on few CTAs want it at once.  us at once /
+  // behind the wait, forwards of 1xHxTx128: 32 CTAs 11.4 / 11.1, 40 11.6 / 11.2, 48 11.8 / 11.7, 56 13.1 / 12.2, 64 12.4 / 11.7, 96 17.0 /
+  // 16.1, on shared heads 15.5 / 14.4; updates: 24 33.0 / 34.3, 32 33.2 / 34.5, 36 59.8 / 60.8, 48 35.2 / 35.9, 56 36.6 / 36.6, 72 to
+  // 128 the same (52.5 / 52.3, 50.8 / 50.8).
+  const bool at_once = gridDim.x <= 48;
   if (at_once) pdl_launch_dependents();
   pdl_wait();
   if (!at_once) pdl_launch_dependents();
