@@ -9,7 +9,7 @@ import saf_inputs as si
 from oracle import saf_oracle as orc
 
 from gpu_util import Layer
-from test_gpu_parity import all_units, check_units, sampled_units
+from test_gpu_parity import _check_gqa_layer, _check_packed_layer, all_units, check_units, sampled_units
 
 pytestmark = pytest.mark.gpu
 
@@ -185,15 +185,23 @@ def test_calibration_mean_pass(T):
         assert np.abs(var.cpu().numpy() - ref).max() <= 1e-6 * np.abs(ref).max()
 
 
-# Query blocks whose even and odd key tiles run in two chains: two tiles, odd and even counts, ragged ends, a row whose second chain
-# sees the diagonal tile only; 12 units of 13 blocks and 32 of 9 mix them with pairs.  fp32 output.
-@pytest.mark.parametrize("B,H,T,D,frozen,o_f32", [
-    (1, 4, 256, 128, (), False), (1, 3, 257, 96, (1,), True), (1, 4, 385, 128, (0,), False), (2, 4, 1025, 128, (3,), True),
-    (1, 12, 1664, 128, (3, 7), False), (2, 16, 1152, 96, (0, 5), False)])
-def test_split_blocks_of_the_wide_forward(B, H, T, D, frozen, o_f32):
-    inp = si.generate(si.Workload("split", B, H, T, D, frozen, -0.05, seed=T + D))
-    units = all_units(inp.wl)
-    check_units(Layer(inp, o_f32=o_f32).run(), units if len(units) <= 12 else sampled_units(inp.wl, 12, seed=5))
+# Query blocks whose even and odd key tiles run in two chains (units of at least four blocks; two and three beside them): odd and
+# even counts, ragged ends, a row whose second chain sees the diagonal tile only; 12 units of 13 blocks and 32 of 9 mix them with
+# pairs.  Shared K/V heads, packed Q/K, fp32 output.
+@pytest.mark.parametrize("B,H,T,D,frozen,o_f32,g,packed", [
+    (1, 4, 256, 128, (), False, 1, False), (1, 3, 257, 96, (1,), True, 1, False), (1, 4, 385, 128, (0,), False, 1, False),
+    (1, 4, 512, 128, (), False, 1, False), (1, 3, 513, 96, (1,), True, 1, False), (2, 4, 1025, 128, (3,), True, 1, False),
+    (1, 8, 700, 128, (2,), False, 4, False), (2, 5, 640, 128, (0, 3), False, 1, True), (1, 4, 900, 96, (1,), False, 2, False),
+    (1, 12, 1664, 128, (3, 7), False, 1, False), (2, 16, 1152, 96, (0, 5), False, 1, False)])
+def test_split_blocks_of_the_wide_forward(B, H, T, D, frozen, o_f32, g, packed):
+    inp = si.generate(si.Workload("split", B, H, T, D, frozen, -0.05, seed=T + D, kv_group=g, packed_qk=packed))
+    L, units = Layer(inp, o_f32=o_f32).run(), all_units(inp.wl)
+    if g > 1:
+        _check_gqa_layer(L, True)
+    elif packed:
+        _check_packed_layer(L, True)
+    else:
+        check_units(L, units if len(units) <= 12 else sampled_units(inp.wl, 12, seed=5))
 
 
 @pytest.mark.parametrize("B,H,T", [(1, 8, 640), (8, 12, 640)])

@@ -1,4 +1,8 @@
-"""GPU tests of how the layer's kernels follow one another on a stream."""
+"""GPU tests of how the library's kernels follow one another on a stream."""
+import os
+import subprocess
+import sys
+
 import pytest
 import torch
 
@@ -43,3 +47,94 @@ def test_forwards_back_to_back_take_no_longer_than_apart(B, H, T, frozen):
     c.saf_set_profiling(0)
     together = _per_call_us(call)
     assert together <= 1.05 * apart, (together, apart)
+
+
+# Passes over two sets of inputs in turn through one context, every pass with outputs of its own and nothing in between, so that a
+# kernel that ran ahead of the one before would meet the other set's intermediate results.
+_PASSES = r"""
+import sys
+sys.path[:0] = sys.argv[1:3]
+import numpy as np, torch
+import paper_2609_34650_b200 as saf
+
+def normal(gen, *shape):
+    return torch.randn(shape, generator=gen, device="cuda", dtype=torch.bfloat16)
+
+def layer(B, H, T, D, frozen, g=1, grads=torch.bfloat16, trainable=False, n=8):
+    mask = np.zeros(H, np.uint8)
+    mask[list(frozen)] = 1
+    ctx, sets, out = saf.Context(0), [], []
+    for seed in range(2):
+        gen = torch.Generator(device="cuda").manual_seed(seed)
+        x = [normal(gen, B, h, T, D) for h in (H, H // g, H // g, H)]
+        rho = -0.02 * torch.arange(T, device="cuda") + 0.1 * torch.randn((H, T), generator=gen, device="cuda")
+        sets.append((*x, torch.randn((H, T), generator=gen, device="cuda"), rho.contiguous(), torch.zeros((H, T), device="cuda")))
+    for _ in range(n):
+        q, k, v, do = sets[0][:4]
+        out.append([torch.zeros_like(do), torch.zeros((B, H, T), device="cuda"), *(torch.zeros(t.shape, device="cuda", dtype=grads) for t in (q, k, v)),
+                    *(torch.zeros((H, T), device="cuda") for _ in range(2))])
+    prob = saf.make_problem(q, T, k_like=k, v_like=v, o_like=do, kv_group=g, H=H, grad_dtype=saf.SAF_F32 if grads == torch.float32 else saf.SAF_BF16)
+    if not trainable:
+        ctx.saf_pattern_prepare(mask, *sets[0][4:])
+    torch.cuda.synchronize()
+    for i, (o, lse, dq, dk, dv, da, dr) in enumerate(out):
+        q, k, v, do, *pattern = sets[i & 1]
+        if trainable:
+            ctx.saf_pattern_prepare(mask, *pattern)
+        else:
+            pattern = sets[0][4:]
+        ctx.saf_hybrid_attn_fwd(prob, q, k, v, mask, *pattern, o, lse)
+        ctx.saf_hybrid_attn_bwd(prob, q, k, v, o, do, lse, mask, *pattern, dq, dk, dv)
+        if trainable:
+            ctx.saf_pattern_grad(prob, v, o, do, mask, *pattern, da, dr)
+    torch.cuda.synchronize()
+    assert ctx.saf_last_device_status()[0] == saf.SAF_OK
+    return out
+
+def calibrate(B, H, T, D, n=3):
+    ctx, mask, out = saf.Context(0), np.zeros(H, np.uint8), []
+    sets = []
+    for seed in range(2):
+        gen = torch.Generator(device="cuda").manual_seed(seed)
+        sets.append([normal(gen, B, H, T, D) for _ in range(3)])
+    for _ in range(n):
+        out.append([torch.zeros((H, T, T), device="cuda"), *(torch.zeros(H, device="cuda", dtype=torch.float64) for _ in range(4)),
+                    torch.zeros((B, H, T), device="cuda"), torch.zeros((B, H, T), device="cuda")])
+    o = torch.zeros_like(sets[0][0])
+    prob = saf.make_problem(o, T, H=H)
+    torch.cuda.synchronize()
+    for i, (mean, sq, pl, var, kl, *lse) in enumerate(out):
+        for j in range(2):
+            q, k, v = sets[(i + j) & 1]
+            ctx.saf_hybrid_attn_fwd(prob, q, k, v, mask, None, None, None, o, lse[j])
+            ctx.saf_calib_accumulate(prob, q, k, lse[j], mean, sq, pl, j)
+        ctx.saf_calib_finalize(H, T, 2 * B, mean, sq, pl, var, kl)
+    torch.cuda.synchronize()
+    assert ctx.saf_last_device_status()[0] == saf.SAF_OK
+    return out
+
+res = [layer(2, 4, 300, 64, (1,)), layer(1, 4, 1100, 64, (0, 2)), layer(2, 4, 333, 96, (1,)), layer(1, 8, 700, 128, (3,), g=4),
+       layer(2, 4, 415, 128, (0, 1), grads=torch.float32, trainable=True), layer(3, 6, 627, 64, (0, 2, 5), trainable=True),
+       layer(2, 4, 1500, 64, (1, 2), trainable=True), calibrate(2, 3, 300, 64), calibrate(2, 4, 261, 128)]
+torch.save([[[t.cpu() for t in p] for p in r] for r in res], sys.argv[3])
+"""
+
+
+def test_results_do_not_depend_on_early_launches(tmp_path):
+    """Calibration, trainable updates and updates with bf16 gradients, with every kernel launched early where the library does
+    so and with none.  Sums by atomics (dQ, shared heads' gradients, pattern gradients, scores) agree to their order of
+    additions; for bf16 results a rounding may then fall the other way here and there."""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    res = []
+    for off in ("0", "1"):
+        path = str(tmp_path / f"res{off}.pt")
+        r = subprocess.run([sys.executable, "-c", _PASSES, root, os.path.join(root, "tests"), path], env=dict(os.environ, SAF_DISABLE_PDL=off),
+                           stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True, timeout=300)
+        assert r.returncode == 0, r.stdout[-2000:]
+        res.append(torch.load(path))
+    tol = {torch.bfloat16: 1e-3, torch.float32: 1e-5, torch.float64: 1e-6}
+    for w, (early, plain) in enumerate(zip(*res)):
+        for i, (a, b) in enumerate(zip(early, plain)):
+            for k, (x, y) in enumerate(zip(a, b)):
+                d, n = (x.double() - y.double()).norm().item(), y.double().norm().item()
+                assert d <= tol[x.dtype] * n, (w, i, k, d, n)
