@@ -430,12 +430,18 @@ void sched_defaults(int wide, int backward, int* frozen_pct, int* overhead_pct, 
 // build_pair_order
 int get_worklist(saf_ctx* ctx, int B, int H, int T, int D, const uint8_t* mask, int kind, int grid, int plan_batch, bool general,
                  cudaStream_t st, const WorklistEntry** out) {
-  for (const WorklistEntry& e : ctx->worklists)
-    if (e.B == B && e.H == H && e.T == T && e.D == D && e.kind == kind && e.grid == grid && e.plan_batch == plan_batch &&
-        e.general == general && std::memcmp(e.mask.data(), mask, H) == 0) {
-      *out = &e;
-      return SAF_OK;
-    }
+  auto find = [&](bool form) -> const WorklistEntry* {
+    for (const WorklistEntry& e : ctx->worklists)
+      if (e.B == B && e.H == H && e.T == T && e.D == D && e.kind == kind && e.grid == grid && e.plan_batch == plan_batch &&
+          e.general == form && std::memcmp(e.mask.data(), mask, H) == 0)
+        return &e;
+    return nullptr;
+  };
+  if ((*out = find(general)) != nullptr) return SAF_OK;
+  // (a capture cannot allocate: there the list of the other form, if that was warmed up, serves as well)
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &capture) != cudaSuccess) cudaGetLastError();
+  if (capture != cudaStreamCaptureStatusNone && (*out = find(!general)) != nullptr) return SAF_OK;
   if (ctx->worklists.size() >= 32) {   // bounded cache: drop the oldest
     cudaStreamSynchronize(st);
     cudaFree(ctx->worklists.front().items_dev);

@@ -86,6 +86,45 @@ def test_patterns_without_prepared_tables_in_paired_items(B, H, T, D):
     check_units(L, [(0, 0), (0, 1), (1, 2), (B - 1, 3), (B - 1, H - 1)], backward=False)
 
 
+@pytest.mark.parametrize("D,T", [(128, 1500), (96, 1337)])
+def test_items_of_a_layer_with_and_without_prepared_tables(D, T):
+    """Two of eight heads frozen, 176 and 192 blocks: without tables their items are longer than the ordinary heads' split blocks
+    and come first; with tables the same context orders them anew."""
+    inp = si.generate(si.Workload("forms", 2, 8, T, D, (1, 6), -0.05, seed=61 + D))
+    L = Layer(inp, backward=False)
+    units = [(0, 0), (0, 1), (1, 1), (0, 6), (1, 6), (1, 3), (1, 7)]
+    saf.saf_pattern_logz_static(0, L.mask, L.alpha, L.rho, L.logZ)
+    for prepare in (False, True):
+        for t in (L.O, L.LSE):
+            t.fill_(float("nan"))
+        L.run(backward=False, prepare=prepare)
+        check_units(L, units, backward=False)
+
+
+def test_a_capture_takes_the_items_of_the_form_that_was_warmed_up():
+    """A forward warmed up with prepared tables and recorded without them (another normaliser pointer): recording allocates
+    nothing."""
+    L = Layer(si.generate(si.Workload("capture", 2, 8, 1500, 128, (1, 6), -0.05, seed=67)), backward=False)
+    c, other = L.ctx, torch.zeros_like(L.logZ)
+    saf.saf_pattern_logz_static(0, L.mask, L.alpha, L.rho, other)
+    call = lambda logZ: c.saf_hybrid_attn_fwd(L.prob, L.Q, L.K, L.V, L.mask, L.alpha, L.rho, logZ, L.O, L.LSE)
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(s):
+        c.saf_pattern_prepare(L.mask, L.alpha, L.rho, L.logZ)
+        call(L.logZ)
+        s.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s):
+            call(other)
+        for t in (L.O, L.LSE):
+            t.fill_(float("nan"))
+        g.replay()
+        s.synchronize()
+    assert c.saf_last_device_status()[0] == saf.SAF_OK
+    check_units(L, [(0, 0), (0, 1), (1, 1), (0, 6), (1, 7)], backward=False)
+
+
 @pytest.mark.parametrize("T", [1, 31, 33, 255, 4096, 4097, 8200])
 @pytest.mark.parametrize("spread", [1.0, 60.0])
 def test_normalisers_at_chunk_edges(T, spread):
