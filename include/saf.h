@@ -183,8 +183,11 @@ int saf_fit_marginals(saf_ctx* ctx, int32_t Hf, int32_t T, const float* mean_att
  * and installation": alpha = 0, rho(d) = log max(eta_rel(d)/(T-d), 1e-9), then `steps` Adam steps (beta1 0.9,
  * beta2 0.999, eps 1e-8, bias-corrected) at learning rate `lr` on
  * L = (1/T)[sum_i log Z(i) - sum_j eta_abs(j) alpha(j) - sum_d eta_rel(d) rho(d)]; the paper uses 400 steps at 0.05).
- * All heads are fitted together; nothing of size T x T is allocated (state: 108 bytes per head and position, held by
- * the context and reused).  Exponentials and the terms of the sums are fp32, Adam and its state fp64.
+ * All heads are fitted together; nothing of size T x T is allocated (state: 108 bytes per head and position, 56 for
+ * T <= 128 and where there is no room for 108, held by the context and reused).  Beyond 128 positions the three sums of a step are fp64 transforms while no normaliser or marginal is
+ * below 2^-28 of the norms of its factors, and else, as up to 128 positions, direct sums of fp32 products (of factors rounded to
+ * fp32 once, in chains of 64; fp64 beyond).  Adam and its state are fp64.  A head with a target that is NaN or infinite has
+ * no finite output after two steps; the others are not affected.
  *   eta_abs, eta_rel : device float64 [Hf, T] (from saf_fit_marginals, or accumulated by the caller)
  *   plogp            : device float64 [Hf] or NULL if kl_out is NULL
  *   alpha_out, rho_out, logZ_out : device float32, row h at offset h*out_stride (out_stride >= T elements): the
@@ -193,8 +196,9 @@ int saf_fit_marginals(saf_ctx* ctx, int32_t Hf, int32_t T, const float* mean_att
  *   kl_out           : device float64 [Hf] or NULL: kappa = mean row KL(P || P^) = L + plogp/T; the paper accepts a
  *                      head when kappa <= 0.2 nats (the caller compares)
  * steps = 0 returns the starting point.  T <= 16384 (SAF_ERR_UNSUPPORTED beyond).  Asynchronous on `stream`
- * (one kernel launch, which keeps its SMs for all steps: 23 ms for 36 heads x 4096 x 400 steps, 0.11 s for 12 heads x
- * 16384; a caller with latency-critical work on the same GPU passes fewer heads or steps at a time). */
+ * (beyond 128 positions two kernel launches, the second for heads handed to the direct sums; each keeps its SMs for all steps:
+ * 5.5 ms for 36 heads x 4096 x 400 steps, 11 ms for 12 heads x 16384; a caller with latency-critical work on the same GPU passes
+ * fewer heads or steps at a time). */
 int saf_fit_compact(saf_ctx* ctx, int32_t Hf, int32_t T, const double* eta_abs, const double* eta_rel,
                     const double* plogp, int32_t steps, double lr, float* alpha_out, float* rho_out, float* logZ_out,
                     int64_t out_stride, double* loss_out, double* kl_out, void* stream);

@@ -10,8 +10,9 @@
 //
 // Nothing of size T x T is formed after the target has been read once.  Beyond 128 positions the Adam steps run in
 // saf_fit_fft.cu, where the three sums of a step are fp64 transforms; the kernel here serves the shortest sequences and goes
-// on with the heads that leave the transforms' bounds.  A thread-block cluster per head runs all Adam steps in one launch, exchanging vectors of length T through distributed shared memory (normalisers)
-// and L2 (parameters), with two cluster barriers per step:
+// on with the heads that leave the transforms' bounds.  A thread-block cluster per head runs all Adam steps in one launch,
+// exchanging vectors of length T through distributed shared memory (normalisers) and L2 (parameters), with two cluster barriers
+// per step:
 //   pass A   rows:      Z(i) = sum_{d<=i} R(d) A(i-d),  W(i) = 1 / Z(i)
 //   pass B   marginals: c(j) = A(j) sum_d R(d) W(j+d)  and  g(d) = R(d) sum_j A(j) W(j+d),
 //            followed in the same thread by the Adam update of alpha(j) / rho(d) (fp64 state)
@@ -285,7 +286,7 @@ struct FitPlan {
 // 58 us per step on 108 SMs, against 100.2 ms for one exponential per pair and sum in two launches per step; 57 % of those
 // SMs' multiply-add peak over everything.  One head of 256 positions: 6.0 us per
 // step (two cluster barriers, L2 round trips of the parameters, fp64 Adam).  Heads of more than 128 positions start in
-// saf_fit_fft_kernel (13.9 us a step of the 36) and come here only from there.
+// saf_fit_fft_kernel (13.6 us a step of the 36) and come here only from there, or where its state or clusters have no room.
 template <int NW, bool PADDED, int RB>
 __global__ void __launch_bounds__(NW * 32, 1)
 saf_fit_kernel(FitState s, int steps, const double* __restrict__ plogp, float* __restrict__ alpha_out,
@@ -596,8 +597,9 @@ saf_fit_kernel(FitState s, int steps, const double* __restrict__ plogp, float* _
 // ------------------------------------------------------------------------------------------------ launchers
 int fit_max_T() { return 16384; }
 
-// Up to 128 positions the direct sums are the shorter of two serial chains (us a step of one head, direct / transforms: 64
-// 5.2 / 4.8, 100 5.1 / 5.2, 256 5.9 / 5.1, 1024 9.1 / 7.5, 4096 22.8 / 10.1)
+// Up to 128 positions the direct sums stay: the two are within 5 % of one another for the head counts of a model (us a step, direct /
+// transforms: one head of 64 5.4 / 5.3, 100 5.1 / 5.3, 128 5.6 / 5.4, 36 of 100 5.2 / 5.3; 150 of 100, more than there are SMs,
+// 10.1 / 5.4), beyond it the transforms are faster (160 5.8 / 5.3, 256 6.2 / 5.4, 1024 9.1 / 7.5, 4096 22.8 / 10.1).
 bool fit_has_transforms(int T) { return T > 128; }
 
 cudaError_t launch_fit_marginals(const float* Abar, float floor_v, double* eta_abs, double* eta_rel, double* plogp,

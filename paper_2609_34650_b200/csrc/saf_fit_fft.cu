@@ -18,13 +18,15 @@
 // that no reordering is needed), the last pass radix 2 or 4 where log2 L is no multiple of three.  After the first pass a
 // sub-transform lies inside a warp.  16-byte pads behind every 8 points keep all passes free of bank conflicts.
 //
-// Bound: latency.  One warp per scheduler works through chains of dependent fp64 operations (the fp64 pipe is 30 % busy for one
-// warp alone), barriers and exchanges.  36 heads of 4096 positions, 400 steps: 13.9 us a step against 59.3 with the
-// direct fp32 sums on 108 SMs; one head: 9.3 against 22.8.  Registers decide much of it: the kernel of eight-CTA clusters
-// spilled 160 bytes a thread and thrashed L1 with them (with less L1 it lost another 12 %); with the owner twiddles in shared
-// memory, the references of the normalisers written out and the peers' addresses computed where they are used, 28 bytes are
-// left (36 x 4096: 6.29 -> 5.91 ms for the whole fit, 1 x 8192: 7.61 -> 6.59, 36 x 8192: 19.6 -> 17.8).  Clusters of up to four
-// keep all of these in registers (with them moved out they measured 1-6 % slower).
+// Bound: latency.  A few warps per scheduler work through chains of dependent fp64 operations (fp64 pipe 13 % busy on the SMs of
+// one head, 24 % with 36), barriers and exchanges.  36 heads of 4096 positions, 400 steps: 13.6 us a step against 59.3 with the
+// direct fp32 sums on 108 SMs; one head: 9.4 against 22.8.  Registers decide much of it: the 512-point kernel of eight-CTA
+// clusters spilled 160 bytes a thread and thrashed L1 with them (with less L1 it lost another 12 %); with the owner twiddles in
+// shared memory, the references of the normalisers written out and the peers' addresses computed where they are used, 24 bytes are
+// left (36 x 4096: 6.29 -> 5.91 ms for the whole fit, 1 x 8192: 7.61 -> 6.59, 36 x 8192: 19.6 -> 17.8).  The larger ones have 128
+// registers a thread and still spill: 68 bytes with 1024 points in clusters of four, 408 and 416 with 1024 and 2048 in
+// clusters of eight (8193 positions and up).  Clusters of up to four keep all of the above in registers (with them moved out they
+// measured 1-6 % slower).
 //
 // Accuracy.  An output's error is up to about 4.5 2^-53 of the 2-norms of its two factors, whatever its own size (measured, T =
 // 4096).  The pattern does not change under alpha(j) -> alpha(j) - k j, rho(d) -> rho(d) - k d, Z(i) -> e^{-k i} Z(i), and
@@ -746,7 +748,9 @@ cudaError_t launch_fit_math(int which, int n, const double* x, double* y, cudaSt
 
 // One transform of 512 points (128 threads, three CTAs per SM) per CTA and as many CTAs as that takes, up to eight: us a step of
 // one head, clusters of 1 / 2 / 4 / 8: 1024 positions 9.2 / 7.5, 2048 14.8 / 11.4 / 8.4, 4096 - / 18.3 / 12.8 / 9.9.  With
-// more heads of 4096 than fit at once (48 clusters of eight), 71 clusters of four do.
+// more heads of 4096 than fit at once (48 clusters of eight), 71 clusters of four do; rounds of them are weighed 18 : 15 (us a step,
+// four / eight: 48 heads 20.0 / 14.8, 49 20.0 / 22.5, 71 20.3 / 27.0, 72 31.6 / 27.1, 142 40.2 / 44.1, 143 49.9 / 44.3, 150
+// 50.5 / 51.3, 240 69.5 / 77.8).  Other lengths have one cluster size each.
 // *launched: false where no such cluster can be resident (then nothing was launched and the direct sums, which run in any
 // cluster size, serve all heads).
 cudaError_t launch_fit_fft(const FitState& s, int Hf, int steps, const double* plogp, float* alpha_out, float* rho_out,
