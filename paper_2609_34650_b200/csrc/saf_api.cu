@@ -1366,6 +1366,7 @@ int saf_fit_compact(saf_ctx* ctx, int32_t Hf, int32_t T, const double* eta_abs, 
   // one int per head (where the device has no room for these, the direct sums do without)
   const size_t n = static_cast<size_t>(Hf) * T, direct_bytes = n * (6 * sizeof(double) + 2 * sizeof(float));
   bool transforms = !ctx->fit_direct && fit_has_transforms(T);
+  ctx->fit_heads = 0;                      // (the steps of the fit before lie in the buffer that is about to change)
   int rc = SAF_ERR_NOMEM;
   if (transforms) {
     rc = ensure(ctx->fit_buf, direct_bytes + n * (6 * sizeof(double) + sizeof(float)) + static_cast<size_t>(Hf) * sizeof(int));
@@ -1385,7 +1386,6 @@ int saf_fit_compact(saf_ctx* ctx, int32_t Hf, int32_t T, const double* eta_abs, 
   s.second = 7 * n;
   s.wref = reinterpret_cast<float*>(d + 13 * n);
   s.resume = transforms ? reinterpret_cast<int*>(s.wref + n) : nullptr;
-  ctx->fit_heads = 0;
   ScopedTimer timer(ctx, SAF_KERNEL_FIT, st);
   if (launch_fit(s, Hf, steps, plogp, alpha_out, rho_out, logZ_out, out_stride, loss_out, kl_out, st) != cudaSuccess)
     return SAF_ERR_CUDA;

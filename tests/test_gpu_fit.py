@@ -465,6 +465,31 @@ def test_a_fit_for_which_only_the_direct_sums_have_room():
         assert np.abs(x[0].cpu().numpy() - w).max() < 2e-4 and torch.equal(x, x[:1].expand(Hf, T))
 
 
+def test_no_handover_steps_of_a_fit_that_failed():
+    """The fit before left its steps in a buffer that the failed call has given back."""
+    T = 300
+    P, ea, er, pl = _oracle_stats(si.mean_attention_maps(1, T, 3))
+    ctx = _ctx()
+    _gpu_fit(ctx, _dev(ea), _dev(er), _dev(pl), 2)
+    assert (ctx.saf_fit_handover(1) == -1).all()
+    Hf = 36000
+    big = [torch.zeros((Hf, T), device="cuda", dtype=torch.float64) for _ in range(2)] + [torch.empty((Hf, T), device="cuda") for _ in range(3)]
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    hold = torch.empty(torch.cuda.mem_get_info()[0] - (300 << 20), device="cuda", dtype=torch.uint8)
+    with pytest.raises(saf.SafError) as e:
+        ctx.saf_fit_compact(Hf, T, big[0], big[1], None, 2, 0.05, *big[2:], T, None, None)
+    assert e.value.code == saf.SAF_ERR_NOMEM
+    for n in (1, Hf):
+        with pytest.raises(saf.SafError) as e:
+            ctx.saf_fit_handover(n)
+        assert e.value.code == saf.SAF_ERR_INVALID_ARG
+    del hold, big
+    torch.cuda.empty_cache()
+    assert np.isfinite(_gpu_fit(ctx, _dev(ea), _dev(er), _dev(pl), 2)[0]).all()
+    assert (ctx.saf_fit_handover(1) == -1).all()
+
+
 @pytest.mark.parametrize("T", [100, 300, 2500])
 @pytest.mark.parametrize("which,value", [(0, float("nan")), (1, float("nan")), (0, float("inf")), (1, float("inf"))])
 def test_a_target_that_is_not_finite_spoils_its_whole_head_and_no_other(T, which, value):
