@@ -126,6 +126,11 @@ int ensure(DevBuf& b, size_t bytes) {
   b.fresh = true;
   return SAF_OK;
 }
+bool capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &s) != cudaSuccess) cudaGetLastError();
+  return s != cudaStreamCaptureStatusNone;
+}
 // Buffers that kernels expect at zero and leave at zero.
 int zero_if_fresh(DevBuf& b, cudaStream_t st) {
   if (!b.fresh) return SAF_OK;
@@ -439,9 +444,7 @@ int get_worklist(saf_ctx* ctx, int B, int H, int T, int D, const uint8_t* mask, 
   };
   if ((*out = find(general)) != nullptr) return SAF_OK;
   // (a capture cannot allocate: there the list of the other form, if that was warmed up, serves as well)
-  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(st, &capture) != cudaSuccess) cudaGetLastError();
-  if (capture != cudaStreamCaptureStatusNone && (*out = find(!general)) != nullptr) return SAF_OK;
+  if (capturing(st) && (*out = find(!general)) != nullptr) return SAF_OK;
   if (ctx->worklists.size() >= 32) {   // bounded cache: drop the oldest
     cudaStreamSynchronize(st);
     cudaFree(ctx->worklists.front().items_dev);
@@ -1363,13 +1366,15 @@ int saf_fit_compact(saf_ctx* ctx, int32_t Hf, int32_t T, const double* eta_abs, 
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   ctx->last_stream = st;
   // State: 6 fp64 and 2 fp32 arrays of [Hf, T]; for the transform form also a second copy of the fp64 ones, another fp32 array and
-  // one int per head (where the device has no room for these, the direct sums do without)
+  // one int per head (where the device has no room for these, the direct sums do without; a capture cannot look for room)
   const size_t n = static_cast<size_t>(Hf) * T, direct_bytes = n * (6 * sizeof(double) + 2 * sizeof(float));
+  const size_t bytes = direct_bytes + n * (6 * sizeof(double) + sizeof(float)) + static_cast<size_t>(Hf) * sizeof(int);
   bool transforms = !ctx->fit_direct && fit_has_transforms(T);
+  if (transforms && ctx->fit_buf.bytes >= direct_bytes && ctx->fit_buf.bytes < bytes && capturing(st)) transforms = false;
   ctx->fit_heads = 0;                      // (the steps of the fit before lie in the buffer that is about to change)
   int rc = SAF_ERR_NOMEM;
   if (transforms) {
-    rc = ensure(ctx->fit_buf, direct_bytes + n * (6 * sizeof(double) + sizeof(float)) + static_cast<size_t>(Hf) * sizeof(int));
+    rc = ensure(ctx->fit_buf, bytes);
     transforms = rc == SAF_OK;
   }
   if (rc == SAF_ERR_NOMEM) rc = ensure(ctx->fit_buf, direct_bytes);

@@ -458,6 +458,14 @@ def test_a_fit_for_which_only_the_direct_sums_have_room():
     ctx.saf_fit_compact(Hf, T, ea_d, er_d, None, 2, 0.05, *out, T, None, None)
     _status(ctx)
     assert (ctx.saf_fit_handover(Hf) == 0).all()
+    s = torch.cuda.Stream()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):                            # (recorded as warmed up)
+        ctx.saf_fit_compact(Hf, T, ea_d, er_d, None, 2, 0.05, *out, T, None, None)
+    for x in out:
+        x.fill_(float("nan"))
+    g.replay()
+    _status(ctx)
     del hold
     torch.cuda.empty_cache()
     want = fo.fit_compact(ea[0], er[0], steps=2)
